@@ -140,63 +140,131 @@ __global__ void k_stats_final(int d, int K, const double* __restrict__ acc,
 
 // ---- network ---------------------------------------------------------------------
 
-__device__ __forceinline__ float ld_op(const float* p) { return *p; }
-__device__ __forceinline__ float ld_op(const __nv_bfloat16* p) { return __bfloat162float(*p); }
+// What the products do with their sums: nothing, add the bias, add it and
+// clip at zero, or keep where the layer's activation was positive (the
+// backward of the clip; `aux` = the activations).
+enum Epi { kPlain, kBias, kBiasRelu, kReluMask };
 
-// C[M x N] = op(A) op(B) (+ bias, relu). op(A)(m, k) = TA ? A[k lda + m] :
-// A[m lda + k]; op(B)(k, n) = TB ? B[n ldb + k] : B[k ldb + n]. 64 x 64
-// tiles, 16-deep K steps through shared memory, 4 x 4 outputs per thread,
-// FP32 accumulation.
-template <bool TA, bool TB, typename BT, int EPI>
-__global__ void __launch_bounds__(256)
+template <int EPI>
+__device__ __forceinline__ float epilogue(float v, const float* aux, int64_t m, int n, int ldc) {
+  if (EPI == kBias || EPI == kBiasRelu) v += aux[n];
+  if (EPI == kBiasRelu) v = fmaxf(v, 0.0f);
+  if (EPI == kReluMask) v = aux[m * ldc + n] > 0.0f ? v : 0.0f;
+  return v;
+}
+
+__device__ __forceinline__ float4 ld4(const float* p) {
+  return __ldg(reinterpret_cast<const float4*>(p));
+}
+__device__ __forceinline__ float4 ld4(const __nv_bfloat16* p) {
+  const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
+  return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
+                     __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
+}
+
+// C[M x N] = op(A) op(B). op(A)(m, k) = TA ? A[k lda + m] : A[m lda + k];
+// op(B)(k, n) = TB ? B[n ldb + k] : B[k ldb + n]; N, the row strides and the
+// untransposed K are multiples of 4. T x T tiles, R x R outputs per thread
+// (rows ty + D i, columns tx + D j), KS-deep K steps through two shared-memory
+// stages (the next step's 16-byte loads in flight while one computes), each
+// operand in shared memory as it lies in memory, so that its 16-byte pieces
+// are stored whole: [row][k] where k is contiguous, else [k][row]. Every
+// output is one FP32 chain over k in increasing order, whatever the tile, so
+// both shapes give the same bits.
+// A batch of 64 has eight 64 x 64 tiles in the first layer (K = 5376), which
+// took 0.7 ms on 8 of 152 SMs; 16 x 16 tiles spread it over 128, where the
+// chain's own latency (5376 dependent FMAs of 4 clocks: 10 us) is the floor.
+template <bool TA, bool TB, typename BT, int EPI, int T, int R, int KS>
+__global__ void __launch_bounds__((T / R) * (T / R))
     k_gemm(int M, int N, int K, const float* __restrict__ A, int lda, const BT* __restrict__ B,
-           int ldb, const float* __restrict__ bias, float* __restrict__ C, int ldc) {
-  __shared__ float As[16][64 + 4], Bs[16][64 + 4];
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += 16) {
-    for (int i = threadIdx.x; i < 64 * 16; i += 256) {
-      int mm, kk;
-      if (TA) { mm = i % 64; kk = i / 64; } else { kk = i % 16; mm = i / 16; }
-      const int m = m0 + mm, k = k0 + kk;
-      As[kk][mm] = (m < M && k < K) ? (TA ? A[(int64_t)k * lda + m] : A[(int64_t)m * lda + k]) : 0.0f;
+           int ldb, const float* __restrict__ aux, float* __restrict__ C, int ldc) {
+  constexpr int D = T / R, NT = D * D, NV = T * KS / 4 / NT;
+  static_assert(T * KS % (4 * NT) == 0 && KS % 4 == 0, "tile");
+  // words of an operand's stage: [k][T + 4] or [T][KS + 4]
+  constexpr int SA = TA ? KS * (T + 4) : T * (KS + 4), SB = TB ? T * (KS + 4) : KS * (T + 4);
+  __shared__ __align__(16) float As[2][SA], Bs[2][SB];
+  const int m0 = blockIdx.y * T, n0 = blockIdx.x * T;
+  const int tx = threadIdx.x % D, ty = threadIdx.x / D;
+  // this thread's 16-byte pieces of a step: 4 along k of one row (kc), or 4
+  // along the rows at one k
+  auto place = [](bool kc, int v, int* row, int* k) {
+    const int id = (int)threadIdx.x + v * NT;
+    *row = kc ? id / (KS / 4) : 4 * (id % (T / 4));
+    *k = kc ? 4 * (id % (KS / 4)) : id / (T / 4);
+  };
+  float4 av[NV], bv[NV];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      int r, k;
+      place(!TA, v, &r, &k);
+      av[v] = make_float4(0, 0, 0, 0);
+      if (k0 + k < K && m0 + r < M)
+        av[v] = TA ? ld4(A + (int64_t)(k0 + k) * lda + m0 + r)
+                   : ld4(A + (int64_t)(m0 + r) * lda + k0 + k);
+      place(TB, v, &r, &k);
+      bv[v] = make_float4(0, 0, 0, 0);
+      if (k0 + k < K && n0 + r < N)
+        bv[v] = TB ? ld4(B + (int64_t)(n0 + r) * ldb + k0 + k)
+                   : ld4(B + (int64_t)(k0 + k) * ldb + n0 + r);
     }
-    for (int i = threadIdx.x; i < 64 * 16; i += 256) {
-      int nn, kk;
-      if (TB) { kk = i % 16; nn = i / 16; } else { nn = i % 64; kk = i / 64; }
-      const int n = n0 + nn, k = k0 + kk;
-      Bs[kk][nn] = (n < N && k < K)
-                       ? (TB ? ld_op(B + (int64_t)n * ldb + k) : ld_op(B + (int64_t)k * ldb + n))
-                       : 0.0f;
+  };
+  auto store = [&](int st) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      int r, k;
+      place(!TA, v, &r, &k);
+      *reinterpret_cast<float4*>(&As[st][TA ? k * (T + 4) + r : r * (KS + 4) + k]) = av[v];
+      place(TB, v, &r, &k);
+      *reinterpret_cast<float4*>(&Bs[st][TB ? r * (KS + 4) + k : k * (T + 4) + r]) = bv[v];
     }
-    __syncthreads();
+  };
+  // four consecutive k of this thread's i-th row (of T, at base t + D i)
+  auto read = [](const float* s, bool kc, int row, int k, float (&v)[4]) {
+    if (kc) {
+      const float4 x = *reinterpret_cast<const float4*>(s + row * (KS + 4) + k);
+      v[0] = x.x;
+      v[1] = x.y;
+      v[2] = x.z;
+      v[3] = x.w;
+    } else {
 #pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      float av[4], bv[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) av[i] = As[kk][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) bv[j] = Bs[kk][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+      for (int c = 0; c < 4; ++c) v[c] = s[(k + c) * (T + 4) + row];
     }
+  };
+  float acc[R][R] = {};
+  fetch(0);
+  store(0);
+  __syncthreads();
+  int st = 0;
+  for (int k0 = 0; k0 < K; k0 += KS, st ^= 1) {
+    const bool more = k0 + KS < K;
+    if (more) fetch(k0 + KS);
+#pragma unroll 4
+    for (int kk = 0; kk < KS; kk += 4) {
+      float xs[R][4], ys[R][4];
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        read(As[st], !TA, ty + D * i, kk, xs[i]);
+        read(Bs[st], TB, tx + D * i, kk, ys[i]);
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+          for (int j = 0; j < R; ++j) acc[i][j] = fmaf(xs[i][c], ys[j][c], acc[i][j]);
+    }
+    if (more) store(st ^ 1);
     __syncthreads();
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty * 4 + i;
-    if (m >= M) continue;
+  for (int i = 0; i < R; ++i) {
+    const int m = m0 + ty + D * i;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx * 4 + j;
-      if (n >= N) continue;
-      float v = acc[i][j];
-      if (EPI >= 1) v += bias[n];
-      if (EPI == 2) v = fmaxf(v, 0.0f);
-      C[(int64_t)m * ldc + n] = v;
+    for (int j = 0; j < R; ++j) {
+      const int n = n0 + tx + D * j;
+      if (m < M && n < N) C[(int64_t)m * ldc + n] = epilogue<EPI>(acc[i][j], aux, m, n, ldc);
     }
   }
 }
@@ -258,31 +326,47 @@ __global__ void k_colsum(const float* __restrict__ X, int rows, int n_cols, floa
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= n_cols) return;
   float s = 0.0f;
+#pragma unroll 16
   for (int r = 0; r < rows; ++r) s += X[(int64_t)r * n_cols + c];
   out[c] = s;
 }
 
-// dH *= (H > 0)
-__global__ void k_relu_bwd(float* dH, const float* __restrict__ H, int64_t n) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n && !(H[i] > 0.0f)) dH[i] = 0.0f;
-}
-
-// One Adam step (Kingma and Ba, 2015); c1 = 1 - b1^t, c2 = 1 - b2^t. wb: the
-// bfloat16 copy the network computes with (null for biases).
-__global__ void k_adam(float* w, float* m, float* v, const float* __restrict__ g,
-                       __nv_bfloat16* wb, int64_t n, float lr, float b1, float b2, float eps,
-                       float c1, float c2) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// One Adam step (Kingma and Ba, 2015) on parameters i .. i + 3 of the packed
+// arrays (W1 | b1 | W2 | b2 | W3 | b3, n in all); c1 = 1 - b1^t, c2 = 1 - b2^t.
+// wb: the packed bfloat16 weights the network computes with (W1 | W2 | W3).
+__global__ void __launch_bounds__(256)
+    k_adam(float* w, float* m, float* v, const float* __restrict__ g, __nv_bfloat16* wb, int64_t n,
+           float lr, float b1, float b2, float eps, float c1, float c2) {
+  const int64_t i = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
   if (i >= n) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.0f - b1) * gi;
-  const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-  w[i] = wi;
-  if (wb) wb[i] = __float2bfloat16_rn(wi);
+  const float4 g4 = *reinterpret_cast<const float4*>(g + i);
+  float4 m4 = *reinterpret_cast<const float4*>(m + i);
+  float4 v4 = *reinterpret_cast<const float4*>(v + i);
+  float4 w4 = *reinterpret_cast<const float4*>(w + i);
+  auto step = [&](float gi, float& mi, float& vi, float& wi) {
+    mi = b1 * mi + (1.0f - b1) * gi;
+    vi = b2 * vi + (1.0f - b2) * gi * gi;
+    wi = wi - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  };
+  step(g4.x, m4.x, v4.x, w4.x);
+  step(g4.y, m4.y, v4.y, w4.y);
+  step(g4.z, m4.z, v4.z, w4.z);
+  step(g4.w, m4.w, v4.w, w4.w);
+  *reinterpret_cast<float4*>(m + i) = m4;
+  *reinterpret_cast<float4*>(v + i) = v4;
+  *reinterpret_cast<float4*>(w + i) = w4;
+  // the layer that holds element i (every boundary is a multiple of 4)
+  constexpr int64_t n1 = (int64_t)kIn * kH, n2 = (int64_t)kH * kH, n3 = (int64_t)kH * kOut;
+  int64_t o = -1;
+  if (i < n1) o = i;
+  else if (i >= n1 + kH && i < n1 + kH + n2) o = i - kH;
+  else if (i >= n1 + n2 + 2 * kH && i < n1 + n2 + n3 + 2 * kH) o = i - 2 * kH;
+  if (o >= 0) {
+    uint2 u;
+    u.x = pack_bf16x2(w4.x, w4.y);
+    u.y = pack_bf16x2(w4.z, w4.w);
+    *reinterpret_cast<uint2*>(wb + o) = u;
+  }
 }
 
 __global__ void k_to_bf16(const float* __restrict__ w, __nv_bfloat16* wb, int64_t n) {
@@ -416,12 +500,17 @@ __global__ void k_gather_rows(const T* __restrict__ src, int64_t cols, const int
 
 __global__ void k_acc_double(double* acc, const double* __restrict__ v) { *acc += *v; }
 
+// 64 x 64 tiles from one CTA per SM of a 152-SM GPU on, 16 x 16 below.
 template <bool TA, bool TB, typename BT, int EPI>
 cudaError_t gemm(int M, int N, int K, const float* A, int lda, const BT* B, int ldb,
-                 const float* bias, float* C, int ldc, cudaStream_t st) {
+                 const float* aux, float* C, int ldc, cudaStream_t st) {
   if (M <= 0 || N <= 0) return cudaSuccess;
-  const dim3 grid((unsigned)((N + 63) / 64), (unsigned)((M + 63) / 64));
-  k_gemm<TA, TB, BT, EPI><<<grid, 256, 0, st>>>(M, N, K, A, lda, B, ldb, bias, C, ldc);
+  auto tiles = [&](int t) { return dim3((unsigned)((N + t - 1) / t), (unsigned)((M + t - 1) / t)); };
+  const dim3 g = tiles(64), s = tiles(16);
+  if ((int64_t)g.x * g.y >= 152 || s.y > 65535)
+    k_gemm<TA, TB, BT, EPI, 64, 4, 16><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, aux, C, ldc);
+  else
+    k_gemm<TA, TB, BT, EPI, 16, 1, 64><<<s, 256, 0, st>>>(M, N, K, A, lda, B, ldb, aux, C, ldc);
   return cudaGetLastError();
 }
 
@@ -457,12 +546,14 @@ cudaError_t launch_node_stats(const Problem& pr, const NodeDesc* nodes, int A,
 cudaError_t launch_mlp_forward(const MlpParams& m, const float* S, int N, MlpWork w,
                                cudaStream_t st) {
   cudaError_t e;
-  if ((e = gemm<false, false, __nv_bfloat16, 2>(N, kH, kIn, S, kIn, m.W1b, kH, m.b1, w.H1, kH, st)))
+  if ((e = gemm<false, false, __nv_bfloat16, kBiasRelu>(N, kH, kIn, S, kIn, m.W1b, kH, m.b1, w.H1,
+                                                       kH, st)))
     return e;
-  if ((e = gemm<false, false, __nv_bfloat16, 2>(N, kH, kH, w.H1, kH, m.W2b, kH, m.b2, w.H2, kH, st)))
+  if ((e = gemm<false, false, __nv_bfloat16, kBiasRelu>(N, kH, kH, w.H1, kH, m.W2b, kH, m.b2, w.H2,
+                                                       kH, st)))
     return e;
-  return gemm<false, false, __nv_bfloat16, 1>(N, kOut, kH, w.H2, kH, m.W3b, kOut, m.b3, w.O,
-                                              kOut, st);
+  return gemm<false, false, __nv_bfloat16, kBias>(N, kOut, kH, w.H2, kH, m.W3b, kOut, m.b3, w.O,
+                                                  kOut, st);
 }
 
 cudaError_t launch_mlp_loss_grad(const MlpParams& m, const float* S, const int32_t* dims,
@@ -473,25 +564,23 @@ cudaError_t launch_mlp_loss_grad(const MlpParams& m, const float* S, const int32
   if ((e = cudaMemsetAsync(loss, 0, sizeof(double), st))) return e;
   k_mlp_loss<<<(unsigned)N, 256, 0, st>>>(w.O, dims, targets, N, w.dO, loss);
   // layer 3: gW3 = H2^T dO, gb3 = colsum dO, dH2 = dO W3^T (x relu')
-  if ((e = gemm<true, false, float, 0>(kH, kOut, N, w.H2, kH, w.dO, kOut, nullptr, g.W3, kOut, st)))
+  if ((e = gemm<true, false, float, kPlain>(kH, kOut, N, w.H2, kH, w.dO, kOut, nullptr, g.W3, kOut, st)))
     return e;
-  k_colsum<<<blocks(kOut), 256, 0, st>>>(w.dO, N, kOut, g.b3);
-  if ((e = gemm<false, true, __nv_bfloat16, 0>(N, kH, kOut, w.dO, kOut, m.W3b, kOut, nullptr,
-                                              w.dH2, kH, st)))
+  k_colsum<<<blocks(kOut, 64), 64, 0, st>>>(w.dO, N, kOut, g.b3);
+  if ((e = gemm<false, true, __nv_bfloat16, kReluMask>(N, kH, kOut, w.dO, kOut, m.W3b, kOut, w.H2,
+                                                      w.dH2, kH, st)))
     return e;
-  k_relu_bwd<<<blocks((int64_t)N * kH), 256, 0, st>>>(w.dH2, w.H2, (int64_t)N * kH);
   // layer 2
-  if ((e = gemm<true, false, float, 0>(kH, kH, N, w.H1, kH, w.dH2, kH, nullptr, g.W2, kH, st)))
+  if ((e = gemm<true, false, float, kPlain>(kH, kH, N, w.H1, kH, w.dH2, kH, nullptr, g.W2, kH, st)))
     return e;
-  k_colsum<<<blocks(kH), 256, 0, st>>>(w.dH2, N, kH, g.b2);
-  if ((e = gemm<false, true, __nv_bfloat16, 0>(N, kH, kH, w.dH2, kH, m.W2b, kH, nullptr, w.dH1,
-                                              kH, st)))
+  k_colsum<<<blocks(kH, 64), 64, 0, st>>>(w.dH2, N, kH, g.b2);
+  if ((e = gemm<false, true, __nv_bfloat16, kReluMask>(N, kH, kH, w.dH2, kH, m.W2b, kH, w.H1, w.dH1,
+                                                      kH, st)))
     return e;
-  k_relu_bwd<<<blocks((int64_t)N * kH), 256, 0, st>>>(w.dH1, w.H1, (int64_t)N * kH);
   // layer 1
-  if ((e = gemm<true, false, float, 0>(kIn, kH, N, S, kIn, w.dH1, kH, nullptr, g.W1, kH, st)))
+  if ((e = gemm<true, false, float, kPlain>(kIn, kH, N, S, kIn, w.dH1, kH, nullptr, g.W1, kH, st)))
     return e;
-  k_colsum<<<blocks(kH), 256, 0, st>>>(w.dH1, N, kH, g.b1);
+  k_colsum<<<blocks(kH, 64), 64, 0, st>>>(w.dH1, N, kH, g.b1);
   return cudaGetLastError();
 }
 
@@ -499,21 +588,10 @@ cudaError_t launch_adam(MlpParams& m, MlpState& s, const MlpGrads& g, int t, flo
                         cudaStream_t st) {
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   const float c1 = (float)(1.0 - pow(0.9, t)), c2 = (float)(1.0 - pow(0.999, t));
-  struct {
-    float* w;
-    float* m;
-    float* v;
-    const float* g;
-    __nv_bfloat16* wb;
-    int64_t n;
-  } parts[6] = {{m.W1, s.mW1, s.vW1, g.W1, m.W1b, (int64_t)kIn * kH},
-                {m.b1, s.mb1, s.vb1, g.b1, nullptr, kH},
-                {m.W2, s.mW2, s.vW2, g.W2, m.W2b, (int64_t)kH * kH},
-                {m.b2, s.mb2, s.vb2, g.b2, nullptr, kH},
-                {m.W3, s.mW3, s.vW3, g.W3, m.W3b, (int64_t)kH * kOut},
-                {m.b3, s.mb3, s.vb3, g.b3, nullptr, kOut}};
-  for (auto& p : parts)
-    k_adam<<<blocks(p.n), 256, 0, st>>>(p.w, p.m, p.v, p.g, p.wb, p.n, lr, b1, b2, eps, c1, c2);
+  // parameters, gradients and moments are packed alike (slm_proposal_create)
+  const int64_t n = (m.b3 + kOut) - m.W1;
+  k_adam<<<blocks(n / 4), 256, 0, st>>>(m.W1, s.mW1, s.vW1, g.W1, m.W1b, n, lr, b1, b2, eps, c1,
+                                        c2);
   return cudaGetLastError();
 }
 

@@ -274,6 +274,16 @@ slm_status stage_in(slm_ctx* c, const T* src, size_t count, DevBuf& buf,
   return SLM_OK;
 }
 
+// A device array the kernels read 16 bytes at a time: as it is when its
+// address allows, else a copy in `buf`.
+slm_status align16(slm_ctx* c, const float** p, size_t count, DevBuf& buf) {
+  if ((reinterpret_cast<uintptr_t>(*p) & 15) == 0) return SLM_OK;
+  CK(ensure(buf, sizeof(float) * count));
+  CK(cudaMemcpyAsync(buf.p, *p, sizeof(float) * count, cudaMemcpyDeviceToDevice, c->stream));
+  *p = static_cast<const float*>(buf.p);
+  return SLM_OK;
+}
+
 int round16(int v) { return (v + 15) / 16 * 16; }
 
 // The tensor-core pass stages all positions of a node in shared memory.
@@ -2956,6 +2966,7 @@ slm_status slm_proposal_forward(slm_ctx* c, const slm_proposal* pp, const float*
   CK(cudaSetDevice(c->device));
   const float* ds;
   if (slm_status s = stage_in(c, stats, (size_t)n * kPropIn, c->ws[W_PS], &ds)) return s;
+  if (slm_status s = align16(c, &ds, (size_t)n * kPropIn, c->ws[W_PS])) return s;
   MlpWork w;
   if (slm_status s = proposal_work(c, n, &w)) return s;
   CK(launch(c, SLM_K_PROPOSAL, 0.0, [&] { return launch_mlp_forward(pp->m, ds, n, w, c->stream); }));
@@ -3023,7 +3034,8 @@ slm_status slm_proposal_train(slm_ctx* c, slm_proposal* pp, const float* stats,
   slm_status s;
   if ((s = stage_in(c, stats, (size_t)n * kPropIn, c->ws[W_PS], &ds)) ||
       (s = stage_in(c, dims, (size_t)n, c->ws[W_PD], &dd)) ||
-      (s = stage_in(c, targets, (size_t)n * kPropD, c->ws[W_PT], &dt)))
+      (s = stage_in(c, targets, (size_t)n * kPropD, c->ws[W_PT], &dt)) ||
+      (s = align16(c, &ds, (size_t)n * kPropIn, c->ws[W_PS])))
     return s;
   const int b = std::min(batch, n);
   MlpWork w;
