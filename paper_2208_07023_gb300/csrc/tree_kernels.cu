@@ -376,32 +376,109 @@ __global__ void k_validate(const int32_t* labels, int64_t n, int K, const int32_
   }
 }
 
-__global__ void k_predict(const float* __restrict__ X, int64_t n, int d, TreeArrays tr,
-                          int n_trees, int H, int B, int K, int crit, int32_t* class_out,
-                          double* value_out, int32_t* leaf_out) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  const float* x = X + s * d;
+// Routes rows through every tree (bin rule of scoring). A CTA takes a tile of
+// rows into shared memory; its warps are RB blocks of 32 rows x WT lanes of
+// trees: a lane walks one row down trees w, w + WT, ... of each chunk of
+// kPredTrees, its leaf ids meeting in shared memory, from which one thread per
+// row counts the votes (or adds the leaf values in tree order). With one
+// thread per row walking every tree from global memory, 100,000 rows x 32
+// through 64 trees of depth 8 took 2.40 ms: too few warps, each waiting on
+// its own row's loads. Features are read 16 bytes at a time (VEC) where d
+// and X's address allow.
+constexpr int kPredTrees = 64;
+constexpr int kPredSmem = 96 * 1024;  // rows kept in shared memory up to this
+
+__host__ __device__ inline int pred_stride(int d, bool vec) { return vec ? d + 4 : d | 1; }
+
+template <bool VEC>
+__global__ void __launch_bounds__(256)
+    k_predict(const float* __restrict__ X, int64_t n, int d, TreeArrays tr, int n_trees, int H,
+              int B, int K, int crit, int32_t* class_out, double* value_out, int32_t* leaf_out,
+              int RB, int WT, int staged) {
+  extern __shared__ __align__(16) float psm[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rb = warp % RB, wt = warp / RB, R = 32 * RB;
+  const int nct = min(n_trees, kPredTrees);
+  int32_t* leaf = reinterpret_cast<int32_t*>(psm);  // [R][nct | 1]
+  const int ls = nct | 1;
+  float* rows = psm + ((R * ls + 3) & ~3);
+  const int stride = pred_stride(d, VEC);
+  const int64_t r0 = (int64_t)blockIdx.x * R;
+  const int nr = (int)min((int64_t)R, n - r0);
+  if (staged) {
+    if (VEC) {
+      const int d4 = d >> 2;
+      for (int q = threadIdx.x; q < nr * d4; q += blockDim.x) {
+        const int r = q / d4, c = q - r * d4;
+        *reinterpret_cast<float4*>(rows + r * stride + 4 * c) =
+            __ldg(reinterpret_cast<const float4*>(X + (r0 + r) * d) + c);
+      }
+    } else {
+      for (int q = threadIdx.x; q < nr * d; q += blockDim.x) {
+        const int r = q / d, c = q - r * d;
+        rows[r * stride + c] = __ldg(X + (r0 + r) * d + c);
+      }
+    }
+    __syncthreads();
+  }
+  const int rl = rb * 32 + lane;  // this lane's row of the tile
+  const bool in = rl < nr;
+  const float* x = staged ? rows + rl * stride : X + (r0 + (in ? rl : 0)) * d;
+  const bool tail = (int)threadIdx.x < nr;  // this thread sums up row threadIdx.x
   int votes[kMaxClasses];
   for (int k = 0; k < kMaxClasses; ++k) votes[k] = 0;
   double vsum = 0.0;
-  for (int t = 0; t < n_trees; ++t) {
-    const int64_t base = (int64_t)t * H;
-    int h = 0;
-    while (h < H && tr.kind[base + h] == 1) {
-      const int64_t slot = base + h;
-      const float* g = tr.dir + slot * d;
-      float acc = 0.0f;
-      for (int j = 0; j < d; ++j) acc = fmaf(__ldg(x + j), __ldg(g + j), acc);
-      const int b = bin_of(acc, tr.zmin[slot], tr.inv_w[slot], B);
-      h = b >= tr.bin[slot] ? 2 * h + 2 : 2 * h + 1;
+  for (int t0 = 0; t0 < n_trees; t0 += kPredTrees) {
+    const int nt = min(kPredTrees, n_trees - t0);
+    if (in)
+      for (int t = wt; t < nt; t += WT) {
+        const int64_t base = (int64_t)(t0 + t) * H;
+        int h = 0;
+        while (h < H && __ldg(tr.kind + base + h) == 1) {
+          const int64_t slot = base + h;
+          const float* g = tr.dir + slot * d;
+          const float zmin = __ldg(tr.zmin + slot), inv_w = __ldg(tr.inv_w + slot);
+          const int eb = __ldg(tr.bin + slot);
+          float acc = 0.0f;
+          if (VEC) {
+#pragma unroll 4
+            for (int j = 0; j < d; j += 4) {
+              const float4 a = *reinterpret_cast<const float4*>(x + j);
+              const float4 b = __ldg(reinterpret_cast<const float4*>(g + j));
+              acc = fmaf(a.x, b.x, acc);
+              acc = fmaf(a.y, b.y, acc);
+              acc = fmaf(a.z, b.z, acc);
+              acc = fmaf(a.w, b.w, acc);
+            }
+          } else {
+#pragma unroll 4
+            for (int j = 0; j < d; ++j) acc = fmaf(x[j], __ldg(g + j), acc);
+          }
+          h = bin_of(acc, zmin, inv_w, B) >= eb ? 2 * h + 2 : 2 * h + 1;
+        }
+        leaf[rl * ls + t] = h;
+      }
+    __syncthreads();
+    if (leaf_out)
+      for (int q = threadIdx.x; q < nr * nt; q += blockDim.x) {
+        const int r = q / nt, t = q - r * nt;
+        leaf_out[(r0 + r) * n_trees + t0 + t] = leaf[r * ls + t];
+      }
+    if (tail) {
+      const int32_t* lf = leaf + threadIdx.x * ls;
+#pragma unroll 4
+      for (int t = 0; t < nt; ++t) {
+        const int64_t slot = (int64_t)(t0 + t) * H + lf[t];
+        if (crit == SLM_MSE)
+          vsum += __ldg(tr.leaf_value + slot);
+        else
+          votes[__ldg(tr.leaf_class + slot)] += 1;
+      }
     }
-    if (leaf_out) leaf_out[s * n_trees + t] = h;
-    if (crit == SLM_MSE)
-      vsum += tr.leaf_value[base + h];
-    else
-      votes[tr.leaf_class[base + h]] += 1;
+    __syncthreads();  // the leaf ids are read
   }
+  if (!tail) return;
+  const int64_t s = r0 + threadIdx.x;
   if (crit == SLM_MSE) {
     if (value_out) value_out[s] = vsum / (double)n_trees;
     if (class_out) class_out[s] = -1;
@@ -543,8 +620,30 @@ cudaError_t launch_predict(const float* X, int64_t n, int d, TreeArrays tr, int 
                            int H, int B, int K, int crit, int32_t* class_out,
                            double* value_out, int32_t* leaf_out, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  k_predict<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(X, n, d, tr, n_trees, H, B, K, crit,
-                                                        class_out, value_out, leaf_out);
+  const bool vec = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+  // as many warps over a tile's trees as there are trees, up to eight; the
+  // rest take more rows, as far as they fit
+  int WT = 1;
+  while (WT < 8 && WT < n_trees) WT *= 2;
+  int RB = 8 / WT;
+  const int ls = (n_trees < kPredTrees ? n_trees : kPredTrees) | 1;
+  auto smem = [&](int rb, bool staged) {
+    return sizeof(float) * ((size_t)((32 * rb * ls + 3) & ~3) +
+                            (staged ? (size_t)32 * rb * pred_stride(d, vec) : 0));
+  };
+  while (RB > 1 && smem(RB, true) > 48 * 1024) RB /= 2;
+  const bool staged = smem(RB, true) <= (size_t)kPredSmem;
+  const size_t sm = smem(RB, staged);
+  const void* f = vec ? (const void*)k_predict<true> : (const void*)k_predict<false>;
+  if (cudaError_t e = allow_smem(f, (int)sm)) return e;
+  const unsigned grid = (unsigned)((n + 32 * RB - 1) / (32 * RB));
+  const int threads = 32 * RB * WT;
+  if (vec)
+    k_predict<true><<<grid, threads, sm, st>>>(X, n, d, tr, n_trees, H, B, K, crit, class_out,
+                                               value_out, leaf_out, RB, WT, staged);
+  else
+    k_predict<false><<<grid, threads, sm, st>>>(X, n, d, tr, n_trees, H, B, K, crit, class_out,
+                                                value_out, leaf_out, RB, WT, staged);
   return cudaGetLastError();
 }
 
