@@ -2716,15 +2716,17 @@ slm_status slm_train_boost(slm_ctx* c, const slm_params* p, const float* X, int6
   CK(ensure(w.F, sizeof(float) * (size_t)n * K));
   CK(ensure(w.r, sizeof(float) * (size_t)n * K));
   CK(ensure(w.v, sizeof(double) * (size_t)n));
-  CK(ensure(w.loss, sizeof(double) * (size_t)(n_rounds > 0 ? n_rounds : 1)));
+  // (32 doubles more: the sums' scratch)
+  CK(ensure(w.loss, sizeof(double) * ((size_t)n_rounds + 32)));
   CK(ensure(w.base, sizeof(float)));
   float* F = static_cast<float*>(w.F.p);
   float* r = static_cast<float*>(w.r.p);
   double* v = static_cast<double*>(w.v.p);
   double* loss = static_cast<double*>(w.loss.p);
+  double* part = loss + n_rounds;
   if (y)
     CK(launch(c, SLM_K_OTHER, 0.0, [&] {
-      return launch_boost_init(dy, n, F, static_cast<float*>(w.base.p), c->stream);
+      return launch_boost_init(dy, n, F, static_cast<float*>(w.base.p), part, c->stream);
     }));
   else
     CK(launch(c, SLM_K_OTHER, 0.0,
@@ -2784,10 +2786,10 @@ slm_status slm_train_boost(slm_ctx* c, const slm_params* p, const float* X, int6
     }
     if (y)
       CK(launch(c, SLM_K_OTHER, 0.0,
-                [&] { return launch_boost_mse(dy, F, n, loss + (m - 1), c->stream); }));
+                [&] { return launch_boost_mse(dy, F, n, loss + (m - 1), part, c->stream); }));
     else
       CK(launch(c, SLM_K_OTHER, 0.0,
-                [&] { return launch_boost_ce(F, dl, n, K, loss + (m - 1), c->stream); }));
+                [&] { return launch_boost_ce(F, dl, n, K, loss + (m - 1), v, part, c->stream); }));
   }
   if (y)
     CK(cudaMemcpyAsync(&b->base, w.base.p, sizeof(float), cudaMemcpyDeviceToHost, c->stream));

@@ -680,49 +680,49 @@ cudaError_t launch_lift(const float* gs, const int32_t* feat, int A, int n, int 
 
 namespace {
 
-constexpr int kBoostThreads = 1024;
+// A sum over n values in a fixed order, whatever the GPU: chain c of 1024
+// adds values c, c + 1024, ... in turn, a shuffle tree adds the 32 chains of a
+// group and another the 32 groups. Each group is a CTA of one warp (the
+// double-precision lanes of 32 SMs instead of one); k_sum_finish adds the
+// groups.
+constexpr int kSumChains = 1024;
+enum SumOf { kSumF, kSumSqDiff, kSumD };
 
-// Sum over one CTA of kBoostThreads in a fixed order: per thread in stride
-// order (done by the caller), then a shuffle tree per warp, then warp 0 over
-// the warps' sums. Thread 0 returns the total.
-__device__ double boost_block_sum(double v) {
-  __shared__ double sh[kBoostThreads / 32];
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-  __syncthreads();
-  v = threadIdx.x < kBoostThreads / 32 ? sh[threadIdx.x] : 0.0;
-  if (threadIdx.x < 32)
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-  return v;
+template <int OF>
+__global__ void __launch_bounds__(32)
+    k_sum_part(const float* __restrict__ y, const float* __restrict__ F,
+               const double* __restrict__ v, int64_t n, double* part) {
+  double s = 0.0;
+#pragma unroll 8
+  for (int64_t i = blockIdx.x * 32 + threadIdx.x; i < n; i += kSumChains) {
+    if (OF == kSumF) s += (double)y[i];
+    if (OF == kSumD) s += v[i];
+    if (OF == kSumSqDiff) {
+      const double di = (double)y[i] - (double)F[i];
+      s += di * di;
+    }
+  }
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-// base = (float)(mean of y), summed in double; F[i] = base.
-__global__ void __launch_bounds__(kBoostThreads)
-    k_boost_init(const float* __restrict__ y, int64_t n, float* F, float* base_out) {
-  __shared__ float s_base;
-  double s = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += kBoostThreads) s += (double)y[i];
-  s = boost_block_sum(s);
+// The mean of n values from their groups' sums, as double and / or float.
+__global__ void __launch_bounds__(32)
+    k_sum_finish(const double* __restrict__ part, int64_t n, double* out, float* fout) {
+  double s = part[threadIdx.x];
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
   if (threadIdx.x == 0) {
-    s_base = (float)(s / (double)n);
-    *base_out = s_base;
+    if (out) *out = s / (double)n;
+    if (fout) *fout = (float)(s / (double)n);
   }
-  __syncthreads();
-  const float b = s_base;
-  for (int64_t i = threadIdx.x; i < n; i += kBoostThreads) F[i] = b;
 }
 
-// Mean over i of (y_i - F_i)^2 in double.
-__global__ void __launch_bounds__(kBoostThreads)
-    k_boost_mse(const float* __restrict__ y, const float* __restrict__ F, int64_t n,
-                double* out) {
-  double s = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += kBoostThreads) {
-    const double di = (double)y[i] - (double)F[i];
-    s += di * di;
-  }
-  s = boost_block_sum(s);
-  if (threadIdx.x == 0) *out = s / (double)n;
+// F[i] = *base.
+__global__ void k_boost_init(float* F, const float* __restrict__ base, int64_t n) {
+  const float b = *base;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x)
+    F[i] = b;
 }
 
 __global__ void k_boost_residual(const float* __restrict__ y, const float* __restrict__ F,
@@ -765,19 +765,16 @@ __global__ void k_softmax_residual(const float* __restrict__ F, const int32_t* _
   }
 }
 
-// Mean over i of -log p_{i, labels_i} (log-sum-exp form) in double.
-__global__ void __launch_bounds__(kBoostThreads)
-    k_boost_ce(const float* __restrict__ F, const int32_t* __restrict__ lab, int64_t n, int K,
-               double* out) {
-  double t = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += kBoostThreads) {
+// v[i] = -log p_{i, labels_i} (log-sum-exp form) in double.
+__global__ void k_boost_ce(const float* __restrict__ F, const int32_t* __restrict__ lab, int64_t n,
+                           int K, double* v) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
     const float* f = F + i * K;
     double mx, sum;
     softmax_row(f, K, &mx, &sum);
-    t += -(((double)f[lab[i]] - mx) - log(sum));
+    v[i] = -(((double)f[lab[i]] - mx) - log(sum));
   }
-  t = boost_block_sum(t);
-  if (threadIdx.x == 0) *out = t / (double)n;
 }
 
 // class_out[i] = argmax over k of F[i*K + k], ties to the lower class.
@@ -805,17 +802,20 @@ unsigned elementwise_blocks(int64_t n) {
 
 }  // namespace
 
-cudaError_t launch_boost_init(const float* y, int64_t n, float* F, float* base_out,
+cudaError_t launch_boost_init(const float* y, int64_t n, float* F, float* base_out, double* part,
                               cudaStream_t st) {
   if (n <= 0) return cudaErrorInvalidValue;
-  k_boost_init<<<1, kBoostThreads, 0, st>>>(y, n, F, base_out);
+  k_sum_part<kSumF><<<32, 32, 0, st>>>(y, nullptr, nullptr, n, part);
+  k_sum_finish<<<1, 32, 0, st>>>(part, n, nullptr, base_out);
+  k_boost_init<<<elementwise_blocks(n), 256, 0, st>>>(F, base_out, n);
   return cudaGetLastError();
 }
 
-cudaError_t launch_boost_mse(const float* y, const float* F, int64_t n, double* out,
+cudaError_t launch_boost_mse(const float* y, const float* F, int64_t n, double* out, double* part,
                              cudaStream_t st) {
   if (n <= 0) return cudaErrorInvalidValue;
-  k_boost_mse<<<1, kBoostThreads, 0, st>>>(y, F, n, out);
+  k_sum_part<kSumSqDiff><<<32, 32, 0, st>>>(y, F, nullptr, n, part);
+  k_sum_finish<<<1, 32, 0, st>>>(part, n, out, nullptr);
   return cudaGetLastError();
 }
 
@@ -841,9 +841,11 @@ cudaError_t launch_softmax_residual(const float* F, const int32_t* labels, int64
 }
 
 cudaError_t launch_boost_ce(const float* F, const int32_t* labels, int64_t n, int K,
-                            double* out, cudaStream_t st) {
+                            double* out, double* v, double* part, cudaStream_t st) {
   if (n <= 0) return cudaErrorInvalidValue;
-  k_boost_ce<<<1, kBoostThreads, 0, st>>>(F, labels, n, K, out);
+  k_boost_ce<<<elementwise_blocks(n), 256, 0, st>>>(F, labels, n, K, v);
+  k_sum_part<kSumD><<<32, 32, 0, st>>>(nullptr, nullptr, v, n, part);
+  k_sum_finish<<<1, 32, 0, st>>>(part, n, out, nullptr);
   return cudaGetLastError();
 }
 
