@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "philox.cuh"
 #include "slm_internal.cuh"
 
 namespace slm {
@@ -291,7 +292,8 @@ __device__ __forceinline__ void mark_improvement(const Problem& pr, const Swarm&
 
 // Algorithm 1, pbest step of particle p after evaluation t (one warp): strict
 // "<" against the particle's best so far; the position is kept on improvement.
-__device__ __forceinline__ void pbest_step(const Problem& pr, const Swarm& sw, int a, int p,
+// Returns (in every lane) whether it improved.
+__device__ __forceinline__ bool pbest_step(const Problem& pr, const Swarm& sw, int a, int p,
                                            int t, const EvalRes& cur) {
   const int lane = threadIdx.x & 31;
   EvalRes* pb = sw.pb + (int64_t)a * pr.Pp + p;
@@ -301,9 +303,43 @@ __device__ __forceinline__ void pbest_step(const Problem& pr, const Swarm& sw, i
     if (imp) *pb = cur;
   }
   imp = __shfl_sync(0xffffffffu, imp, 0);
-  if (!imp) return;
+  if (!imp) return false;
   const int64_t o = ((int64_t)a * pr.Pp + p) * pr.d;
   for (int j = lane; j < pr.d; j += 32) sw.pbest[o + j] = sw.pos[o + j];
+  return true;
+}
+
+// The terms of Eq. pso-1 for particle pi of node a that do not depend on gB,
+// after the pbest step of evaluation t (one warp; t < T): for every feature j,
+// ic = omega v + (c1 r1)(pB - x) and s2 = c2 r2, r1 and r2 the draws of the
+// move to t + 1 (counter (uid, t + 1, pi, j/4)), each operation rounded as in
+// move_item; k_step finishes the move with v' = ic + s2 (gB - x), x' = x + v'.
+__device__ __forceinline__ void premove_particle(const Problem& pr, const Swarm& sw, uint32_t uid,
+                                                 int a, int t, int pi) {
+  const int lane = threadIdx.x & 31;
+  const int d = pr.d, d4 = (d + 3) >> 2;
+  const SwarmCoef& co = sw.co;
+  const uint32_t k0 = (uint32_t)co.seed, k1 = (uint32_t)(co.seed >> 32);
+  const int64_t row = ((int64_t)a * pr.Pp + pi) * d;
+  const float* x = sw.pos + row;
+  const float* v = sw.vel + row;
+  const float* pb = sw.pbest + row;
+  for (int q = lane; q < d4; q += 32) {
+    const U4 r1 = philox4x32_10(uid, (uint32_t)(t + 1), (uint32_t)pi,
+                                (uint32_t)q | (kR1 << 24), k0, k1);
+    const U4 r2 = philox4x32_10(uid, (uint32_t)(t + 1), (uint32_t)pi,
+                                (uint32_t)q | (kR2 << 24), k0, k1);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int j = 4 * q + c;
+      if (j >= d) break;
+      const float xj = x[j];
+      const float inertia = __fmul_rn(co.inertia, v[j]);
+      const float cog = __fmul_rn(__fmul_rn(co.c1, uniform24(r1.v[c])), __fsub_rn(pb[j], xj));
+      sw.ic[row + j] = __fadd_rn(inertia, cog);
+      sw.s2[row + j] = __fmul_rn(co.c2, uniform24(r2.v[c]));
+    }
+  }
 }
 
 

@@ -637,39 +637,6 @@ __device__ __forceinline__ void move_item(const Problem& pr, const Swarm& sw, co
   if (sw.posb) store_posb4(sw.posb, Pp, pr.dp, a, pi, 4 * q, xn);
 }
 
-// The terms of Eq. pso-1 for particle pi of node a that do not depend on gB,
-// after the pbest step of evaluation t (one warp; t < T): for every feature j,
-// ic = omega v + (c1 r1)(pB - x) and s2 = c2 r2, r1 and r2 the draws of the
-// move to t + 1 (counter (uid, t + 1, pi, j/4)), each operation rounded as in
-// move_item; k_step finishes the move with v' = ic + s2 (gB - x), x' = x + v'.
-__device__ __forceinline__ void premove_particle(const Problem& pr, const Swarm& sw, uint32_t uid,
-                                                 int a, int t, int pi) {
-  const int lane = threadIdx.x & 31;
-  const int d = pr.d, d4 = (d + 3) >> 2;
-  const SwarmCoef& co = sw.co;
-  const uint32_t k0 = (uint32_t)co.seed, k1 = (uint32_t)(co.seed >> 32);
-  const int64_t row = ((int64_t)a * pr.Pp + pi) * d;
-  const float* x = sw.pos + row;
-  const float* v = sw.vel + row;
-  const float* pb = sw.pbest + row;
-  for (int q = lane; q < d4; q += 32) {
-    const U4 r1 = philox4x32_10(uid, (uint32_t)(t + 1), (uint32_t)pi,
-                                (uint32_t)q | (kR1 << 24), k0, k1);
-    const U4 r2 = philox4x32_10(uid, (uint32_t)(t + 1), (uint32_t)pi,
-                                (uint32_t)q | (kR2 << 24), k0, k1);
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int j = 4 * q + c;
-      if (j >= d) break;
-      const float xj = x[j];
-      const float inertia = __fmul_rn(co.inertia, v[j]);
-      const float cog = __fmul_rn(__fmul_rn(co.c1, uniform24(r1.v[c])), __fsub_rn(pb[j], xj));
-      sw.ic[row + j] = __fadd_rn(inertia, cog);
-      sw.s2[row + j] = __fmul_rn(co.c2, uniform24(r2.v[c]));
-    }
-  }
-}
-
 // Fuzzy memberships of the evolutionary factor f in the adaptive PSO states
 // (1 exploration, 2 exploitation, 3 convergence, 4 jumping out).
 __device__ float apso_mu(int state, float f) {
@@ -2000,10 +1967,11 @@ __global__ void k_bootstrap(uint64_t seed, uint32_t tree, int64_t n,
 
 // ---- MSE moments ------------------------------------------------------------------
 
-__global__ void k_mse_init(int A, unsigned long long* acc_w, int32_t* acc_y) {
+__global__ void k_mse_init(int A, unsigned long long* acc_w, int32_t* acc_y, MseNode* mnode) {
   const int a = blockIdx.x * blockDim.x + threadIdx.x;
   if (a >= A) return;
   acc_w[a] = 0ull;
+  if (mnode) mnode[a] = MseNode{};
   acc_y[2 * a] = INT_MAX;
   acc_y[2 * a + 1] = INT_MIN;
 }
@@ -2054,9 +2022,12 @@ __global__ void __launch_bounds__(kTS)
 __global__ void __launch_bounds__(kTS)
     k_mse_moments(Problem pr, const WorkTile* __restrict__ tiles,
                   const unsigned long long* __restrict__ acc_w, const int32_t* __restrict__ acc_y,
-                  long long* m1, long long* m2, double* mscale) {
+                  long long* m1, long long* m2, double* mscale, uint32_t* mq, MseNode* mnode) {
+  __shared__ unsigned long long s_s, s_q;
   const WorkTile wt = tiles[blockIdx.x];
   const int a = wt.node;
+  if (threadIdx.x == 0) s_s = s_q = 0ull;
+  __syncthreads();
   const double W = (double)acc_w[a];
   float c = 0.0f;
   double D = 0.0;
@@ -2078,12 +2049,59 @@ __global__ void __launch_bounds__(kTS)
     mscale[2 * a] = ldexp(1.0, -s);
     mscale[2 * a + 1] = ldexp(1.0, t - 2 * s);
   }
-  if ((int)threadIdx.x >= wt.rows) return;
-  const int64_t e = wt.row0 + threadIdx.x;
-  const double w = pr.w ? (double)pr.w[e] : 1.0;
-  const double v = (double)pr.y[e] - (double)c;
-  m1[e] = llrint(w * v * ldexp(1.0, s));
-  m2[e] = llrint(w * v * v * ldexp(1.0, 2 * s - t));
+  // bits dropped by the 30-bit targets: |m1| <= D 2^s < 2^eb for one entry
+  int eb = 0;
+  if (D > 0.0) frexp(D * (1.0 + 0x1p-40) * ldexp(1.0, s), &eb);
+  const int qs = eb > 28 ? eb - 28 : 0;
+  long long v1 = 0, v2 = 0;
+  if ((int)threadIdx.x < wt.rows) {
+    const int64_t e = wt.row0 + threadIdx.x;
+    const double w = pr.w ? (double)pr.w[e] : 1.0;
+    const double v = (double)pr.y[e] - (double)c;
+    v1 = llrint(w * v * ldexp(1.0, s));
+    v2 = llrint(w * v * v * ldexp(1.0, 2 * s - t));
+    m1[e] = v1;
+    m2[e] = v2;
+    if (mq) {
+      const long long q = qs > 0 ? (v1 + (1ll << (qs - 1))) >> qs : v1;
+      mq[e] = (uint32_t)(min(max(q, -(1ll << 29)), (1ll << 29) - 1) + (1ll << 29));
+    }
+  }
+  if (!mnode) return;
+  // the node's sums of both moments (the units' scale from every tile alike)
+  unsigned long long s1 = (unsigned long long)v1, s2 = (unsigned long long)v2;
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    s1 += __shfl_xor_sync(0xffffffffu, s1, off);
+    s2 += __shfl_xor_sync(0xffffffffu, s2, off);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(&s_s, s1);
+    atomicAdd(&s_q, s2);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    atomicAdd(reinterpret_cast<unsigned long long*>(&mnode[a].S), s_s);
+    atomicAdd(reinterpret_cast<unsigned long long*>(&mnode[a].Q), s_q);
+    mnode[a].inv = ldexp(1.0, qs - s);  // one unit of the rounded targets
+  }
+}
+
+// Per node: the constants of the rounded scores (MseNode) from its sums; W
+// its entries.
+__global__ void k_mse_nodes(int A, const unsigned long long* __restrict__ acc_w,
+                            const double* __restrict__ mscale, MseNode* mnode) {
+  const int a = blockIdx.x * blockDim.x + threadIdx.x;
+  if (a >= A) return;
+  MseNode m = mnode[a];
+  const double n = (double)acc_w[a], f1 = mscale[2 * a], f2 = mscale[2 * a + 1];
+  const double sf = (double)m.S * f1, unit = m.inv;
+  m.base = n > 0.0 ? (double)m.Q * f2 - sf * sf / n : 0.0;
+  m.inv = n > 0.0 && unit > 0.0 ? 1.0 / (n * unit * unit) : 0.0;
+  m.flat = m.S == 0 && m.Q == 0;
+  // targets that are not finite, or scales out of range: score every edge
+  m.full = !isfinite(m.base) || !isfinite(m.inv) || !(m.inv > 0.0);
+  mnode[a] = m;
 }
 
 }  // namespace
@@ -2092,12 +2110,14 @@ __global__ void __launch_bounds__(kTS)
 
 cudaError_t launch_mse_moments(const Problem& pr, const WorkTile* tiles, int n_tiles, int A,
                                unsigned long long* acc_w, int32_t* acc_y, long long* m1,
-                               long long* m2, double* mscale, cudaStream_t st) {
+                               long long* m2, double* mscale, cudaStream_t st, uint32_t* mq,
+                               MseNode* mnode) {
   if (A <= 0) return cudaSuccess;
-  k_mse_init<<<(A + 255) / 256, 256, 0, st>>>(A, acc_w, acc_y);
+  k_mse_init<<<(A + 255) / 256, 256, 0, st>>>(A, acc_w, acc_y, mnode);
   if (n_tiles > 0) {
     k_mse_range<<<n_tiles, kTS, 0, st>>>(pr, tiles, acc_w, acc_y);
-    k_mse_moments<<<n_tiles, kTS, 0, st>>>(pr, tiles, acc_w, acc_y, m1, m2, mscale);
+    k_mse_moments<<<n_tiles, kTS, 0, st>>>(pr, tiles, acc_w, acc_y, m1, m2, mscale, mq, mnode);
+    if (mnode) k_mse_nodes<<<(A + 255) / 256, 256, 0, st>>>(A, acc_w, mscale, mnode);
   }
   return cudaGetLastError();
 }

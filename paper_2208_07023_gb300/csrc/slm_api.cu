@@ -41,7 +41,7 @@ enum Slot {
   // SLM_PROJ_BF16_TOPK
   W_XB, S_POSB, S_MTILES, S_SEL, S_INV, S_POSK, S_Z2, S_ZMM2, S_CUR2,
   // MSE moments
-  S_M1, S_M2, S_MACCW, S_MACCY, S_MSCALE,
+  S_M1, S_M2, S_MACCW, S_MACCY, S_MSCALE, S_MQ, S_MNODE, S_GNEED,
   // learned proposal: node statistics, network work space, training data
   S_PSTATS, S_PYR, S_PACC, S_PWK, S_PWORK, S_PLOSS, W_PS, W_PD, W_PT, W_PIDX, W_PBS, W_PBD,
   W_PBT, W_PRHO, W_PMU, W_PPOS,
@@ -462,12 +462,22 @@ slm_status setup_scoring(slm_ctx* c, Problem& pr, int A,
     pr.m1 = ws_ptr<long long>(c, S_M1);
     pr.m2 = ws_ptr<long long>(c, S_M2);
     pr.mscale = ws_ptr<double>(c, S_MSCALE);
+    pr.mq = nullptr;
+    pr.mnode = nullptr;
+    uint32_t* mq = nullptr;
+    MseNode* mnode = nullptr;
+    if (!pr.w && c->class_hist) {  // scored from the rounded targets (mse_kernels.cu)
+      CK(ensure(c->ws[S_MQ], sizeof(uint32_t) * ne));
+      CK(ensure(c->ws[S_MNODE], sizeof(MseNode) * (size_t)A));
+      pr.mq = mq = ws_ptr<uint32_t>(c, S_MQ);
+      pr.mnode = mnode = ws_ptr<MseNode>(c, S_MNODE);
+    }
     CK(launch(c, SLM_K_NODE_STATS, 0.0, [&] {
       return launch_mse_moments(pr, ws_ptr<WorkTile>(c, S_TILES), (int)tiles.size(), A,
                                 ws_ptr<unsigned long long>(c, S_MACCW),
                                 ws_ptr<int32_t>(c, S_MACCY), ws_ptr<long long>(c, S_M1),
                                 ws_ptr<long long>(c, S_M2), ws_ptr<double>(c, S_MSCALE),
-                                c->stream);
+                                c->stream, mq, mnode);
     }));
   }
   sw->cur = ws_ptr<EvalRes>(c, S_CUR);
@@ -497,6 +507,10 @@ slm_status setup_swarm(slm_ctx* c, Problem& pr, int A, int T, bool want_trace,
   CK(cudaMemsetAsync(c->ws[S_DONE].p, 0, sizeof(int32_t) * (size_t)A, c->stream));
   if (want_trace) CK(ensure(c->ws[S_TRACE], sizeof(double) * (size_t)A * (T + 1)));
   CK(ensure(c->ws[S_APSO], sizeof(ApsoState) * (size_t)A));
+  if (pr.mq) {
+    CK(ensure(c->ws[S_GNEED], sizeof(float) * (size_t)A * pr.Pp));
+    s.gneed = ws_ptr<float>(c, S_GNEED);
+  }
   s.pos = ws_ptr<float>(c, S_POS);
   s.vel = ws_ptr<float>(c, S_VEL);
   s.pbest = ws_ptr<float>(c, S_PBEST);
@@ -538,6 +552,8 @@ struct Bf16Plan {
   // k), splits S_fast / S_fast_k, the c ln c table of entropy scans
   bool fast = false;
   int S_fast = 1, S_fast_k = 1;
+  int S_large = 1, S_large_k = 1;  // the same for a HistPlan's large list
+  int64_t max_len = 0;             // largest node
   const double* xtab = nullptr;
 };
 
@@ -562,6 +578,7 @@ struct HistPlan {
 struct ClsPlan {
   bool on = false;
   int S = 1, S_large = 1;
+  int64_t max_len = 0;  // largest node of the batch
   const double* xtab = nullptr;
 };
 
@@ -573,12 +590,14 @@ slm_status setup_hist_plan(slm_ctx* c, const Problem& pr, const std::vector<Node
   *plan = HistPlan{};
   const bool subset = !in.empty();
   auto member = [&](int a) { return !subset || in[a] != 0; };
-  const bool warp_ok = c->small_node_max > 0 && hist_warp_ok(pr);
+  const bool lazy = mse_lazy_ok(pr);
+  const bool warp_ok = c->small_node_max > 0 && (lazy || hist_warp_ok(pr));
+  const int small_max = lazy ? std::min(c->small_node_max, mse_warp_max()) : c->small_node_max;
   std::vector<int32_t> large, small;
   int64_t max_large = 0;
   for (int a = 0; a < (int)nodes.size(); ++a) {
     if (!member(a)) continue;
-    if (warp_ok && nodes[a].seg_len <= c->small_node_max) {
+    if (warp_ok && nodes[a].seg_len <= small_max) {
       small.push_back(a);
       plan->pairs_small += (double)nodes[a].seg_len * pr.P;
     } else {
@@ -713,6 +732,41 @@ struct StepPlan {
   int sh = 0;  // tile shape of k_step
 };
 
+// The latency-oriented histogram kernels of a search on A nodes (of list[],
+// when set) of at most max_len entries: regression from the rounded targets
+// where the search has them (unweighted), else k_hist_cls / k_hist_mse.
+bool fast_hist_ok(const Problem& pr, int64_t max_len) {
+  return hist_cls_ok(pr) &&
+         (mse_lazy_ok(pr) && mse_lazy_fits(max_len) ? true : hist_cls_fits(pr, max_len));
+}
+
+cudaError_t prepare_fast_hist(const Problem& pr) {
+  if (mse_lazy_ok(pr))
+    if (cudaError_t e = prepare_mse_lazy(pr)) return e;
+  return prepare_hist_cls(pr);
+}
+
+int fast_hist_split(const Problem& pr, int A, int64_t max_len, int n_sm) {
+  return mse_lazy_ok(pr) ? mse_lazy_split(pr, A, max_len, n_sm)
+                         : hist_cls_split(pr, A, max_len, n_sm);
+}
+
+cudaError_t launch_fast_hist(const Problem& pr, const Swarm& sw, const NodeDesc* dn, int A,
+                             int64_t max_len, int S, int t, int do_update, const double* xtab,
+                             cudaStream_t st, const int32_t* list = nullptr) {
+  return mse_lazy_ok(pr)
+             ? launch_mse_lazy(pr, sw, dn, A, max_len, S, t, do_update, st, list)
+             : launch_hist_cls(pr, sw, dn, A, S, t, do_update, xtab, st, list);
+}
+
+// The warp-per-particle histogram kernels.
+cudaError_t launch_small_hist(const Problem& pr, const Swarm& sw, const NodeDesc* dn,
+                              const int32_t* list, int n, int t, int do_update,
+                              cudaStream_t st) {
+  return pr.crit == SLM_MSE ? launch_mse_warp(pr, sw, dn, list, n, t, do_update, st)
+                            : launch_hist_warp(pr, sw, dn, list, n, t, do_update, st);
+}
+
 // One scoring pass of every (node, particle) of a batch; with a swarm
 // (co != null) the pass ends with the swarm update of iteration t.
 slm_status score_batch(slm_ctx* c, const Problem& pr, const Swarm& sw_in,
@@ -740,6 +794,25 @@ slm_status score_batch(slm_ctx* c, const Problem& pr, const Swarm& sw_in,
   if (bp && bp->on) {
     // bfloat16 scores of every particle on the tensor cores
     const Bf16Plan& b = *bp;
+    // a scoring pass of the search: large nodes, then small ones
+    auto pass = [&](const Problem& q, const Swarm& w, int Sf, int Sl, double prs) -> slm_status {
+      if (!(hp && hp->on)) {
+        CK(launch(c, SLM_K_HIST_SCAN, prs, [&] {
+          return launch_fast_hist(q, w, dn, A, b.max_len, Sf, t, 0, b.xtab, c->stream);
+        }));
+        return SLM_OK;
+      }
+      if (hp->n_large)
+        CK(launch(c, SLM_K_HIST_SCAN, prs * hp->pairs_large / pairs, [&] {
+          return launch_fast_hist(q, w, dn, hp->n_large, hp->max_large, Sl, t, 0, b.xtab,
+                                  c->stream, hp->large);
+        }));
+      if (hp->n_small)
+        CK(launch(c, SLM_K_HIST_SCAN, prs * hp->pairs_small / pairs, [&] {
+          return launch_small_hist(q, w, dn, hp->small, hp->n_small, t, 0, c->stream);
+        }));
+      return SLM_OK;
+    };
     if (!co)  // a search's positions are converted by its swarm kernels
       CK(launch(c, SLM_K_TOPK, 0.0, [&] {
         return launch_to_mma_layout(sw.pos, (int64_t)A * pr.Pp, pr.d, pr.dp, pr.Pp, A, b.posb,
@@ -750,11 +823,13 @@ slm_status score_batch(slm_ctx* c, const Problem& pr, const Swarm& sw_in,
         return launch_project_mma(pr, sw, ws_ptr<WorkTile>(c, S_MTILES), b.n_mtiles, b.posb,
                                   b.grid, c->stream);
       }));
-    CK(launch(c, SLM_K_HIST_SCAN, pairs, [&] {
-      return b.fast && !bins_out
-                 ? launch_hist_cls(pr, sw, dn, A, b.S_fast, t, 0, b.xtab, c->stream)
-                 : launch_hist_scan(pr, sw, dn, A, S, bins_out, t, 0, c->stream);
-    }));
+    if (b.fast && !bins_out) {
+      if (slm_status s = pass(pr, sw, b.S_fast, b.S_large, pairs)) return s;
+    } else {
+      CK(launch(c, SLM_K_HIST_SCAN, pairs, [&] {
+        return launch_hist_scan(pr, sw, dn, A, S, bins_out, t, 0, c->stream);
+      }));
+    }
     if (b.k > 0) {
       // FP32 re-scores of the k best of each node (selected by the last
       // histogram CTA of the node) replace theirs
@@ -763,11 +838,13 @@ slm_status score_batch(slm_ctx* c, const Problem& pr, const Swarm& sw_in,
           return launch_project(b.pr_k, b.sw_k, dt, n_tiles, cap, c->stream, 0, false,
                                 c->tma ? A : 0);
         }));
-      CK(launch(c, SLM_K_HIST_SCAN, b.pairs_k, [&] {
-        return b.fast
-                   ? launch_hist_cls(b.pr_k, b.sw_k, dn, A, b.S_fast_k, t, 0, b.xtab, c->stream)
-                   : launch_hist_scan(b.pr_k, b.sw_k, dn, A, b.S_k, nullptr, t, 0, c->stream);
-      }));
+      if (b.fast) {
+        if (slm_status s = pass(b.pr_k, b.sw_k, b.S_fast_k, b.S_large_k, b.pairs_k)) return s;
+      } else {
+        CK(launch(c, SLM_K_HIST_SCAN, b.pairs_k, [&] {
+          return launch_hist_scan(b.pr_k, b.sw_k, dn, A, b.S_k, nullptr, t, 0, c->stream);
+        }));
+      }
       CK(launch(c, SLM_K_TOPK, 0.0, [&] {
         return launch_merge(pr, sw, A, b.sw_k.cur, b.kp, b.inv, t, co ? 1 : 0, c->stream);
       }));
@@ -786,18 +863,19 @@ slm_status score_batch(slm_ctx* c, const Problem& pr, const Swarm& sw_in,
   if (hp && hp->on && !bins_out) {
     if (hp->n_large)
       CK(launch(c, SLM_K_HIST_SCAN, hp->pairs_large, [&] {
-        return cls ? launch_hist_cls(pr, sw, dn, hp->n_large, cp->S_large, t, co ? 1 : 0,
-                                     cp->xtab, c->stream, hp->large)
+        return cls ? launch_fast_hist(pr, sw, dn, hp->n_large, hp->max_large, cp->S_large, t,
+                                      co ? 1 : 0, cp->xtab, c->stream, hp->large)
                    : launch_hist_scan(pr, sw, dn, hp->n_large, hp->S_large, nullptr, t,
                                       co ? 1 : 0, c->stream, hp->large);
       }));
     if (hp->n_small)
       CK(launch(c, SLM_K_HIST_SCAN, hp->pairs_small, [&] {
-        return launch_hist_warp(pr, sw, dn, hp->small, hp->n_small, t, co ? 1 : 0, c->stream);
+        return launch_small_hist(pr, sw, dn, hp->small, hp->n_small, t, co ? 1 : 0, c->stream);
       }));
   } else {
     CK(launch(c, SLM_K_HIST_SCAN, pairs, [&] {
-      return cls ? launch_hist_cls(pr, sw, dn, A, cp->S, t, co ? 1 : 0, cp->xtab, c->stream)
+      return cls ? launch_fast_hist(pr, sw, dn, A, cp->max_len, cp->S, t, co ? 1 : 0, cp->xtab,
+                                    c->stream)
                  : launch_hist_scan(pr, sw, dn, A, S, bins_out, t, co ? 1 : 0, c->stream);
     }));
   }
@@ -1167,6 +1245,7 @@ struct KeyWriter {
     put(p.X); put(p.Xg); put(p.gidx); put(p.lab); put(p.y); put(p.w); put(p.E); put(p.Ez);
     put(p.d); put(p.crit); put(p.K); put(p.B); put(p.min_leaf); put(p.P); put(p.Pp);
     put(p.G); put(p.Xb); put(p.dp); put(p.m1); put(p.m2); put(p.mscale);
+    put(p.mq); put(p.mnode);
   }
   void swarm(const Swarm& w) {
     put(w.pos); put(w.vel); put(w.pbest); put(w.gbest); put(w.cur); put(w.pb); put(w.gb);
@@ -1174,7 +1253,7 @@ struct KeyWriter {
     put(w.T); put(w.sel); put(w.k); put(w.tk_sel); put(w.tk_inv); put(w.tk_pos);
     put(w.tk_k); put(w.tk_kp); put(w.posb); put(w.apso); put(w.ic); put(w.s2);
     put(w.co.inertia); put(w.co.c1); put(w.co.c2); put(w.co.seed); put(w.node_step);
-    put(w.n_nodes); put(w.imp);
+    put(w.n_nodes); put(w.imp); put(w.gneed);
   }
 };
 
@@ -1259,13 +1338,14 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
   if (bp.on && bp.k > 0 && c->class_hist && hist_cls_ok(pr) && hist_cls_ok(bp.pr_k)) {
     int64_t len = 0;
     for (const NodeDesc& nd : nodes) len = std::max<int64_t>(len, nd.seg_len);
-    if (hist_cls_fits(pr, len)) {
-      CK(prepare_hist_cls(bp.pr_k));  // (shared-memory limits are only raised)
-      CK(prepare_hist_cls(pr));
+    if (fast_hist_ok(pr, len)) {
+      CK(prepare_fast_hist(bp.pr_k));  // (shared-memory limits are only raised)
+      CK(prepare_fast_hist(pr));
       bp.fast = true;
+      bp.max_len = len;
       if (pr.crit == SLM_ENTROPY) bp.xtab = xlogx_table(c->device);
-      bp.S_fast = hist_cls_split(pr, A, len, c->n_sm);
-      bp.S_fast_k = hist_cls_split(bp.pr_k, A, len, c->n_sm);
+      bp.S_fast = fast_hist_split(pr, A, len, c->n_sm);
+      bp.S_fast_k = fast_hist_split(bp.pr_k, A, len, c->n_sm);
     }
   }
   if (p->seeded) {
@@ -1386,19 +1466,28 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
     slm_ctx::Tiles tl{};
     if (!bp.on && !stp.on && (s = pick_tiles(c, pr, sw, (int)tiles.size(), A, &tl))) return s;
     HistPlan hp;
-    if (!bp.on && (s = setup_hist_plan(c, pr, nodes, in, &hp))) return s;
+    // (the BF16 form has a warp-per-particle kernel for regression only)
+    if ((!bp.on || (bp.fast && mse_lazy_ok(pr))) && (s = setup_hist_plan(c, pr, nodes, in, &hp)))
+      return s;
+    if (bp.fast && hp.on && hp.n_large) {
+      bp.S_large = fast_hist_split(pr, hp.n_large, hp.max_large, c->n_sm);
+      bp.S_large_k = fast_hist_split(bp.pr_k, hp.n_large, hp.max_large, c->n_sm);
+    }
     ClsPlan cp;
     int64_t max_len = 0;
     for (const NodeDesc& nd : nodes) max_len = std::max<int64_t>(max_len, nd.seg_len);
-    if (c->class_hist && !bp.on && hist_cls_ok(pr) && hist_cls_fits(pr, max_len)) {
-      CK(prepare_hist_cls(pr));
+    if (c->class_hist && !bp.on && fast_hist_ok(pr, max_len)) {
+      CK(prepare_fast_hist(pr));
       cp.on = true;
+      cp.max_len = max_len;
       cp.xtab = xlogx_table(c->device);
       if (hp.on && hp.n_large)
-        cp.S_large = hist_cls_split(pr, hp.n_large, hp.max_large, c->n_sm);
+        cp.S_large = fast_hist_split(pr, hp.n_large, hp.max_large, c->n_sm);
     }
-    if (!bp.on && !hp.on &&
-        (s = pick_split(c, pr, sw, nodes, (int)tiles.size(), tl, &S, cp.on ? &cp : nullptr)))
+    if (cp.on && mse_lazy_ok(pr))
+      S = mse_lazy_split(pr, A, max_len, c->n_sm);
+    else if (!bp.on && !hp.on &&
+             (s = pick_split(c, pr, sw, nodes, (int)tiles.size(), tl, &S, cp.on ? &cp : nullptr)))
       return s;
     cp.S = S;
     // every node scored by k_hist_cls: its last CTA per node takes the gbest
@@ -1420,6 +1509,8 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
       kw.put(bp.on); kw.put(bp.k); kw.put(bp.kp); kw.put(bp.n_mtiles); kw.put(bp.grid);
       kw.put(bp.S_k); kw.put(bp.pairs_k); kw.put(bp.posb); kw.put(bp.sel); kw.put(bp.inv);
       kw.put(bp.fast); kw.put(bp.S_fast); kw.put(bp.S_fast_k); kw.put(bp.xtab);
+      kw.put(bp.S_large); kw.put(bp.S_large_k); kw.put(bp.max_len); kw.put(cp.max_len);
+      kw.put(hp.max_large);
       kw.put(hp.on); kw.put(hp.large); kw.put(hp.n_large); kw.put(hp.S_large);
       kw.put(hp.pairs_large); kw.put(hp.small); kw.put(hp.n_small); kw.put(hp.pairs_small);
       kw.put(hp.moved); kw.put(hp.n_moved);
@@ -3002,7 +3093,8 @@ slm_status slm_proposal_loss_grad(slm_ctx* c, const slm_proposal* pp, const floa
   slm_status s;
   if ((s = stage_in(c, stats, (size_t)n * kPropIn, c->ws[W_PS], &ds)) ||
       (s = stage_in(c, dims, (size_t)n, c->ws[W_PD], &dd)) ||
-      (s = stage_in(c, targets, (size_t)n * kPropD, c->ws[W_PT], &dt)))
+      (s = stage_in(c, targets, (size_t)n * kPropD, c->ws[W_PT], &dt)) ||
+      (s = align16(c, &ds, (size_t)n * kPropIn, c->ws[W_PS])))
     return s;
   MlpWork w;
   if ((s = proposal_work(c, n, &w))) return s;

@@ -102,6 +102,20 @@ struct Problem {
   const long long* m1;
   const long long* m2;
   const double* mscale;
+  // MSE, unweighted searches: w (y - c) rounded to 30 bits, stored + 2^29,
+  // and per node the constants of the scores formed from it (mse_kernels.cu)
+  const uint32_t* mq;
+  const struct MseNode* mnode;
+};
+
+// One regression node's sums of both fixed-point moments and what relates
+// its between-children sum of squares G (in squared units of the rounded
+// targets, see mse_kernels.cu) to the loss: loss n =
+// base - G / inv. flat: every target equal; full: score every edge exactly.
+struct MseNode {
+  long long S, Q;
+  double base, inv;
+  int32_t flat, full;
 };
 
 // Codes of the kernels' error word (Swarm::err). Both mean that a bounded
@@ -179,6 +193,9 @@ struct Swarm {
   // histogram kernels, reset by the kernel that takes the gbest step); the
   // gbest step skips its argmin when it is 0, since gB then stays
   int32_t* imp;
+  // regression searches scored from the rounded targets: the G an edge must
+  // reach to improve each particle's best (set at every pbest improvement)
+  float* gneed;  // [A, Pp]
 };
 
 // Adaptive PSO state of one node (Sec. III-B): evolutionary state 1..4
@@ -244,6 +261,24 @@ int hist_cls_split(const Problem& pr, int A, int64_t max_len, int n_sm);
 cudaError_t launch_hist_cls(const Problem& pr, const Swarm& sw, const NodeDesc* nodes, int A,
                             int S, int t, int do_update, const double* xtab, cudaStream_t st,
                             const int32_t* list = nullptr);
+// Histograms and scans of unweighted regression searches, scores, pbest
+// steps and move terms as launch_hist_scan except that a score that cannot
+// improve its particle's best is recorded as invalid (mse_kernels.cu): a
+// (node, particle) per cluster of S CTAs (nodes of at most max_len entries,
+// mse_lazy_fits, S at least mse_lazy_min_split), or per warp (the nodes
+// list[] names, of at most mse_warp_max() entries).
+bool mse_lazy_ok(const Problem& pr);
+bool mse_lazy_fits(int64_t max_len);
+int mse_lazy_min_split(int64_t max_len);
+int mse_lazy_split(const Problem& pr, int A, int64_t max_len, int n_sm);
+int mse_warp_max();
+cudaError_t prepare_mse_lazy(const Problem& pr);
+cudaError_t launch_mse_lazy(const Problem& pr, const Swarm& sw, const NodeDesc* nodes, int A,
+                            int64_t max_len, int S, int t, int do_update, cudaStream_t st,
+                            const int32_t* list = nullptr);
+cudaError_t launch_mse_warp(const Problem& pr, const Swarm& sw, const NodeDesc* nodes,
+                            const int32_t* list, int n_nodes, int t, int do_update,
+                            cudaStream_t st);
 // Persistent search of classification nodes whose rows fit in shared memory:
 // all T + 1 iterations in one launch, a cluster of S (1..8) CTAs per node of
 // list[n_nodes] (A: the batch's node count, the gbest buffers' stride).
@@ -344,10 +379,12 @@ cudaError_t launch_merge(const Problem& pr, const Swarm& sw, int A, const EvalRe
 // index): per node the range of y and the weight W (acc_w[A], acc_y[A, 2]),
 // then per entry m1 = round(w (y-c) 2^s), m2 = round(w (y-c)^2 2^(2s-t)),
 // with c the node's mid-range and s, t chosen so each node sum stays below
-// 2^61; mscale[A, 2] = 2^-s, 2^(t-2s).
+// 2^61; mscale[A, 2] = 2^-s, 2^(t-2s). Unweighted: mq, mnode (when set) as
+// Problem::mq and Problem::mnode.
 cudaError_t launch_mse_moments(const Problem& pr, const WorkTile* tiles, int n_tiles, int A,
                                unsigned long long* acc_w, int32_t* acc_y, long long* m1,
-                               long long* m2, double* mscale, cudaStream_t st);
+                               long long* m2, double* mscale, cudaStream_t st,
+                               uint32_t* mq = nullptr, MseNode* mnode = nullptr);
 cudaError_t launch_swarm_uniforms(uint64_t seed, uint32_t uid, uint32_t t,
                                   int P, int d, uint32_t purpose, float* u,
                                   cudaStream_t st);

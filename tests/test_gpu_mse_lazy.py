@@ -1,0 +1,77 @@
+"""Regression scores from the 30-bit rounded targets (mse_kernels.cu) are those
+of the staged-copy kernel, bit for bit: an edge's rounded interval may only
+rule it out, and every edge left is scored exactly. Sizes at the edges of the
+kernels: the largest warp node (2,048 entries) and the smallest cluster node,
+slices around the switch from 8 to 32 copies per bin, the largest slice of a
+single CTA, bins per lane of every width, and targets that leave many edges
+(two values, one value, one far outlier)."""
+import numpy as np
+import pytest
+
+from paper_2208_07023_gb300 import workloads as W
+from tests.gpu_util import context, gpu_params
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctxs():
+    a, b = context(), context()
+    b.set_class_hist(False)  # the staged-copy kernel scores every particle
+    yield a, b
+    a.set_small_nodes()
+    a.close()
+    b.close()
+
+
+def _targets(kind, wl):
+    y = wl.y.copy()
+    if kind == "two":
+        return (y > 0.3).astype(np.float32) * 0.9 - 0.1
+    if kind == "one":
+        return np.full_like(y, 0.25)
+    if kind == "outlier":
+        y[len(y) // 2] = 3e6
+    if kind == "offset":
+        y = (y * np.float32(1e-3) + np.float32(500)).astype(np.float32)
+    return y
+
+
+@pytest.mark.parametrize("n,B,min_leaf,kind", [
+    (2048, 256, 1, "plain"), (2049, 256, 1, "plain"), (2047, 200, 5, "plain"),
+    (65, 33, 1, "plain"), (3, 16, 1, "plain"), (700, 2, 1, "plain"),
+    (1500, 64, 1, "two"), (1500, 100, 1, "one"), (1800, 256, 1, "outlier"),
+    (1900, 128, 3, "offset"), (8190, 32, 1, "two"), (9000, 256, 1, "one"),
+    (40001, 256, 5, "plain"), (40001, 256, 1, "outlier"), (70003, 128, 1, "offset"),
+    (131003, 256, 20, "plain"),
+])
+@pytest.mark.parametrize("warp", [False, True])
+def test_search_identical_to_the_exact_histogram(ctxs, n, B, min_leaf, kind, warp):
+    from paper_2208_07023_gb300 import binding as S
+    a, b = ctxs
+    a.set_small_nodes(4096 if warp else 0, 0)
+    wl = W.tanh_regression(n, 6, seed=n % 83)
+    y = _targets(kind, wl)
+    p = gpu_params(S, "mse", 0, 19, 9, B, min_leaf=min_leaf, seed=3)
+    ra = a.node_split(p, wl.X, y=y, node_uid=8, want_trace=True)
+    rb = b.node_split(p, wl.X, y=y, node_uid=8, want_trace=True)
+    assert np.array_equal(ra["trace"], rb["trace"])
+    assert np.array_equal(ra["gbest"].view(np.uint32), rb["gbest"].view(np.uint32))
+    for k in ("valid", "bin", "loss", "n_left", "n_right", "particle", "iter_of_best"):
+        assert ra[k] == rb[k], k
+
+
+@pytest.mark.parametrize("proj,apso", [("fp32", False), ("bf16", False), ("fp32", True)])
+def test_tree_identical_to_the_exact_histogram(ctxs, proj, apso):
+    """Levels of hundreds of small nodes (a warp each), beside large ones."""
+    from paper_2208_07023_gb300 import binding as S
+    a, b = ctxs
+    a.set_small_nodes()
+    wl = W.tanh_regression(12000, 9, seed=5)
+    p = S.make_params("mse", 0, n_particles=24, n_iters=6, n_bins=200, min_leaf=4, max_depth=9,
+                      seed=5, proj=S.SLM_PROJ_BF16_TOPK if proj == "bf16" else S.SLM_PROJ_FP32,
+                      topk=5, apso=apso)
+    ga, gb = (c.train_tree(p, wl.X, y=wl.y).export(0) for c in (a, b))
+    for k in ga:
+        assert np.array_equal(ga[k], gb[k]), k
+    assert (ga["kind"] == 1).sum() > 200
