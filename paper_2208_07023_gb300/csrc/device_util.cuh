@@ -202,9 +202,10 @@ __device__ __forceinline__ EvalRes ldcg_res(const EvalRes* r) {
 // smallest loss are then compared exactly (better(), index ties), which gives
 // the result of an exact argmin over all candidates.
 __device__ __forceinline__ uint64_t loss_key(const EvalRes& e) {
-  // losses are >= 0: their bit patterns order like their values; invalid
-  // scores last
-  return e.valid ? (uint64_t)__double_as_longlong(e.loss) : ~0ull;
+  // the doubles' order as unsigned integers (a squared-error loss of a perfect
+  // split can round to just below zero); invalid scores last
+  const uint64_t u = (uint64_t)__double_as_longlong(e.loss);
+  return !e.valid ? ~0ull : (u >> 63) ? ~u : u | 0x8000000000000000ull;
 }
 
 // The warp's choice among its lanes' candidates: lane l proposes particle bi

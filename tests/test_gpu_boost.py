@@ -309,3 +309,24 @@ def test_cls_boost_round_forest_views(ctx):
             assert np.allclose(vg, vo, rtol=1e-12, atol=1e-12)
             F[:, k] = (F[:, k] + np.float32(0.5) * vo.astype(np.float32)).astype(np.float32)
     b.free()
+
+
+@pytest.mark.parametrize("seed", range(8))
+def test_perfect_splits_of_two_valued_targets(ctx, seed):
+    """Two-valued targets (a class's residuals) that a hyperplane separates:
+    many particles reach a perfect split, whose squared error is zero up to a
+    rounding of either sign. The gbest step must keep the smallest loss (a
+    negative one too), or gB and its recorded split part and the partition
+    refuses the node."""
+    from paper_2208_07023_gb300 import binding as S
+    rng = np.random.default_rng(seed)
+    X = rng.standard_normal((3000, 3)).astype(np.float32)
+    s = X[:, 0] - 0.3 * X[:, 1]
+    X[:, 0] += np.where(s > 0, 0.7, -0.7).astype(np.float32)  # a gap between the sides
+    y = np.where(s > 0, 0.9, -0.1).astype(np.float32)
+    for P in (40, 100):  # folded, not folded
+        p = gpu_params(S, "mse", 0, P, 40, 64, min_leaf=20, max_depth=1, seed=seed)
+        r = ctx.node_split(p, X, y=y, node_uid=0, want_trace=True)
+        assert r["loss"] == r["trace"].min()
+        g = ctx.train_tree(p, X, y=y).export(0)
+        assert g["n_left"][0] == r["n_left"] and np.array_equal(g["dir"][0], r["gbest"])
