@@ -523,8 +523,8 @@ slm_status slm_kernel_stats(slm_ctx* ctx, int32_t kernel, int64_t* launches,
  * node of a graph counts as one launch). */
 slm_status slm_launch_count(slm_ctx* ctx, int64_t* launches);
 
-/* Projection tiles. on = 1 (the default): the FP32 projection of a search
- * runs with the tile shape (particles per group: 8, 16, 24, 32 or 48 dividing
+/* Projection tiles. on = 1 (the default): the row-major FP32 projection
+ * (searches with slm_set_fused_step off) runs with the tile shape (particles per group: 8, 16, 24, 32 or 48 dividing
  * P rounded up to 16; 1 or 2 CTAs per SM; rows from the level copy or, in
  * bagged forests, gathered from the base rows) that was fastest when the first
  * search of the same shape (d, padded P, log2 of the 256-row tiles) timed
@@ -607,35 +607,32 @@ slm_status slm_set_graphs(slm_ctx* ctx, int32_t on);
  * issuing thread, 128-byte swizzle); on = 0: by per-thread asynchronous
  * copies. The projected values are identical either way. */
 slm_status slm_set_projection_tma(slm_ctx* ctx, int32_t on);
-/* on = 1 (the default) or 2: plain FP32 searches (no adaptive PSO, no BF16
- * form, no persistent node search) whose padded swarm is 16, 32, 48 or 64
- * particles, whose positions fit in 96 KB of shared memory and for which
- * no projection tiles are forced (slm_force_tiles) fold the
- * swarm move of Eq. pso-1 into the projection: one iteration is the
- * projection (which first takes the gbest step of the previous evaluation,
- * Algorithm 1, and moves every particle) and the histogram pass (which
- * leaves the gB-independent terms of the next move), two launches instead
- * of three, and each row tile is projected onto all particles at once.
- * With on = 1 only a batch whose projection is at most 4 waves of row
- * tiles (of 128 or 256 rows) on the GPU is folded: there the iteration is
- * latency-bound and the saved launch pays; longer projections (many nodes,
- * or one very large node) run faster unfolded, with the tuned projection.
- * on = 2 folds every eligible batch; on = 0 none (the projection,
- * histogram and move kernels). Results are identical either way.
+/* on = 1 (the default) or 2: FP32 searches of whole batches (no BF16 form, no
+ * persistent node search, no projection tiles forced by slm_force_tiles)
+ * project from the rows laid out in blocks of 32, feature-major, once per
+ * search (a second copy of the batch's rows; searches without room for it
+ * use the kernels of on = 0). Plain searches (no adaptive PSO) whose padded
+ * swarm is 16, 32, 48 or 64 particles and whose positions fit in 96 KB of
+ * shared memory may also fold the swarm move of Eq. pso-1 into this
+ * projection: one iteration is the projection (which first takes the gbest
+ * step of the previous evaluation, Algorithm 1, and moves every particle)
+ * and the histogram pass (which leaves the gB-independent terms of the next
+ * move), two launches instead of three. With on = 1 only a batch of at most
+ * 48 blocks per SM and one node per SM is folded: there the iteration is
+ * latency-bound and the saved launch pays. on = 2 folds every eligible
+ * batch; on = 0 none, with the tuned row-major projection, histogram and
+ * move kernels. Results are identical either way.
  * *searches (optional) = searches run folded so far. SLM_EINVAL for other
  * values of on. */
 slm_status slm_set_fused_step(slm_ctx* ctx, int32_t on, int64_t* searches);
 /* Tile shape of the folded projection: shape = -1 (the default) picks, per
- * batch, the shape with the least estimated work per CTA (units per CTA x
- * (rows per unit x particles per unit / swarm width + a fixed cost of 32
- * rows per unit); on ties, half-swarm units where each CTA takes one unit,
- * else larger row tiles), so a short node is spread over
- * more CTAs; 0, 1, 2 force 128-256, 64-128 or 32-64 rows per tile with every
- * particle in a unit, 3, 4, 5 the same with half the particles of a swarm of
- * 32 or 64 (by swarm width; a width without the forced shape takes shape
- * 0). Results are identical for every shape. *last (optional) = the shape
- * of the last folded batch (-1 before the first). SLM_EINVAL for other
- * values of shape. */
+ * batch, the shape with the least estimated time of its longest CTA; 0, 1, 2
+ * force 384, 192 or 96 rows per CTA at a time (12 warps, 1, 2 or 4 of them
+ * sharing a block's particles) with every particle in a unit, 3, 4, 5 the
+ * same with half the particles of a swarm of 32 or 64 (a width without the
+ * forced shape takes shape 0). Results are identical for every shape. *last
+ * (optional) = the shape of the last folded batch (-1 before the first).
+ * SLM_EINVAL for other values of shape. */
 slm_status slm_set_step_shape(slm_ctx* ctx, int32_t shape, int32_t* last);
 /* on != 0 (the default): the searches of the FP32 form score each
  * iteration with the latency-oriented histogram kernels (entries loaded 16

@@ -15,6 +15,15 @@ namespace {
 
 // ---- small helpers -----------------------------------------------------------
 
+// Reads a kernel parameter here: a launch starts with its parameters to be
+// fetched into the constant cache, and reading them before pdl_wait() keeps
+// those misses off the chain that starts there.
+template <class T>
+__device__ __forceinline__ void touch(const T* p) {
+  asm volatile("" ::"l"(p));
+}
+__device__ __forceinline__ void touch(int v) { asm volatile("" ::"r"(v)); }
+
 // Programmatic dependent launch: the next kernel of the stream may begin
 // launching once every CTA of this grid has passed pdl_trigger(); pdl_wait()
 // blocks until the previous grid has completed and its writes are visible.
@@ -201,11 +210,21 @@ __device__ __forceinline__ EvalRes ldcg_res(const EvalRes* r) {
 // units in the last place of each other. The candidates within 8 ulps of the
 // smallest loss are then compared exactly (better(), index ties), which gives
 // the result of an exact argmin over all candidates.
-__device__ __forceinline__ uint64_t loss_key(const EvalRes& e) {
+__device__ __forceinline__ uint64_t loss_key(double loss) {
   // the doubles' order as unsigned integers (a squared-error loss of a perfect
-  // split can round to just below zero); invalid scores last
-  const uint64_t u = (uint64_t)__double_as_longlong(e.loss);
-  return !e.valid ? ~0ull : (u >> 63) ? ~u : u | 0x8000000000000000ull;
+  // split can round to just below zero)
+  const uint64_t u = (uint64_t)__double_as_longlong(loss);
+  return (u >> 63) ? ~u : u | 0x8000000000000000ull;
+}
+__device__ __forceinline__ uint64_t loss_key(const EvalRes& e) {
+  return e.valid ? loss_key(e.loss) : ~0ull;  // invalid scores last
+}
+
+// Records a particle's score (index ci of [A, Pp]), with its key in searches
+// that keep them.
+__device__ __forceinline__ void store_score(const Swarm& sw, int64_t ci, const EvalRes& res) {
+  sw.cur[ci] = res;
+  if (sw.keys) sw.keys[ci] = loss_key(res);
 }
 
 // The warp's choice among its lanes' candidates: lane l proposes particle bi

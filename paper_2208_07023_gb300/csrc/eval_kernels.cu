@@ -1270,7 +1270,7 @@ __global__ void __launch_bounds__(kThreads, 3)
     res.inv_w = inv_w;
   }
   if (threadIdx.x == 0) {
-    sw.cur[(int64_t)a * pr.Pp + p] = res;
+    store_score(sw, (int64_t)a * pr.Pp + p, res);
     zz[0] = INT_MAX;  // ready for the next iteration
     zz[1] = INT_MIN;
     if (do_update) mark_improvement(pr, sw, a, t, res);
@@ -1538,7 +1538,7 @@ __global__ void __launch_bounds__(kThreads)
     res.inv_w = inv_w;
   }
   if (lane == 0) {
-    sw.cur[(int64_t)a * pr.Pp + p] = res;
+    store_score(sw, (int64_t)a * pr.Pp + p, res);
     zz[0] = INT_MAX;  // ready for the next iteration
     zz[1] = INT_MIN;
     if (do_update) mark_improvement(pr, sw, a, t, res);

@@ -476,7 +476,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 
   // ---- score, range reset, pbest step, the next move's gB-independent terms
   if (threadIdx.x == 0) {
-    sw.cur[ci] = res;
+    store_score(sw, ci, res);
     zz[0] = INT_MAX;  // ready for the next iteration
     zz[1] = INT_MIN;
     int imp = 0;
@@ -929,7 +929,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   if (threadIdx.x == 0) {
     for (int q = 0; q < np; ++q) {
       const int64_t ci = ci0 + q;
-      sw.cur[ci] = res[q];
+      store_score(sw, ci, res[q]);
       zz0[2 * q] = INT_MAX;  // ready for the next iteration
       zz0[2 * q + 1] = INT_MIN;
       int imp = 0;

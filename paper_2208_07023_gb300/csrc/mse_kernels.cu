@@ -510,7 +510,7 @@ __global__ void __launch_bounds__(kThreads, 3)
       res.zmin = zmin;
       res.inv_w = inv_w;
     }
-    sw.cur[ci] = res;
+    store_score(sw, ci, res);
     zz[0] = INT_MAX;  // ready for the next iteration
     zz[1] = INT_MIN;
     int imp = 0;
@@ -823,7 +823,7 @@ __global__ void __launch_bounds__(kThreads, 4)
       res.inv_w = inv_w;
     }
     if (lane == 0) {
-      sw.cur[ci] = res;
+      store_score(sw, ci, res);
       zz[0] = INT_MAX;  // ready for the next iteration
       zz[1] = INT_MIN;
       if (do_update) mark_improvement(pr, sw, a, t, res);

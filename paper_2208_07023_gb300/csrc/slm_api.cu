@@ -28,11 +28,9 @@ struct DevBuf {
   size_t cap = 0;
 };
 
-// A level's search folds the move into the projection when its projection
-// is at most this many waves of row-tile units (slm_set_fused_step, on = 1).
-constexpr int kFusedMaxWaves = 4;
-// The fixed cost of one folded projection unit, in rows of work.
-constexpr int kStepUnitRows = 32;
+// A plain search's move is folded into its projection when the batch has at
+// most this many blocks of 32 rows per CTA of the projection's grid.
+constexpr int kFoldMaxBlocks = 48;
 
 enum Slot {
   W_X, W_LAB, W_Y, W_IDX, W_W, W_BINS, W_XL, W_LABL, W_YL,
@@ -55,7 +53,7 @@ enum Slot {
   S_APSO,
   // the projection with the move folded in: second position buffer, the
   // gB-independent move terms, its row tiles
-  S_POS2, S_IC, S_S2, S_STILES, S_IMP,
+  S_POS2, S_IC, S_S2, S_XT, S_RUNS, S_IMP, S_KEYS,
   // probabilistic search: every candidate's vector and score, the rank
   // tables, the best so far, the pruning's state
   S_PRALL, S_PRSC, S_PRTAB, S_PRBEST, S_PRUNE,
@@ -721,16 +719,77 @@ slm_status setup_bf16(slm_ctx* c, const Problem& pr, const std::vector<NodeDesc>
   return SLM_OK;
 }
 
-// A plain FP32 search whose move is folded into the projection (k_step):
+// A search projected from blocked rows (k_step): with the move folded in,
 // positions alternate between pos[0] and pos[1] by iteration parity.
 struct StepPlan {
-  bool on = false;
+  bool on = false, fold = false;
   float* pos[2] = {nullptr, nullptr};
-  const WorkTile* tiles = nullptr;
-  int n_tiles = 0;
-  int grid = 0;
-  int sh = 0;  // tile shape of k_step
+  const StepRun* runs = nullptr;
+  int n_runs = 0;
+  StepConfig cfg;
 };
+
+// The CTAs' runs of blocks. With no more (node, slice) pairs than CTAs each
+// pair gets CTAs of its own in proportion to its blocks (a CTA that forms two
+// nodes' positions one after the other takes about 5 us longer than the
+// rest); else equal shares of the blocks in order, a pair that a run opens
+// counted as four blocks more.
+std::vector<StepRun> plan_runs(const std::vector<NodeDesc>& nodes, int slices, int grid) {
+  std::vector<StepRun> runs;
+  runs.reserve((size_t)grid);
+  const int A = (int)nodes.size();
+  auto blocks = [&](int a) { return (nodes[a].seg_len + 31) / 32; };
+  int64_t total = 0;
+  for (int a = 0; a < A; ++a) total += (int64_t)blocks(a) * slices;
+  if ((int64_t)A * slices <= grid) {
+    // the fewest blocks per CTA at which the pairs' CTAs fit the grid
+    int64_t lo = std::max<int64_t>(1, (total + grid - 1) / grid), hi = 1;
+    for (int a = 0; a < A; ++a) hi = std::max<int64_t>(hi, blocks(a));
+    hi = std::max(hi, lo);
+    while (lo < hi) {
+      const int64_t m = (lo + hi) / 2;
+      int64_t n = 0;
+      for (int a = 0; a < A; ++a) n += (blocks(a) + m - 1) / m * slices;
+      if (n <= grid)
+        hi = m;
+      else
+        lo = m + 1;
+    }
+    for (int a = 0; a < A; ++a) {
+      const int nb = blocks(a), k = (int)((nb + lo - 1) / lo);
+      for (int q = 0; q < slices; ++q)
+        for (int i = 0; i < k; ++i) {
+          const int b0 = (int)((int64_t)nb * i / k), b1 = (int)((int64_t)nb * (i + 1) / k);
+          if (b1 > b0) runs.push_back(StepRun{a, q, b0, b1 - b0});
+        }
+    }
+    return runs;
+  }
+  const int64_t open = 4;
+  const int64_t cost = total + open * A * slices;
+  int64_t done = 0;  // cost up to the current block
+  int64_t share = 0;  // shares handed out
+  for (int a = 0; a < A; ++a) {
+    const int nb = blocks(a);
+    for (int q = 0; q < slices; ++q) {
+      for (int b = 0; b < nb;) {
+        // a run starts where the cost passes the next share's start
+        if (runs.empty() || done * grid >= share * cost) {
+          runs.push_back(StepRun{a, q, b, 0});
+          share = std::max<int64_t>(share + 1, done * grid / std::max<int64_t>(cost, 1) + 1);
+        }
+        if (b == 0) done += open;
+        // blocks up to the next share's start
+        const int64_t next = (share * cost + grid - 1) / grid;
+        const int take = (int)std::min<int64_t>(nb - b, std::max<int64_t>(1, next - done));
+        runs.back().count += take;
+        b += take;
+        done += take;
+      }
+    }
+  }
+  return runs;
+}
 
 // The latency-oriented histogram kernels of a search on A nodes (of list[],
 // when set) of at most max_len entries: regression from the rounded targets
@@ -780,15 +839,17 @@ slm_status score_batch(slm_ctx* c, const Problem& pr, const Swarm& sw_in,
   const int cap = c->cur.cps * c->n_sm;
   Swarm sw = sw_in;
   if (sp && sp->on) {
-    // iteration t: move (t > 0) and project in one launch; the histogram
-    // kernels score x_t in pos[t & 1] and leave the next move's terms (or,
-    // with node_step, move the swarm into pos[(t + 1) & 1] themselves)
-    sw.pos = sp->pos[t & 1];
-    sw.pos_next = sp->pos[(t + 1) & 1];
-    const float* prev = sw.node_step ? sw.pos : sp->pos[t > 0 ? (t - 1) & 1 : 0];
+    // folded: iteration t's move (t > 0) and projection in one launch; the
+    // histogram kernels score x_t in pos[t & 1] and leave the next move's
+    // terms (or, with node_step, move the swarm into pos[(t + 1) & 1])
+    const float* prev = sw.pos;
+    if (sp->fold) {
+      sw.pos = sp->pos[t & 1];
+      sw.pos_next = sp->pos[(t + 1) & 1];
+      prev = sw.node_step ? sw.pos : sp->pos[t > 0 ? (t - 1) & 1 : 0];
+    }
     CK(launch(c, SLM_K_PROJECT, pairs, [&] {
-      return launch_step(pr, sw, prev, dn, A, sp->tiles, sp->n_tiles, sp->grid, sp->sh, t,
-                         c->stream);
+      return launch_step(sp->cfg, pr, sw, prev, dn, A, sp->runs, sp->n_runs, t, c->stream);
     }));
   }
   if (bp && bp->on) {
@@ -890,7 +951,7 @@ slm_status score_batch(slm_ctx* c, const Problem& pr, const Swarm& sw_in,
     }));
   // k_apso moves the adaptive swarm itself; a folded move needs only the
   // gbest step of the last evaluation
-  if (co && !sw.apso && (!(sp && sp->on) || (t == sw.T && !sw.node_step)))
+  if (co && !sw.apso && (!(sp && sp->fold) || (t == sw.T && !sw.node_step)))
     CK(launch(c, SLM_K_SWARM_UPDATE, 0.0, [&] {
       return launch_move(psw, sw, dn, A, t, *co, c->stream, hp ? hp->moved : nullptr,
                          hp ? hp->n_moved : 0);
@@ -1245,7 +1306,7 @@ struct KeyWriter {
     put(p.X); put(p.Xg); put(p.gidx); put(p.lab); put(p.y); put(p.w); put(p.E); put(p.Ez);
     put(p.d); put(p.crit); put(p.K); put(p.B); put(p.min_leaf); put(p.P); put(p.Pp);
     put(p.G); put(p.Xb); put(p.dp); put(p.m1); put(p.m2); put(p.mscale);
-    put(p.mq); put(p.mnode);
+    put(p.mq); put(p.mnode); put(p.Xt);
   }
   void swarm(const Swarm& w) {
     put(w.pos); put(w.vel); put(w.pbest); put(w.gbest); put(w.cur); put(w.pb); put(w.gb);
@@ -1253,7 +1314,7 @@ struct KeyWriter {
     put(w.T); put(w.sel); put(w.k); put(w.tk_sel); put(w.tk_inv); put(w.tk_pos);
     put(w.tk_k); put(w.tk_kp); put(w.posb); put(w.apso); put(w.ic); put(w.s2);
     put(w.co.inertia); put(w.co.c1); put(w.co.c2); put(w.co.seed); put(w.node_step);
-    put(w.n_nodes); put(w.imp); put(w.gneed);
+    put(w.n_nodes); put(w.imp); put(w.gneed); put(w.keys);
   }
 };
 
@@ -1381,82 +1442,106 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
     if (!joined) CK(cudaEventRecord(c->ev_join, st));
     c->last_node_search = S;
   }
-  // plain FP32 searches of whole batches: the move folded into the projection
+  // FP32 searches of whole batches: projected from blocked rows, the move of
+  // a plain search folded in where the batch is short
   StepPlan stp;
-  if (n_res == 0 && c->fused_step && !c->forced.pg && !bp.on && !p->apso && step_ok(pr)) {
+  if (n_res == 0 && c->fused_step && !c->forced.pg && !bp.on) {
+    // (nodes in the order of their segments: the blocks' places are disjoint)
     bool every = true;
-    for (int a = 0; a < A; ++a) every = every && nodes[a].seg_len > 0;
-    auto units = [&](int rows) {
-      int64_t u = 0;
-      for (int a = 0; a < A; ++a) u += (nodes[a].seg_len + rows - 1) / rows;
-      return u;
-    };
-    // a unit of half the particles costs half the rows' work
-    // Tile shape: the least estimated time per CTA, units per CTA x (rows
-    // per unit + a unit's fixed cost, about kStepUnitRows rows' worth:
-    // staging, z stores, range reductions), larger row tiles on ties; a
-    // short node is spread over more CTAs by smaller tiles. Every shape gives
-    // the same z (the same fused multiply-adds per z).
-    int sh = 0, grid = 0, best_tie = 0;
-    int64_t best = -1;
-    const int want = c->step_shape >= 0 && step_rows(pr, c->step_shape) <= 0 ? 0 : c->step_shape;
-    for (int k = 0; k < kStepShapeCount; ++k) {
-      const int rows = step_rows(pr, k);
-      if (rows <= 0 || (want >= 0 && k != want)) continue;
-      CK(prepare_step_kernels(pr, k));
-      const int g = step_grid(pr, k, c->n_sm);
-      if (g <= 0) continue;
-      const int sl = step_slices(pr, k);
-      const int64_t u = units(rows) * sl, runs = (u + g - 1) / g;
-      const int64_t per = runs * (rows / sl + kStepUnitRows);
-      // equal estimates: where every CTA takes one unit, the half-swarm
-      // units (each CTA moves half the particles); else the larger tiles
-      const int tie = runs == 1 ? (sl > 1 ? 0 : 1) : (sl > 1 ? 1 : 0);
-      if (best < 0 || per < best || (per == best && tie < best_tie)) {
-        best = per;
-        best_tie = tie;
-        sh = k;
-        grid = g;
+    for (int a = 0; a < A; ++a)
+      every = every && nodes[a].seg_len > 0 &&
+              (a == 0 || nodes[a].seg_start >= nodes[a - 1].seg_start + nodes[a - 1].seg_len);
+    int64_t blocks = 0;
+    for (int a = 0; a < A; ++a) blocks += (nodes[a].seg_len + 31) / 32;
+    StepConfig cfg;
+    int sh = -1, grid = 0;
+    if (every && !p->apso && step_ok(pr)) {
+      // Folding pays where the chain is latency-bound: up to kFoldMaxBlocks
+      // blocks per CTA (100,000 x 32 rows, P = 48: 28 us an iteration folded,
+      // 30 not; 1,000,000 rows: 173 and 167), and where no CTA forms two
+      // nodes' positions one after the other (a 30,011 x 50 regression tree:
+      // 22.6 ms, 23.1 when its levels of more nodes than CTAs fold too).
+      StepConfig c0;
+      step_config(pr, 0, &c0);
+      CK(prepare_step(c0));
+      const int g0 = step_grid(c0, c->n_sm);
+      const bool short_level = blocks <= (int64_t)kFoldMaxBlocks * g0 && A <= g0;
+      if (c->fused_step == 2 || short_level) {
+        StepConfig want;
+        const bool forced = c->step_shape >= 0;
+        const int f = forced && step_config(pr, c->step_shape, &want) ? c->step_shape : 0;
+        // The shape of the least estimated time: the warps' blocks one after
+        // another (8 clocks per feature and particle of a thread, and the
+        // shared-memory latency that one warp does not hide), or the SM's
+        // FP32 pipes when its warps are many; and the slice's move.
+        double best = 0.0;
+        for (int k = 0; k < kStepShapeCount; ++k) {
+          StepConfig q;
+          if ((forced && k != f) || !step_config(pr, k, &q)) continue;
+          CK(prepare_step(q));
+          const int g = step_grid(q, c->n_sm);
+          if (g <= 0) continue;
+          const int64_t units = blocks * q.slices, m = (units + g - 1) / g;
+          const int64_t ctas = std::min<int64_t>(g, units);
+          const double rounds = (double)((m + q.row_warps - 1) / q.row_warps);
+          const double per_sm = (double)m * ((ctas + c->n_sm - 1) / c->n_sm) * q.pb / 4.0;
+          const double lat = rounds * pr.d * (8.0 * q.qp + 12.0);
+          const double thr = std::max(1.0, per_sm) * pr.d * 8.0 * q.qp;
+          const double est = std::max(lat, thr) + 8.0 * q.qp * q.pb * pr.d / 10.0;
+          if (grid == 0 || est < best) {
+            best = est;
+            sh = k;
+            cfg = q;
+            grid = g;
+          }
+        }
       }
     }
-    const int rows = step_rows(pr, sh), slices = step_slices(pr, sh);
-    std::vector<WorkTile> st;
-    if (grid > 0)
-      for (int a = 0; a < A; ++a)
-        for (int q = 0; q < slices; ++q)
-          for (int r = 0; r < nodes[a].seg_len; r += rows)
-            st.push_back(WorkTile{a, nodes[a].seg_start + r, std::min(rows, nodes[a].seg_len - r),
-                                  q * (pr.Pp / slices)});
-    // Folding pays where the chain is latency-bound: a level whose
-    // projection is a few waves of units (a tree's levels of one or a few
-    // large nodes). Long projections (many nodes, or one very large node)
-    // keep the tuned projection and the separate move, where each row tile
-    // is not paired with the re-formed positions of its node. Measured in
-    // waves of the largest tile shape.
-    const int g0 = step_grid(pr, 0, c->n_sm);
-    const bool short_level = g0 > 0 && units(step_rows(pr, 0)) <= (int64_t)kFusedMaxWaves * g0;
-    if (every && grid > 0 && !st.empty() && (c->fused_step == 2 || short_level)) {
+    if (every && grid == 0 && step_config(pr, -1, &cfg, blocks / A)) {
+      CK(prepare_step(cfg));
+      grid = step_grid(cfg, c->n_sm);
+    }
+    if (grid > 0) {
+      const cudaError_t e = ensure(c->ws[S_XT], sizeof(float) * (size_t)step_rows_floats(pr, A));
+      if (e == cudaErrorMemoryAllocation) {
+        (void)cudaGetLastError();  // no room for a second copy of the rows
+        grid = 0;
+      } else {
+        CK(e);
+      }
+    }
+    if (grid > 0) {
+      const std::vector<StepRun> runs = plan_runs(nodes, cfg.slices, grid);
+      CK(ensure(c->ws[S_RUNS], sizeof(StepRun) * runs.size()));
+      CK(cudaMemcpyAsync(c->ws[S_RUNS].p, runs.data(), sizeof(StepRun) * runs.size(),
+                         cudaMemcpyHostToDevice, c->stream));
+      pr.Xt = ws_ptr<float>(c, S_XT);
+      CK(launch(c, SLM_K_GATHER, 0.0, [&] {
+        return launch_block_rows(pr, ws_ptr<WorkTile>(c, S_TILES), (int)tiles.size(),
+                                 ws_ptr<float>(c, S_XT), c->stream);
+      }));
+      stp.on = true;
+      stp.runs = ws_ptr<StepRun>(c, S_RUNS);
+      stp.n_runs = (int)runs.size();
+      stp.cfg = cfg;
+      stp.fold = sh >= 0;
+    }
+    if (stp.fold) {
       const size_t apd = (size_t)A * pr.Pp * pr.d;
       CK(ensure(c->ws[S_POS2], sizeof(float) * apd));
       CK(ensure(c->ws[S_IC], sizeof(float) * apd));
       CK(ensure(c->ws[S_S2], sizeof(float) * apd));
-      CK(ensure(c->ws[S_STILES], sizeof(WorkTile) * st.size()));
       CK(ensure(c->ws[S_IMP], sizeof(int32_t) * 2 * (size_t)A));
       CK(cudaMemsetAsync(c->ws[S_IMP].p, 0, sizeof(int32_t) * 2 * (size_t)A, c->stream));
-      CK(cudaMemcpyAsync(c->ws[S_STILES].p, st.data(), sizeof(WorkTile) * st.size(),
-                         cudaMemcpyHostToDevice, c->stream));
-      stp.on = true;
       stp.pos[0] = sw.pos;
       stp.pos[1] = ws_ptr<float>(c, S_POS2);
-      stp.tiles = ws_ptr<WorkTile>(c, S_STILES);
-      stp.n_tiles = (int)st.size();
-      stp.grid = grid;
-      stp.sh = sh;
       c->last_step_shape = sh;
       sw.ic = ws_ptr<float>(c, S_IC);
       sw.s2 = ws_ptr<float>(c, S_S2);
       sw.co = co;
       sw.imp = ws_ptr<int32_t>(c, S_IMP);
+      CK(ensure(c->ws[S_KEYS], sizeof(uint64_t) * (size_t)A * pr.Pp));
+      sw.keys = ws_ptr<uint64_t>(c, S_KEYS);
       sw.n_nodes = A;
       c->fused_searches += 1;
     }
@@ -1492,7 +1577,7 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
     cp.S = S;
     // every node scored by k_hist_cls: its last CTA per node takes the gbest
     // step and moves the swarm
-    if (stp.on && cp.on && !hp.on && c->node_step && pr.crit != SLM_MSE) sw.node_step = 1;
+    if (stp.fold && cp.on && !hp.on && c->node_step && pr.crit != SLM_MSE) sw.node_step = 1;
     c->last_split = S;
     c->cur = tl;
     c->last = tl;
@@ -1514,8 +1599,8 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
       kw.put(hp.on); kw.put(hp.large); kw.put(hp.n_large); kw.put(hp.S_large);
       kw.put(hp.pairs_large); kw.put(hp.small); kw.put(hp.n_small); kw.put(hp.pairs_small);
       kw.put(hp.moved); kw.put(hp.n_moved);
-      kw.put(stp.on); kw.put(stp.pos[1]); kw.put(stp.tiles); kw.put(stp.n_tiles);
-      kw.put(stp.grid); kw.put(cp.on); kw.put(cp.S); kw.put(cp.S_large); kw.put(cp.xtab);
+      kw.put(stp.on); kw.put(stp.fold); kw.put(stp.pos[1]); kw.put(stp.runs);
+      kw.put(stp.n_runs); kw.put(stp.cfg.fn); kw.put(stp.cfg.slices); kw.put(cp.on); kw.put(cp.S); kw.put(cp.S_large); kw.put(cp.xtab);
       if (bp.on) {
         kw.problem(bp.pr_k);
         kw.swarm(bp.sw_k);
@@ -3128,8 +3213,7 @@ slm_status slm_proposal_train(slm_ctx* c, slm_proposal* pp, const float* stats,
   slm_status s;
   if ((s = stage_in(c, stats, (size_t)n * kPropIn, c->ws[W_PS], &ds)) ||
       (s = stage_in(c, dims, (size_t)n, c->ws[W_PD], &dd)) ||
-      (s = stage_in(c, targets, (size_t)n * kPropD, c->ws[W_PT], &dt)) ||
-      (s = align16(c, &ds, (size_t)n * kPropIn, c->ws[W_PS])))
+      (s = stage_in(c, targets, (size_t)n * kPropD, c->ws[W_PT], &dt)))
     return s;
   const int b = std::min(batch, n);
   MlpWork w;

@@ -106,6 +106,9 @@ struct Problem {
   // and per node the constants of the scores formed from it (mse_kernels.cu)
   const uint32_t* mq;
   const struct MseNode* mnode;
+  // a search's rows in blocks of 32, feature-major (step_kernels.cu): node
+  // a's first block at row seg_start + 32 a; null where there are none
+  const float* Xt;
 };
 
 // One regression node's sums of both fixed-point moments and what relates
@@ -196,6 +199,9 @@ struct Swarm {
   // regression searches scored from the rounded targets: the G an edge must
   // reach to improve each particle's best (set at every pbest improvement)
   float* gneed;  // [A, Pp]
+  // folded searches: each score's loss as an ordered integer (loss_key), so
+  // that the gbest step reads 8 bytes a particle instead of its record
+  uint64_t* keys;  // [A, Pp]
 };
 
 // Adaptive PSO state of one node (Sec. III-B): evolutionary state 1..4
@@ -307,31 +313,45 @@ cudaError_t launch_hist_warp(const Problem& pr, const Swarm& sw, const NodeDesc*
 cudaError_t launch_apso(const Problem& pr, const Swarm& sw, const NodeDesc* nodes, int A,
                         int t, SwarmCoef co, cudaStream_t st, const int32_t* list = nullptr,
                         int n_list = 0);
-// The projection of iteration t with the swarm move folded in (classification
-// or MSE searches in the FP32 form): for t > 0 every CTA first takes the gbest
+// The projection of iteration t from blocked rows (pr.Xt, step_kernels.cu).
+// Folded (StepConfig of a shape): for t > 0 every CTA first takes the gbest
 // step of evaluation t - 1 of each node it projects (the rule of k_move) and
-// forms the node's positions x_t = x + (ic + s2 (gB - x)) from pos_prev (the
-// positions of t - 1) in shared memory; the CTA holding the node's first row
-// tile writes x_t to sw.pos, v_t to sw.vel and the gbest records. Then z and
-// the ranges of every (row tile, all particles) unit, as k_project (the same
-// fused multiply-adds). tiles: for every node in order, for each of its
-// step_slices(pr, sh) particle slices (WorkTile::pad = the slice's first
-// particle), its step_rows(pr, sh)-row tiles; every node with at least one.
-// sh picks the tile shape (0: the largest row tile with every particle;
-// 1, 2: smaller row tiles; 3-5: the same with half the particles per unit;
-// step_rows 0 when the swarm width has no such shape). The gbest step of
-// the last evaluation is left to launch_move(t = T). With sw.node_step the
-// histogram kernel has moved the swarm already: k_step loads the positions
-// of t from pos_prev.
+// forms its slice's positions x_t = x + (ic + s2 (gB - x)) from pos_prev (the
+// positions of t - 1) in shared memory; the CTA holding a slice's first block
+// writes x_t to sw.pos, v_t to sw.vel and (slice 0) the gbest records. With
+// sw.node_step the histogram kernel has moved the swarm already: the positions
+// of t come from pos_prev. The gbest step of the last evaluation is left to
+// launch_move(t = T). Not folded (sh = -1): the positions are sw.pos. Then z
+// and the ranges of every (block, slice), as k_project (the same fused
+// multiply-adds). runs[n_runs]: each CTA's blocks, a contiguous run in (node,
+// slice, block) order starting at block blk of (node, slice), count >= 1
+// blocks over following slices and nodes; every node has at least one row.
+struct StepRun {
+  int32_t node, slice, blk, count;
+};
 constexpr int kStepShapeCount = 6;
+struct StepConfig {
+  const void* fn = nullptr;
+  int qp = 0, pb = 0;     // particles per thread, warps sharing a slice
+  int slices = 1;         // of 8 qp pb particles each
+  int row_warps = 0;      // blocks a CTA takes at a time
+  int threads = 0;
+  size_t smem = 0;
+};
 bool step_ok(const Problem& pr);
-int step_rows(const Problem& pr, int sh);
-int step_slices(const Problem& pr, int sh);
-int step_grid(const Problem& pr, int sh, int n_sm);
-cudaError_t prepare_step_kernels(const Problem& pr, int sh);
-cudaError_t launch_step(const Problem& pr, const Swarm& sw, const float* pos_prev,
-                        const NodeDesc* nodes, int A, const WorkTile* tiles, int n_tiles,
-                        int grid, int sh, int t, cudaStream_t st);
+// Shape sh (0 .. 5) of the folded projection, or (sh = -1) the unfolded one
+// for nodes of about `blocks` blocks of 32 rows.
+bool step_config(const Problem& pr, int sh, StepConfig* c, int64_t blocks = 1 << 20);
+cudaError_t prepare_step(const StepConfig& c);
+int step_grid(const StepConfig& c, int n_sm);
+// Blocked rows of A nodes: the array's floats; filled from pr.X (tiles: the
+// nodes' kTS-row tiles).
+int64_t step_rows_floats(const Problem& pr, int A);
+cudaError_t launch_block_rows(const Problem& pr, const WorkTile* tiles, int n_tiles, float* Xt,
+                              cudaStream_t st);
+cudaError_t launch_step(const StepConfig& c, const Problem& pr, const Swarm& sw,
+                        const float* pos_prev, const NodeDesc* nodes, int A, const StepRun* runs,
+                        int n_runs, int t, cudaStream_t st);
 // gbest step of iteration t and (t < T) the Eq. pso-1 move of every particle
 // of A nodes to iteration t+1 (of the n_list nodes list[] names, when set).
 cudaError_t launch_move(const Problem& pr, const Swarm& sw, const NodeDesc* nodes,

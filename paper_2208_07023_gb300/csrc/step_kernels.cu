@@ -1,37 +1,40 @@
-// One iteration's projection of the FP32 swarm search with the swarm move
-// folded in (Sec. III-A, Eq. pso-1 and Algorithm 1; Sec. II-A, Eq. 1).
+// The projection z = X_node . x_p of a search's iteration (Sec. II-A, Eq. 1)
+// from blocked rows, with the swarm move folded in (Sec. III-A, Eq. pso-1 and
+// Algorithm 1) or from positions a separate kernel moved.
 //
-// A search iteration t is two launches: k_step (gbest step of evaluation t-1,
-// the move to x_t, z = X_node . x_t and the per-particle ranges) and a
+// Blocked rows. A search reads its rows T + 1 times, so they are laid out once
+// for these reads (k_block_rows): blocks of 32 rows of one node, feature-major
+// ([d][32] floats, rows past the node zero), node a's first block at row
+// seg_start + 32 a of the array. A block streams through shared memory as
+// whole 2 KB chunks without an address computed per row, whatever d is, and a
+// thread's four consecutive rows at one feature are one 16-byte word: two
+// pairs of rows for the packed FP32 multiply-add (fma.rn.f32x2: two
+// independent FMAs, each rounded as fmaf; half the issue slots, which with
+// shared-memory reads and address arithmetic were what bounded the earlier
+// row-major kernel, at 2.2 instructions per FMA).
+//
+// Units. A warp takes a block and the 8 QP particles of a slice (thread tile 8
+// rows x QP particles: every x pair meets QP particles, every position 8 rows),
+// or PB warps share the slice. A CTA takes a contiguous run of blocks in
+// (node, slice, block) order, so its warps read one set of positions, in
+// shared memory, feature-major. Every z is the sequential fused multiply-add
+// over the features in increasing order, for every shape.
+//
+// Fold. An iteration t of a folded search is two launches: k_step (gbest step
+// of evaluation t-1, the move to x_t, z and the per-particle ranges) and a
 // histogram kernel (bins, threshold scan, pbest step, and the gB-independent
-// terms of the next move). k_step's unit is one tile of rows of one node with
-// ALL of the node's particles, so every row tile is read from L2 once per
-// iteration; the node's positions live in shared memory for the whole unit.
-//
-// The move needs gB, which needs every particle's score, so it cannot run in
-// the histogram kernel that produces those scores. Every CTA that projects a
-// node therefore takes the node's gbest step itself (a warp argmin over P
-// scores) and forms the node's new positions from the terms the histogram
-// kernel left: x' = x + (ic + s2 (gB - x)), three operations per element. The
-// CTA holding the node's first row tile writes x' and v' back (into the
-// other of two position buffers, so the other CTAs still read x) together
-// with the gbest records, exactly as k_move would.
-//
-// Each CTA of the persistent grid takes a contiguous run of units; it forms a
-// node's positions once for all its consecutive units of that node. The row
-// tiles stream through a ring of shared-memory stages (the copies of the next
-// NS - 1 feature chunks in flight, one barrier per chunk), and a finished
-// unit's z leaves through per-warp staging rows, so that each store writes
-// whole 128-byte rows of a particle.
-//
-// Thread tile: 4 rows (sg + 8i) x PJ particles (pg + 4j) per thread; a warp
-// covers 32 rows x 4 PJ particles; the CTA's 8 warps are RB = 8 / PB row
-// blocks x PB particle blocks, so a unit is 32 RB rows x 4 PJ PB = Pp
-// particles. Every z is the sequential fused multiply-add over the features
-// of k_project (bit-identical results).
+// terms of the next move). The move needs gB, which needs every particle's
+// score, so every CTA that projects a node takes the node's gbest step itself
+// (a warp argmin over P scores) and forms its slice's new positions from the
+// terms the histogram kernel left: x' = x + (ic + s2 (gB - x)). The CTA
+// holding the slice's first block writes x' and v' back (into the other of two
+// position buffers, so the other CTAs still read x), and slice 0's the gbest
+// records, exactly as k_move would.
 #include <cuda_runtime.h>
 #include <float.h>
 #include <limits.h>
+
+#include <algorithm>
 
 #include "device_util.cuh"
 #include "slm_internal.cuh"
@@ -39,497 +42,750 @@
 namespace slm {
 namespace {
 
-constexpr int kStepMaxPosBytes = 96 * 1024;  // the node's positions in shared memory
-// Floats per particle of a warp's z staging rows: 32 rows and 8 of padding,
-// so that the four particles a warp stages fall on distinct banks.
-constexpr int kZS = 40;
+constexpr int kStepMaxPosBytes = 96 * 1024;  // a slice's positions in shared memory
+constexpr int kBR = 32;                      // rows of a block
+constexpr int kSC = 16;                      // features of a staged chunk (2 KB)
+constexpr int kStepStages = 3;               // a warp's ring of chunks
+// Warps of a CTA and registers of a thread. Folded: one CTA per SM, so that a
+// node's positions and move terms (48 KB at P = d = 64) are read once per SM;
+// 120 registers leave room for the histogram kernel's CTAs beside it, whose
+// programmatic launch then overlaps (8 warps, two CTAs per SM: the
+// 50,000 x 64 tree 17.5 ms instead of 15.9). Unfolded: two CTAs per SM, so
+// that one's change of node overlaps the other's products, with small rings:
+// the carveout they leave to L1 is the one the histogram kernel beside them
+// runs with, and its entries' labels and targets hit there (with 96 KB rings
+// two SLM Boost rounds took 83 ms instead of 72).
+constexpr int kFoldWarps = 12, kProjWarps = 8;
+constexpr int kFoldRegs = 120, kFoldRegsWide = 152, kProjRegs = 128;  // wide: QP > 6
 
-// Positions in shared memory, chunk-major: feature j of particle p at
-// (j / kKC) * Pp * kXS + p * kXS + j % kKC, so that the particles a thread
-// reads sit at compile-time offsets and the four particles a warp reads at
-// one feature fall on distinct banks (rows kXS = 36 floats apart). Features
-// past d and particles past P stay zero.
-__host__ __device__ inline size_t step_pos_floats(int Pp, int d) {
-  return (size_t)((d + kKC - 1) / kKC) * Pp * kXS;
+// Two packed FP32 fused multiply-adds, each rounded to nearest like fmaf.
+__device__ __forceinline__ void fma2(uint64_t& c, uint64_t a, uint64_t b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;\n" : "+l"(c) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;\n" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};\n" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+// (lo, hi) -> (hi, lo)
+__device__ __forceinline__ uint64_t swap2(uint64_t v) {
+  const float2 f = unpack2(v);
+  return pack2(f.y, f.x);
 }
 
-// Row-tile stages in the ring: the copies of the next NS - 1 steps are in
-// flight while a step computes (fewer for the larger row tiles, so that two
-// CTAs still fit on an SM).
-__host__ __device__ constexpr int step_stages(int RT) { return RT <= 64 ? 4 : RT <= 128 ? 3 : 2; }
+// Where particle r (0 .. 8 QP - 1) of a warp's slice sits in the row of
+// feature k. Lane group g (8 of them) owns particles 4g .. 4g + 3 of the
+// first 32 and W g .. W g + W - 1 of the rest (W = QP - 4, or QP below 4);
+// the groups' words are permuted by a key that changes every four features,
+// so that the 16-byte move stores of one particle's features spread over the
+// banks while a warp's reads at one feature stay distinct.
+template <int QP>
+__device__ __forceinline__ int pos_slot(int r, int k) {
+  const int key = (k >> 2) & 7;
+  if (QP >= 4 && r < 32) return (((r >> 2) ^ key) << 2) + (r & 3);
+  constexpr int W = QP >= 4 ? (QP > 4 ? QP - 4 : 1) : QP, B0 = QP >= 4 ? 32 : 0;
+  const int q = r - B0;
+  return B0 + ((q / W) ^ key) * W + q % W;
+}
 
-template <int PJ, int PB>
-__global__ void __launch_bounds__(kThreads, 2)
-    k_step(Problem pr, Swarm sw, const float* __restrict__ pos_prev,
-           const NodeDesc* __restrict__ nodes, int A, const WorkTile* __restrict__ tiles,
-           int n_units, int t) {
-  constexpr int RB = 8 / PB;   // 32-row blocks of a unit
-  constexpr int RT = 32 * RB;  // rows of a unit
-  constexpr int PPB = 4 * PJ;  // particles of a particle block
-  constexpr int PU = PPB * PB;  // particles of a unit (a slice of the swarm, or all of it)
-  constexpr int NS = step_stages(RT);
-  static_assert(PJ % 2 == 0 && RB * PB == 8 && NS >= 2, "tile shape");
+// The blocked rows; one CTA per 256-row tile (which starts a multiple of 256
+// rows into its node), a warp per block.
+__global__ void __launch_bounds__(256)
+    k_block_rows(const float* __restrict__ X, int d, const WorkTile* __restrict__ tiles,
+                 float* __restrict__ Xt) {
+  __shared__ float s[8][32][33];
+  const WorkTile wt = tiles[blockIdx.x];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int r0 = warp * 32;
+  if (r0 >= wt.rows) return;
+  const int nr = min(32, wt.rows - r0);
+  float* out = Xt + ((int64_t)wt.row0 + r0 + 32 * (int64_t)wt.node) * d;
+  for (int k0 = 0; k0 < d; k0 += 32) {
+    const int kc = min(32, d - k0);
+#pragma unroll 8
+    for (int r = 0; r < 32; ++r) {
+      float v = 0.0f;
+      if (r < nr && lane < kc) v = __ldg(X + ((int64_t)wt.row0 + r0 + r) * d + k0 + lane);
+      s[warp][r][lane] = v;
+    }
+    __syncwarp();
+#pragma unroll 8
+    for (int k = 0; k < 32; ++k)
+      if (k < kc) out[(int64_t)(k0 + k) * 32 + lane] = s[warp][lane][k];
+    __syncwarp();
+  }
+}
+
+template <int QP, int PB, bool FOLD>
+__global__ void __launch_bounds__(32 * (FOLD ? kFoldWarps : kProjWarps))
+    __maxnreg__(FOLD ? (QP > 6 ? kFoldRegsWide : kFoldRegs) : kProjRegs) k_step(Problem pr, Swarm sw, const float* pos_prev, const NodeDesc* __restrict__ nodes, int A,
+           const StepRun* __restrict__ runs, int n_slices, uint32_t inv_d, int t) {
+  constexpr int NW = FOLD ? kFoldWarps : kProjWarps, NT = 32 * NW;
+  constexpr int PW = 8 * QP;             // particles of a warp
+  constexpr int PU = PW * PB;            // particles of a slice
+  constexpr int RB = NW / PB;            // row warps
+  constexpr int NS = kStepStages;
+  constexpr int TF = FOLD ? 8 : 16;      // features of an unrolled turn
+  constexpr int W = QP >= 4 ? QP - 4 : QP;  // particles per lane beyond the first four
+  static_assert(RB * PB == NW && QP >= 1 && QP <= 8 && PU <= 64, "tile shape");
   extern __shared__ __align__(16) float sm[];
-  __shared__ int s_lo[64], s_hi[64];  // ordered-int range of each particle
+  __shared__ int s_lo[64], s_hi[64];  // ordered-int range of each particle of the slice
   __shared__ int s_best;
   const int d = pr.d, Pp = pr.Pp, P = pr.P;
-  float* xs = sm;                                   // [NS][RT][kXS] row-tile stages
-  float* ps = sm + NS * RT * kXS;                   // the node's positions, chunk-major
-  float* gs = ps + step_pos_floats(Pp, d);          // the node's gB (d floats, padded to 4)
-  float* zst = gs + ((d + 3) & ~3);                 // [8 warps][4][kZS] z staging rows
-  pdl_trigger();
-  const int nk = (d + kKC - 1) / kKC;
-  const int cstride = Pp * kXS;   // floats per feature chunk of the positions
-  const bool vec = (d & 3) == 0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int sg = lane & 7, pg = lane >> 3;
-  const int rb = warp % RB, pbk = warp / RB;
-  // a contiguous run of units per CTA (the tiles are in node order), so that
-  // consecutive units of a CTA mostly share a node and its moved positions
-  const int u0 = (int)(((int64_t)blockIdx.x * n_units) / gridDim.x);
-  const int my_units = (int)(((int64_t)(blockIdx.x + 1) * n_units) / gridDim.x) - u0;
-  const int n_st = my_units * nk;
+  const int rg = lane & 3, pg = lane >> 2;  // rows 4 rg.. and 16 + 4 rg..; particle group
+  // (rotated by CTA, so that the warps that take one block more fall on
+  // different schedulers of an SM)
+  const int rw = (warp + blockIdx.x) % RB, pbk = warp / RB;
+  float* xs = sm + warp * (NS * kSC * kBR);           // this warp's ring of chunks
+  float* ps = sm + NW * NS * kSC * kBR;               // [PB][d][PW] positions
+  float* gs = ps + (size_t)PU * d;                    // the node's gB (d floats)
+  pdl_trigger();
+  const StepRun run = runs[blockIdx.x];
+  const int nk = (d + kSC - 1) / kSC;
 
-  // rows of step s (unit s / nk, feature chunk s % nk) into its ring stage;
-  // rows past the tile and features past d arrive as zeros. One commit group
-  // per step, empty past the last.
-  auto stage = [&](int s) {
-    if (s < n_st) {
-      float* xb = xs + (s % NS) * (RT * kXS);
-      const int ui = s / nk, c = s - ui * nk;
-      const WorkTile wt = tiles[u0 + ui];
-      const int k0 = c * kKC, kc = min(kKC, d - k0);
-      if (vec) {
-        for (int q = threadIdx.x; q < RT * (kKC / 4); q += kThreads) {
-          const int r = q >> 3, cc = (q & 7) * 4;
-          const bool ok = r < wt.rows && cc < kc;
-          const float* src = ok ? row_of(pr, wt.row0 + r) + k0 + cc : pr.X;
-          cp_async16(xb + r * kXS + cc, src, ok ? 16 : 0);
-        }
-      } else {
-        for (int q = threadIdx.x; q < RT * kKC; q += kThreads) {
-          const int r = q >> 5, cc = q & 31;
-          const bool ok = r < wt.rows && cc < kc;
-          const float* src = ok ? row_of(pr, wt.row0 + r) + k0 + cc : pr.X;
-          cp_async4(xb + r * kXS + cc, src, ok ? 4 : 0);
-        }
+  // ---- the warp's chunks in order: blocks rw, rw + RB, ... of each (node,
+  // slice) of the run, the features of a block in chunks
+  int f_node = run.node, f_slice = run.slice, f_left = run.count;
+  int f_b = 0, f_end = 0;         // the open (node, slice)'s next block and end
+  const float* f_src = pr.Xt;     // this lane's place in the open block's next chunk
+  int f_rem = 0;                  // floats of the block from there on
+  const int blk_floats = kBR * d;
+  auto f_open = [&](int first) {  // blocks of the open (node, slice)
+    const NodeDesc nd = nodes[f_node];
+    const int nb = (nd.seg_len + kBR - 1) / kBR;
+    const int take = min(f_left, nb - first);
+    f_b = first + rw;
+    f_end = first + take;
+    f_left -= take;
+    f_src = pr.Xt + ((int64_t)nd.seg_start + 32 * (int64_t)f_node + (int64_t)f_b * kBR) * d +
+            4 * lane;
+    f_rem = blk_floats - 4 * lane;
+  };
+  f_open(run.blk);
+  float* f_dst = xs + 4 * lane;
+  float* const f_dst_end = f_dst + NS * kSC * kBR;
+  auto stage = [&] {
+    while (f_b >= f_end && f_left > 0) {  // the next (node, slice)
+      if (++f_slice == n_slices) {
+        f_slice = 0;
+        ++f_node;
+      }
+      f_open(0);
+    }
+    if (f_b < f_end) {
+#pragma unroll
+      for (int i = 0; i < kSC * kBR / 128; ++i)
+        if (f_rem > 128 * i) cp_async16(f_dst + 128 * i, f_src + 128 * i, 16);
+      f_src += kSC * kBR;
+      f_rem -= kSC * kBR;
+      if (f_rem + 4 * lane <= 0) {  // (the same for every lane) the next block
+        const int used = blk_floats - 4 * lane - f_rem;
+        f_b += RB;
+        f_src += (int64_t)RB * blk_floats - used;
+        f_rem += used;
       }
     }
     cp_async_commit();
+    f_dst += kSC * kBR;
+    if (f_dst == f_dst_end) f_dst -= NS * kSC * kBR;
   };
 
   if (threadIdx.x < 64) {
     s_lo[threadIdx.x] = INT_MAX;
     s_hi[threadIdx.x] = INT_MIN;
   }
-  // Within a search the rows and tiles are written before the first
+  // Within a search the blocked rows and runs are written before the first
   // iteration's launch, so iterations t > 0 start fetching them before the
   // previous kernel's results are visible.
   if (t > 0)
-    for (int s = 0; s < NS - 1; ++s) stage(s);
-  // padding features and particles of the positions stay zero
-  for (int i = threadIdx.x; i < nk * cstride; i += kThreads) ps[i] = 0.0f;
+#pragma unroll 1
+    for (int s = 0; s < NS - 1; ++s) stage();
+  // positions of particles past the swarm stay zero
+  for (int i = threadIdx.x; i < PU * d; i += NT) ps[i] = 0.0f;
+  touch(sw.pos);
+  touch(sw.z);
+  touch(sw.zmm);
+  touch(sw.node_step);
+  if (FOLD) {
+    touch(pos_prev);
+    touch(sw.vel);
+    touch(sw.gbest);
+    touch(sw.cur);
+    touch(sw.gb);
+    touch(sw.trace);
+    touch(sw.ic);
+    touch(sw.s2);
+    touch(sw.imp);
+    touch(sw.keys);
+  }
+  touch(pr.crit);
+  touch((int)pr.Ez);
+  __syncthreads();
   pdl_wait();
   if (t == 0)
-    for (int s = 0; s < NS - 1; ++s) stage(s);
+#pragma unroll 1
+    for (int s = 0; s < NS - 1; ++s) stage();
 
-  // The positions of node a for iteration t in ps (and, from the CTA that
-  // holds the node's first row tile, in sw.pos / sw.vel with the gbest
-  // records of evaluation t - 1).
-  // desig: this CTA holds the first row tile of its slice (particles pg0 ..
-  // pg0 + PU - 1) of node a; the slice's positions go back to memory from
-  // there, and the node's gbest records from slice 0's
+  // A slice's rows [particle][feature] start on 16 bytes whatever d is (its
+  // first particle is a multiple of 8) and are read and moved four words at a
+  // time; with d % 4 == 0 the four belong to one particle. f / d of a word
+  // index f < 2^17 by the launcher's factor.
+  const bool vec = (d & 3) == 0;
+  auto quot = [](int e, uint32_t inv) { return inv ? (int)__umulhi((uint32_t)e, inv) : e; };
+  auto put = [&](int pl, int k, float v) {  // particle pl of the slice
+    const int pb = pl / PW;
+    ps[(pb * d + k) * PW + pos_slot<QP>(pl - pb * PW, k)] = v;
+  };
+  // words 4 e .. 4 e + 3 of the slice's rows, np particles
+  auto put4 = [&](int e, int np, const float4& v) {
+    int pl = quot(4 * e, inv_d), j = 4 * e - pl * d;
+    if (vec) {
+      put(pl, j, v.x);
+      put(pl, j + 1, v.y);
+      put(pl, j + 2, v.z);
+      put(pl, j + 3, v.w);
+      return;
+    }
+    const float w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      if (pl < np) put(pl, j, w[c]);
+      if (++j == d) {
+        j = 0;
+        ++pl;
+      }
+    }
+  };
+
+  // The positions of node a's slice (particles pg0 .. pg0 + PU - 1) for
+  // iteration t in ps; desig: this CTA holds the slice's first block.
   auto node_positions = [&](int a, int pg0, bool desig) {
     const int64_t nb = (int64_t)a * Pp * d;
-    const bool desig0 = desig && pg0 == 0;
-    const int p_lo = min(pg0, P), p_hi = min(P, pg0 + PU);  // the slice's particles
-    if (t == 0 || sw.node_step) {  // the histogram kernel moved the swarm
-      for (int e = threadIdx.x; e < P * d; e += kThreads) {
-        const int p = e / d, j = e - p * d;
-        ps[(j / kKC) * cstride + p * kXS + j % kKC] = pos_prev[nb + e];
-      }
+    const int np = min(P, pg0 + PU) - pg0;  // the slice's particles
+    const int64_t o0 = nb + (int64_t)pg0 * d;
+    const int n4 = (np * d + 3) >> 2;
+    if (!FOLD || t == 0 || sw.node_step) {  // another kernel moved the swarm
+      const float* src = (FOLD ? pos_prev : sw.pos) + o0;
+#pragma unroll 4
+      for (int e = threadIdx.x; e < n4; e += NT)
+        put4(e, np, __ldcg(reinterpret_cast<const float4*>(src) + e));
       __syncthreads();
       return;
     }
-    // Positions of t - 1 go by asynchronous copies straight into ps (moved
-    // there in place) and the recorded gB into gs; the move terms to
-    // registers; all before the gbest step. After a gbest change gB is the
-    // new best particle's position of t - 1 (it beat every pbest, so its own
-    // pbest became that position), which ps then holds: the move needs
-    // nothing more from global memory.
-    const int d4 = d >> 2, items = vec ? P * d4 : 0;
-    // the slice's elements (the positions of every particle are copied: gB
-    // may be any particle's)
-    const int e_lo = vec ? p_lo * d4 : 0, e_hi = vec ? p_hi * d4 : 0;
-    if (vec) {
-      for (int e = threadIdx.x; e < items; e += kThreads) {
-        const int p = e / d4, j = 4 * (e - p * d4);
-        cp_async16(ps + (j / kKC) * cstride + p * kXS + j % kKC, pos_prev + nb + 4 * (int64_t)e,
-                   16);
-      }
-      for (int q = threadIdx.x; q < d4; q += kThreads)
-        cp_async16(gs + 4 * q, sw.gbest + (int64_t)a * d + 4 * q, 16);
-      cp_async_commit();
-    }
-    // the move terms: every element of the thread in flight at once when
-    // they fit kPre float4 per thread, else two at a time
-    constexpr int kPre = 4;
-    const bool pre = e_hi - e_lo <= kPre * kThreads;
-    float4 ia[kPre], sa[kPre];
-    auto load_terms = [&](int e0, int n) {
-#pragma unroll
-      for (int u = 0; u < kPre; ++u) {
-        const int e = e0 + u * kThreads;
-        if (u < n && e < e_hi) {
-          const int64_t o = nb + 4 * (int64_t)e;  // element (p, 4q) of the node's rows
-          ia[u] = __ldcg(reinterpret_cast<const float4*>(sw.ic + o));
-          sa[u] = __ldcg(reinterpret_cast<const float4*>(sw.s2 + o));
-        }
-      }
-    };
-    load_terms(e_lo + threadIdx.x, pre ? kPre : 2);
-    // gbest step of evaluation t - 1 (k_move's rule and double buffering),
-    // its inputs loaded together: the node's scores (two per lane), the
-    // improvement flag and the recorded gbest score
-    if (warp == 0) {
-      const EvalRes* cur = sw.cur + (int64_t)a * Pp;
-      const EvalRes e0 = lane < P ? cur[lane] : invalid_res();
-      const EvalRes e1 = lane + 32 < P ? cur[lane + 32] : invalid_res();
-      // the argmin only when a particle beat gB in evaluation t - 1 (every
-      // particle is a candidate at evaluation 0)
-      const bool any = t == 1 || !sw.imp || __ldcg(sw.imp + (int64_t)((t - 1) & 1) * A + a) != 0;
-      const EvalRes gold = sw.gb[(int64_t)(t & 1) * A + a];
-      EvalRes be = gold;
-      int bi = -1;
-      if (any) {
-        int ci = -1;
-        EvalRes ce = invalid_res();
-        if (lane < P) gbest_consider(pr, gold, t - 1, lane, e0, &ci, &ce);
-        if (lane + 32 < P) gbest_consider(pr, gold, t - 1, lane + 32, e1, &ci, &ce);
-        bi = gbest_select(pr, ci, ce, &be);
-      }
-      if (lane == 0) {
-        s_best = bi;
-        if (desig0 && sw.imp) sw.imp[(int64_t)(t & 1) * A + a] = 0;  // evaluation t's flag
-        if (desig0) {
-          const EvalRes g = bi >= 0 ? be : gold;
-          sw.gb[(int64_t)((t - 1) & 1) * A + a] = g;
-          if (bi >= 0) {
-            sw.gpart[a] = bi;
-            sw.giter[a] = t - 1;
-          }
-          if (sw.trace)
-            sw.trace[(int64_t)a * (sw.T + 1) + (t - 1)] =
-                g.valid ? g.loss : __longlong_as_double(0x7ff0000000000000LL);
-        }
-      }
-    }
-    if (vec) cp_async_wait<0>();
-    __syncthreads();
-    const int bi = s_best;
-    if (vec) {
-      // gB into gs before any position is overwritten
-      if (bi >= 0)
-        for (int j = threadIdx.x; j < d; j += kThreads)
-          gs[j] = ps[(j / kKC) * cstride + bi * kXS + j % kKC];
-      __syncthreads();
-      if (desig0 && bi >= 0)
-        for (int j = threadIdx.x; j < d; j += kThreads) sw.gbest[(int64_t)a * d + j] = gs[j];
-      // x' = x + (ic + s2 (gB - x)), v' = ic + s2 (gB - x), one rounding each
-      auto move4 = [&](int e, const float4& ic, const float4& s2) {
-        const int p = e / d4, j = 4 * (e - p * d4);
-        float* xp = ps + (j / kKC) * cstride + p * kXS + j % kKC;
-        const float4 x = *reinterpret_cast<const float4*>(xp);
-        const float4 g = *reinterpret_cast<const float4*>(gs + j);
-        float4 vn, xn;
-        vn.x = __fadd_rn(ic.x, __fmul_rn(s2.x, __fsub_rn(g.x, x.x)));
-        vn.y = __fadd_rn(ic.y, __fmul_rn(s2.y, __fsub_rn(g.y, x.y)));
-        vn.z = __fadd_rn(ic.z, __fmul_rn(s2.z, __fsub_rn(g.z, x.z)));
-        vn.w = __fadd_rn(ic.w, __fmul_rn(s2.w, __fsub_rn(g.w, x.w)));
-        xn.x = __fadd_rn(x.x, vn.x);
-        xn.y = __fadd_rn(x.y, vn.y);
-        xn.z = __fadd_rn(x.z, vn.z);
-        xn.w = __fadd_rn(x.w, vn.w);
-        if (desig) {
-          const int64_t o = nb + 4 * (int64_t)e;
-          *reinterpret_cast<float4*>(sw.pos + o) = xn;
-          *reinterpret_cast<float4*>(sw.vel + o) = vn;
-        }
-        *reinterpret_cast<float4*>(xp) = xn;
-      };
-      if (pre) {
+    if constexpr (FOLD) {
+      const bool desig0 = desig && pg0 == 0;
+      // All inputs in flight before any is used: the slice's positions of
+      // t - 1 and move terms, the recorded gB, and (warp 0) the node's scores
+      // (two per lane), improvement flag and gbest score.
+      constexpr int kPre = 3;
+      float4 xa[kPre], ia[kPre], sa[kPre];
+      auto load_terms = [&](int e0) {
 #pragma unroll
         for (int u = 0; u < kPre; ++u) {
-          const int e = e_lo + threadIdx.x + u * kThreads;
-          if (e < e_hi) move4(e, ia[u], sa[u]);
-        }
-      } else {
-        for (int e0 = e_lo + threadIdx.x; e0 < e_hi; e0 += 2 * kThreads) {
-          if (e0 != e_lo + (int)threadIdx.x) load_terms(e0, 2);
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int e = e0 + u * kThreads;
-            if (e < e_hi) move4(e, ia[u], sa[u]);
+          const int e = e0 + u * NT;
+          if (e < n4) {
+            xa[u] = __ldcg(reinterpret_cast<const float4*>(pos_prev + o0) + e);
+            ia[u] = __ldcg(reinterpret_cast<const float4*>(sw.ic + o0) + e);
+            sa[u] = __ldcg(reinterpret_cast<const float4*>(sw.s2 + o0) + e);
           }
         }
-      }
-    } else {
-      // a new best improved its pbest in evaluation t - 1: gB is that row
-      const float* gsrc = bi >= 0 ? sw.pbest + nb + (int64_t)bi * d : sw.gbest + (int64_t)a * d;
-      if (desig0 && bi >= 0)
-        for (int j = threadIdx.x; j < d; j += kThreads) sw.gbest[(int64_t)a * d + j] = gsrc[j];
-      for (int e = p_lo * d + (int)threadIdx.x; e < p_hi * d; e += kThreads) {
-        const int p = e / d, j = e - p * d;
-        const int64_t o = nb + e;
-        const float x = pos_prev[o];
-        const float vn = __fadd_rn(sw.ic[o], __fmul_rn(sw.s2[o], __fsub_rn(gsrc[j], x)));
-        const float xn = __fadd_rn(x, vn);
-        if (desig) {
-          sw.pos[o] = xn;
-          sw.vel[o] = vn;
+      };
+      const float* gb_row = sw.gbest + (int64_t)a * d;
+      if (warp == 0) {
+        // gbest step of evaluation t - 1 (k_move's rule and double
+        // buffering): nothing when no particle beat gB in evaluation t - 1;
+        // else the particle of the smallest loss key where that decides (no
+        // other within 8 ulps of it, nor gB), else by the exact records
+        const EvalRes* cur = sw.cur + (int64_t)a * Pp;
+        const EvalRes* gold_at = sw.gb + (int64_t)(t & 1) * A + a;
+        const int flag =
+            t == 1 || !sw.imp ? 1 : __ldcg(sw.imp + (int64_t)((t - 1) & 1) * A + a);
+        const uint64_t* kp = sw.keys + (int64_t)a * Pp;
+        const uint64_t k0 = lane < P ? __ldcg(kp + lane) : ~0ull;
+        const uint64_t k1 = lane + 32 < P ? __ldcg(kp + lane + 32) : ~0ull;
+        const double gl = __ldcg(&gold_at->loss);
+        const int gv = __ldcg(&gold_at->valid);
+        load_terms(threadIdx.x);
+        int bi = -1;
+        if (flag != 0) {
+          const uint64_t km = k0 < k1 ? k0 : k1;
+          const uint32_t h = __reduce_min_sync(0xffffffffu, (uint32_t)(km >> 32));
+          const uint32_t l = __reduce_min_sync(
+              0xffffffffu, (uint32_t)(km >> 32) == h ? (uint32_t)km : 0xffffffffu);
+          const uint64_t kmin = ((uint64_t)h << 32) | l;
+          const uint64_t near = kmin > ~0ull - 8 ? ~0ull : kmin + 8;
+          const unsigned n0 = __ballot_sync(0xffffffffu, k0 <= near);
+          const unsigned n1 = __ballot_sync(0xffffffffu, k1 <= near);
+          const uint64_t kg = gv ? loss_key(gl) : ~0ull;
+          if (t > 1 && __popc(n0) + __popc(n1) == 1 && near < kg) {
+            bi = n0 ? __ffs(n0) - 1 : 31 + __ffs(n1);
+          } else {
+            const EvalRes gold = ldcg_res(gold_at);
+            int ci = -1;
+            EvalRes ce = invalid_res(), be = gold;
+            for (int p = lane; p < P; p += 32)
+              gbest_consider(pr, gold, t - 1, p, ldcg_res(cur + p), &ci, &ce);
+            bi = gbest_select(pr, ci, ce, &be);
+          }
         }
-        ps[(j / kKC) * cstride + p * kXS + j % kKC] = xn;
+        if (lane == 0) {
+          s_best = bi;
+          if (desig0) {
+            if (sw.imp) sw.imp[(int64_t)(t & 1) * A + a] = 0;  // evaluation t's flag
+            const EvalRes g = ldcg_res(bi >= 0 ? cur + bi : gold_at);
+            sw.gb[(int64_t)((t - 1) & 1) * A + a] = g;
+            if (bi >= 0) {
+              sw.gpart[a] = bi;
+              sw.giter[a] = t - 1;
+            }
+            if (sw.trace)
+              sw.trace[(int64_t)a * (sw.T + 1) + (t - 1)] =
+                  g.valid ? g.loss : __longlong_as_double(0x7ff0000000000000LL);
+          }
+        }
+      } else {
+        load_terms(threadIdx.x);
+        for (int j = threadIdx.x - 32; j < d; j += NT - 32) gs[j] = __ldcg(gb_row + j);
       }
+      __syncthreads();
+      // After a gbest change gB is the new best particle's position of t - 1
+      // (it beat every pbest, so its own pbest became that position).
+      const int bi = s_best;
+      if (bi >= 0) {
+        if (n4 <= kPre * NT && bi >= pg0 && bi < pg0 + np && vec) {
+#pragma unroll
+          for (int u = 0; u < kPre; ++u) {  // from the thread that holds it
+            const int e = threadIdx.x + u * NT, j = 4 * e - (bi - pg0) * d;
+            if (e < n4 && j >= 0 && j < d) {
+              *reinterpret_cast<float4*>(gs + j) = xa[u];
+              if (desig0) *reinterpret_cast<float4*>(sw.gbest + (int64_t)a * d + j) = xa[u];
+            }
+          }
+        } else {
+          for (int j = threadIdx.x; j < d; j += NT) {
+            const float g = __ldcg(pos_prev + nb + (int64_t)bi * d + j);
+            gs[j] = g;
+            if (desig0) sw.gbest[(int64_t)a * d + j] = g;
+          }
+        }
+        __syncthreads();
+      }
+      // x' = x + (ic + s2 (gB - x)), v' = ic + s2 (gB - x), one rounding each
+      auto move1 = [](float x, float ic, float s2, float g, float* v) {
+        *v = __fadd_rn(ic, __fmul_rn(s2, __fsub_rn(g, x)));
+        return __fadd_rn(x, *v);
+      };
+      for (int e0 = threadIdx.x; e0 < n4; e0 += kPre * NT) {
+        if (e0 != (int)threadIdx.x) load_terms(e0);
+#pragma unroll
+        for (int u = 0; u < kPre; ++u) {
+          const int e = e0 + u * NT;
+          if (e >= n4) break;
+          const float4 x = xa[u], ic = ia[u], s2 = sa[u];
+          float4 g;
+          {
+            int j = 4 * e - quot(4 * e, inv_d) * d;
+            if (vec) {
+              g = *reinterpret_cast<const float4*>(gs + j);
+            } else {
+              auto next = [&] {
+                const float v = gs[j];
+                j = j + 1 == d ? 0 : j + 1;
+                return v;
+              };
+              g.x = next();
+              g.y = next();
+              g.z = next();
+              g.w = next();
+            }
+          }
+          float4 vn, xn;
+          xn.x = move1(x.x, ic.x, s2.x, g.x, &vn.x);
+          xn.y = move1(x.y, ic.y, s2.y, g.y, &vn.y);
+          xn.z = move1(x.z, ic.z, s2.z, g.z, &vn.z);
+          xn.w = move1(x.w, ic.w, s2.w, g.w, &vn.w);
+          if (desig) {  // (words past the last particle are padding)
+            reinterpret_cast<float4*>(sw.pos + o0)[e] = xn;
+            reinterpret_cast<float4*>(sw.vel + o0)[e] = vn;
+          }
+          put4(e, np, xn);
+        }
+      }
+      __syncthreads();
     }
-    __syncthreads();
   };
 
-  // the CTA's range of each particle of node a, into the node's ranges
-  auto flush_ranges = [&](int a) {
-    if ((int)threadIdx.x < P && s_lo[threadIdx.x] != INT_MAX) {
-      int* zz = sw.zmm + ((int64_t)a * Pp + threadIdx.x) * 2;
+  // the CTA's range of each particle of node a's slice, into the node's
+  auto flush_ranges = [&](int a, int pg0) {
+    if ((int)threadIdx.x < PU && s_lo[threadIdx.x] != INT_MAX) {
+      int* zz = sw.zmm + ((int64_t)a * Pp + pg0 + threadIdx.x) * 2;
       atomicMin(zz, s_lo[threadIdx.x]);
       atomicMax(zz + 1, s_hi[threadIdx.x]);
-    }
-    if (threadIdx.x < 64) {
       s_lo[threadIdx.x] = INT_MAX;
       s_hi[threadIdx.x] = INT_MIN;
     }
   };
+  // particle j of this lane, of the slice
+  auto my_particle = [&](int j) {
+    return pbk * PW +
+           (QP >= 4 ? (j < 4 ? 4 * pg + j : 32 + W * pg + j - 4) : W * pg + j);
+  };
 
-  float acc[4][PJ];
-  int cur_a = -1, cur_pg = -1;
-  float* zw = zst + warp * (4 * kZS);  // this warp's staging rows
   const bool z16 = ((reinterpret_cast<uintptr_t>(sw.z) | (uintptr_t)pr.Ez * 4) & 15) == 0;
-
-  for (int s = 0; s < n_st; ++s) {
-    const int ui = s / nk, c = s - ui * nk;
-    const WorkTile wt = tiles[u0 + ui];
-    cp_async_wait<NS - 2>();
-    // step s's rows are in place, and every warp is done with step s - 1
-    // (its stage, the positions of its node, its ranges)
-    __syncthreads();
-    if (c == 0) {  // a unit starts (no sum is live through the move)
+  int slot = 0;
+  int a = run.node, slice = run.slice, left = run.count, first = run.blk;
+  while (left > 0) {
+    const NodeDesc nd = nodes[a];
+    const int nb = (nd.seg_len + kBR - 1) / kBR;
+    const int take = min(left, nb - first);
+    const int pg0 = slice * PU;
+    node_positions(a, pg0, first == 0);
+    for (int b = first + rw; b < first + take; b += RB) {
+      uint64_t acc[4][QP];
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < PJ; ++j) acc[i][j] = 0.0f;
-      if (wt.node != cur_a || wt.pad != cur_pg) {
-        if (cur_a >= 0) flush_ranges(cur_a);
-        cur_a = wt.node;
-        cur_pg = wt.pad;
-        node_positions(cur_a, cur_pg, wt.row0 == nodes[cur_a].seg_start);
-      }
-    }
-    stage(s + NS - 1);  // into the stage step s - 1 read
-    const float* xr = xs + (s % NS) * (RT * kXS) + (rb * 32 + sg) * kXS;
-    const float* ar = ps + c * cstride + (cur_pg + pbk * PPB + pg) * kXS;
-    // features 4 ch .. 4 ch + 3 of the chunk: feature-outer within each pair
-    // of particles, so every accumulator takes the features in increasing order
-    auto fma4 = [&](int ch) {
-      float4 xv[4];
+        for (int j = 0; j < QP; ++j) acc[i][j] = 0ull;
+      const float* ar0 = ps + pbk * d * PW;
+      // One feature's operands: rows 4 rg .. + 3 and 16 + 4 rg .. + 3 in pairs
+      // (x0, x1), the positions in pairs (a0, a1). A pair of rows meets a pair
+      // of positions in two packed multiply-adds, straight (x0 a0, x1 a1) and
+      // crossed (x0 a1, x1 a0): one swap per pair of positions instead of a
+      // copy of every position into both halves, which took the multiply-add
+      // pipe as long as half of the products did. (An odd last position is
+      // copied.)
+      struct Operands {
+        ulonglong2 x0, x1;
+        uint64_t a[(QP + 1) / 2];
+      };
+      for (int c = 0; c < nk; ++c) {
+        cp_async_wait<NS - 2>();
+        __syncwarp();  // the chunk is in place; every lane is done with the last one
+        const float* xr = xs + slot * (kSC * kBR) + 4 * rg;
+        slot = slot + 1 == NS ? 0 : slot + 1;
+        const int k0 = c * kSC;
+        const float* ar = ar0 + k0 * PW;
+        auto read = [&](Operands& o, int k, int key) {
+          o.x0 = *reinterpret_cast<const ulonglong2*>(xr + k * kBR);
+          o.x1 = *reinterpret_cast<const ulonglong2*>(xr + k * kBR + 16);
+          const float* ak = ar + k * PW;
+          constexpr int J0 = QP >= 4 ? 4 : 0;
+          if constexpr (QP >= 4) {
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(ak + ((pg ^ key) << 2));
+            o.a[0] = v.x;
+            o.a[1] = v.y;
+          }
+          if constexpr (W == 4) {
+            const ulonglong2 v =
+                *reinterpret_cast<const ulonglong2*>(ak + 32 + ((pg ^ key) << 2));
+            o.a[2] = v.x;
+            o.a[3] = v.y;
+          } else if constexpr (W == 2) {
+            o.a[J0 / 2] = *reinterpret_cast<const uint64_t*>(ak + 8 * J0 + ((pg ^ key) << 1));
+          } else if constexpr (W == 3) {
+            const float* aw = ak + 8 * J0 + (pg ^ key) * W;
+            o.a[J0 / 2] = pack2(aw[0], aw[1]);
+            o.a[J0 / 2 + 1] = pack2(aw[2], aw[2]);
+          } else if constexpr (W == 1) {
+            const float v = ak[8 * J0 + (pg ^ key)];
+            o.a[J0 / 2] = pack2(v, v);
+          }
+        };
+        auto feature = [&](const Operands& o) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        xv[i] = *reinterpret_cast<const float4*>(xr + i * 8 * kXS + 4 * ch);
-#pragma unroll
-      for (int j = 0; j < PJ; j += 2) {
-        const float4 a0 = *reinterpret_cast<const float4*>(ar + j * 4 * kXS + 4 * ch);
-        const float4 a1 = *reinterpret_cast<const float4*>(ar + (j + 1) * 4 * kXS + 4 * ch);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          acc[i][j] = fmaf(xv[i].x, a0.x, acc[i][j]);
-          acc[i][j + 1] = fmaf(xv[i].x, a1.x, acc[i][j + 1]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          acc[i][j] = fmaf(xv[i].y, a0.y, acc[i][j]);
-          acc[i][j + 1] = fmaf(xv[i].y, a1.y, acc[i][j + 1]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          acc[i][j] = fmaf(xv[i].z, a0.z, acc[i][j]);
-          acc[i][j + 1] = fmaf(xv[i].z, a1.z, acc[i][j + 1]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          acc[i][j] = fmaf(xv[i].w, a0.w, acc[i][j]);
-          acc[i][j + 1] = fmaf(xv[i].w, a1.w, acc[i][j + 1]);
-        }
-      }
-    };
-    const int kc4 = (min(kKC, d - c * kKC) + 3) >> 2;  // 16-byte chunks of features
-    if (kc4 == kKC / 4) {
-#pragma unroll(PJ <= 4 ? 2 : 1)
-      for (int ch = 0; ch < kKC / 4; ++ch) fma4(ch);
-    } else {
+          for (int m = 0; m < QP / 2; ++m) {
+            const uint64_t as = swap2(o.a[m]);
+            fma2(acc[0][2 * m], o.x0.x, o.a[m]);
+            fma2(acc[1][2 * m], o.x0.y, o.a[m]);
+            fma2(acc[2][2 * m], o.x1.x, o.a[m]);
+            fma2(acc[3][2 * m], o.x1.y, o.a[m]);
+            fma2(acc[0][2 * m + 1], o.x0.x, as);
+            fma2(acc[1][2 * m + 1], o.x0.y, as);
+            fma2(acc[2][2 * m + 1], o.x1.x, as);
+            fma2(acc[3][2 * m + 1], o.x1.y, as);
+          }
+          if constexpr (QP & 1) {
+            fma2(acc[0][QP - 1], o.x0.x, o.a[QP / 2]);
+            fma2(acc[1][QP - 1], o.x0.y, o.a[QP / 2]);
+            fma2(acc[2][QP - 1], o.x1.x, o.a[QP / 2]);
+            fma2(acc[3][QP - 1], o.x1.y, o.a[QP / 2]);
+          }
+        };
+        const int kc = min(kSC, d - k0);
+        Operands o[2];
+        const int key0 = (k0 >> 2) & 7;  // (a chunk's keys do not wrap)
+        read(o[0], 0, key0);
+        stage();  // into the slot of the chunk before this one
+        // TF features a turn, the next one's operands read ahead
+        int k = 0;
 #pragma unroll 1
-      for (int ch = 0; ch < kc4; ++ch) fma4(ch);
-    }
-    if (c == nk - 1) {
-      // unit complete: the ranges into the CTA's; z out through the warp's
-      // staging rows, so that every store writes whole rows of a particle
-      // (four 128-byte rows per 16-byte store when aligned, else one per
-      // 4-byte store) instead of 32-byte pieces of four rows
-      const int rw = wt.rows - rb * 32;  // rows of the warp's block in the tile
-      const int64_t zrow = wt.row0 + rb * 32;
-      const bool v16 = z16 && rw >= 32 && (zrow & 3) == 0;
+        for (; k + TF <= kc; k += TF) {
+          const int key = key0 + (k >> 2);
 #pragma unroll
-      for (int j = 0; j < PJ; ++j) {
-        const int pb0 = cur_pg + pbk * PPB + 4 * j;  // the warp's particles pb0 .. pb0 + 3
-        const int p = pb0 + pg;
-        float lo = FLT_MAX, hi = -FLT_MAX;
-        bool any = false;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          if (sg + 8 * i < rw) {
-            const float z = acc[i][j];
-            lo = z < lo ? z : lo;
-            hi = z > hi ? z : hi;
-            any = true;
+          for (int i = 0; i < TF; ++i) {
+            if (i + 1 < TF)
+              read(o[(i + 1) & 1], k + i + 1, key + ((i + 1) >> 2));
+            else if (k + TF < kc)
+              read(o[0], k + TF, key + TF / 4);
+            feature(o[i & 1]);
           }
         }
-        int olo = any ? f2ord(lo) : INT_MAX, ohi = any ? f2ord(hi) : INT_MIN;
-#pragma unroll
-        for (int off = 1; off < 8; off <<= 1) {
-          olo = min(olo, __shfl_xor_sync(0xffffffffu, olo, off));
-          ohi = max(ohi, __shfl_xor_sync(0xffffffffu, ohi, off));
+#pragma unroll 1
+        for (; k < kc; ++k) {
+          feature(o[0]);
+          if (k + 1 < kc) read(o[0], k + 1, key0 + ((k + 1) >> 2));
         }
-        if (sg == 0 && olo != INT_MAX && p < P) {
-          atomicMin(&s_lo[p], olo);
-          atomicMax(&s_hi[p], ohi);
-        }
-        __syncwarp();  // the previous particles' staging rows are read
+      }
+      // block complete: its ranges into the CTA's, z out (16 bytes a store
+      // where the block is whole and aligned)
+      const int nr = min(kBR, nd.seg_len - b * kBR);
+      const int64_t zrow = (int64_t)nd.seg_start + b * kBR;
+      const bool whole = nr == kBR;
+      const bool v16 = z16 && whole && (zrow & 3) == 0;
+      float* zp = sw.z + (int64_t)(pg0 + my_particle(0)) * pr.Ez + zrow + 4 * rg;
+      constexpr int QR = (QP + 3) & ~3;  // particles of the range exchange
+      float lo[QR], hi[QR];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) zw[pg * kZS + sg + 8 * i] = acc[i][j];
-        __syncwarp();
+      for (int j = 0; j < QR; ++j) {
+        lo[j] = FLT_MAX;
+        hi[j] = -FLT_MAX;
+      }
+#pragma unroll
+      for (int j = 0; j < QP; ++j) {
+        const int p = pg0 + my_particle(j);
+        if (j > 0) zp += j == 4 && QP > 4 ? (int64_t)(my_particle(4) - my_particle(3)) * pr.Ez : pr.Ez;
+        // rows' pairs of particle j: the straight sums' halves of its own
+        // parity and the crossed sums' of the other (an odd last particle has
+        // both halves)
+        auto rows = [&](const uint64_t (&c)[QP]) {
+          if (j == QP - 1 && (QP & 1)) return unpack2(c[j]);
+          const float2 s0 = unpack2(c[j & ~1]), s1 = unpack2(c[j | 1]);
+          return (j & 1) ? make_float2(s1.x, s0.y) : make_float2(s0.x, s1.y);
+        };
+        const float2 v0 = rows(acc[0]), v1 = rows(acc[1]), v2 = rows(acc[2]), v3 = rows(acc[3]);
+        if (whole) {
+          lo[j] = fminf(lo[j], fminf(fminf(fminf(v0.x, v0.y), fminf(v1.x, v1.y)),
+                               fminf(fminf(v2.x, v2.y), fminf(v3.x, v3.y))));
+          hi[j] = fmaxf(hi[j], fmaxf(fmaxf(fmaxf(v0.x, v0.y), fmaxf(v1.x, v1.y)),
+                               fmaxf(fmaxf(v2.x, v2.y), fmaxf(v3.x, v3.y))));
+        }
         if (v16) {
-          const int q = lane >> 3, r4 = 4 * (lane & 7);
-          const float4 v = *reinterpret_cast<const float4*>(zw + q * kZS + r4);
-          if (pb0 + q < P) *reinterpret_cast<float4*>(sw.z + (int64_t)(pb0 + q) * pr.Ez + zrow + r4) = v;
+          if (p < P) {
+            *reinterpret_cast<float4*>(zp) = make_float4(v0.x, v0.y, v1.x, v1.y);
+            *reinterpret_cast<float4*>(zp + 16) = make_float4(v2.x, v2.y, v3.x, v3.y);
+          }
         } else {
+          const float v[8] = {v0.x, v0.y, v1.x, v1.y, v2.x, v2.y, v3.x, v3.y};
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (lane < rw && pb0 + q < P) sw.z[(int64_t)(pb0 + q) * pr.Ez + zrow + lane] = zw[q * kZS + lane];
+          for (int i = 0; i < 8; ++i) {
+            const int off = (i & 3) + 16 * (i >> 2);
+            if (4 * rg + off < nr) {
+              if (!whole) {
+                lo[j] = fminf(lo[j], v[i]);
+                hi[j] = fmaxf(hi[j], v[i]);
+              }
+              if (p < P) zp[off] = v[i];
+            }
+          }
+        }
+      }
+      // The four lanes that share these particles (rg) exchange ranges,
+      // halving their particles each time: every lane ends with QR / 4
+      // particles' ranges over all the block's rows (3 QR / 2 shuffles; a
+      // reduction of each particle by every lane takes 4 QR).
+#pragma unroll
+      for (int j = 0; j < QR / 2; ++j) {
+        const bool up = rg & 1;
+        const float sl = up ? lo[j] : lo[j + QR / 2], sh = up ? hi[j] : hi[j + QR / 2];
+        const float kl = up ? lo[j + QR / 2] : lo[j], kh = up ? hi[j + QR / 2] : hi[j];
+        lo[j] = fminf(kl, __shfl_xor_sync(0xffffffffu, sl, 1));
+        hi[j] = fmaxf(kh, __shfl_xor_sync(0xffffffffu, sh, 1));
+      }
+#pragma unroll
+      for (int j = 0; j < QR / 4; ++j) {
+        const bool up = rg & 2;
+        const float sl = up ? lo[j] : lo[j + QR / 4], sh = up ? hi[j] : hi[j + QR / 4];
+        const float kl = up ? lo[j + QR / 4] : lo[j], kh = up ? hi[j + QR / 4] : hi[j];
+        lo[j] = fminf(kl, __shfl_xor_sync(0xffffffffu, sl, 2));
+        hi[j] = fmaxf(kh, __shfl_xor_sync(0xffffffffu, sh, 2));
+        const int jj = (rg & 1) * (QR / 2) + (rg >> 1) * (QR / 4) + j;
+        const int pl = my_particle(jj);
+        if (jj < QP && pg0 + pl < P) {
+          atomicMin(&s_lo[pl], f2ord(lo[j]));
+          atomicMax(&s_hi[pl], f2ord(hi[j]));
         }
       }
     }
+    __syncthreads();  // every warp's ranges are in; the positions are read
+    flush_ranges(a, pg0);
+    left -= take;
+    first = 0;
+    if (++slice == n_slices) {
+      slice = 0;
+      ++a;
+    }
   }
-  __syncthreads();  // every warp's ranges are in
-  if (cur_a >= 0) flush_ranges(cur_a);
 }
 
-// Tile shapes of a padded swarm, largest row tile first: (PJ, PB), rows per
-// unit 32 (8 / PB), particles per unit 4 PJ PB. Shapes 0-2 take every
-// particle in a unit; shapes 3-5 take half of them (two slices of a swarm of
-// 32 or 64), so a short node is spread over twice the CTAs with half the
-// move and projection each. The smaller tiles spread a short node further.
-constexpr int kStepShapes = 6;
-
-bool step_shape(int Pp, int sh, int* PJ, int* PB) {
-  static const int tab[4][3][2] = {
-      {{4, 1}, {2, 2}, {0, 0}},   // 16 particles per unit
-      {{8, 1}, {4, 2}, {2, 4}},   // 32
-      {{6, 2}, {0, 0}, {0, 0}},   // 48
-      {{8, 2}, {4, 4}, {2, 8}}};  // 64
-  if (Pp % 16 || Pp < 16 || Pp > 64 || sh < 0 || sh >= kStepShapes) return false;
-  const int pu = sh < 3 ? Pp : Pp / 2;  // particles per unit
-  if (pu % 16) return false;
-  const int* e = tab[pu / 16 - 1][sh % 3];
-  *PJ = e[0];
-  *PB = e[1];
-  return e[0] > 0;
+// Tile shapes of a folded search's padded swarm: particles per thread and
+// particle warps. Shapes 0-2 take every particle in a unit, on 384, 192 or 96
+// rows of the CTA; shapes 3-5 take half of them (two slices of a swarm of 32
+// or 64), so a short node is spread over twice the CTAs with half the move
+// and projection each.
+bool step_shape(const Problem& pr, int sh, int* QP, int* PB) {
+  const int Pp = pr.Pp;
+  if (Pp % 16 || Pp < 16 || Pp > 64 || sh < 0 || sh >= kStepShapeCount) return false;
+  const int pu = sh < 3 ? Pp : Pp / 2;
+  if ((sh >= 3 && Pp != 32 && Pp != 64) || pu % 16) return false;
+  *PB = 1 << (sh % 3);
+  if (pu == 48) {
+    *QP = (pr.P + 7) / 8;  // 5 or 6
+    return *PB == 1;
+  }
+  *QP = pu / 8 / *PB;
+  return *QP >= 1;
 }
 
-size_t step_smem(const Problem& pr, int sh) {
-  int PJ = 0, PB = 0;
-  if (!step_shape(pr.Pp, sh, &PJ, &PB)) return 0;
-  const int RT = 32 * (8 / PB);
-  return sizeof(float) * ((size_t)step_stages(RT) * RT * kXS + step_pos_floats(pr.Pp, pr.d) +
-                          (size_t)((pr.d + 3) & ~3) + (size_t)8 * 4 * kZS);
+// The unfolded projection's slices: the fewest of at most 64 particles whose
+// positions fit, each shared by as many warps (1, 2 or 4) as leaves a row
+// warp for each of the `blocks` of a node: small nodes' blocks would leave
+// the other warps idle.
+bool proj_shape(const Problem& pr, int64_t blocks, int* QP, int* PB, int* slices) {
+  for (int n = (pr.P + 63) / 64; n <= pr.P; ++n) {
+    const int q = ((pr.P + n - 1) / n + 7) / 8;
+    if ((size_t)8 * q * pr.d * sizeof(float) <= (size_t)kStepMaxPosBytes) {
+      *PB = 1;
+      while (*PB < 4 && blocks * *PB * 2 <= kProjWarps && q > *PB) *PB *= 2;
+      *QP = (q + *PB - 1) / *PB;
+      *slices = (pr.P + 8 * *QP * *PB - 1) / (8 * *QP * *PB);
+      return true;
+    }
+    if (q == 1) break;
+  }
+  return false;
 }
 
-template <class F>
-cudaError_t step_dispatch(int Pp, int sh, F&& f) {
-  int PJ = 0, PB = 0;
-  if (!step_shape(Pp, sh, &PJ, &PB)) return cudaErrorInvalidValue;
-  switch (PJ * 16 + PB) {
-    case 4 * 16 + 1: return f(k_step<4, 1>);
-    case 2 * 16 + 2: return f(k_step<2, 2>);
-    case 8 * 16 + 1: return f(k_step<8, 1>);
-    case 4 * 16 + 2: return f(k_step<4, 2>);
-    case 2 * 16 + 4: return f(k_step<2, 4>);
-    case 6 * 16 + 2: return f(k_step<6, 2>);
-    case 8 * 16 + 2: return f(k_step<8, 2>);
-    case 4 * 16 + 4: return f(k_step<4, 4>);
-    case 2 * 16 + 8: return f(k_step<2, 8>);
-    default: return cudaErrorInvalidValue;
+size_t step_smem(int d, int pu, int warps) {
+  return sizeof(float) * ((size_t)warps * kStepStages * kSC * kBR + (size_t)pu * d +
+                          (size_t)((d + 3) & ~3));
+}
+
+const void* step_fn(int QP, int PB) {
+  switch (QP * 16 + PB) {
+    case 8 * 16 + 1: return (const void*)k_step<8, 1, true>;
+    case 6 * 16 + 1: return (const void*)k_step<6, 1, true>;
+    case 5 * 16 + 1: return (const void*)k_step<5, 1, true>;
+    case 4 * 16 + 1: return (const void*)k_step<4, 1, true>;
+    case 4 * 16 + 2: return (const void*)k_step<4, 2, true>;
+    case 2 * 16 + 1: return (const void*)k_step<2, 1, true>;
+    case 2 * 16 + 2: return (const void*)k_step<2, 2, true>;
+    case 2 * 16 + 4: return (const void*)k_step<2, 4, true>;
+    case 1 * 16 + 1: return (const void*)k_step<1, 1, true>;
+    case 1 * 16 + 2: return (const void*)k_step<1, 2, true>;
+    case 1 * 16 + 4: return (const void*)k_step<1, 4, true>;
+    default: return nullptr;
+  }
+}
+
+const void* proj_fn(int QP, int PB) {
+  switch (QP * 16 + PB) {
+    case 1 * 16 + 1: return (const void*)k_step<1, 1, false>;
+    case 2 * 16 + 1: return (const void*)k_step<2, 1, false>;
+    case 3 * 16 + 1: return (const void*)k_step<3, 1, false>;
+    case 4 * 16 + 1: return (const void*)k_step<4, 1, false>;
+    case 5 * 16 + 1: return (const void*)k_step<5, 1, false>;
+    case 6 * 16 + 1: return (const void*)k_step<6, 1, false>;
+    case 7 * 16 + 1: return (const void*)k_step<7, 1, false>;
+    case 8 * 16 + 1: return (const void*)k_step<8, 1, false>;
+    case 1 * 16 + 2: return (const void*)k_step<1, 2, false>;
+    case 2 * 16 + 2: return (const void*)k_step<2, 2, false>;
+    case 3 * 16 + 2: return (const void*)k_step<3, 2, false>;
+    case 4 * 16 + 2: return (const void*)k_step<4, 2, false>;
+    case 1 * 16 + 4: return (const void*)k_step<1, 4, false>;
+    case 2 * 16 + 4: return (const void*)k_step<2, 4, false>;
+    default: return nullptr;
   }
 }
 
 }  // namespace
 
 bool step_ok(const Problem& pr) {
-  int PJ = 0, PB = 0;
-  return step_shape(pr.Pp, 0, &PJ, &PB) &&
-         step_pos_floats(pr.Pp, pr.d) * sizeof(float) <= (size_t)kStepMaxPosBytes;
+  int QP = 0, PB = 0;
+  return step_shape(pr, 0, &QP, &PB) &&
+         (size_t)8 * QP * PB * pr.d * sizeof(float) <= (size_t)kStepMaxPosBytes;
 }
 
-int step_rows(const Problem& pr, int sh) {
-  int PJ = 0, PB = 0;
-  return step_shape(pr.Pp, sh, &PJ, &PB) ? 32 * (8 / PB) : 0;
+bool step_config(const Problem& pr, int sh, StepConfig* c, int64_t blocks) {
+  int QP = 0, PB = 0, slices = 1;
+  if (sh >= 0) {
+    if (!step_shape(pr, sh, &QP, &PB)) return false;
+    slices = (pr.P + 8 * QP * PB - 1) / (8 * QP * PB);
+    c->fn = step_fn(QP, PB);
+  } else {
+    if (!proj_shape(pr, blocks, &QP, &PB, &slices)) return false;
+    c->fn = proj_fn(QP, PB);
+  }
+  c->qp = QP;
+  c->pb = PB;
+  c->slices = slices;
+  const int warps = sh >= 0 ? kFoldWarps : kProjWarps;
+  c->threads = 32 * warps;
+  c->row_warps = warps / PB;
+  c->smem = step_smem(pr.d, 8 * QP * PB, warps);
+  return c->fn != nullptr;
 }
 
-int step_slices(const Problem& pr, int sh) {
-  int PJ = 0, PB = 0;
-  return step_shape(pr.Pp, sh, &PJ, &PB) ? pr.Pp / (4 * PJ * PB) : 0;
-}
+cudaError_t prepare_step(const StepConfig& c) { return allow_smem(c.fn, (int)c.smem); }
 
-cudaError_t prepare_step_kernels(const Problem& pr, int sh) {
-  return step_dispatch(pr.Pp, sh, [&](auto fn) {
-    return allow_smem((const void*)fn, (int)step_smem(pr, sh));
-  });
-}
-
-int step_grid(const Problem& pr, int sh, int n_sm) {
+int step_grid(const StepConfig& c, int n_sm) {
   int per_sm = 0;
-  const cudaError_t e = step_dispatch(pr.Pp, sh, [&](auto fn) {
-    return occupancy(&per_sm, (const void*)fn, kThreads, step_smem(pr, sh));
-  });
-  if (e != cudaSuccess) {
+  if (occupancy(&per_sm, c.fn, c.threads, c.smem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
   return per_sm * n_sm;
 }
 
-cudaError_t launch_step(const Problem& pr, const Swarm& sw, const float* pos_prev,
-                        const NodeDesc* nodes, int A, const WorkTile* tiles, int n_tiles,
-                        int grid, int sh, int t, cudaStream_t st) {
+int64_t step_rows_floats(const Problem& pr, int A) { return (pr.E + 32 * (int64_t)A) * pr.d; }
+
+cudaError_t launch_block_rows(const Problem& pr, const WorkTile* tiles, int n_tiles, float* Xt,
+                              cudaStream_t st) {
   if (n_tiles <= 0) return cudaSuccess;
-  if (!step_ok(pr) || grid <= 0) return cudaErrorInvalidValue;
+  k_block_rows<<<(unsigned)n_tiles, 256, 0, st>>>(pr.X, pr.d, tiles, Xt);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_step(const StepConfig& c, const Problem& pr, const Swarm& sw,
+                        const float* pos_prev, const NodeDesc* nodes, int A, const StepRun* runs,
+                        int n_runs, int t, cudaStream_t st) {
+  if (n_runs <= 0) return cudaSuccess;
+  if (!pr.Xt) return cudaErrorInvalidValue;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(n_tiles < grid ? n_tiles : grid), 1, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = step_smem(pr, sh);
+  cfg.gridDim = dim3((unsigned)n_runs, 1, 1);
+  cfg.blockDim = dim3((unsigned)c.threads, 1, 1);
+  cfg.dynamicSmemBytes = c.smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return step_dispatch(pr.Pp, sh, [&](auto fn) {
-    return cudaLaunchKernelEx(&cfg, fn, pr, sw, pos_prev, nodes, A, tiles, n_tiles, t);
-  });
+  int n_slices = c.slices;
+  // ceil(2^32 / v): __umulhi(e, .) = e / v exactly for e v < 2^32; 0 (no
+  // factor of 32 bits) for v = 1
+  auto factor = [](uint32_t v) {
+    return v > 1 ? (uint32_t)(((1ull << 32) + v - 1) / v) : 0u;
+  };
+  uint32_t inv_d = factor((uint32_t)pr.d);
+  void* args[] = {(void*)&pr, (void*)&sw, (void*)&pos_prev, (void*)&nodes, (void*)&A,
+                  (void*)&runs, (void*)&n_slices, (void*)&inv_d, (void*)&t};
+  return cudaLaunchKernelExC(&cfg, c.fn, args);
 }
 
 }  // namespace slm

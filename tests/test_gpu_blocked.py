@@ -1,0 +1,62 @@
+"""The projection from blocked rows, not folded (the default where a batch is
+long, has more nodes than CTAs, runs adaptive PSO or a swarm that does not
+fold): the results of the row-major projection bit for bit. Swarm widths of
+every particles-per-thread variant, several slices, slices cut down because
+their positions would not fit, feature counts around the 16-feature chunks
+and odd ones, nodes smaller than a block, and levels of many small nodes
+(several warps sharing a block)."""
+import numpy as np
+import pytest
+
+from paper_2208_07023_gb300 import workloads as W
+from tests.gpu_util import context, gpu_params
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctxs():
+    a, b = context(), context()
+    b.set_fused_step(False)
+    yield a, b
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("n,d,P,apso", [
+    (3001, 17, 65, False),    # two slices of 40
+    (2000, 16, 100, False),
+    (700, 1, 256, False),     # four slices of 64, one feature
+    (900, 1024, 70, False),   # slices cut to the positions' room
+    (333, 300, 128, False),
+    (31, 5, 80, False),       # less than one block
+    (5000, 23, 7, True), (4097, 33, 15, True), (2500, 50, 23, True), (2500, 48, 31, True),
+    (1200, 15, 39, True), (1200, 31, 47, True), (800, 64, 55, True), (4100, 12, 63, True),
+])
+def test_search_identical_blocked_and_row_major(ctxs, n, d, P, apso):
+    from paper_2208_07023_gb300 import binding as S
+    a, b = ctxs
+    wl = W.gmm(n, d, 3, seed=d + P)
+    p = S.make_params("gini", 3, n_particles=P, n_iters=4, n_bins=64, min_leaf=2, seed=3,
+                      apso=apso)
+    before = a.set_fused_step(True)
+    ra = a.node_split(p, wl.X, labels=wl.labels, node_uid=9, want_trace=True)
+    assert a.set_fused_step(True) == before  # not folded
+    rb = b.node_split(p, wl.X, labels=wl.labels, node_uid=9, want_trace=True)
+    assert np.array_equal(ra["trace"], rb["trace"])
+    assert np.array_equal(ra["gbest"].view(np.uint32), rb["gbest"].view(np.uint32))
+    for k in ("bin", "q_num", "q_den", "n_left", "particle", "iter_of_best"):
+        assert ra[k] == rb[k], k
+
+
+@pytest.mark.parametrize("P,d", [(24, 9), (64, 20), (40, 33), (16, 6)])
+def test_many_small_nodes_identical(ctxs, P, d):
+    """More nodes than CTAs: runs of several nodes, 1, 2 or 4 warps a block."""
+    from paper_2208_07023_gb300 import binding as S
+    a, b = ctxs
+    wl = W.tanh_regression(9000, d, seed=P)
+    p = gpu_params(S, "mse", 0, P, 3, 64, min_leaf=4, max_depth=10, seed=2)
+    ga, gb = (c.train_tree(p, wl.X, y=wl.y).export(0) for c in (a, b))
+    for k in ga:
+        assert np.array_equal(ga[k], gb[k]), k
+    assert (ga["kind"] == 1).sum() > 500
