@@ -39,6 +39,7 @@
 #include <limits.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "device_util.cuh"
 #include "philox.cuh"
@@ -60,7 +61,7 @@ constexpr int kMqOffset = 1 << 29;  // targets are stored as q + 2^29, |q| <= 2^
 // whose merge is cheaper on short slices (at most 1,100 per copy).
 constexpr int kMseSlice = 65000;
 constexpr int kMseSliceFew = 8192;
-constexpr int kMseMaxCluster = 8;
+constexpr int kMseMaxCluster = 16;
 constexpr int kMseWarps = kThreads / 32;
 constexpr int kMseGroup = 4;  // edges scored per masked pass
 // Slack of G for the double-precision rounding of two losses, in squared
@@ -196,20 +197,25 @@ __global__ void __launch_bounds__(kThreads, 3)
   const int n = r_end - r_begin;
   const bool g16 = (e0 & 3) == 0;  // 16-byte loads: groups of four entries
   const int n4 = g16 ? n >> 2 : 0;
-  constexpr int U = 4;  // groups in flight per thread
-  float4 zv[U];
-  uint4 uv[U];
-  auto load_groups = [&](int g0) {
+  // Two sets of U groups per thread, one on its way while the other is
+  // binned (with one set of four a thread waited out a memory round trip
+  // every 16 entries: 75 us on 200,000 entries x 64 particles).
+  constexpr int U = 2;
+  struct Groups {
+    float4 z[U];
+    uint4 u[U];
+  } ga, gc;
+  auto load_groups = [&](Groups& q, int g0) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int g = g0 + u * kThreads;
       if (g < n4) {
-        zv[u] = __ldcg(reinterpret_cast<const float4*>(zs) + g);
-        uv[u] = __ldg(reinterpret_cast<const uint4*>(us) + g);
+        q.z[u] = __ldcg(reinterpret_cast<const float4*>(zs) + g);
+        q.u[u] = __ldg(reinterpret_cast<const uint4*>(us) + g);
       }
     }
   };
-  load_groups(threadIdx.x);
+  load_groups(ga, threadIdx.x);
   const int64_t prow0 = ci * d;
   float need = 0.0f;
   if (upd) {
@@ -250,16 +256,21 @@ __global__ void __launch_bounds__(kThreads, 3)
       atomicAdd(hA + i, 1u | ((u & ((1u << kMqLoBits) - 1u)) << kMqCntBits));
       atomicAdd(hB + i, u >> kMqLoBits);
     };
-    for (int g0 = threadIdx.x; g0 < n4; g0 += U * kThreads) {
-      if (g0 != (int)threadIdx.x) load_groups(g0);
+    auto bin_groups = [&](const Groups& q, int g0) {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         if (g0 + u * kThreads >= n4) break;
-        add(zv[u].x, uv[u].x);
-        add(zv[u].y, uv[u].y);
-        add(zv[u].z, uv[u].z);
-        add(zv[u].w, uv[u].w);
+        add(q.z[u].x, q.u[u].x);
+        add(q.z[u].y, q.u[u].y);
+        add(q.z[u].z, q.u[u].z);
+        add(q.z[u].w, q.u[u].w);
       }
+    };
+    for (int g0 = threadIdx.x; g0 < n4; g0 += 2 * U * kThreads) {
+      load_groups(gc, g0 + U * kThreads);
+      bin_groups(ga, g0);
+      load_groups(ga, g0 + 2 * U * kThreads);
+      bin_groups(gc, g0 + U * kThreads);
     }
     for (int i = (n4 << 2) + (int)threadIdx.x; i < n; i += kThreads)
       add(__ldcg(zs + i), __ldg(us + i));
@@ -308,23 +319,25 @@ __global__ void __launch_bounds__(kThreads, 3)
   const MseNode mn = pr.mnode[a];
   EvalRes res = invalid_res();
   // exact scores of the edges in sc.dec_e: this rank's masked sums into rank 0
-  auto masked_pass = [&](int nc) {
-    int ed[kMseGroup];
+  auto masked_edges = [&](auto edges, int nc) {
+    constexpr int N = decltype(edges)::value;
+    int ed[N];
 #pragma unroll
-    for (int c = 0; c < kMseGroup; ++c) ed[c] = c < nc ? sc.dec_e[c] : 0;
-    unsigned long long as[kMseGroup] = {}, aq[kMseGroup] = {};
-    uint32_t an[kMseGroup] = {};
+    for (int c = 0; c < N; ++c) ed[c] = c < nc ? sc.dec_e[c] : 0;
+    unsigned long long as[N] = {}, aq[N] = {};
+    uint32_t an[N] = {};
     auto take = [&](float z, long long v1, long long v2) {
       const int bz = bin_of(z, zmin, inv_w, B);
 #pragma unroll
-      for (int c = 0; c < kMseGroup; ++c)
-        if (c < nc && bz < ed[c]) {
+      for (int c = 0; c < N; ++c)
+        if (bz < ed[c]) {
           as[c] += (unsigned long long)v1;
           aq[c] += (unsigned long long)v2;
           an[c] += 1u;
         }
     };
     if (ok) {
+#pragma unroll 2
       for (int g = threadIdx.x; g < n4; g += kThreads) {
         const float4 z4 = __ldcg(reinterpret_cast<const float4*>(zs) + g);
         const longlong2 a0 = __ldg(reinterpret_cast<const longlong2*>(m1) + 2 * g);
@@ -343,7 +356,7 @@ __global__ void __launch_bounds__(kThreads, 3)
     unsigned long long* dq = S > 1 ? cl.map_shared_rank(sc.acc_q, 0) : sc.acc_q;
     unsigned int* dn = S > 1 ? cl.map_shared_rank(sc.acc_n, 0) : sc.acc_n;
 #pragma unroll
-    for (int c = 0; c < kMseGroup; ++c) {
+    for (int c = 0; c < N; ++c) {
       if (c >= nc) break;
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) {
@@ -357,6 +370,12 @@ __global__ void __launch_bounds__(kThreads, 3)
         atomicAdd(dn + c, an[c]);
       }
     }
+  };
+  auto masked_pass = [&](int nc) {  // (mostly one edge)
+    if (nc == 1)
+      masked_edges(std::integral_constant<int, 1>{}, 1);
+    else
+      masked_edges(std::integral_constant<int, kMseGroup>{}, nc);
   };
   auto all_sync = [&] {
     if (S > 1)
@@ -629,25 +648,36 @@ __global__ void __launch_bounds__(kThreads, 4)
       atomicAdd(hB + i, u >> kMqLoBits);
     };
     constexpr int U = 2;
-    for (int g0 = lane; g0 < n4; g0 += 32 * U) {
-      float4 zv[U];
-      uint4 uv[U];
+    struct Groups {
+      float4 z[U];
+      uint4 u[U];
+    } ga, gc;
+    auto load = [&](Groups& q, int g0) {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int g = g0 + 32 * u;
         if (g < n4) {
-          zv[u] = __ldcg(reinterpret_cast<const float4*>(zs) + g);
-          uv[u] = __ldg(reinterpret_cast<const uint4*>(us) + g);
+          q.z[u] = __ldcg(reinterpret_cast<const float4*>(zs) + g);
+          q.u[u] = __ldg(reinterpret_cast<const uint4*>(us) + g);
         }
       }
+    };
+    auto bin_groups = [&](const Groups& q, int g0) {
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         if (g0 + 32 * u >= n4) break;
-        add(zv[u].x, uv[u].x);
-        add(zv[u].y, uv[u].y);
-        add(zv[u].z, uv[u].z);
-        add(zv[u].w, uv[u].w);
+        add(q.z[u].x, q.u[u].x);
+        add(q.z[u].y, q.u[u].y);
+        add(q.z[u].z, q.u[u].z);
+        add(q.z[u].w, q.u[u].w);
       }
+    };
+    load(ga, lane);
+    for (int g0 = lane; g0 < n4; g0 += 64 * U) {
+      load(gc, g0 + 32 * U);
+      bin_groups(ga, g0);
+      load(ga, g0 + 64 * U);
+      bin_groups(gc, g0 + 32 * U);
     }
     for (int i = (n4 << 2) + lane; i < n; i += 32) add(__ldcg(zs + i), __ldg(us + i));
   }
@@ -734,19 +764,21 @@ __global__ void __launch_bounds__(kThreads, 4)
         ++nc;
       }
     }
-    if (nc > 0) {
-      unsigned long long as[kMseGroup] = {}, aq[kMseGroup] = {};
-      uint32_t an[kMseGroup] = {};
+    auto masked_edges = [&](auto edges) {
+      constexpr int N = decltype(edges)::value;
+      unsigned long long as[N] = {}, aq[N] = {};
+      uint32_t an[N] = {};
       auto take = [&](float z, long long v1, long long v2) {
         const int bz = bin_of(z, zmin, inv_w, B);
 #pragma unroll
-        for (int c = 0; c < kMseGroup; ++c)
-          if (c < nc && bz < ed[c]) {
+        for (int c = 0; c < N; ++c)
+          if (bz < ed[c]) {
             as[c] += (unsigned long long)v1;
             aq[c] += (unsigned long long)v2;
             an[c] += 1u;
           }
       };
+#pragma unroll 1
       for (int g = lane; g < n4; g += 32) {
         const float4 z4 = __ldcg(reinterpret_cast<const float4*>(zs) + g);
         const longlong2 a0 = __ldg(reinterpret_cast<const longlong2*>(m1) + 2 * g);
@@ -761,7 +793,7 @@ __global__ void __launch_bounds__(kThreads, 4)
       for (int i = (n4 << 2) + lane; i < n; i += 32)
         take(__ldcg(zs + i), __ldg(m1 + i), __ldg(m2 + i));
 #pragma unroll
-      for (int c = 0; c < kMseGroup; ++c) {
+      for (int c = 0; c < N; ++c) {
         if (c >= nc) break;
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
@@ -771,7 +803,11 @@ __global__ void __launch_bounds__(kThreads, 4)
         an[c] = __reduce_add_sync(0xffffffffu, an[c]);
         if (lane == 0) sc.job[warp][c] = MseEdge{(long long)as[c], (long long)aq[c], an[c], ed[c]};
       }
-    }
+    };
+    if (nc == 1)  // (most often)
+      masked_edges(std::integral_constant<int, 1>{});
+    else if (nc > 1)
+      masked_edges(std::integral_constant<int, kMseGroup>{});
     if (lane == 0) sc.nc[warp] = nc;
     first = false;
     __syncthreads();
@@ -885,24 +921,24 @@ int mse_warp_max() { return kMqEntries; }
 bool mse_lazy_fits(int64_t max_len) { return max_len <= (int64_t)kMseMaxCluster * (kMseSlice - 4); }
 
 int mse_lazy_min_split(int64_t max_len) {
-  int S = 1;
-  while (S < kMseMaxCluster && max_len > (int64_t)S * (kMseSlice - 4)) S *= 2;
-  return S;
+  return (int)std::min<int64_t>(kMseMaxCluster,
+                                std::max<int64_t>(1, (max_len + kMseSlice - 5) / (kMseSlice - 4)));
 }
 
 cudaError_t prepare_mse_lazy(const Problem& pr) {
-  for (int C : {8, 32})
+  for (int C : {8, 32}) {
     if (cudaError_t e = allow_smem(mse_fn(C), (int)mse_hist_smem(pr, C))) return e;
+    if (cudaError_t e = allow_cluster(mse_fn(C))) return e;
+  }
   return allow_smem((const void*)k_mse_warp, (int)mse_warp_smem(pr));
 }
 
 int mse_lazy_split(const Problem& pr, int A, int64_t max_len, int n_sm) {
-  int S = mse_lazy_min_split(max_len);
-  // up to one wave of CTAs at two per SM, slices of at least 1024 entries
-  while (2 * S <= kMseMaxCluster && (int64_t)A * pr.P * (2 * S) <= 2 * (int64_t)n_sm &&
-         max_len / (2 * S) >= 1024)
-    S *= 2;
-  return S;
+  // as many slices as one wave of CTAs (three per SM) takes, of at least 2048
+  // entries
+  const int64_t wave = 3 * (int64_t)n_sm / ((int64_t)A * pr.P);
+  const int64_t S = std::min<int64_t>({wave, max_len / 2048, kMseMaxCluster});
+  return (int)std::max<int64_t>(S, mse_lazy_min_split(max_len));
 }
 
 cudaError_t launch_mse_lazy(const Problem& pr, const Swarm& sw, const NodeDesc* nodes, int A,
