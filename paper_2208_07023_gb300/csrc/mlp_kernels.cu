@@ -269,6 +269,80 @@ __global__ void __launch_bounds__((T / R) * (T / R))
   }
 }
 
+// A layer's forward product on few rows: C[M x N] = A[M x K] B[K x N] (+ bias,
+// clipped), 16 x 16 tiles, two adjacent outputs per thread, operands through
+// a ring of kFwdStages shared-memory stages of 128 k (asynchronous copies, two
+// stages in flight while one computes). K and N are multiples of 16. One FP32
+// chain per output over k in increasing order: k_gemm's bits. The chain is
+// what bounds it (K = 5376: 5376 dependent FMAs of 4 clocks, 10 us); with
+// k_gemm's two register-staged steps of 64 the first layer took 95 us, most
+// of it waiting for each step's loads; now 40 us at 64 rows, the shared-memory
+// loads and 2 FMAs per k being issued by only 4 warps per SM.
+constexpr int kFwdK = 128, kFwdStages = 3;
+constexpr int kFwdA = 16 * (kFwdK + 4);          // floats: [16 rows][128 k + 4]
+constexpr int kFwdBytes = kFwdA * 4 + kFwdK * 16 * 2;  // and [128 k][16 columns] bfloat16
+
+template <int EPI>
+__global__ void __launch_bounds__(128)
+    k_gemm_fwd(int M, int N, int K, const float* __restrict__ A, const __nv_bfloat16* __restrict__ B,
+               const float* __restrict__ bias, float* __restrict__ C) {
+  __shared__ __align__(16) unsigned char sm[kFwdStages][kFwdBytes];
+  const int m0 = blockIdx.y * 16, n0 = blockIdx.x * 16;
+  const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
+  const int ns = (K + kFwdK - 1) / kFwdK;
+  auto stage = [&](int s) {
+    if (s < ns) {
+      float* a = reinterpret_cast<float*>(sm[s % kFwdStages]);
+      unsigned char* b = sm[s % kFwdStages] + kFwdA * 4;
+      const int k0 = s * kFwdK, kc = min(kFwdK, K - k0);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {  // 16 rows x 32 pieces
+        const int id = (int)threadIdx.x + 128 * i, r = id >> 5, k = 4 * (id & 31);
+        const bool in = k < kc && m0 + r < M;
+        cp_async16(a + r * (kFwdK + 4) + k, in ? A + (int64_t)(m0 + r) * K + k0 + k : A,
+                   in ? 16 : 0);
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {  // 128 k x 2 pieces
+        const int id = (int)threadIdx.x + 128 * i, k = id >> 1, h = id & 1;
+        const bool in = k < kc;
+        cp_async16(b + k * 32 + 16 * h, in ? B + (int64_t)(k0 + k) * N + n0 + 8 * h : B,
+                   in ? 16 : 0);
+      }
+    }
+    cp_async_commit();
+  };
+#pragma unroll
+  for (int s = 0; s < kFwdStages - 1; ++s) stage(s);
+  float c0 = 0.0f, c1 = 0.0f;
+  for (int s = 0; s < ns; ++s) {
+    cp_async_wait<kFwdStages - 2>();
+    __syncthreads();  // stage s is in place; every thread is done with s - 1
+    stage(s + kFwdStages - 1);
+    const float* a = reinterpret_cast<const float*>(sm[s % kFwdStages]) + ty * (kFwdK + 4);
+    const uint32_t* b =
+        reinterpret_cast<const uint32_t*>(sm[s % kFwdStages] + kFwdA * 4) + tx;
+    const int kc = min(kFwdK, K - s * kFwdK);
+#pragma unroll 4
+    for (int k = 0; k < kc; k += 4) {
+      const float4 x = *reinterpret_cast<const float4*>(a + k);
+      const uint32_t w0 = b[8 * k], w1 = b[8 * k + 8], w2 = b[8 * k + 16], w3 = b[8 * k + 24];
+      c0 = fmaf(x.x, __uint_as_float(w0 << 16), c0);
+      c1 = fmaf(x.x, __uint_as_float(w0 & 0xffff0000u), c1);
+      c0 = fmaf(x.y, __uint_as_float(w1 << 16), c0);
+      c1 = fmaf(x.y, __uint_as_float(w1 & 0xffff0000u), c1);
+      c0 = fmaf(x.z, __uint_as_float(w2 << 16), c0);
+      c1 = fmaf(x.z, __uint_as_float(w2 & 0xffff0000u), c1);
+      c0 = fmaf(x.w, __uint_as_float(w3 << 16), c0);
+      c1 = fmaf(x.w, __uint_as_float(w3 & 0xffff0000u), c1);
+    }
+  }
+  const int m = m0 + ty, n = n0 + 2 * tx;
+  if (m < M)
+    *reinterpret_cast<float2*>(C + (int64_t)m * N + n) =
+        make_float2(epilogue<EPI>(c0, bias, m, n, N), epilogue<EPI>(c1, bias, m, n + 1, N));
+}
+
 __device__ __forceinline__ double block_sum(double v, double* sh) {
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
@@ -321,14 +395,20 @@ __global__ void __launch_bounds__(256)
   if (j == 0) atomicAdd(loss, (1.0 - c * c / q + spread / kP) / N);
 }
 
-// out[n] = sum over rows of X[rows x n_cols] column n.
-__global__ void k_colsum(const float* __restrict__ X, int rows, int n_cols, float* out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= n_cols) return;
+// The bias gradients: column sums over the batch's rows of dO, dH2 and dH1,
+// one thread per column.
+__global__ void __launch_bounds__(64)
+    k_bias_grads(const float* __restrict__ dO, const float* __restrict__ dH2,
+                 const float* __restrict__ dH1, int rows, float* b3, float* b2, float* b1) {
+  const int c0 = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c0 >= kOut + 2 * kH) return;
+  const int l = c0 < kOut ? 0 : c0 < kOut + kH ? 1 : 2;
+  const int n = l == 0 ? kOut : kH, c = l == 0 ? c0 : (c0 - kOut) % kH;
+  const float* X = l == 0 ? dO : l == 1 ? dH2 : dH1;
   float s = 0.0f;
-#pragma unroll 16
-  for (int r = 0; r < rows; ++r) s += X[(int64_t)r * n_cols + c];
-  out[c] = s;
+#pragma unroll 32
+  for (int r = 0; r < rows; ++r) s += X[(int64_t)r * n + c];
+  (l == 0 ? b3 : l == 1 ? b2 : b1)[c] = s;
 }
 
 // One Adam step (Kingma and Ba, 2015) on parameters i .. i + 3 of the packed
@@ -543,17 +623,26 @@ cudaError_t launch_node_stats(const Problem& pr, const NodeDesc* nodes, int A,
   return cudaGetLastError();
 }
 
+// A layer's forward product: few rows by k_gemm_fwd (below one 64 x 64 tile
+// per SM of a 152-SM GPU), else k_gemm.
+template <int EPI>
+cudaError_t gemm_fwd(int M, int N, int K, const float* A, const __nv_bfloat16* B,
+                     const float* bias, float* C, cudaStream_t st) {
+  const int64_t tiles = (int64_t)((N + 63) / 64) * ((M + 63) / 64);
+  if (M <= 0) return cudaSuccess;
+  if (tiles >= 152) return gemm<false, false, __nv_bfloat16, EPI>(M, N, K, A, K, B, N, bias, C, N, st);
+  k_gemm_fwd<EPI><<<dim3((unsigned)(N / 16), (unsigned)((M + 15) / 16)), 128, 0, st>>>(
+      M, N, K, A, B, bias, C);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_mlp_forward(const MlpParams& m, const float* S, int N, MlpWork w,
                                cudaStream_t st) {
+  static_assert(kIn % 16 == 0 && kH % 16 == 0 && kOut % 16 == 0, "k_gemm_fwd's tiles");
   cudaError_t e;
-  if ((e = gemm<false, false, __nv_bfloat16, kBiasRelu>(N, kH, kIn, S, kIn, m.W1b, kH, m.b1, w.H1,
-                                                       kH, st)))
-    return e;
-  if ((e = gemm<false, false, __nv_bfloat16, kBiasRelu>(N, kH, kH, w.H1, kH, m.W2b, kH, m.b2, w.H2,
-                                                       kH, st)))
-    return e;
-  return gemm<false, false, __nv_bfloat16, kBias>(N, kOut, kH, w.H2, kH, m.W3b, kOut, m.b3, w.O,
-                                                  kOut, st);
+  if ((e = gemm_fwd<kBiasRelu>(N, kH, kIn, S, m.W1b, m.b1, w.H1, st))) return e;
+  if ((e = gemm_fwd<kBiasRelu>(N, kH, kH, w.H1, m.W2b, m.b2, w.H2, st))) return e;
+  return gemm_fwd<kBias>(N, kOut, kH, w.H2, m.W3b, m.b3, w.O, st);
 }
 
 cudaError_t launch_mlp_loss_grad(const MlpParams& m, const float* S, const int32_t* dims,
@@ -566,21 +655,19 @@ cudaError_t launch_mlp_loss_grad(const MlpParams& m, const float* S, const int32
   // layer 3: gW3 = H2^T dO, gb3 = colsum dO, dH2 = dO W3^T (x relu')
   if ((e = gemm<true, false, float, kPlain>(kH, kOut, N, w.H2, kH, w.dO, kOut, nullptr, g.W3, kOut, st)))
     return e;
-  k_colsum<<<blocks(kOut, 64), 64, 0, st>>>(w.dO, N, kOut, g.b3);
   if ((e = gemm<false, true, __nv_bfloat16, kReluMask>(N, kH, kOut, w.dO, kOut, m.W3b, kOut, w.H2,
                                                       w.dH2, kH, st)))
     return e;
   // layer 2
   if ((e = gemm<true, false, float, kPlain>(kH, kH, N, w.H1, kH, w.dH2, kH, nullptr, g.W2, kH, st)))
     return e;
-  k_colsum<<<blocks(kH, 64), 64, 0, st>>>(w.dH2, N, kH, g.b2);
   if ((e = gemm<false, true, __nv_bfloat16, kReluMask>(N, kH, kH, w.dH2, kH, m.W2b, kH, w.H1, w.dH1,
                                                       kH, st)))
     return e;
   // layer 1
   if ((e = gemm<true, false, float, kPlain>(kIn, kH, N, S, kIn, w.dH1, kH, nullptr, g.W1, kH, st)))
     return e;
-  k_colsum<<<blocks(kH, 64), 64, 0, st>>>(w.dH1, N, kH, g.b1);
+  k_bias_grads<<<blocks(kOut + 2 * kH, 64), 64, 0, st>>>(w.dO, w.dH2, w.dH1, N, g.b3, g.b2, g.b1);
   return cudaGetLastError();
 }
 

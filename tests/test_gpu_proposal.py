@@ -92,6 +92,20 @@ def test_forward_matches_oracle(ctx):
         prop.free()
 
 
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 130, 1215])
+def test_forward_rows_do_not_depend_on_the_batch(ctx, n):
+    # few rows run in 16 x 16 tiles, 1,216 rows and more (for the hidden
+    # layers) in 64 x 64 tiles: one chain of the same order per output
+    m = rand_net(9)
+    s, _, _ = rand_batch(10, 1300)
+    p = ctx.proposal()
+    try:
+        p.set(m)
+        assert np.array_equal(p.forward(s[:n]), p.forward(s)[:n])
+    finally:
+        p.free()
+
+
 def test_loss_and_gradient_match_oracle(ctx):
     m = rand_net(4)
     prop = ctx.proposal(seed=3)
