@@ -181,3 +181,31 @@ def test_regression_pairs_of_particles_per_block(ctxs):
     assert (g["kind"] == 1).sum() >= 64  # levels of 32+ nodes x 127 particles were scored
     fa.free()
     fb.free()
+
+
+@pytest.mark.parametrize("crit,P,B,K,d,bf16", [
+    ("gini", 33, 128, 5, 12, False),    # 528 pairs: an odd swarm, the last block one particle
+    ("entropy", 40, 50, 7, 13, False),
+    ("gini", 48, 256, 10, 70, False),
+    ("gini", 32, 256, 10, 830, False),  # 512 pairs, too much memory for two particles
+    ("gini", 64, 64, 3, 32, True),      # the BF16 form's passes (top k by the last block)
+])
+def test_classification_pairs_of_particles_per_block(ctxs, ctx_step, crit, P, B, K, d, bf16):
+    """Batches of 512 node-particle pairs and more score two particles per
+    block: the same forests as the staged-copy kernel."""
+    from paper_2208_07023_gb300 import binding as S
+    a, b = ctxs
+    wl = W.gmm(2501 if d > 100 else 9001, d, K, seed=21)
+    kw = dict(proj=S.SLM_PROJ_BF16_TOPK, topk=16) if bf16 else {}
+    p = S.make_params(crit, K, n_particles=P, n_iters=5, n_bins=B, min_leaf=4, seed=5,
+                      max_depth=3, n_trees=16, bootstrap=True, **kw)
+    fb = b.train_tree(p, wl.X, labels=wl.labels)
+    for c in (a, ctx_step):
+        c.set_small_nodes(0, 0)  # every level through the classification kernel
+        try:
+            fa = c.train_tree(p, wl.X, labels=wl.labels)
+        finally:
+            c.set_small_nodes()
+        same_tree(fa, fb, 16)
+        fa.free()
+    fb.free()
