@@ -132,6 +132,11 @@ __global__ void __launch_bounds__(32 * (FOLD ? kFoldWarps : kProjWarps))
   constexpr int NS = kStepStages;
   constexpr int TF = FOLD ? 8 : 16;      // features of an unrolled turn
   constexpr int W = QP >= 4 ? QP - 4 : QP;  // particles per lane beyond the first four
+  // Ranges are exchanged once per (node, slice) where two registers a particle
+  // are free, else after each block (64 trees on 100,000 x 32 rows, P = 48:
+  // 219 us instead of 253; with QP = 8 they spill: 112 us instead of 99 in
+  // the first levels of SLM Boost, and the folded kernels lose 2%).
+  constexpr bool kRun = !FOLD && QP <= 6;
   static_assert(RB * PB == NW && QP >= 1 && QP <= 8 && PU <= 64, "tile shape");
   extern __shared__ __align__(16) float sm[];
   __shared__ int s_lo[64], s_hi[64];  // ordered-int range of each particle of the slice
@@ -446,6 +451,46 @@ __global__ void __launch_bounds__(32 * (FOLD ? kFoldWarps : kProjWarps))
     const int take = min(left, nb - first);
     const int pg0 = slice * PU;
     node_positions(a, pg0, first == 0);
+    // this lane's ranges of its particles, over the warp's blocks (kRun) or a
+    // block
+    constexpr int QR = (QP + 3) & ~3;  // particles of the range exchange
+    float lo[QR], hi[QR];
+    auto reset_ranges = [&] {
+#pragma unroll
+      for (int j = 0; j < QR; ++j) {
+        lo[j] = FLT_MAX;
+        hi[j] = -FLT_MAX;
+      }
+    };
+    auto exchange_ranges = [&] {
+      // The four lanes that share these particles (rg) exchange ranges,
+      // halving their particles each time: every lane ends with QR / 4
+      // particles' ranges over all the warp's rows (3 QR / 2 shuffles; a
+      // reduction of each particle by every lane takes 4 QR).
+#pragma unroll
+      for (int j = 0; j < QR / 2; ++j) {
+        const bool up = rg & 1;
+        const float sl = up ? lo[j] : lo[j + QR / 2], sh = up ? hi[j] : hi[j + QR / 2];
+        const float kl = up ? lo[j + QR / 2] : lo[j], kh = up ? hi[j + QR / 2] : hi[j];
+        lo[j] = fminf(kl, __shfl_xor_sync(0xffffffffu, sl, 1));
+        hi[j] = fmaxf(kh, __shfl_xor_sync(0xffffffffu, sh, 1));
+      }
+#pragma unroll
+      for (int j = 0; j < QR / 4; ++j) {
+        const bool up = rg & 2;
+        const float sl = up ? lo[j] : lo[j + QR / 4], sh = up ? hi[j] : hi[j + QR / 4];
+        const float kl = up ? lo[j + QR / 4] : lo[j], kh = up ? hi[j + QR / 4] : hi[j];
+        lo[j] = fminf(kl, __shfl_xor_sync(0xffffffffu, sl, 2));
+        hi[j] = fmaxf(kh, __shfl_xor_sync(0xffffffffu, sh, 2));
+        const int jj = (rg & 1) * (QR / 2) + (rg >> 1) * (QR / 4) + j;
+        const int pl = my_particle(jj);
+        if (jj < QP && pg0 + pl < P) {
+          atomicMin(&s_lo[pl], f2ord(lo[j]));
+          atomicMax(&s_hi[pl], f2ord(hi[j]));
+        }
+      }
+    };
+    if (kRun) reset_ranges();
     for (int b = first + rw; b < first + take; b += RB) {
       uint64_t acc[4][QP];
 #pragma unroll
@@ -542,20 +587,14 @@ __global__ void __launch_bounds__(32 * (FOLD ? kFoldWarps : kProjWarps))
           if (k + 1 < kc) read(o[0], k + 1, key0 + ((k + 1) >> 2));
         }
       }
-      // block complete: its ranges into the CTA's, z out (16 bytes a store
+      // block complete: its ranges into the lane's, z out (16 bytes a store
       // where the block is whole and aligned)
       const int nr = min(kBR, nd.seg_len - b * kBR);
       const int64_t zrow = (int64_t)nd.seg_start + b * kBR;
       const bool whole = nr == kBR;
       const bool v16 = z16 && whole && (zrow & 3) == 0;
+      if (!kRun) reset_ranges();
       float* zp = sw.z + (int64_t)(pg0 + my_particle(0)) * pr.Ez + zrow + 4 * rg;
-      constexpr int QR = (QP + 3) & ~3;  // particles of the range exchange
-      float lo[QR], hi[QR];
-#pragma unroll
-      for (int j = 0; j < QR; ++j) {
-        lo[j] = FLT_MAX;
-        hi[j] = -FLT_MAX;
-      }
 #pragma unroll
       for (int j = 0; j < QP; ++j) {
         const int p = pg0 + my_particle(j);
@@ -595,33 +634,9 @@ __global__ void __launch_bounds__(32 * (FOLD ? kFoldWarps : kProjWarps))
           }
         }
       }
-      // The four lanes that share these particles (rg) exchange ranges,
-      // halving their particles each time: every lane ends with QR / 4
-      // particles' ranges over all the block's rows (3 QR / 2 shuffles; a
-      // reduction of each particle by every lane takes 4 QR).
-#pragma unroll
-      for (int j = 0; j < QR / 2; ++j) {
-        const bool up = rg & 1;
-        const float sl = up ? lo[j] : lo[j + QR / 2], sh = up ? hi[j] : hi[j + QR / 2];
-        const float kl = up ? lo[j + QR / 2] : lo[j], kh = up ? hi[j + QR / 2] : hi[j];
-        lo[j] = fminf(kl, __shfl_xor_sync(0xffffffffu, sl, 1));
-        hi[j] = fmaxf(kh, __shfl_xor_sync(0xffffffffu, sh, 1));
-      }
-#pragma unroll
-      for (int j = 0; j < QR / 4; ++j) {
-        const bool up = rg & 2;
-        const float sl = up ? lo[j] : lo[j + QR / 4], sh = up ? hi[j] : hi[j + QR / 4];
-        const float kl = up ? lo[j + QR / 4] : lo[j], kh = up ? hi[j + QR / 4] : hi[j];
-        lo[j] = fminf(kl, __shfl_xor_sync(0xffffffffu, sl, 2));
-        hi[j] = fmaxf(kh, __shfl_xor_sync(0xffffffffu, sh, 2));
-        const int jj = (rg & 1) * (QR / 2) + (rg >> 1) * (QR / 4) + j;
-        const int pl = my_particle(jj);
-        if (jj < QP && pg0 + pl < P) {
-          atomicMin(&s_lo[pl], f2ord(lo[j]));
-          atomicMax(&s_hi[pl], f2ord(hi[j]));
-        }
-      }
+      if (!kRun) exchange_ranges();
     }
+    if (kRun && rw < take) exchange_ranges();
     __syncthreads();  // every warp's ranges are in; the positions are read
     flush_ranges(a, pg0);
     left -= take;
