@@ -618,7 +618,7 @@ slm_status slm_set_projection_tma(slm_ctx* ctx, int32_t on);
  * step of the previous evaluation, Algorithm 1, and moves every particle)
  * and the histogram pass (which leaves the gB-independent terms of the next
  * move), two launches instead of three. With on = 1 only a batch of at most
- * 48 blocks per SM and one node per SM is folded: there the iteration is
+ * 24 blocks per SM and one node per SM is folded: there the iteration is
  * latency-bound and the saved launch pays. on = 2 folds every eligible
  * batch; on = 0 none, with the tuned row-major projection, histogram and
  * move kernels. Results are identical either way.

@@ -30,7 +30,7 @@ struct DevBuf {
 
 // A plain search's move is folded into its projection when the batch has at
 // most this many blocks of 32 rows per CTA of the projection's grid.
-constexpr int kFoldMaxBlocks = 48;
+constexpr int kFoldMaxBlocks = 24;
 
 enum Slot {
   W_X, W_LAB, W_Y, W_IDX, W_W, W_BINS, W_XL, W_LABL, W_YL,
@@ -1457,8 +1457,9 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
     int sh = -1, grid = 0;
     if (every && !p->apso && step_ok(pr)) {
       // Folding pays where the chain is latency-bound: up to kFoldMaxBlocks
-      // blocks per CTA (100,000 x 32 rows, P = 48: 28 us an iteration folded,
-      // 30 not; 1,000,000 rows: 173 and 167), and where no CTA forms two
+      // blocks per CTA (100,000 x 32 rows, P = 48: 25 us an iteration folded,
+      // 27 not; 200,000 x 128 rows, P = 64, third to sixth level: 125 to 142
+      // and 119 to 132; 400,000 x 32, P = 32: 69 and 45), and where no CTA forms two
       // nodes' positions one after the other (a 30,011 x 50 regression tree:
       // 22.6 ms, 23.1 when its levels of more nodes than CTAs fold too).
       StepConfig c0;
@@ -1472,8 +1473,12 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
         const int f = forced && step_config(pr, c->step_shape, &want) ? c->step_shape : 0;
         // The shape of the least estimated time: the warps' blocks one after
         // another (8 clocks per feature and particle of a thread, and the
-        // shared-memory latency that one warp does not hide), or the SM's
-        // FP32 pipes when its warps are many; and the slice's move.
+        // shared-memory latency that one warp does not hide), or those of
+        // the scheduler with the most warps' worth (8 clocks more a feature:
+        // its reads and swaps, which a narrow tile repeats for fewer
+        // products); and the slice's move. Without the 8 clocks halves of a
+        // swarm of 32 looked as cheap as whole ones: 30,000 x 500 rows took
+        // 55 us an iteration instead of 45, 50,000 x 128 27 instead of 24.
         double best = 0.0;
         for (int k = 0; k < kStepShapeCount; ++k) {
           StepConfig q;
@@ -1484,9 +1489,9 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
           const int64_t units = blocks * q.slices, m = (units + g - 1) / g;
           const int64_t ctas = std::min<int64_t>(g, units);
           const double rounds = (double)((m + q.row_warps - 1) / q.row_warps);
-          const double per_sm = (double)m * ((ctas + c->n_sm - 1) / c->n_sm) * q.pb / 4.0;
+          const int64_t per_sm = (m * ((ctas + c->n_sm - 1) / c->n_sm) * q.pb + 3) / 4;
           const double lat = rounds * pr.d * (8.0 * q.qp + 12.0);
-          const double thr = std::max(1.0, per_sm) * pr.d * 8.0 * q.qp;
+          const double thr = (double)per_sm * pr.d * (8.0 * q.qp + 8.0);
           const double est = std::max(lat, thr) + 8.0 * q.qp * q.pb * pr.d / 10.0;
           if (grid == 0 || est < best) {
             best = est;
