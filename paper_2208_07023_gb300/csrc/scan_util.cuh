@@ -184,41 +184,64 @@ __device__ EvalRes block_scan_mse(const uint32_t* cnt, const long long* s, const
 
 // The whole CTA selects node a's tk_k best particles by sw.cur (ties to the
 // lower index; rank = particles strictly better, or equal and lower) and
-// gathers their positions. scratch: P EvalRes + 2 P ints of shared memory.
+// gathers their positions. scratch: P EvalRes + P keys of shared memory.
+//
+// It is the tail of the last CTA to score a node, so its length is what
+// counts: a warp ranks a particle against 32 others at a time, by their loss
+// keys and by better() only where these are within 8 ulps (equal losses, and
+// Gini's rationals closer than their doubles) or not a number; one warp
+// compacts the taken particles by ballots.
 __device__ __noinline__ void topk_select(const Problem& pr, const Swarm& sw, int a,
                                          unsigned char* scratch) {
-  EvalRes* s_sc = reinterpret_cast<EvalRes*>(scratch);
-  int* s_take = reinterpret_cast<int*>(s_sc + pr.P);
-  int* s_sel = s_take + pr.P;
+  EvalRes* s_sc = reinterpret_cast<EvalRes*>(scratch);  // (bin: taken)
+  uint64_t* s_key = reinterpret_cast<uint64_t*>(s_sc + pr.P);
+  int* s_sel = reinterpret_cast<int*>(s_key);  // once the keys are read
   const int P = pr.P, Pp = pr.Pp, d = pr.d, k = sw.tk_k, kp = sw.tk_kp;
-  for (int p = threadIdx.x; p < P; p += blockDim.x) s_sc[p] = ldcg_res(sw.cur + (int64_t)a * Pp + p);
-  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  constexpr uint64_t kNan = ~0ull - 1;
   for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    const EvalRes me = s_sc[p];
+    const EvalRes e = ldcg_res(sw.cur + (int64_t)a * Pp + p);
+    s_sc[p] = e;
+    const bool nan = ((uint64_t)__double_as_longlong(e.loss) << 1) > 0xffe0000000000000ull;
+    s_key[p] = e.valid && nan ? kNan : loss_key(e);
+  }
+  __syncthreads();
+  for (int p = warp; p < P; p += nw) {
+    const uint64_t km = s_key[p];
     int rank = 0;
-    for (int q = 0; q < P; ++q) {
-      if (q == p) continue;
-      const EvalRes o = s_sc[q];
-      if (better(o, me, pr.crit) || (q < p && !better(me, o, pr.crit))) ++rank;
+    for (int q = lane; q < P; q += 32) {
+      const uint64_t ko = s_key[q];
+      bool first = ko < km;  // q ranks before p
+      if ((first ? km - ko : ko - km) <= 8 || ko == kNan || km == kNan)
+        first = better(s_sc[q], s_sc[p], pr.crit) ||
+                (q < p && !better(s_sc[p], s_sc[q], pr.crit));
+      rank += q != p && first;
     }
-    s_take[p] = rank < k;
+    rank = __reduce_add_sync(0xffffffffu, rank);
+    if (lane == 0) s_sc[p].bin = rank < k;
   }
   __syncthreads();
-  for (int p = threadIdx.x; p < Pp; p += blockDim.x) {
-    int q = -1;
-    if (p < P && s_take[p]) {
-      q = 0;
-      for (int j = 0; j < p; ++j) q += s_take[j];
-      s_sel[q] = p;
-      sw.tk_sel[(int64_t)a * k + q] = p;
+  if (warp == 0) {
+    int n = 0;  // taken so far
+    for (int p0 = 0; p0 < Pp; p0 += 32) {
+      const int p = p0 + lane;
+      const bool take = p < P && s_sc[p].bin;
+      const unsigned m = __ballot_sync(0xffffffffu, take);
+      const int q = take ? n + __popc(m & ((1u << lane) - 1u)) : -1;
+      if (take) {
+        s_sel[q] = p;
+        sw.tk_sel[(int64_t)a * k + q] = p;
+      }
+      if (p < Pp) sw.tk_inv[(int64_t)a * Pp + p] = q;
+      n += __popc(m);
     }
-    sw.tk_inv[(int64_t)a * Pp + p] = q;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < kp * d; e += blockDim.x) {
-    const int q = e / d, j = e - q * d;
-    sw.tk_pos[((int64_t)a * kp + q) * d + j] =
-        q < k ? sw.pos[((int64_t)a * Pp + s_sel[q]) * d + j] : 0.0f;
+  for (int q = warp; q < kp; q += nw) {
+    const float* src = sw.pos + ((int64_t)a * Pp + (q < k ? s_sel[q] : 0)) * d;
+    float* dst = sw.tk_pos + ((int64_t)a * kp + q) * d;
+#pragma unroll 4
+    for (int j = lane; j < d; j += 32) dst[j] = q < k ? src[j] : 0.0f;
   }
 }
 
