@@ -2024,42 +2024,54 @@ __global__ void __launch_bounds__(kTS)
                   const unsigned long long* __restrict__ acc_w, const int32_t* __restrict__ acc_y,
                   long long* m1, long long* m2, double* mscale, uint32_t* mq, MseNode* mnode) {
   __shared__ unsigned long long s_s, s_q;
+  __shared__ double s_f1, s_f2;
+  __shared__ float s_c;
+  __shared__ int s_qs;
   const WorkTile wt = tiles[blockIdx.x];
   const int a = wt.node;
-  if (threadIdx.x == 0) s_s = s_q = 0ull;
-  __syncthreads();
-  const double W = (double)acc_w[a];
-  float c = 0.0f;
-  double D = 0.0;
-  if (acc_y[2 * a] != INT_MAX) {
-    const double ylo = ord2f(acc_y[2 * a]), yhi = ord2f(acc_y[2 * a + 1]);
-    c = (float)(0.5 * (ylo + yhi));
-    // rounding is monotone: every |y - c| below is at most D
-    D = fmax(yhi - (double)c, (double)c - ylo);
-  }
-  int s = 0, t = 0;
-  if (W > 0.0 && D > 0.0) {
-    int e1, e2;
-    frexp(W * D * (1.0 + 0x1p-40), &e1);      // W D < 2^e1
-    frexp(W * D * D * (1.0 + 0x1p-40), &e2);  // W D^2 < 2^e2
-    s = 61 - e1;
-    t = e2 + 2 * s - 61;
-  }
-  if (threadIdx.x == 0) {  // identical from every tile of the node
+  if (threadIdx.x == 0) {  // (double precision: two lanes per clock per SM)
+    s_s = s_q = 0ull;
+    const double W = (double)acc_w[a];
+    float c = 0.0f;
+    double D = 0.0;
+    if (acc_y[2 * a] != INT_MAX) {
+      const double ylo = ord2f(acc_y[2 * a]), yhi = ord2f(acc_y[2 * a + 1]);
+      c = (float)(0.5 * (ylo + yhi));
+      // rounding is monotone: every |y - c| below is at most D
+      D = fmax(yhi - (double)c, (double)c - ylo);
+    }
+    int s = 0, t = 0;
+    if (W > 0.0 && D > 0.0) {
+      int e1, e2;
+      frexp(W * D * (1.0 + 0x1p-40), &e1);      // W D < 2^e1
+      frexp(W * D * D * (1.0 + 0x1p-40), &e2);  // W D^2 < 2^e2
+      s = 61 - e1;
+      t = e2 + 2 * s - 61;
+    }
+    // identical from every tile of the node
     mscale[2 * a] = ldexp(1.0, -s);
     mscale[2 * a + 1] = ldexp(1.0, t - 2 * s);
+    // bits dropped by the 30-bit targets: |m1| <= D 2^s < 2^eb for one entry
+    int eb = 0;
+    s_f1 = ldexp(1.0, s);
+    s_f2 = ldexp(1.0, 2 * s - t);
+    if (D > 0.0) frexp(D * (1.0 + 0x1p-40) * s_f1, &eb);
+    const int qs = eb > 28 ? eb - 28 : 0;
+    s_c = c;
+    s_qs = qs;
+    if (mnode) mnode[a].inv = ldexp(1.0, qs - s);  // one unit of the rounded targets
   }
-  // bits dropped by the 30-bit targets: |m1| <= D 2^s < 2^eb for one entry
-  int eb = 0;
-  if (D > 0.0) frexp(D * (1.0 + 0x1p-40) * ldexp(1.0, s), &eb);
-  const int qs = eb > 28 ? eb - 28 : 0;
+  __syncthreads();
+  const float c = s_c;
+  const double f1 = s_f1, f2 = s_f2;
+  const int qs = s_qs;
   long long v1 = 0, v2 = 0;
   if ((int)threadIdx.x < wt.rows) {
     const int64_t e = wt.row0 + threadIdx.x;
     const double w = pr.w ? (double)pr.w[e] : 1.0;
     const double v = (double)pr.y[e] - (double)c;
-    v1 = llrint(w * v * ldexp(1.0, s));
-    v2 = llrint(w * v * v * ldexp(1.0, 2 * s - t));
+    v1 = llrint(w * v * f1);
+    v2 = llrint(w * v * v * f2);
     m1[e] = v1;
     m2[e] = v2;
     if (mq) {
@@ -2083,7 +2095,6 @@ __global__ void __launch_bounds__(kTS)
   if (threadIdx.x == 0) {
     atomicAdd(reinterpret_cast<unsigned long long*>(&mnode[a].S), s_s);
     atomicAdd(reinterpret_cast<unsigned long long*>(&mnode[a].Q), s_q);
-    mnode[a].inv = ldexp(1.0, qs - s);  // one unit of the rounded targets
   }
 }
 

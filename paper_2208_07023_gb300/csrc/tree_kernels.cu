@@ -8,12 +8,18 @@
 // right ("+") iff bin(gB . x) >= b*, i.e. z >= t_b.
 //
 // Every per-level pass runs over the same kTS-row tiles of the entry-ordered
-// level arrays (one CTA per tile), followed by a one-thread-per-node kernel
+// level arrays (one CTA per tile), followed by a one-warp-per-node kernel
 // where a per-node decision is needed, so shallow levels with a few large
-// nodes keep the whole GPU busy.
+// nodes keep the whole GPU busy. The passes over rows are bound by DRAM, the
+// per-node kernels by the chain over a large node's tiles. At 200,000 x 128
+// rows, with loads one at a time and 64-bit shared atomics before, and now:
+// side of every entry and decision 142 and 47 us a level, scatter 80 and 34,
+// statistics 99 and 53, the first gather 128 and 32.
 #include <cuda_runtime.h>
 #include <limits.h>
 #include <math.h>
+
+#include <type_traits>
 
 #include "slm_internal.cuh"
 
@@ -22,6 +28,7 @@ namespace slm {
 namespace {
 
 constexpr int kTT = kTS;  // threads per CTA = rows per tile
+constexpr int kNodeWarps = 4;  // nodes per CTA of the per-node kernels
 
 __device__ __forceinline__ int bin_of(float z, float zmin, float inv_w, int B) {
   const float off = __fsub_rn(z, zmin);
@@ -37,12 +44,89 @@ __device__ __forceinline__ int f2ord(float f) {
 }
 
 // gB . x as one fmaf per feature in increasing order from +0, the same
-// sequence the scoring kernels run.
+// sequence the scoring kernels run. Rows of whole 16-byte words (v4) are read
+// eight words ahead of their products, a 128-byte line per thread.
 __device__ __forceinline__ float project_row(const float* __restrict__ x,
-                                             const float* __restrict__ g, int d) {
+                                             const float* __restrict__ g, int d, bool v4) {
   float acc = 0.0f;
-  for (int j = 0; j < d; ++j) acc = fmaf(__ldg(x + j), g[j], acc);
+  int j = 0;
+  if (v4) {
+    constexpr int U = 8;
+    for (; j + 4 * U <= d; j += 4 * U) {
+      float4 v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) v[u] = __ldg(reinterpret_cast<const float4*>(x + j) + u);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        acc = fmaf(v[u].x, g[j + 4 * u], acc);
+        acc = fmaf(v[u].y, g[j + 4 * u + 1], acc);
+        acc = fmaf(v[u].z, g[j + 4 * u + 2], acc);
+        acc = fmaf(v[u].w, g[j + 4 * u + 3], acc);
+      }
+    }
+  }
+#pragma unroll 8
+  for (; j < d; ++j) acc = fmaf(__ldg(x + j), g[j], acc);
   return acc;
+}
+
+// The weight of a tile's entries, in total or per class, in two 32-bit
+// halves: a tile's kTS = 256 entries of up to 2^32 - 1 add up to less than
+// 2^24 in each (64-bit shared atomics retry in a loop).
+struct TileWeight {
+  uint32_t lo, hi;
+  __device__ __forceinline__ void add(uint32_t w) {
+    atomicAdd(&lo, w & 0xffffu);
+    if (w >> 16) atomicAdd(&hi, w >> 16);
+  }
+  __device__ __forceinline__ unsigned long long sum() const {
+    return (unsigned long long)lo + ((unsigned long long)hi << 16);
+  }
+};
+// the same over a warp, in every lane
+__device__ __forceinline__ unsigned long long warp_weight(uint32_t w) {
+  return (unsigned long long)__reduce_add_sync(0xffffffffu, w & 0xffffu) +
+         ((unsigned long long)__reduce_add_sync(0xffffffffu, w >> 16) << 16);
+}
+
+// Copies the rows of a tile (its thread r: row r of src to row s_to[r] of
+// dst), 16 bytes a lane where rows and arrays allow.
+__device__ __forceinline__ void copy_rows(const float* __restrict__ src, const int* s_from,
+                                          float* __restrict__ dst, const int* s_to, int rows,
+                                          int d) {
+  const bool v4 = (d & 3) == 0 && ((reinterpret_cast<uintptr_t>(src) |
+                                    reinterpret_cast<uintptr_t>(dst)) & 15) == 0;
+  auto run = [&](auto* out, const auto* in, int w) {  // w words a row
+    using T = std::remove_const_t<std::remove_pointer_t<decltype(out)>>;
+    constexpr int U = 8;  // words in flight per thread
+    const int step_r = kTT / w, step_j = kTT - step_r * w;
+    int r = (int)threadIdx.x / w, j = (int)threadIdx.x - r * w;
+    while (r < rows) {
+      T v[U];
+      int64_t o[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        o[u] = -1;
+        if (r < rows) {
+          v[u] = __ldg(in + (int64_t)s_from[r] * w + j);
+          o[u] = (int64_t)s_to[r] * w + j;
+        }
+        r += step_r;
+        j += step_j;
+        if (j >= w) {
+          j -= w;
+          ++r;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (o[u] >= 0) out[o[u]] = v[u];
+    }
+  };
+  if (v4)
+    run(reinterpret_cast<float4*>(dst), reinterpret_cast<const float4*>(src), d >> 2);
+  else
+    run(dst, src, d);
 }
 
 // Block-wide exclusive scan of one int per thread (kTT threads); returns the
@@ -83,75 +167,116 @@ __global__ void __launch_bounds__(kTT)
     k_stats_tiles(Problem pr, const WorkTile* __restrict__ tiles, LevelAcc acc) {
   const WorkTile wt = tiles[blockIdx.x];
   const int K = pr.K;
-  __shared__ unsigned long long s_cnt[kMaxClasses];
-  __shared__ unsigned long long s_w;
+  __shared__ TileWeight s_cnt[kMaxClasses];
+  __shared__ unsigned long long s_w[kTT / 32];
   __shared__ double s_sy[kTT], s_sq[kTT];
   __shared__ int s_lo, s_hi;
-  if (threadIdx.x < kMaxClasses) s_cnt[threadIdx.x] = 0;
+  const bool mse = pr.crit == SLM_MSE;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x < kMaxClasses) s_cnt[threadIdx.x] = TileWeight{0u, 0u};
   if (threadIdx.x == 0) {
-    s_w = 0;
     s_lo = INT_MAX;
     s_hi = INT_MIN;
   }
   __syncthreads();
   const int r = threadIdx.x;
   double sy = 0.0, sq = 0.0;
+  uint32_t w = 0;
+  int lo = INT_MAX, hi = INT_MIN;
   if (r < wt.rows) {
     const int64_t e = (int64_t)wt.row0 + r;
-    const uint32_t w = pr.w ? pr.w[e] : 1u;
-    atomicAdd(&s_w, (unsigned long long)w);
-    if (pr.crit == SLM_MSE) {
+    w = pr.w ? pr.w[e] : 1u;
+    if (mse) {
       const float yv = pr.y[e];
       sy = (double)w * (double)yv;
       sq = sy * (double)yv;
-      atomicMin(&s_lo, f2ord(yv));
-      atomicMax(&s_hi, f2ord(yv));
+      lo = hi = f2ord(yv);
     } else {
-      atomicAdd(&s_cnt[pr.lab[e]], (unsigned long long)w);
+      s_cnt[pr.lab[e]].add(w);
     }
   }
-  s_sy[threadIdx.x] = sy;
-  s_sq[threadIdx.x] = sq;
-  __syncthreads();
-  for (int off = kTT / 2; off > 0; off >>= 1) {  // fixed order: deterministic
-    if (threadIdx.x < off) {
-      s_sy[threadIdx.x] += s_sy[threadIdx.x + off];
-      s_sq[threadIdx.x] += s_sq[threadIdx.x + off];
+  const unsigned long long ww = warp_weight(w);
+  if (lane == 0) s_w[warp] = ww;
+  if (mse) {
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) {
+      atomicMin(&s_lo, lo);
+      atomicMax(&s_hi, hi);
     }
+    s_sy[threadIdx.x] = sy;
+    s_sq[threadIdx.x] = sq;
+    __syncthreads();
+    for (int off = kTT / 2; off > 0; off >>= 1) {  // fixed order: deterministic
+      if (threadIdx.x < off) {
+        s_sy[threadIdx.x] += s_sy[threadIdx.x + off];
+        s_sq[threadIdx.x] += s_sq[threadIdx.x + off];
+      }
+      __syncthreads();
+    }
+  } else {
     __syncthreads();
   }
   const int l = wt.node;
-  if (threadIdx.x < K && pr.crit != SLM_MSE && s_cnt[threadIdx.x])
-    atomicAdd(&acc.cls[(int64_t)l * K + threadIdx.x], s_cnt[threadIdx.x]);
+  if (threadIdx.x < K && !mse && s_cnt[threadIdx.x].sum())
+    atomicAdd(&acc.cls[(int64_t)l * K + threadIdx.x], s_cnt[threadIdx.x].sum());
   if (threadIdx.x == 0) {
-    atomicAdd(&acc.w[l], s_w);
-    acc.tile_s[2 * blockIdx.x] = s_sy[0];
-    acc.tile_s[2 * blockIdx.x + 1] = s_sq[0];
-    if (pr.crit == SLM_MSE && s_lo != INT_MAX) {
+    unsigned long long tw = 0;
+    for (int i = 0; i < kTT / 32; ++i) tw += s_w[i];
+    atomicAdd(&acc.w[l], tw);
+    if (mse) {
+      acc.tile_s[2 * blockIdx.x] = s_sy[0];
+      acc.tile_s[2 * blockIdx.x + 1] = s_sq[0];
+    }
+    if (mse && s_lo != INT_MAX) {
       atomicMin(&acc.ylo[l], s_lo);
       atomicMax(&acc.yhi[l], s_hi);
     }
   }
 }
 
-// One thread per level node: leaf value, splittable flag, parent sums.
+// One warp per level node: leaf value, splittable flag, parent sums. The
+// tiles' target sums are added in tile order, 32 tiles fetched at a time,
+// lane 0 the first moments and lane 1 the second (one thread fetching them
+// one after the other took 92 us at 200,000 entries).
 __global__ void k_stats_finish(Problem pr, const LevelNode* __restrict__ nodes,
                                const int32_t* __restrict__ tile0, int L, LevelAcc acc,
                                TreeArrays tr, int max_depth, double* par,
                                int32_t* splittable) {
-  const int l = blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ double s_t[kNodeWarps][64];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int l = blockIdx.x * kNodeWarps + warp;
   if (l >= L) return;
   const LevelNode nd = nodes[l];
   const int K = pr.K;
   const unsigned long long nw = acc.w[l];
   const int slot = nd.slot;
   bool pure;
+  double sy = 0.0, sq = 0.0;
   if (pr.crit == SLM_MSE) {
-    double sy = 0.0, sq = 0.0;
-    for (int t = tile0[l]; t < tile0[l + 1]; ++t) {
-      sy += acc.tile_s[2 * t];
-      sq += acc.tile_s[2 * t + 1];
+    const int t1 = 2 * tile0[l + 1];
+    double v = 0.0;
+    int o = 2 * tile0[l];
+    double n0 = o + lane < t1 ? acc.tile_s[o + lane] : 0.0;
+    double n1 = o + 32 + lane < t1 ? acc.tile_s[o + 32 + lane] : 0.0;
+    for (; o < t1; o += 64) {
+      s_t[warp][lane] = n0;
+      s_t[warp][lane + 32] = n1;
+      __syncwarp();
+      if (o + 64 + lane < t1) n0 = acc.tile_s[o + 64 + lane];
+      if (o + 96 + lane < t1) n1 = acc.tile_s[o + 96 + lane];
+      const int m = min(64, t1 - o);
+      if (lane < 2) {
+#pragma unroll 8
+        for (int i = lane; i < m; i += 2) v += s_t[warp][i];
+      }
+      __syncwarp();
     }
+    sy = v;
+    sq = __shfl_sync(0xffffffffu, v, 1);
+  }
+  if (lane != 0) return;
+  if (pr.crit == SLM_MSE) {
     tr.leaf_value[slot] = nw ? sy / (double)nw : 0.0;
     tr.leaf_class[slot] = -1;
     pure = !(acc.yhi[l] > acc.ylo[l]);
@@ -188,44 +313,45 @@ __global__ void __launch_bounds__(kTT)
   const EvalRes gb = sw.gb[a];
   const int d = pr.d, K = pr.K;
   extern __shared__ float s_g[];  // [d]
-  __shared__ unsigned long long s_lk[kMaxClasses];
-  __shared__ unsigned long long s_wl;
-  __shared__ int s_n;
+  __shared__ TileWeight s_lk[kMaxClasses];
+  __shared__ unsigned long long s_wl[kTT / 32];
   if (!gb.valid) {
     if (threadIdx.x == 0) tile_left[blockIdx.x] = 0;
     return;
   }
   for (int j = threadIdx.x; j < d; j += kTT) s_g[j] = sw.gbest[(int64_t)a * d + j];
-  if (threadIdx.x < kMaxClasses) s_lk[threadIdx.x] = 0;
-  if (threadIdx.x == 0) {
-    s_wl = 0;
-    s_n = 0;
-  }
+  if (threadIdx.x < kMaxClasses) s_lk[threadIdx.x] = TileWeight{0u, 0u};
   __syncthreads();
   const int r = threadIdx.x;
+  uint32_t wl = 0;
+  int left = 0;
+  const bool v4 = (d & 3) == 0 && (reinterpret_cast<uintptr_t>(pr.X) & 15) == 0;
   if (r < wt.rows) {
     const int64_t e = (int64_t)wt.row0 + r;
-    const float z = project_row(pr.X + e * d, s_g, d);
+    const float z = project_row(pr.X + e * d, s_g, d, v4);
     const int b = bin_of(z, gb.zmin, gb.inv_w, pr.B);
     const int right = b >= gb.bin;
     side[e] = (uint8_t)right;
     if (!right) {
-      const uint32_t w = pr.w ? pr.w[e] : 1u;
-      atomicAdd(&s_n, 1);
-      atomicAdd(&s_wl, (unsigned long long)w);
-      if (pr.crit != SLM_MSE) atomicAdd(&s_lk[pr.lab[e]], (unsigned long long)w);
+      left = 1;
+      wl = pr.w ? pr.w[e] : 1u;
+      if (pr.crit != SLM_MSE) s_lk[pr.lab[e]].add(wl);
     }
   }
-  __syncthreads();
-  if (threadIdx.x < K && pr.crit != SLM_MSE && s_lk[threadIdx.x])
-    atomicAdd(&acc.lk[(int64_t)a * K + threadIdx.x], s_lk[threadIdx.x]);
+  const unsigned long long ww = warp_weight(wl);
+  if ((threadIdx.x & 31) == 0) s_wl[threadIdx.x >> 5] = ww;
+  const int n_left = __syncthreads_count(left);
+  if (threadIdx.x < K && pr.crit != SLM_MSE && s_lk[threadIdx.x].sum())
+    atomicAdd(&acc.lk[(int64_t)a * K + threadIdx.x], s_lk[threadIdx.x].sum());
   if (threadIdx.x == 0) {
-    tile_left[blockIdx.x] = s_n;
-    if (s_wl) atomicAdd(&acc.wl[a], s_wl);
+    tile_left[blockIdx.x] = n_left;
+    unsigned long long tw = 0;
+    for (int i = 0; i < kTT / 32; ++i) tw += s_wl[i];
+    if (tw) atomicAdd(&acc.wl[a], tw);
   }
 }
 
-// One thread per searched node: zero-gain test, internal-node fields, tile
+// One warp per searched node: zero-gain test, internal-node fields, tile
 // bases of the scatter. out3[a] = {split?, left entries, right entries}.
 __global__ void k_decide(Problem pr, Swarm sw, const NodeDesc* __restrict__ snodes,
                          const int32_t* __restrict__ map, const int32_t* __restrict__ tile0,
@@ -233,26 +359,38 @@ __global__ void k_decide(Problem pr, Swarm sw, const NodeDesc* __restrict__ snod
                          const unsigned long long* __restrict__ node_cls,
                          const double* __restrict__ par, PartAcc acc, TreeArrays tr,
                          int32_t* out3, int32_t* status) {
-  const int a = blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const int a = blockIdx.x * kNodeWarps + (threadIdx.x >> 5);
   if (a >= A) return;
   const NodeDesc nd = snodes[a];
   const EvalRes gb = sw.gb[a];
   const int d = pr.d, K = pr.K;
   int nl_entries = 0;
-  for (int t = tile0[a]; t < tile0[a + 1]; ++t) {
-    tile_base[t] = nl_entries;
-    nl_entries += gb.valid ? tile_left[t] : 0;
+  const int t1 = tile0[a + 1];
+  for (int t0 = tile0[a]; t0 < t1; t0 += 32) {
+    const int t = t0 + lane;
+    const int v = t < t1 && gb.valid ? tile_left[t] : 0;
+    int incl = v;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, off);
+      if (lane >= off) incl += u;
+    }
+    if (t < t1) tile_base[t] = nl_entries + incl - v;
+    nl_entries += __shfl_sync(0xffffffffu, incl, 31);
   }
-  out3[3 * a + 1] = nl_entries;
-  out3[3 * a + 2] = nd.seg_len - nl_entries;
+  if (lane == 0) {
+    out3[3 * a + 1] = nl_entries;
+    out3[3 * a + 2] = nd.seg_len - nl_entries;
+  }
   if (!gb.valid) {
-    out3[3 * a] = 0;
+    if (lane == 0) out3[3 * a] = 0;
     return;
   }
   const int l = map[a];
   const unsigned long long wleft = acc.wl[a];
   const unsigned long long nw = (unsigned long long)(gb.nl + gb.nr);
-  if (wleft != (unsigned long long)gb.nl) atomicExch(status, 2);  // must agree
+  if (lane == 0 && wleft != (unsigned long long)gb.nl) atomicExch(status, 2);  // must agree
   // Zero gain: children keep the parent's class mix (Gini and entropy are
   // strictly concave), or the MSE does not drop below the parent's.
   bool no_gain;
@@ -261,16 +399,19 @@ __global__ void k_decide(Problem pr, Swarm sw, const NodeDesc* __restrict__ snod
     const double parent = (sq - sy * sy / (double)nw) / (double)nw;
     no_gain = !(gb.loss < parent);
   } else {
-    no_gain = true;
-    for (int k = 0; k < K; ++k)
-      if (acc.lk[(int64_t)a * K + k] * nw != node_cls[(int64_t)l * K + k] * wleft)
-        no_gain = false;
+    bool differs = false;
+    for (int k = lane; k < K; k += 32)
+      differs |= acc.lk[(int64_t)a * K + k] * nw != node_cls[(int64_t)l * K + k] * wleft;
+    no_gain = !__any_sync(0xffffffffu, differs);
   }
-  out3[3 * a] = no_gain ? 0 : 1;
+  if (lane == 0) out3[3 * a] = no_gain ? 0 : 1;
   if (no_gain) return;
   const int slot = nd.slot;
+#pragma unroll 4
+  for (int j = lane; j < d; j += 32)
+    tr.dir[(int64_t)slot * d + j] = sw.gbest[(int64_t)a * d + j];
+  if (lane != 0) return;
   tr.kind[slot] = 1;
-  for (int j = 0; j < d; ++j) tr.dir[(int64_t)slot * d + j] = sw.gbest[(int64_t)a * d + j];
   tr.zmin[slot] = gb.zmin;
   tr.inv_w[slot] = gb.inv_w;
   tr.bin[slot] = gb.bin;
@@ -292,7 +433,7 @@ __global__ void __launch_bounds__(kTT)
   if (dl < 0) return;
   const int d = pr.d;
   __shared__ int sbuf[kTT / 32 + 1];
-  __shared__ int s_dst[kTT];
+  __shared__ int s_src[kTT], s_dst[kTT];
   const int r = threadIdx.x;
   const bool in = r < wt.rows;
   const int64_t e = (int64_t)wt.row0 + r;
@@ -304,6 +445,7 @@ __global__ void __launch_bounds__(kTT)
   const int base_r = rows_before - base_l;
   if (in) {
     const int32_t pos = is_left ? dl + base_l + rank_l : dr + base_r + (r - rank_l);
+    s_src[r] = (int)e;
     s_dst[r] = pos;
     nx.idx[pos] = idx_cur[e];
     if (nx.lab) nx.lab[pos] = pr.lab[e];
@@ -311,10 +453,7 @@ __global__ void __launch_bounds__(kTT)
     if (nx.w) nx.w[pos] = pr.w[e];
   }
   __syncthreads();
-  for (int q = threadIdx.x; q < wt.rows * d; q += kTT) {
-    const int rr = q / d, j = q - rr * d;
-    nx.X[(int64_t)s_dst[rr] * d + j] = pr.X[((int64_t)wt.row0 + rr) * d + j];
-  }
+  copy_rows(pr.X, s_src, nx.X, s_dst, wt.rows, d);
 }
 
 __global__ void __launch_bounds__(kTT)
@@ -340,19 +479,24 @@ __global__ void __launch_bounds__(kTT)
   if (threadIdx.x == 0) counts[t] = count;
 }
 
-__global__ void k_gather(const float* __restrict__ X, const int32_t* __restrict__ labels,
-                         const float* __restrict__ y, const int32_t* __restrict__ idx,
-                         int64_t E, int d, float* Xl, int32_t* lab_l, float* y_l) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= E * d) return;
-  const int64_t e = q / d;
-  const int j = (int)(q - e * d);
-  const int64_t s = idx[e];
-  Xl[q] = X[s * d + j];
-  if (j == 0) {
+// A CTA per kTT entries.
+__global__ void __launch_bounds__(kTT)
+    k_gather(const float* __restrict__ X, const int32_t* __restrict__ labels,
+             const float* __restrict__ y, const int32_t* __restrict__ idx, int64_t E, int d,
+             float* Xl, int32_t* lab_l, float* y_l) {
+  __shared__ int s_src[kTT], s_dst[kTT];
+  const int64_t e0 = (int64_t)blockIdx.x * kTT;
+  const int rows = (int)min((int64_t)kTT, E - e0);
+  if ((int)threadIdx.x < rows) {
+    const int64_t e = e0 + threadIdx.x;
+    const int s = idx[e];
+    s_src[threadIdx.x] = s;
+    s_dst[threadIdx.x] = (int)threadIdx.x;
     if (lab_l) lab_l[e] = labels[s];
     if (y_l) y_l[e] = y[s];
   }
+  __syncthreads();
+  copy_rows(X, s_src, Xl + e0 * d, s_dst, rows, d);
 }
 
 // idx[c * stride + i] = i for i < n, c < copies.
@@ -547,7 +691,7 @@ cudaError_t launch_node_stats(const Problem& pr, const LevelNode* nodes, int L,
   if (n_tiles > 0) k_stats_tiles<<<n_tiles, kTT, 0, st>>>(pr, tiles, acc);
   cudaError_t e = cudaGetLastError();
   if (e) return e;
-  k_stats_finish<<<(L + 127) / 128, 128, 0, st>>>(pr, nodes, tile0, L, acc, tr, max_depth,
+  k_stats_finish<<<(L + kNodeWarps - 1) / kNodeWarps, 32 * kNodeWarps, 0, st>>>(pr, nodes, tile0, L, acc, tr, max_depth,
                                                   par, splittable);
   return cudaGetLastError();
 }
@@ -568,7 +712,7 @@ cudaError_t launch_decide(const Problem& pr, const Swarm& sw, const NodeDesc* sn
                           PartAcc acc, TreeArrays tr, int32_t* out3, int32_t* status,
                           cudaStream_t st) {
   if (A <= 0) return cudaSuccess;
-  k_decide<<<(A + 127) / 128, 128, 0, st>>>(pr, sw, snodes, map, tile0, A, tile_left,
+  k_decide<<<(A + kNodeWarps - 1) / kNodeWarps, 32 * kNodeWarps, 0, st>>>(pr, sw, snodes, map, tile0, A, tile_left,
                                             tile_base, node_cls, par, acc, tr, out3, status);
   return cudaGetLastError();
 }
@@ -595,7 +739,7 @@ cudaError_t launch_gather(const float* X, const int32_t* labels, const float* y,
                           float* y_l, cudaStream_t st) {
   const int64_t total = E * d;
   if (total <= 0) return cudaSuccess;
-  k_gather<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(X, labels, y, idx, E, d, Xl,
+  k_gather<<<(unsigned)((E + kTT - 1) / kTT), kTT, 0, st>>>(X, labels, y, idx, E, d, Xl,
                                                            lab_l, y_l);
   return cudaGetLastError();
 }

@@ -1,0 +1,46 @@
+"""The per-level tree kernels (statistics, sides, decisions, scatter, gather)
+at the widths where their row copies and products change form: rows of whole
+16-byte words and not, up to and beyond the 256 words that a block copies at a time, and the
+32-feature turns of the side's product with and without a remainder; nodes of
+one and several 256-row tiles, more than 64 of them (the per-node kernels'
+fetches). Trees equal the oracle's."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2208_07023_gb300 import workloads as W
+from tests.gpu_util import context, gpu_params, oracle_params
+from tests.test_gpu_parity import _check_tree_up_to_near_ties, _compare_tree
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = context()
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("crit,n,d", [
+    ("gini", 17000, 1), ("gini", 2000, 4), ("gini", 700, 31), ("gini", 700, 36),
+    ("gini", 600, 261), ("gini", 513, 1024),
+    ("mse", 17000, 2), ("mse", 8300, 32), ("mse", 255, 257),
+])
+def test_tree_matches_oracle(ctx, crit, n, d):
+    from paper_2208_07023_gb300 import binding as S
+    K, B = (5, 32) if crit == "gini" else (0, 32)
+    wl = W.gmm(n, d, K, seed=d) if K else W.tanh_regression(n, d, seed=d)
+    lab, y = (wl.labels, None) if K else (None, wl.y)
+    gp = gpu_params(S, crit, K, 16, 3, B, min_leaf=5, max_depth=3, seed=4)
+    op = oracle_params(O, crit, K, 16, 3, B, min_leaf=5, max_depth=3, seed=4)
+    g = ctx.train_tree(gp, wl.X, labels=lab, y=y).export(0)
+    r = O.train_tree(op, wl.X, lab, y)
+    assert (r.kind == 1).any()
+    if K:
+        inner, present = _compare_tree(g, r, d)
+        assert np.array_equal(g["loss"][inner], r.loss[inner])
+        assert np.array_equal(g["leaf_class"][present], r.leaf_class[present])
+    elif _check_tree_up_to_near_ties(g, r, op, wl.X, None, wl.y) == 0:
+        present = r.kind >= 0
+        assert np.allclose(g["leaf_value"][present], r.leaf_value[present], rtol=1e-12, atol=1e-12)
