@@ -531,6 +531,16 @@ int batch_split(slm_ctx* c, const Problem& pr, const std::vector<NodeDesc>& node
   return hist_split(pr, (int)nodes.size(), max_len, c->n_sm, hist_max_cluster(pr));
 }
 
+// A search projected from blocked rows (k_step): with the move folded in,
+// positions alternate between pos[0] and pos[1] by iteration parity.
+struct StepPlan {
+  bool on = false, fold = false;
+  float* pos[2] = {nullptr, nullptr};
+  const StepRun* runs = nullptr;
+  int n_runs = 0;
+  StepConfig cfg;
+};
+
 // The reduced-precision pass of SLM_PROJ_BF16_TOPK: bfloat16 scores of all
 // particles on the tensor cores, then FP32 re-scores of the k best per node.
 struct Bf16Plan {
@@ -540,6 +550,7 @@ struct Bf16Plan {
   int grid = 0;          // k_project_mma grid
   int S_k = 1;           // cluster split of the re-scoring histogram pass
   double pairs_k = 0.0;
+  StepPlan step_k;       // the re-scores projected from blocked rows
   Problem pr_k{};        // the re-scoring problem: P = k
   Swarm sw_k{};          // its view: compact positions, z, ranges, scores
   uint16_t* posb = nullptr;
@@ -719,16 +730,6 @@ slm_status setup_bf16(slm_ctx* c, const Problem& pr, const std::vector<NodeDesc>
   return SLM_OK;
 }
 
-// A search projected from blocked rows (k_step): with the move folded in,
-// positions alternate between pos[0] and pos[1] by iteration parity.
-struct StepPlan {
-  bool on = false, fold = false;
-  float* pos[2] = {nullptr, nullptr};
-  const StepRun* runs = nullptr;
-  int n_runs = 0;
-  StepConfig cfg;
-};
-
 // The CTAs' runs of blocks. With no more (node, slice) pairs than CTAs each
 // pair gets CTAs of its own in proportion to its blocks (a CTA that forms two
 // nodes' positions one after the other takes about 5 us longer than the
@@ -789,6 +790,34 @@ std::vector<StepRun> plan_runs(const std::vector<NodeDesc>& nodes, int slices, i
     }
   }
   return runs;
+}
+
+// Blocked rows of the batch and the runs of a projection from them
+// (plan->on; off when there is no room for a second copy of the rows).
+slm_status plan_step(slm_ctx* c, Problem& pr, const std::vector<NodeDesc>& nodes,
+                     const std::vector<WorkTile>& tiles, const StepConfig& cfg, int grid,
+                     StepPlan* plan) {
+  const cudaError_t e =
+      ensure(c->ws[S_XT], sizeof(float) * (size_t)step_rows_floats(pr, (int)nodes.size()));
+  if (e == cudaErrorMemoryAllocation) {
+    (void)cudaGetLastError();
+    return SLM_OK;
+  }
+  CK(e);
+  const std::vector<StepRun> runs = plan_runs(nodes, cfg.slices, grid);
+  CK(ensure(c->ws[S_RUNS], sizeof(StepRun) * runs.size()));
+  CK(cudaMemcpyAsync(c->ws[S_RUNS].p, runs.data(), sizeof(StepRun) * runs.size(),
+                     cudaMemcpyHostToDevice, c->stream));
+  pr.Xt = ws_ptr<float>(c, S_XT);
+  CK(launch(c, SLM_K_GATHER, 0.0, [&] {
+    return launch_block_rows(pr, ws_ptr<WorkTile>(c, S_TILES), (int)tiles.size(),
+                             ws_ptr<float>(c, S_XT), c->stream);
+  }));
+  plan->on = true;
+  plan->runs = ws_ptr<StepRun>(c, S_RUNS);
+  plan->n_runs = (int)runs.size();
+  plan->cfg = cfg;
+  return SLM_OK;
 }
 
 // The latency-oriented histogram kernels of a search on A nodes (of list[],
@@ -894,7 +923,12 @@ slm_status score_batch(slm_ctx* c, const Problem& pr, const Swarm& sw_in,
     if (b.k > 0) {
       // FP32 re-scores of the k best of each node (selected by the last
       // histogram CTA of the node) replace theirs
-      if (n_tiles)
+      if (b.step_k.on)
+        CK(launch(c, SLM_K_PROJECT, b.pairs_k, [&] {
+          return launch_project_few(b.step_k.cfg, b.pr_k, b.sw_k, dn, b.step_k.runs,
+                                    b.step_k.n_runs, c->stream);
+        }));
+      else if (n_tiles)
         CK(launch(c, SLM_K_PROJECT, b.pairs_k, [&] {
           return launch_project(b.pr_k, b.sw_k, dt, n_tiles, cap, c->stream, 0, false,
                                 c->tma ? A : 0);
@@ -1445,17 +1479,25 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
   // FP32 searches of whole batches: projected from blocked rows, the move of
   // a plain search folded in where the batch is short
   StepPlan stp;
-  if (n_res == 0 && c->fused_step && !c->forced.pg && !bp.on) {
-    // (nodes in the order of their segments: the blocks' places are disjoint)
-    bool every = true;
-    for (int a = 0; a < A; ++a)
-      every = every && nodes[a].seg_len > 0 &&
-              (a == 0 || nodes[a].seg_start >= nodes[a - 1].seg_start + nodes[a - 1].seg_len);
+  // (nodes in the order of their segments: the blocks' places are disjoint)
+  bool every = n_res == 0 && c->fused_step && !c->forced.pg;
+  for (int a = 0; a < A; ++a)
+    every = every && nodes[a].seg_len > 0 &&
+            (a == 0 || nodes[a].seg_start >= nodes[a - 1].seg_start + nodes[a - 1].seg_len);
+  if (every && bp.on && bp.k > 0) {  // the BF16 form's FP32 re-scores
+    StepConfig cfg;
+    if (few_config(bp.pr_k, &cfg)) {
+      CK(prepare_step(cfg));
+      const int grid = step_grid(cfg, c->n_sm);
+      if (grid > 0 && (s = plan_step(c, bp.pr_k, nodes, tiles, cfg, grid, &bp.step_k))) return s;
+    }
+  }
+  if (every && !bp.on) {
     int64_t blocks = 0;
     for (int a = 0; a < A; ++a) blocks += (nodes[a].seg_len + 31) / 32;
     StepConfig cfg;
     int sh = -1, grid = 0;
-    if (every && !p->apso && step_ok(pr)) {
+    if (!p->apso && step_ok(pr)) {
       // Folding pays where the chain is latency-bound: up to kFoldMaxBlocks
       // blocks per CTA (100,000 x 32 rows, P = 48: 25 us an iteration folded,
       // 27 not; 200,000 x 128 rows, P = 64, third to sixth level: 125 to 142
@@ -1502,35 +1544,12 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
         }
       }
     }
-    if (every && grid == 0 && step_config(pr, -1, &cfg, blocks / A)) {
+    if (grid == 0 && step_config(pr, -1, &cfg, blocks / A)) {
       CK(prepare_step(cfg));
       grid = step_grid(cfg, c->n_sm);
     }
-    if (grid > 0) {
-      const cudaError_t e = ensure(c->ws[S_XT], sizeof(float) * (size_t)step_rows_floats(pr, A));
-      if (e == cudaErrorMemoryAllocation) {
-        (void)cudaGetLastError();  // no room for a second copy of the rows
-        grid = 0;
-      } else {
-        CK(e);
-      }
-    }
-    if (grid > 0) {
-      const std::vector<StepRun> runs = plan_runs(nodes, cfg.slices, grid);
-      CK(ensure(c->ws[S_RUNS], sizeof(StepRun) * runs.size()));
-      CK(cudaMemcpyAsync(c->ws[S_RUNS].p, runs.data(), sizeof(StepRun) * runs.size(),
-                         cudaMemcpyHostToDevice, c->stream));
-      pr.Xt = ws_ptr<float>(c, S_XT);
-      CK(launch(c, SLM_K_GATHER, 0.0, [&] {
-        return launch_block_rows(pr, ws_ptr<WorkTile>(c, S_TILES), (int)tiles.size(),
-                                 ws_ptr<float>(c, S_XT), c->stream);
-      }));
-      stp.on = true;
-      stp.runs = ws_ptr<StepRun>(c, S_RUNS);
-      stp.n_runs = (int)runs.size();
-      stp.cfg = cfg;
-      stp.fold = sh >= 0;
-    }
+    if (grid > 0 && (s = plan_step(c, pr, nodes, tiles, cfg, grid, &stp))) return s;
+    stp.fold = stp.on && sh >= 0;
     if (stp.fold) {
       const size_t apd = (size_t)A * pr.Pp * pr.d;
       CK(ensure(c->ws[S_POS2], sizeof(float) * apd));
@@ -1597,7 +1616,8 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
       kw.put(pairs);
       kw.put(dn); kw.put(ws_ptr<WorkTile>(c, S_TILES)); kw.put(ws_ptr<WorkTile>(c, S_MTILES));
       kw.put(bp.on); kw.put(bp.k); kw.put(bp.kp); kw.put(bp.n_mtiles); kw.put(bp.grid);
-      kw.put(bp.S_k); kw.put(bp.pairs_k); kw.put(bp.posb); kw.put(bp.sel); kw.put(bp.inv);
+      kw.put(bp.S_k); kw.put(bp.pairs_k); kw.put(bp.step_k.on); kw.put(bp.step_k.runs);
+      kw.put(bp.step_k.n_runs); kw.put(bp.step_k.cfg.slices); kw.put(bp.posb); kw.put(bp.sel); kw.put(bp.inv);
       kw.put(bp.fast); kw.put(bp.S_fast); kw.put(bp.S_fast_k); kw.put(bp.xtab);
       kw.put(bp.S_large); kw.put(bp.S_large_k); kw.put(bp.max_len); kw.put(cp.max_len);
       kw.put(hp.max_large);

@@ -342,6 +342,11 @@ bool step_ok(const Problem& pr);
 // Shape sh (0 .. 5) of the folded projection, or (sh = -1) the unfolded one
 // for nodes of about `blocks` blocks of 32 rows.
 bool step_config(const Problem& pr, int sh, StepConfig* c, int64_t blocks = 1 << 20);
+// Few particles (unfolded, slices of 8): k_project_few.
+bool few_config(const Problem& pr, StepConfig* c);
+cudaError_t launch_project_few(const StepConfig& c, const Problem& pr, const Swarm& sw,
+                               const NodeDesc* nodes, const StepRun* runs, int n_runs,
+                               cudaStream_t st);
 cudaError_t prepare_step(const StepConfig& c);
 int step_grid(const StepConfig& c, int n_sm);
 // Blocked rows of A nodes: the array's floats; filled from pr.X (tiles: the

@@ -94,7 +94,8 @@ __device__ __forceinline__ int pos_slot(int r, int k) {
 }
 
 // The blocked rows; one CTA per 256-row tile (which starts a multiple of 256
-// rows into its node), a warp per block.
+// rows into its node), a warp per block. Bound by DRAM (204 MB at 200,000 x
+// 128 rows: 41 us).
 __global__ void __launch_bounds__(256)
     k_block_rows(const float* __restrict__ X, int d, const WorkTile* __restrict__ tiles,
                  float* __restrict__ Xt) {
@@ -107,12 +108,12 @@ __global__ void __launch_bounds__(256)
   float* out = Xt + ((int64_t)wt.row0 + r0 + 32 * (int64_t)wt.node) * d;
   for (int k0 = 0; k0 < d; k0 += 32) {
     const int kc = min(32, d - k0);
-#pragma unroll 8
-    for (int r = 0; r < 32; ++r) {
-      float v = 0.0f;
-      if (r < nr && lane < kc) v = __ldg(X + ((int64_t)wt.row0 + r0 + r) * d + k0 + lane);
-      s[warp][r][lane] = v;
-    }
+    float v[32];  // 32 loads on their way (8: 125 us at 200,000 x 128 rows)
+    const float* x = X + ((int64_t)wt.row0 + r0) * d + k0 + lane;
+#pragma unroll
+    for (int r = 0; r < 32; ++r) v[r] = r < nr && lane < kc ? __ldg(x + (int64_t)r * d) : 0.0f;
+#pragma unroll
+    for (int r = 0; r < 32; ++r) s[warp][r][lane] = v[r];
     __syncwarp();
 #pragma unroll 8
     for (int k = 0; k < 32; ++k)
@@ -648,6 +649,145 @@ __global__ void __launch_bounds__(32 * (FOLD ? kFoldWarps : kProjWarps))
   }
 }
 
+// The projection of few particles (slices of 8): a thread takes two rows and
+// all 8, so every x is read once, straight from the blocked rows (8 bytes per
+// lane, eight features on their way while eight are multiplied), and a slice's
+// positions at one feature are two broadcast words. A warp takes two blocks
+// at a time. Bound by waiting for the rows: the FP32 re-scores of the BF16
+// form, 200,000 x 128 rows and 8 particles, take 33 us (102 MB; four blocks a
+// warp 36), by the row-major kernel (row tiles through shared memory) 39.
+constexpr int kFewWarps = 8, kFewP = 8, kFewF = 8;
+constexpr int kFewBlocks = 2;  // blocks of a warp
+
+__global__ void __launch_bounds__(32 * kFewWarps, 3)
+    k_project_few(Problem pr, Swarm sw, const NodeDesc* __restrict__ nodes,
+                  const StepRun* __restrict__ runs, int n_slices) {
+  constexpr int NT = 32 * kFewWarps;
+  extern __shared__ __align__(16) float sm[];  // [d][8] positions
+  __shared__ int s_lo[kFewP], s_hi[kFewP];
+  const int d = pr.d, P = pr.P;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int blk = lane >> 4, rl = 2 * (lane & 15);  // this lane's block of the two, its rows
+  pdl_trigger();
+  const StepRun run = runs[blockIdx.x];
+  const bool z16 = ((reinterpret_cast<uintptr_t>(sw.z) | (uintptr_t)pr.Ez * 4) & 15) == 0;
+  const int nc = (d + kFewF - 1) / kFewF;  // chunks of features
+  if (threadIdx.x < kFewP) {
+    s_lo[threadIdx.x] = INT_MAX;
+    s_hi[threadIdx.x] = INT_MIN;
+  }
+  pdl_wait();
+  int a = run.node, slice = run.slice, left = run.count, first = run.blk;
+  while (left > 0) {
+    const NodeDesc nd = nodes[a];
+    const int nb = (nd.seg_len + kBR - 1) / kBR;
+    const int take = min(left, nb - first);
+    const int pg0 = slice * kFewP, np = min(P - pg0, kFewP);
+    const float* src = sw.pos + ((int64_t)a * pr.Pp + pg0) * d;
+    for (int i = threadIdx.x; i < kFewP * d; i += NT) {
+      const int q = i / d, k = i - q * d;
+      sm[k * kFewP + q] = q < np ? __ldcg(src + i) : 0.0f;
+    }
+    __syncthreads();
+    float lo[kFewP], hi[kFewP];
+#pragma unroll
+    for (int q = 0; q < kFewP; ++q) {
+      lo[q] = FLT_MAX;
+      hi[q] = -FLT_MAX;
+    }
+    for (int u = kFewBlocks * warp; u < take; u += kFewBlocks * kFewWarps) {
+      const int b = first + u + blk;  // this lane's block
+      const bool in = u + blk < take;
+      const float* x = pr.Xt +
+                       ((int64_t)nd.seg_start + 32 * (int64_t)a + (int64_t)b * kBR) * d + rl;
+      float2 v[2][kFewF];
+      auto load = [&](float2 (&w)[kFewF], int c) {
+#pragma unroll
+        for (int i = 0; i < kFewF; ++i) {
+          const int k = c * kFewF + i;
+          w[i] = in && k < d ? __ldcg(reinterpret_cast<const float2*>(x + (int64_t)k * kBR))
+                             : make_float2(0.f, 0.f);
+        }
+      };
+      // rows in pairs, straight and crossed with the particles' pairs (see
+      // k_step): acc[2 j] = (r0 p0, r1 p1), acc[2 j + 1] = (r1 p0, r0 p1)
+      uint64_t acc[kFewP];
+#pragma unroll
+      for (int q = 0; q < kFewP; ++q) acc[q] = 0ull;
+      auto multiply = [&](const float2 (&w)[kFewF], int c) {
+        const float* ps = sm + c * kFewF * kFewP;
+        const int kc = d - c * kFewF;  // (a product past d could turn -0 into 0)
+#pragma unroll
+        for (int i = 0; i < kFewF; ++i) {
+          if (i >= kc) break;
+          const ulonglong2 a0 = *reinterpret_cast<const ulonglong2*>(ps + i * kFewP);
+          const ulonglong2 a1 = *reinterpret_cast<const ulonglong2*>(ps + i * kFewP + 4);
+          const uint64_t av[4] = {a0.x, a0.y, a1.x, a1.y};
+          const uint64_t x = pack2(w[i].x, w[i].y), y = pack2(w[i].y, w[i].x);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            fma2(acc[2 * j], x, av[j]);
+            fma2(acc[2 * j + 1], y, av[j]);
+          }
+        }
+      };
+      load(v[0], 0);
+      for (int c = 0; c < nc; c += 2) {
+        load(v[1], c + 1);
+        multiply(v[0], c);
+        if (c + 1 >= nc) break;
+        load(v[0], c + 2);
+        multiply(v[1], c + 1);
+      }
+      const int nr = in ? min(kBR, nd.seg_len - b * kBR) : 0;
+      const int64_t zrow = (int64_t)nd.seg_start + (int64_t)b * kBR + rl;
+      const bool v8 = z16 && nr == kBR && (zrow & 1) == 0;
+#pragma unroll
+      for (int q = 0; q < kFewP; ++q) {
+        const float2 s0 = unpack2(acc[q & ~1]), s1 = unpack2(acc[q | 1]);
+        const float r0 = (q & 1) ? s1.y : s0.x, r1 = (q & 1) ? s0.y : s1.x;
+        float* zp = sw.z + (int64_t)(pg0 + q) * pr.Ez + zrow;
+        if (rl < nr) {
+          lo[q] = fminf(lo[q], r0);
+          hi[q] = fmaxf(hi[q], r0);
+          if (!v8 && q < np) zp[0] = r0;
+        }
+        if (rl + 1 < nr) {
+          lo[q] = fminf(lo[q], r1);
+          hi[q] = fmaxf(hi[q], r1);
+          if (!v8 && q < np) zp[1] = r1;
+        }
+        if (v8 && q < np) *reinterpret_cast<float2*>(zp) = make_float2(r0, r1);
+      }
+    }
+    if (kFewBlocks * warp < take) {  // (the warp had blocks)
+#pragma unroll
+      for (int q = 0; q < kFewP; ++q) {
+        const int l = __reduce_min_sync(0xffffffffu, f2ord(lo[q]));
+        const int h = __reduce_max_sync(0xffffffffu, f2ord(hi[q]));
+        if (lane == q) {
+          atomicMin(&s_lo[q], l);
+          atomicMax(&s_hi[q], h);
+        }
+      }
+    }
+    __syncthreads();  // every warp's ranges are in; the positions are read
+    if ((int)threadIdx.x < np && s_lo[threadIdx.x] != INT_MAX) {
+      int* zz = sw.zmm + ((int64_t)a * pr.Pp + pg0 + threadIdx.x) * 2;
+      atomicMin(zz, s_lo[threadIdx.x]);
+      atomicMax(zz + 1, s_hi[threadIdx.x]);
+      s_lo[threadIdx.x] = INT_MAX;
+      s_hi[threadIdx.x] = INT_MIN;
+    }
+    left -= take;
+    first = 0;
+    if (++slice == n_slices) {
+      slice = 0;
+      ++a;
+    }
+  }
+}
+
 // Tile shapes of a folded search's padded swarm: particles per thread and
 // particle warps. Shapes 0-2 take every particle in a unit, on 384, 192 or 96
 // rows of the CTA; shapes 3-5 take half of them (two slices of a swarm of 32
@@ -754,6 +894,37 @@ bool step_config(const Problem& pr, int sh, StepConfig* c, int64_t blocks) {
   c->row_warps = warps / PB;
   c->smem = step_smem(pr.d, 8 * QP * PB, warps);
   return c->fn != nullptr;
+}
+
+bool few_config(const Problem& pr, StepConfig* c) {
+  c->fn = nullptr;
+  c->qp = 1;
+  c->pb = 1;
+  c->slices = (pr.P + kFewP - 1) / kFewP;
+  c->threads = 32 * kFewWarps;
+  c->row_warps = kFewWarps;
+  c->smem = sizeof(float) * (size_t)pr.d * kFewP;
+  if (c->smem > (size_t)kStepMaxPosBytes) return false;
+  c->fn = (const void*)k_project_few;
+  return true;
+}
+
+cudaError_t launch_project_few(const StepConfig& c, const Problem& pr, const Swarm& sw,
+                               const NodeDesc* nodes, const StepRun* runs, int n_runs,
+                               cudaStream_t st) {
+  if (n_runs <= 0) return cudaSuccess;
+  if (!pr.Xt) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)n_runs, 1, 1);
+  cfg.blockDim = dim3((unsigned)c.threads, 1, 1);
+  cfg.dynamicSmemBytes = c.smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_project_few, pr, sw, nodes, runs, c.slices);
 }
 
 cudaError_t prepare_step(const StepConfig& c) { return allow_smem(c.fn, (int)c.smem); }

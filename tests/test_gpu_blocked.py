@@ -60,3 +60,35 @@ def test_many_small_nodes_identical(ctxs, P, d):
     for k in ga:
         assert np.array_equal(ga[k], gb[k]), k
     assert (ga["kind"] == 1).sum() > 500
+
+
+@pytest.mark.parametrize("n,d,P,k", [
+    (5000, 32, 64, 8),
+    (3001, 17, 48, 8),    # odd feature count, a ragged last block
+    (4099, 9, 40, 3),     # fewer than 8 re-scored
+    (2500, 65, 64, 16),   # two slices
+    (700, 8, 32, 20),     # three, the last of four
+    (30, 5, 24, 8),       # less than one block
+    (1500, 600, 32, 8),
+])
+@pytest.mark.parametrize("crit", ["gini", "mse"])
+def test_bf16_rescores_identical(ctxs, crit, n, d, P, k):
+    """The FP32 re-scores of the BF16 form from blocked rows (a thread takes
+    two rows and eight particles): the row-major kernel's."""
+    from paper_2208_07023_gb300 import binding as S
+    a, b = ctxs
+    if crit == "gini":
+        wl = W.gmm(n, d, 4, seed=d)
+        kw = dict(labels=wl.labels)
+    else:
+        wl = W.tanh_regression(n, d, seed=d)
+        kw = dict(y=wl.y)
+    p = S.make_params(crit, 4 if crit == "gini" else 0, n_particles=P, n_iters=4, n_bins=64,
+                      min_leaf=2, seed=3, max_depth=4, proj=S.SLM_PROJ_BF16_TOPK, topk=k)
+    ra, rb = (c.node_split(p, wl.X, node_uid=9, want_trace=True, **kw) for c in (a, b))
+    assert np.array_equal(ra["trace"], rb["trace"])
+    assert np.array_equal(ra["gbest"].view(np.uint32), rb["gbest"].view(np.uint32))
+    assert ra["particle"] == rb["particle"] and ra["bin"] == rb["bin"]
+    ga, gb = (c.train_tree(p, wl.X, **kw).export(0) for c in (a, b))
+    for key in ga:
+        assert np.array_equal(ga[key], gb[key]), key
