@@ -684,22 +684,43 @@ __device__ float apso_mu(int state, float f) {
 // 4. the move of Eq. pso-1 with these factors.
 //
 // Layout: positions feature-major in shared memory (row k holds feature k of
-// the Pq = P rounded up to 4 particles, 16-byte aligned), so a thread's 4 x 4
-// tile of (i, j) pairs reads two float4 per feature and the lanes of a warp
-// (consecutive j blocks) read consecutive 16-byte words. The rows i are taken
+// the Pq = P rounded up to 4 particles, 16-byte aligned), so a thread's 2 x 2
+// tile of (i, j) pairs reads two float2 per feature and the lanes of a warp
+// (consecutive j blocks) read consecutive words (4 x 4 tiles left most of the
+// threads idle and each with 16 square roots: 12,000 clocks). The rows i are taken
 // in chunks of apso_rows(P, d) whose square roots go to a buffer of stride
-// Pq + 1, from which thread r adds row r without bank conflicts.
+// Pq + 1, from which thread r adds row r without bank conflicts. When one
+// chunk holds every row the tiles below the diagonal are the others' mirror
+// (x_j - x_i is x_i - x_j negated, its square the same).
+//
+// One CTA runs a chain of short phases, so latency is what bounds it: what
+// depends on no result of the evaluation (the Philox draws of the first
+// kApsoItems move items of a thread, elitist learning's step) is done before
+// the wait for the previous kernel, and the positions, gB, the elite slot
+// (asynchronous copies into shared memory, where they fit beside the rest)
+// and those items' velocities and personal bests are on their way while warp
+// 0 takes the gbest step (by the loss keys). 40 particles of 33 features, us a
+// launch: 22.4 with every phase loading for itself, 20.4 with the early loads,
+// 18.0 with the keys and 2 x 2 tiles, 16.3 with every row in one chunk.
 __host__ __device__ inline int apso_pq(int P) { return (P + 3) & ~3; }
+constexpr int kApsoItems = 3;
 
 __host__ __device__ inline size_t apso_smem(int P, int d, int R) {
   const int Pq = apso_pq(P);
   return sizeof(float) * ((size_t)d * Pq + (size_t)R * (Pq + 1));
 }
+// with rows of stride Pq + 4 (4 lanes a bank instead of 32 in the transposing
+// copies) and the elite's and gB's vectors
+__host__ __device__ inline size_t apso_smem_wide(int P, int d, int R) {
+  return apso_smem(P, d, R) + sizeof(float) * 6 * (size_t)d;
+}
+constexpr size_t kApsoMaxSmem = 227 * 1024 - 2048;  // less the static part
 
-// Rows per chunk: the largest of 64, 32, 16, 8, 4 (not above Pq) whose
-// buffers fit in 227 KB; 0 if none does.
+// Rows per chunk: all Pq, else the largest of 64, 32, 16, 8, 4 (not above Pq)
+// whose buffers fit in 227 KB; 0 if none does.
 inline int apso_rows(int P, int d) {
   const int Pq = apso_pq(P);
+  if (apso_smem_wide(P, d, Pq) <= kApsoMaxSmem) return Pq;
   for (int R = 64; R >= 4; R >>= 1)
     if (R <= Pq && apso_smem(P, d, R) <= 227 * 1024) return R;
   return apso_smem(P, d, 4) <= 227 * 1024 ? 4 : 0;
@@ -707,39 +728,170 @@ inline int apso_rows(int P, int d) {
 
 __global__ void __launch_bounds__(256)
     k_apso(Problem pr, Swarm sw, const NodeDesc* __restrict__ nodes, int t, SwarmCoef co,
-           const int32_t* __restrict__ list, int A, int R) {
+           const int32_t* __restrict__ list, int A, int R, int wide) {
   extern __shared__ __align__(16) float asm_[];
   __shared__ float s_di[kMaxParticles];
   __shared__ int s_gp;
-  pdl_trigger();
-  pdl_wait();
   __shared__ int s_mode, s_w, s_wpb, s_k;
   __shared__ float s_g, s_c[3];
+  pdl_trigger();
   const int a = list ? list[blockIdx.x] : (int)blockIdx.x;
   const int P = pr.P, d = pr.d, Pp = pr.Pp, Pq = apso_pq(P);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t cb = (int64_t)a * Pp;
   float* pos = sw.pos + cb * d;
+  float* vel = sw.vel + cb * d;
   float* pbp = sw.pbest + cb * d;
   float* gbp = sw.gbest + (int64_t)a * d;
   float* erow = pos + (int64_t)P * d;  // the elite candidate's slot
+  const uint32_t uid = nodes[a].uid;
+  const uint32_t k0 = (uint32_t)co.seed, k1 = (uint32_t)(co.seed >> 32);
+  const int d4 = (d + 3) >> 2, n_items = P * d4;
+  const int ldx = wide ? Pq + 4 : Pq;
+  float* xt = asm_;                     // [d][ldx] current positions, feature-major
+  float* rw = asm_ + (size_t)d * ldx;   // [R][Pq + 1] square roots of a chunk of rows
+  float* e_sm = rw + (size_t)R * (Pq + 1);  // wide: [d] the elite candidate, [d] gB
+  float* g_sm = e_sm + d;
+  // the draws of particle pi's features 4q .. 4q + 3
+  auto draw = [&](int item, float (&u1)[4], float (&u2)[4]) {
+    const int pi = item / d4, q = item - pi * d4;
+    const U4 r1 = philox4x32_10(uid, (uint32_t)(t + 1), (uint32_t)pi,
+                                (uint32_t)q | (kR1 << 24), k0, k1);
+    const U4 r2 = philox4x32_10(uid, (uint32_t)(t + 1), (uint32_t)pi,
+                                (uint32_t)q | (kR2 << 24), k0, k1);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      u1[c] = uniform24(r1.v[c]);
+      u2[c] = uniform24(r2.v[c]);
+    }
+  };
+  float delta = 0.0f;  // thread 0
+  float u1[kApsoItems][4], u2[kApsoItems][4], pv[kApsoItems][4], pp[kApsoItems][4];
+  if (t < sw.T) {
+#pragma unroll
+    for (int m = 0; m < kApsoItems; ++m) {
+      const int item = threadIdx.x + m * 256;
+      if (item < n_items) draw(item, u1[m], u2[m]);
+    }
+    if (threadIdx.x == 0) {
+      const U4 r = philox4x32_10(uid, (uint32_t)t, 0u, kApso << 24, k0, k1);
+      delta = __fadd_rn(0.05f, __fmul_rn(0.05f, uniform24(r.v[0])));
+    }
+    if (threadIdx.x == 32) {
+      // elitist learning's step: coordinate k = floor(u1 d), g = sqrt(-2
+      // ln(1 - u2)) cos(2 pi u3) (Box-Muller, in double, rounded to float)
+      const U4 r = philox4x32_10(uid, (uint32_t)t, 0u, kApso << 24, k0, k1);
+      s_k = (int)__dmul_rn((double)uniform24(r.v[1]), (double)d);
+      s_g =
+          (float)__dmul_rn(sqrt(__dmul_rn(-2.0, log((double)__fsub_rn(1.0f, uniform24(r.v[2]))))),
+                           cos(__dmul_rn(6.283185307179586, (double)uniform24(r.v[3]))));
+    }
+    // columns of the particles past P
+    for (int e = threadIdx.x; e < (Pq - P) * d; e += blockDim.x) {
+      const int k = e / (Pq - P);
+      xt[(size_t)k * ldx + P + (e - k * (Pq - P))] = 0.0f;
+    }
+  }
+  pdl_wait();
+  if (t < sw.T) {
+    {
+      // row-major reads, feature-major writes; element e = i d + k
+      const int step_i = 256 / d, step_k = 256 - step_i * d;
+      int i = (int)threadIdx.x / d, k = (int)threadIdx.x - i * d;
+      for (int e = threadIdx.x; e < P * d; e += 256) {
+        cp_async4(xt + (size_t)k * ldx + i, pos + e, 4);
+        i += step_i;
+        k += step_k;
+        if (k >= d) {
+          k -= d;
+          ++i;
+        }
+      }
+      if (wide)
+        for (int j = threadIdx.x; j < d; j += 256) {
+          cp_async4(e_sm + j, erow + j, 4);
+          cp_async4(g_sm + j, gbp + j, 4);
+        }
+      cp_async_commit();
+    }
+#pragma unroll
+    for (int m = 0; m < kApsoItems; ++m) {
+      const int item = threadIdx.x + m * 256;
+      const int pi = item / d4, j0 = 4 * (item - pi * d4);
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (item < n_items && j0 + c < d) {
+          pv[m][c] = __ldcg(vel + (int64_t)pi * d + j0 + c);
+          pp[m][c] = __ldcg(pbp + (int64_t)pi * d + j0 + c);
+        }
+    }
+  }
   // 1. gbest step of evaluation t (the rule of k_move), then the elite
   // candidate scored in this evaluation: gB and the gB particle's personal
   // best if strictly better, else the worst particle's position (and its
   // personal best if better than it)
+  ApsoState st{};
   if (warp == 0) {
+    // the particles' loss keys decide the best and the worst unless several
+    // lie within 8 ulps of them (or of gB): then the exact comparisons do
+    constexpr int kPer = kMaxParticles / 32;
+    const EvalRes* cur = sw.cur + cb;
+    uint64_t key[kPer];
     const EvalRes gold = sw.gb[(int64_t)((t + 1) & 1) * A + a];
-    EvalRes be;
-    const int bi = gbest_argmin(pr, sw.cur + cb, gold, t, &be);
-    const int pending = sw.apso[a].pending;
-    const int wi = pending ? worst_argmax(pr, sw.cur + cb) : -1;
+    const EvalRes ee = cur[P];
+    const int gp0 = sw.gpart[a], gi0 = sw.giter[a];
+    st = sw.apso[a];
+    uint64_t kmin = ~0ull, kmax = 0ull;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      const int p = lane + 32 * i;
+      key[i] = ~0ull;
+      if (p < P) {
+        key[i] = cur[p].valid ? loss_key(cur[p].loss) : ~0ull;
+        kmin = min(kmin, key[i]);
+        kmax = max(kmax, key[i]);
+      }
+    }
+    {
+      const uint32_t h = __reduce_min_sync(0xffffffffu, (uint32_t)(kmin >> 32));
+      const uint32_t l = __reduce_min_sync(
+          0xffffffffu, (uint32_t)(kmin >> 32) == h ? (uint32_t)kmin : 0xffffffffu);
+      kmin = ((uint64_t)h << 32) | l;
+      const uint32_t hx = __reduce_max_sync(0xffffffffu, (uint32_t)(kmax >> 32));
+      const uint32_t lx = __reduce_max_sync(
+          0xffffffffu, (uint32_t)(kmax >> 32) == hx ? (uint32_t)kmax : 0u);
+      kmax = ((uint64_t)hx << 32) | lx;
+    }
+    const uint64_t near = kmin > ~0ull - 8 ? ~0ull : kmin + 8, far = kmax < 8 ? 0ull : kmax - 8;
+    int nb = 0, nw = 0, pb0 = -1, pw0 = -1;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      if (32 * i >= P) break;
+      const bool in = lane + 32 * i < P;
+      const unsigned mb = __ballot_sync(0xffffffffu, in && key[i] <= near);
+      const unsigned mw = __ballot_sync(0xffffffffu, in && key[i] >= far);
+      if (mb && nb == 0) pb0 = 32 * i + __ffs(mb) - 1;
+      if (mw && nw == 0) pw0 = 32 * i + __ffs(mw) - 1;
+      nb += __popc(mb);
+      nw += __popc(mw);
+    }
+    EvalRes be = gold;
+    int bi = -1;
+    const uint64_t kg = loss_key(gold);
+    if (t > 0 && nb == 1 && near < kg) {
+      bi = pb0;
+      be = cur[bi];
+    } else if (t == 0 || !gold.valid || kmin <= (kg > ~0ull - 8 ? ~0ull : kg + 8)) {
+      bi = gbest_argmin(pr, cur, gold, t, &be);
+    }
+    const int pending = st.pending;
+    const int wi = !pending ? -1 : nw == 1 ? pw0 : worst_argmax(pr, cur);
     if (lane == 0) {
       EvalRes gnew = bi >= 0 ? be : gold;
-      const int gp = bi >= 0 ? bi : sw.gpart[a];
-      int git = bi >= 0 ? t : sw.giter[a];
+      const int gp = bi >= 0 ? bi : gp0;
+      int git = bi >= 0 ? t : gi0;
       int mode = bi >= 0 ? 1 : 0, wr = -1, wpb = 0;
       if (pending) {
-        const EvalRes ee = sw.cur[cb + P];
         if (better(ee, gnew, pr.crit)) {
           gnew = ee;
           git = t;
@@ -767,84 +919,111 @@ __global__ void __launch_bounds__(256)
       s_wpb = wpb;
     }
   }
+  cp_async_wait<0>();
   __syncthreads();
+  const int gp = s_gp, mode = s_mode, w = s_w, wpb = s_wpb;
+  const bool sm = wide && t < sw.T;
+  const float* er = sm ? e_sm : erow;
   for (int j = threadIdx.x; j < d; j += blockDim.x) {
-    if (s_mode == 1) {
-      gbp[j] = pbp[(int64_t)s_gp * d + j];
-    } else if (s_mode == 2) {
-      gbp[j] = erow[j];
-      pbp[(int64_t)s_gp * d + j] = erow[j];
+    if (mode != 0) {
+      // (a new best improved its personal best in this evaluation: that row
+      // is its position)
+      const float g =
+          mode == 2 ? er[j] : sm ? xt[(size_t)j * ldx + gp] : pbp[(int64_t)gp * d + j];
+      gbp[j] = g;
+      if (sm) g_sm[j] = g;
+      if (mode == 2) pbp[(int64_t)gp * d + j] = g;
     }
-    if (s_w >= 0) {
-      pos[(int64_t)s_w * d + j] = erow[j];
-      if (s_wpb) pbp[(int64_t)s_w * d + j] = erow[j];
+    if (w >= 0) {
+      const float e = er[j];
+      pos[(int64_t)w * d + j] = e;
+      if (t < sw.T) xt[(size_t)j * ldx + w] = e;
+      if (wpb) pbp[(int64_t)w * d + j] = e;
     }
   }
   if (t >= sw.T) return;
   __syncthreads();
+  const float* gv = sm ? g_sm : gbp;
   // 2. the evolutionary state of the current positions
-  float* xt = asm_;             // [d][Pq] current positions, feature-major
-  float* rw = asm_ + d * Pq;    // [R][Pq + 1] square roots of a chunk of rows
-  // consecutive threads take consecutive particles of one feature: the
-  // shared-memory writes go to consecutive banks (the global reads are
-  // strided but hit L2: the positions were written by the last move)
-  for (int e = threadIdx.x; e < Pq * d; e += blockDim.x) {
-    const int k = e / Pq, i = e - k * Pq;
-    xt[e] = i < P ? pos[(int64_t)i * d + k] : 0.0f;
-  }
-  __syncthreads();
-  const int nJ = Pq >> 2, ld = Pq + 1;
+  const int nJ = Pq >> 1, ld = Pq + 1;
+  const bool once = R >= P;  // one chunk: tiles on and above the diagonal
   for (int c0 = 0; c0 < P; c0 += R) {
-    const int rows = min(R, P - c0), nI = (rows + 3) >> 2;
-    for (int u = threadIdx.x; u < nI * nJ; u += blockDim.x) {
-      const int ib = u / nJ, jb = u - ib * nJ;
-      const int i0 = c0 + 4 * ib, j0 = 4 * jb;
-      float s2[4][4];
-#pragma unroll
-      for (int p = 0; p < 4; ++p)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) s2[p][q] = 0.0f;
-#pragma unroll 2
-      for (int k = 0; k < d; ++k) {
-        const float4 xi = *reinterpret_cast<const float4*>(xt + k * Pq + i0);
-        const float4 xj = *reinterpret_cast<const float4*>(xt + k * Pq + j0);
-        const float vi[4] = {xi.x, xi.y, xi.z, xi.w}, vj[4] = {xj.x, xj.y, xj.z, xj.w};
-#pragma unroll
-        for (int p = 0; p < 4; ++p)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const float diff = __fsub_rn(vi[p], vj[q]);
-            s2[p][q] = fmaf(diff, diff, s2[p][q]);
-          }
+    const int rows = min(R, P - c0), nI = (rows + 1) >> 1;
+    const int n_tiles = once ? nJ * (nJ + 1) / 2 : nI * nJ;
+    for (int u = threadIdx.x; u < n_tiles; u += blockDim.x) {
+      int ib = u / nJ, jb = u - ib * nJ;
+      // on and above the diagonal: rows nJ - 1 - r and r + 1 (of nJ - r and
+      // r columns less) make up one row of nJ + 1, folded
+      if (once) {
+        ib = u / (nJ + 1);
+        jb = u - ib * (nJ + 1);
+        if (jb < nJ - ib) {
+          jb += ib;
+        } else {
+          jb -= nJ - ib;
+          ib = nJ - 1 - ib;
+          jb += ib;
+        }
       }
+      const int i0 = c0 + 2 * ib, j0 = 2 * jb;
+      float s00 = 0.0f, s01 = 0.0f, s10 = 0.0f, s11 = 0.0f;
+      const float *xi = xt + i0, *xj = xt + j0;
+#pragma unroll 8
+      for (int k = 0; k < d; ++k) {
+        const float2 vi = *reinterpret_cast<const float2*>(xi);
+        const float2 vj = *reinterpret_cast<const float2*>(xj);
+        xi += ldx;
+        xj += ldx;
+        const float d00 = __fsub_rn(vi.x, vj.x), d01 = __fsub_rn(vi.x, vj.y);
+        const float d10 = __fsub_rn(vi.y, vj.x), d11 = __fsub_rn(vi.y, vj.y);
+        s00 = fmaf(d00, d00, s00);
+        s01 = fmaf(d01, d01, s01);
+        s10 = fmaf(d10, d10, s10);
+        s11 = fmaf(d11, d11, s11);
+      }
+      const float r[2][2] = {{__fsqrt_rn(s00), __fsqrt_rn(s01)}, {__fsqrt_rn(s10), __fsqrt_rn(s11)}};
 #pragma unroll
-      for (int p = 0; p < 4; ++p)
+      for (int p = 0; p < 2; ++p)
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (i0 + p < c0 + rows && j0 + q < P)
-            rw[(i0 + p - c0) * ld + j0 + q] = __fsqrt_rn(s2[p][q]);
+        for (int q = 0; q < 2; ++q)
+          if (i0 + p < c0 + rows && j0 + q < P) {
+            rw[(i0 + p - c0) * ld + j0 + q] = r[p][q];
+            if (once && ib != jb) rw[(j0 + q) * ld + i0 + p] = r[p][q];
+          }
     }
     __syncthreads();
     if ((int)threadIdx.x < rows) {
       const int i = c0 + threadIdx.x;
       const float* ri = rw + threadIdx.x * ld;
       float acc = 0.0f;
-      for (int j = 0; j < P; ++j)
-        if (j != i) acc = __fadd_rn(acc, ri[j]);
+#pragma unroll 8
+      for (int j = 0; j < P; ++j) {
+        const float s = __fadd_rn(acc, ri[j]);
+        acc = j != i ? s : acc;
+      }
       s_di[i] = P > 1 ? __fdiv_rn(acc, (float)(P - 1)) : 0.0f;
     }
     __syncthreads();
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float dmin = s_di[0], dmax = s_di[0];
-    for (int i = 1; i < P; ++i) {
-      dmin = s_di[i] < dmin ? s_di[i] : dmin;
-      dmax = s_di[i] > dmax ? s_di[i] : dmax;
+  float dmin = 0.0f, dmax = 0.0f;
+  if (warp == 0) {
+    // the smallest and largest d_i (not-a-number: as if scanned from d_0 on,
+    // a first one stays)
+    dmin = dmax = s_di[0];
+    for (int i = lane; i < P; i += 32) {
+      dmin = fminf(dmin, s_di[i]);
+      dmax = fmaxf(dmax, s_di[i]);
     }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      dmin = fminf(dmin, __shfl_xor_sync(0xffffffffu, dmin, off));
+      dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, off));
+    }
+    if (s_di[0] != s_di[0]) dmin = dmax = s_di[0];
+  }
+  if (threadIdx.x == 0) {
     const float dg = s_di[s_gp];
     const float f = dmax > dmin ? __fdiv_rn(__fsub_rn(dg, dmin), __fsub_rn(dmax, dmin)) : 0.0f;
-    ApsoState st = sw.apso[a];
     float mu[5];
     int cand[4], nc = 0;
     for (int q = 1; q <= 4; ++q) {
@@ -868,9 +1047,6 @@ __global__ void __launch_bounds__(256)
           if (mu[cand[q]] > mu[state]) state = cand[q];
       }
     }
-    const uint32_t k0 = (uint32_t)co.seed, k1 = (uint32_t)(co.seed >> 32);
-    const U4 r = philox4x32_10(nodes[a].uid, (uint32_t)t, 0u, kApso << 24, k0, k1);
-    const float delta = __fadd_rn(0.05f, __fmul_rn(0.05f, uniform24(r.v[0])));
     const float h = __fmul_rn(0.5f, delta);
     float c1 = st.c1, c2 = st.c2;
     if (state == 1) {
@@ -903,15 +1079,6 @@ __global__ void __launch_bounds__(256)
     s_c[0] = st.w;
     s_c[1] = st.c1;
     s_c[2] = st.c2;
-  } else if (threadIdx.x == 32) {
-    // elitist learning's step, beside thread 0's state update: coordinate
-    // k = floor(u1 d), g = sqrt(-2 ln(1 - u2)) cos(2 pi u3) (Box-Muller, in
-    // double, rounded to float)
-    const uint32_t k0 = (uint32_t)co.seed, k1 = (uint32_t)(co.seed >> 32);
-    const U4 r = philox4x32_10(nodes[a].uid, (uint32_t)t, 0u, kApso << 24, k0, k1);
-    s_k = (int)__dmul_rn((double)uniform24(r.v[1]), (double)d);
-    s_g = (float)__dmul_rn(sqrt(__dmul_rn(-2.0, log((double)__fsub_rn(1.0f, uniform24(r.v[2]))))),
-                           cos(__dmul_rn(6.283185307179586, (double)uniform24(r.v[3]))));
   }
   __syncthreads();
   // 3. in the convergence state the next elite candidate: gB with
@@ -919,18 +1086,55 @@ __global__ void __launch_bounds__(256)
   if (s_mode) {
     const float sigma = __fsub_rn(1.0f, __fmul_rn(0.9f, __fdiv_rn((float)t, (float)sw.T)));
     for (int j = threadIdx.x; j < d; j += blockDim.x)
-      erow[j] = j == s_k ? __fadd_rn(gbp[j], __fmul_rn(__fmul_rn(2.0f, sigma), s_g)) : gbp[j];
+      erow[j] = j == s_k ? __fadd_rn(gv[j], __fmul_rn(__fmul_rn(2.0f, sigma), s_g)) : gv[j];
   }
   // 4. the move of Eq. pso-1 to iteration t + 1 with the adaptive factors
   // (k_move's step, here by this node's CTA)
-  SwarmCoef cm = co;
-  cm.inertia = s_c[0];
-  cm.c1 = s_c[1];
-  cm.c2 = s_c[2];
-  const int d4 = (d + 3) >> 2;
-  const uint32_t uid = nodes[a].uid;
-  for (int item = threadIdx.x; item < P * d4; item += blockDim.x)
-    move_item(pr, sw, cm, uid, a, t, item / d4, item - (item / d4) * d4, pbp, gbp);
+  const float cw = s_c[0], c1 = s_c[1], c2 = s_c[2];
+  auto move = [&](int item, const float (&r1)[4], const float (&r2)[4], const float (&v)[4],
+                  const float (&pb)[4]) {
+    const int pi = item / d4, j0 = 4 * (item - pi * d4);
+    float xn[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int j = j0 + c;
+      if (j >= d) break;
+      const float x = xt[(size_t)j * ldx + pi];
+      const float inertia = __fmul_rn(cw, v[c]);
+      const float cog = __fmul_rn(__fmul_rn(c1, r1[c]), __fsub_rn(pb[c], x));
+      const float soc = __fmul_rn(__fmul_rn(c2, r2[c]), __fsub_rn(gv[j], x));
+      const float vn = __fadd_rn(__fadd_rn(inertia, cog), soc);
+      vel[(int64_t)pi * d + j] = vn;
+      xn[c] = __fadd_rn(x, vn);
+      pos[(int64_t)pi * d + j] = xn[c];
+    }
+    if (sw.posb) store_posb4(sw.posb, Pp, pr.dp, a, pi, j0, xn);
+  };
+#pragma unroll
+  for (int m = 0; m < kApsoItems; ++m) {
+    const int item = threadIdx.x + m * 256;
+    if (item >= n_items) break;
+    const int pi = item / d4, j0 = 4 * (item - pi * d4);
+    // the elite candidate may have become this particle's personal best
+    // since it was read
+    if ((mode == 2 && pi == gp) || (wpb && pi == w))
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (j0 + c < d) pp[m][c] = pbp[(int64_t)pi * d + j0 + c];
+    move(item, u1[m], u2[m], pv[m], pp[m]);
+  }
+  for (int item = threadIdx.x + kApsoItems * 256; item < n_items; item += 256) {
+    const int pi = item / d4, j0 = 4 * (item - pi * d4);
+    float r1[4], r2[4], v[4], pb[4];
+    draw(item, r1, r2);
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      if (j0 + c < d) {
+        v[c] = vel[(int64_t)pi * d + j0 + c];
+        pb[c] = pbp[(int64_t)pi * d + j0 + c];
+      }
+    move(item, r1, r2, v, pb);
+  }
 }
 
 // Algorithm 1's gbest step after evaluation t, then (t < T) the synchronous
@@ -2449,7 +2653,8 @@ cudaError_t launch_apso(const Problem& pr, const Swarm& sw, const NodeDesc* node
   if (n_nodes <= 0 || !sw.apso) return cudaSuccess;
   const int R = apso_rows(pr.P, pr.d);
   if (R == 0) return cudaErrorInvalidValue;
-  const size_t smem = apso_smem(pr.P, pr.d, R);
+  const int wide = apso_smem_wide(pr.P, pr.d, R) <= kApsoMaxSmem;
+  const size_t smem = wide ? apso_smem_wide(pr.P, pr.d, R) : apso_smem(pr.P, pr.d, R);
   cudaError_t e = allow_smem((const void*)k_apso, (int)smem);
   if (e) return e;
   cudaLaunchConfig_t cfg = {};
@@ -2462,7 +2667,7 @@ cudaError_t launch_apso(const Problem& pr, const Swarm& sw, const NodeDesc* node
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_apso, pr, sw, nodes, t, co, list, A, R);
+  return cudaLaunchKernelEx(&cfg, k_apso, pr, sw, nodes, t, co, list, A, R, wide);
 }
 
 cudaError_t launch_move(const Problem& pr, const Swarm& sw, const NodeDesc* nodes, int A,

@@ -129,3 +129,27 @@ def test_unsupported_apso_is_rejected(ctx):
     with pytest.raises(S.SlmError) as e:
         ctx.node_split(p, wl.X, labels=wl.labels)
     assert e.value.status == S.SLM_EINVAL
+
+
+@pytest.mark.parametrize("crit,K,B,d,n,P,T", [
+    ("gini", 3, 32, 40, 600, 62, 30),     # every row in one chunk, a half tile
+    ("entropy", 2, 32, 24, 500, 100, 20), # more move items than a thread fetches ahead
+    ("gini", 2, 32, 16, 400, 254, 12),    # chunks of 64 rows
+    ("gini", 2, 32, 980, 300, 52, 12),    # no room for the elite's and gB's vectors
+    ("gini", 2, 32, 1, 300, 17, 20),      # one feature
+])
+def test_apso_layouts_match_oracle(ctx, crit, K, B, d, n, P, T):
+    """Every memory layout of the adaptive step's kernel (whether or not the
+    short search reaches the convergence state and tries an elite)."""
+    from paper_2208_07023_gb300 import binding as S
+    wl = W.single_node(n, d, seed=3) if K == 2 else W.gmm(n, d, K, seed=P + d)
+    g = ctx.node_split(params(S, crit, K, P, T, B, min_leaf=2, seed=21), wl.X, labels=wl.labels,
+                       node_uid=12, want_trace=True)
+    r = O.node_split(oparams(crit, K, P, T, B, min_leaf=2, seed=21), wl.X, wl.labels, node_uid=12)
+    stop = r.split["first_near_tie"]
+    upto = T + 1 if stop < 0 else stop
+    assert np.array_equal(g["trace"][:upto], r.trace_loss[:upto])
+    if stop < 0:
+        assert np.array_equal(g["gbest"].astype(np.float64), r.gbest)
+        assert (g["particle"], g["iter_of_best"], g["bin"]) == \
+            (r.split["particle"], r.split["iter_of_best"], r.split["bin"])
