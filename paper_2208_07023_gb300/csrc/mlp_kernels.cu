@@ -276,8 +276,10 @@ __global__ void __launch_bounds__((T / R) * (T / R))
 // chain per output over k in increasing order: k_gemm's bits. The chain is
 // what bounds it (K = 5376: 5376 dependent FMAs of 4 clocks, 10 us); with
 // k_gemm's two register-staged steps of 64 the first layer took 95 us, most
-// of it waiting for each step's loads; now 40 us at 64 rows, the shared-memory
-// loads and 2 FMAs per k being issued by only 4 warps per SM.
+// of it waiting for each step's loads; 33 us now at 64 rows (40 with four k of
+// the loop unrolled instead of 128): the loads, conversions and 2 FMAs per k are
+// issued by only 4 warps per SM. More stages or operands read further ahead
+// change nothing.
 constexpr int kFwdK = 128, kFwdStages = 3;
 constexpr int kFwdA = 16 * (kFwdK + 4);          // floats: [16 rows][128 k + 4]
 constexpr int kFwdBytes = kFwdA * 4 + kFwdK * 16 * 2;  // and [128 k][16 columns] bfloat16
@@ -323,7 +325,7 @@ __global__ void __launch_bounds__(128)
     const uint32_t* b =
         reinterpret_cast<const uint32_t*>(sm[s % kFwdStages] + kFwdA * 4) + tx;
     const int kc = min(kFwdK, K - s * kFwdK);
-#pragma unroll 4
+#pragma unroll 32
     for (int k = 0; k < kc; k += 4) {
       const float4 x = *reinterpret_cast<const float4*>(a + k);
       const uint32_t w0 = b[8 * k], w1 = b[8 * k + 8], w2 = b[8 * k + 16], w3 = b[8 * k + 24];
@@ -354,24 +356,59 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
   return s;
 }
 
+// Two sums over the block's threads, each block_sum's (the warps' butterflies,
+// then the warps in order); the warps from `active` on hold zeros.
+struct Sums2 {
+  double v[2][8], s[2];
+};
+__device__ __forceinline__ double2 block_sum2(double a, double b, int active, Sums2& sh) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp < active) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, off);
+      b += __shfl_xor_sync(0xffffffffu, b, off);
+    }
+  }
+  if (lane == 0) {
+    sh.v[0][warp] = warp < active ? a : 0.0;
+    sh.v[1][warp] = warp < active ? b : 0.0;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    double s = 0.0;
+    for (int i = 0; i < 8; ++i) s += sh.v[threadIdx.x][i];
+    sh.s[threadIdx.x] = s;
+  }
+  __syncthreads();
+  return make_double2(sh.s[0], sh.s[1]);
+}
+
 // One block (256 threads) per sample r: its loss (added into *loss, already
-// divided by N) and dL/do (divided by N) in double.
+// divided by N) and dL/do (divided by N) in double. Bound by the double
+// pipes (two lanes per clock per SM): the sums run in pairs, added up by one
+// warp, and only warps with features of the sample divide (64 samples of 64
+// features: 19.6 us with every warp summing and dividing, 14.6 now).
 __global__ void __launch_bounds__(256)
     k_mlp_loss(const float* __restrict__ O, const int32_t* __restrict__ dims,
                const float* __restrict__ targets, int N, float* dO, double* loss) {
-  __shared__ double sh[8];
+  __shared__ Sums2 sh0, sh1, sh2;
   const int r = blockIdx.x, j = threadIdx.x;
   const float* o = O + (int64_t)r * kOut;
   const float* a = targets + (int64_t)r * kD;
-  const int d = dims[r];
+  const int d = dims[r], wd = (d + 31) >> 5;  // warps with features
   const double oj = j < d ? (double)o[j] : 0.0, aj = j < d ? (double)a[j] : 0.0;
-  const double c = block_sum(oj * aj, sh);
-  const double mm = block_sum(oj * oj, sh);
+  const double2 cm = block_sum2(oj * aj, oj * oj, wd, sh0);
+  const double c = cm.x, mm = cm.y;
   const double q = mm + 1e-12, sg = c >= 0.0 ? 1.0 : -1.0;
   const double nm = sqrt(mm);
-  const double mh = mm > 0.0 ? oj / nm : 0.0, uj = mh - sg * aj;
-  const double delta = mm > 0.0 ? sqrt(block_sum(j < d ? uj * uj : 0.0, sh)) : 1.0;
-  const double hu = block_sum(j < d ? mh * uj : 0.0, sh);
+  double mh = 0.0, uj = 0.0;
+  if (j < d) {
+    mh = mm > 0.0 ? oj / nm : 0.0;
+    uj = mh - sg * aj;
+  }
+  const double2 uh = block_sum2(uj * uj, mh * uj, wd, sh1);
+  const double delta = mm > 0.0 ? sqrt(uh.x) : 1.0, hu = uh.y;
   // spread: radii i < 64 on threads 0..63
   double pin = 0.0, dld = 0.0;
   if (j < kP) {
@@ -384,14 +421,15 @@ __global__ void __launch_bounds__(256)
     const double dl_drho = (u >= 0.0 ? -tau : 1.0 - tau) / kP;
     dO[(int64_t)r * kOut + kD + j] = (float)(dl_drho / (1.0 + exp(-x)) / N);
   }
-  const double spread = block_sum(pin, sh);
-  const double dl_ddelta = block_sum(dld, sh);
-  double g = 0.0;
+  const double2 sd = block_sum2(pin, dld, (kP + 31) >> 5, sh2);
+  const double spread = sd.x, dl_ddelta = sd.y;
+  float g32 = 0.0f;
   if (j < d) {
-    g = -2.0 * c * aj / q + 2.0 * c * c * oj / (q * q);
+    double g = -2.0 * c * aj / q + 2.0 * c * c * oj / (q * q);
     if (mm > 0.0 && delta > 0.0) g += dl_ddelta * (uj - mh * hu) / (nm * delta);
+    g32 = (float)(g / N);
   }
-  dO[(int64_t)r * kOut + j] = (float)(g / N);
+  dO[(int64_t)r * kOut + j] = g32;
   if (j == 0) atomicAdd(loss, (1.0 - c * c / q + spread / kP) / N);
 }
 
