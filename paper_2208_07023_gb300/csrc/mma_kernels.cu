@@ -7,15 +7,15 @@
 // rows of one node at a time. One thread issues tcgen05.mma (kind::f16, BF16
 // A and B, FP32 accumulator in tensor memory, M = 128, N = P', K = 16 per
 // instruction) on operands that 1D bulk copies stage in shared memory; the
-// four warps read the accumulator back with tcgen05.ld (warp w owns TMEM lanes
-// 32w..32w+31 = rows of the tile), store z to the L2-resident z buffer and
+// eight warps read the accumulator back with tcgen05.ld (warp w owns TMEM lanes
+// 32 (w mod 4) .. + 31 = rows of the tile, and every second 16 columns), store z to the L2-resident z buffer and
 // fold each particle's range. The level's rows are converted to bfloat16 once
 // per level, directly into the operand layout, so a tile chunk is one
 // contiguous copy; the positions are converted once per iteration.
 //
 // Then, per node, the k particles with the best such score (selected by the
-// last histogram CTA of the node) are re-scored on the FP32 projection (the
-// k_project / k_hist_scan path) and k_merge writes their scores over the
+// last histogram CTA of the node) are re-scored on an FP32 projection
+// (k_project_few) and k_merge writes their scores over the
 // reduced ones, takes every particle's pbest step and the gbest step among
 // the re-scored particles (Algorithm 1).
 #include <cuda_bf16.h>
@@ -29,7 +29,12 @@ namespace slm {
 namespace {
 
 constexpr int kMmaKC = 128;       // features per staged chunk of a tile
-constexpr int kMmaThreads = 128;  // four warps: the 128 TMEM lanes
+// Eight warps: two for each quadrant of the 128 TMEM lanes, each with every
+// second group of 16 columns. The epilogue (two warp reductions and a store per
+// column and warp) bounds the kernel: 200,000 x 128 rows, 64 particles took
+// 36 us with four warps and a test per element, 30 without the tests in whole
+// tiles, 24.5 with eight warps (24 with sixteen).
+constexpr int kMmaThreads = 256;
 
 // ---- tensor memory and tcgen05 -------------------------------------------------
 
@@ -143,8 +148,8 @@ __host__ __device__ inline uint32_t mma_tmem_cols(int Pp) {
 // issues the MMAs of an item as soon as it lands and commits them to
 // free[s] (stage reusable) and, after the tile's last chunk, to acc[u & 1]:
 // the accumulator is double-buffered in tensor memory, so the MMAs of tile
-// u+1 run while the four warps read tile u back. The positions of a node are
-// staged once per node. Each warp keeps a running range per column in shared
+// u+1 run while the warps read tile u back. The positions of a node are
+// staged once per node. Each quadrant keeps a running range per column in shared
 // memory, folded into global memory once per node.
 __global__ void __launch_bounds__(kMmaThreads)
     k_project_mma(Problem pr, Swarm sw, const WorkTile* __restrict__ tiles, int n_tiles,
@@ -153,7 +158,7 @@ __global__ void __launch_bounds__(kMmaThreads)
   __shared__ __align__(8) uint64_t bar_full[2], bar_free[2], bar_acc[2], bar_b;
   __shared__ uint32_t s_tmem;
   __shared__ int s_err;
-  __shared__ int s_lo[kMmaThreads / 32][kMaxParticles], s_hi[kMmaThreads / 32][kMaxParticles];
+  __shared__ int s_lo[4][kMaxParticles], s_hi[4][kMaxParticles];  // by quadrant
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int P = pr.P, Pp = pr.Pp, dp = pr.dp;
   const uint32_t stage = mma_stage_bytes(dp);
@@ -178,10 +183,11 @@ __global__ void __launch_bounds__(kMmaThreads)
     mbar_init_fence();
     s_err = 0;
   }
-  for (int p = lane; p < Pp; p += 32) {  // each warp its own running range
-    s_lo[warp][p] = INT_MAX;
-    s_hi[warp][p] = INT_MIN;
-  }
+  if (warp < 4)
+    for (int p = lane; p < Pp; p += 32) {
+      s_lo[warp][p] = INT_MAX;
+      s_hi[warp][p] = INT_MIN;
+    }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -255,30 +261,41 @@ __global__ void __launch_bounds__(kMmaThreads)
     if (tid == 0 && ti + 1 < my_tiles) mma_tile(ti + 1);
     if (!mbar_wait(&bar_acc[ti & 1], (uint32_t)((ti >> 1) & 1), kWaitPolls)) s_err = 1;
     tc_fence_after();
-    // epilogue: accumulator row r = 32 warp + lane holds z of every particle
-    const int r = warp * 32 + lane;
+    // epilogue: accumulator row r holds z of every particle; a warp reads the
+    // 32 rows of its quadrant (warp mod 4) and every second 16 columns
+    const int quad = warp & 3;
+    const int r = quad * 32 + lane;
     const bool rv = r < wt.rows;
     float* zrow = sw.z + wt.row0 + r;
-    const uint32_t t_row = tmem + (uint32_t)(ti & 1) * cols + ((uint32_t)(warp * 32) << 16);
-    for (int cb = 0; cb < Pp / 16; ++cb) {
+    const uint32_t t_row = tmem + (uint32_t)(ti & 1) * cols + ((uint32_t)(quad * 32) << 16);
+    // a whole tile and 16 columns of particles: nothing to test per element
+    const bool whole = wt.rows == kMmaRows;
+    for (int cb = warp >> 2; cb < Pp / 16; cb += kMmaThreads / 128) {
       uint32_t v[16];
       tmem_ld16(t_row + (uint32_t)(cb * 16), v);
       int my_lo = INT_MAX, my_hi = INT_MIN;  // lane j < 16: column cb*16 + j
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const int p = cb * 16 + j;
+      float* zp = zrow + (int64_t)(cb * 16) * pr.Ez;
+      auto column = [&](int j, bool in, bool out) {
         const float z = __uint_as_float(v[j]);
         const int oz = f2ord(z);
-        const int lo = __reduce_min_sync(0xffffffffu, rv ? oz : INT_MAX);
-        const int hi = __reduce_max_sync(0xffffffffu, rv ? oz : INT_MIN);
-        if (rv && p < P) zrow[(int64_t)p * pr.Ez] = z;
+        const int lo = __reduce_min_sync(0xffffffffu, in ? oz : INT_MAX);
+        const int hi = __reduce_max_sync(0xffffffffu, in ? oz : INT_MIN);
+        if (out) *zp = z;
+        zp += pr.Ez;
         my_lo = lane == j ? lo : my_lo;
         my_hi = lane == j ? hi : my_hi;
+      };
+      if (whole && cb * 16 + 16 <= P) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) column(j, true, true);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) column(j, rv, rv && cb * 16 + j < P);
       }
       if (lane < 16) {
         const int p = cb * 16 + lane;
-        s_lo[warp][p] = min(s_lo[warp][p], my_lo);
-        s_hi[warp][p] = max(s_hi[warp][p], my_hi);
+        s_lo[quad][p] = min(s_lo[quad][p], my_lo);
+        s_hi[quad][p] = max(s_hi[quad][p], my_hi);
       }
     }
     tc_fence_before();
@@ -289,7 +306,7 @@ __global__ void __launch_bounds__(kMmaThreads)
       for (int p = tid; p < P; p += kMmaThreads) {
         int lo = INT_MAX, hi = INT_MIN;
 #pragma unroll
-        for (int w = 0; w < kMmaThreads / 32; ++w) {
+        for (int w = 0; w < 4; ++w) {
           lo = min(lo, s_lo[w][p]);
           hi = max(hi, s_hi[w][p]);
           s_lo[w][p] = INT_MAX;

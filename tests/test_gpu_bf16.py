@@ -237,3 +237,14 @@ def test_bf16_rejects_bad_topk_and_sizes(ctx):
     with pytest.raises(S.SlmError) as e:
         ctx.node_split(bf16_gpu_params(S, "gini", 2, 256, 3, 16, topk=8), Xw, labels=lab)
     assert e.value.status == S.SLM_EUNSUPPORTED
+
+
+@pytest.mark.parametrize("n,d,P", [
+    (384, 32, 16),    # whole row tiles, one group of columns: a quadrant's second warp idle
+    (128, 16, 40),    # three groups, the last partly particles
+    (1000, 33, 64),   # a ragged last tile
+    (1280, 64, 250),  # the widest accumulator
+])
+def test_bf16_epilogue_tiles(ctx, n, d, P):
+    """Whole and ragged row tiles and column groups of the tensor-core pass."""
+    test_bf16_scores_follow_bins(ctx, "gini", 3, 32, d, n, None, P, False)
