@@ -560,11 +560,12 @@ slm_status slm_set_node_search(slm_ctx* ctx, int32_t on);
 /* CTAs per node of the context's last search in the persistent kernel, 0 if
  * the last search used the per-iteration kernels. */
 slm_status slm_last_node_search(slm_ctx* ctx, int32_t* ctas_per_node);
-/* Histogram kernels of classification searches (FP32 form): when a level's
+/* Histogram kernels of the searches: when a level's
  * nodes of at most max_entries entries (default 4096) give at least
  * min_pairs (node, particle) pairs (-1, the default: 2 x SMs x 8, enough
  * warps to fill the GPU), they are scored one warp per (node, particle)
- * from memory; the other nodes (all nodes otherwise) by clusters of CTAs
+ * from memory (classification in the FP32 form; unweighted regression up to
+ * 2,048 entries, also in the BF16 form); the other nodes (all nodes otherwise) by clusters of CTAs
  * staging the node through shared memory. max_entries = 0 sends every node
  * to the clusters. Scores are identical either way. SLM_EINVAL for
  * max_entries < 0 or min_pairs < -1. */
@@ -637,10 +638,12 @@ slm_status slm_set_step_shape(slm_ctx* ctx, int32_t shape, int32_t* last);
 /* on != 0 (the default): the searches of the FP32 form score each
  * iteration with the latency-oriented histogram kernels (entries loaded 16
  * bytes at a time with several in flight; classification: class-major
- * histograms scanned one warp per class; regression, for nodes of at most
- * 257,740 entries: two particles per block, the fixed-point bin moments
- * added as 32-bit pieces into lane copies; the pbest step spread over the
- * block; the BF16 form's regression passes too); on = 0: with
+ * histograms scanned one warp per class, two particles per block in large
+ * batches; unweighted regression: targets rounded to 30 bits bound every
+ * edge's score, and only those that can matter are scored exactly; weighted
+ * regression, for nodes of at most 257,740 entries: the fixed-point bin
+ * moments added as 32-bit pieces into lane copies; the pbest step spread over
+ * the block; the BF16 form's passes too); on = 0: with
  * the staged-copy histogram kernel that also serves bins output and the
  * BF16 form. node_step != 0: in folded classification searches
  * (slm_set_fused_step) whose nodes all take that kernel, the last block to

@@ -11,8 +11,9 @@
 //
 // Data layout. A batch's rows are stored entry-ordered and contiguous (the
 // level-resident copy X_l[E, d]: each node is a segment of consecutive rows),
-// with entry-aligned labels / targets / multiplicities. One iteration is two
-// kernels plus the swarm update:
+// with entry-aligned labels / targets / multiplicities. The general kernels
+// (the default searches take the projection of step_kernels.cu and the
+// histograms of hist_kernels.cu and mse_kernels.cu):
 //  * k_project: z[p][e] = X_l[e] . x_p for all entries and particles, once.
 //    A persistent grid walks (tile of kTS = 256 rows, group of PG = 8..48
 //    particles, picked per problem shape by the autotuner) work units; rows and positions stream through shared memory

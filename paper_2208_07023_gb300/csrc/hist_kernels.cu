@@ -711,8 +711,9 @@ __global__ void __launch_bounds__(kThreads, NP == 1 ? 2 : 4)
   }
 }
 
-// Histogram and threshold scan of regression searches in the FP32 form
-// (Sec. II-A, Eqs. 3-4 with the squared error): per bin the weight and the
+// Histogram and threshold scan of weighted (bagged) regression searches
+// (Sec. II-A, Eqs. 3-4 with the squared error; unweighted ones take the
+// kernels of mse_kernels.cu): per bin the weight and the
 // fixed-point sums of w (y - c) and w (y - c)^2. Shared-memory atomics are
 // 32-bit only (64-bit ones run several times slower on this GPU): each
 // 64-bit moment v is added as three pieces, v mod 2^16, (v >> 16) mod 2^16
