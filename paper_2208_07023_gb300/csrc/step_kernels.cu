@@ -131,7 +131,11 @@ __global__ void __launch_bounds__(32 * (FOLD ? kFoldWarps : kProjWarps))
   constexpr int PU = PW * PB;            // particles of a slice
   constexpr int RB = NW / PB;            // row warps
   constexpr int NS = kStepStages;
-  constexpr int TF = FOLD ? 8 : 16;      // features of an unrolled turn
+  // Features of an unrolled turn: a whole chunk. (Folded, us a launch with 8, 16:
+  // 12.6, 11.3 on 7,321 x 23 rows, 17.7, 17.2 on 50,000 x 64, 16.8, 16.1 on
+  // 30,011 x 50; unfolded with 8: 87 instead of 78 on 200,000 x 128. A turn of 4
+  // for the rest of a chunk costs the others registers: 85 there.)
+  constexpr int TF = 16;
   constexpr int W = QP >= 4 ? QP - 4 : QP;  // particles per lane beyond the first four
   // Ranges are exchanged once per (node, slice) where two registers a particle
   // are free, else after each block (64 trees on 100,000 x 32 rows, P = 48:
