@@ -67,10 +67,10 @@ HBM_PEAK_GBS, BF16_PEAK_TFLOPS, PEAK_SOURCE = _measured_peaks()
 # launch over its pairs, profiles/), each valid only for the kernel source it
 # was taken from: (bytes per pair, source file, sha256 of that file).
 TRAFFIC = {
-    "project": (12945152 / 3.2e6, "step_kernels.cu",
-                "6f7aa4390ba6326c3a0f7e2e133cae0165c0f104276e7fc53b374ce71d178241"),
-    "hist_scan": (13066496 / 3.2e6, "hist_kernels.cu",
-                  "503a69c3a12c5b8fac4578b88d018a05729810e190770abfa551f1af9538117e"),
+    "project": (16464128 / 3.2e6, "step_kernels.cu",
+                "2fe5bf2588f2bcc6a2d548f57ddbaf6a9b26c948ab42b930cd13fa26df68857e"),
+    "hist_scan": (13067008 / 3.2e6, "hist_kernels.cu",
+                  "cd01add82b7f135f633e18f9d46bd3d011001fb0cb83be2dda9a70edbb538620"),
 }
 
 
