@@ -330,9 +330,11 @@ __global__ void __launch_bounds__(kMmaThreads)
 
 // ---- merge of the re-scored particles ----------------------------------------------------
 
-// Grid (node, group of 8 particles): warp w of block y merges particle
-// 8 y + w and takes its pbest step; block y = 0 also takes the node's gbest
-// step among the re-scored particles, from their FP32 scores in cur2.
+// Grid (node, group of 8 particles, and in a search one more): warp w of block
+// y merges particle 8 y + w and takes its pbest step; the last block takes the
+// node's gbest step among the re-scored particles, from their FP32 scores in
+// cur2, beside the merges instead of after one block's (a chain of dependent
+// loads each; on 200,000 x 128 rows 9.0 and 6.0 us a launch).
 __global__ void __launch_bounds__(256)
     k_merge(Problem pr, Swarm sw, const EvalRes* __restrict__ cur2, int kp,
             const int32_t* __restrict__ inv, int t, int do_update) {
@@ -342,52 +344,30 @@ __global__ void __launch_bounds__(256)
   const int a = blockIdx.x, A = gridDim.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int Pp = pr.Pp, d = pr.d;
-  const int p = blockIdx.y * 8 + warp;
-  if (p < pr.P) {
-    const int q = inv[(int64_t)a * Pp + p];
-    const EvalRes e = q >= 0 ? cur2[(int64_t)a * kp + q] : sw.cur[(int64_t)a * Pp + p];
-    if (q >= 0 && lane == 0) sw.cur[(int64_t)a * Pp + p] = e;
-    if (do_update) pbest_step(pr, sw, a, p, t, e);
+  if (!do_update || blockIdx.y + 1 < gridDim.y) {
+    const int p = blockIdx.y * 8 + warp;
+    if (p < pr.P) {
+      const int q = inv[(int64_t)a * Pp + p];
+      const EvalRes e = q >= 0 ? cur2[(int64_t)a * kp + q] : sw.cur[(int64_t)a * Pp + p];
+      if (q >= 0 && lane == 0) sw.cur[(int64_t)a * Pp + p] = e;
+      if (do_update) pbest_step(pr, sw, a, p, t, e);
+    }
+    return;
   }
-  if (!do_update || blockIdx.y != 0) return;
   if (warp == 0) {
     // gbest step among the re-scored particles: the best strictly better
     // than the gbest of iteration t-1 (at t = 0 any), ties to the lower index
     const EvalRes gold = sw.gb[(int64_t)((t + 1) & 1) * A + a];
     int bi = -1;
     EvalRes be = invalid_res();
-    for (int q = lane; q < sw.k; q += 32) {
-      const int pq = sw.sel[(int64_t)a * sw.k + q];
-      const EvalRes e = cur2[(int64_t)a * kp + q];
-      if (!(t == 0 || better(e, gold, pr.crit))) continue;
-      if (bi < 0 || better(e, be, pr.crit)) {
-        bi = pq;
-        be = e;
-      }
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-      const EvalRes o = shfl_res(be, lane ^ off);
-      bool take;
-      if (oi < 0)
-        take = false;
-      else if (bi < 0)
-        take = true;
-      else if (better(o, be, pr.crit))
-        take = true;
-      else if (better(be, o, pr.crit))
-        take = false;
-      else
-        take = oi < bi;
-      if (take) {
-        bi = oi;
-        be = o;
-      }
-    }
+    for (int q = lane; q < sw.k; q += 32)
+      gbest_consider(pr, gold, t, sw.sel[(int64_t)a * sw.k + q], cur2[(int64_t)a * kp + q], &bi,
+                     &be);
+    EvalRes best = gold;
+    bi = gbest_select(pr, bi, be, &best);
     if (lane == 0) {
       s_best = bi;
-      const EvalRes g = bi >= 0 ? be : gold;
+      const EvalRes g = bi >= 0 ? best : gold;
       sw.gb[(int64_t)(t & 1) * A + a] = g;
       if (bi >= 0) {
         sw.gpart[a] = bi;
@@ -483,7 +463,7 @@ cudaError_t launch_merge(const Problem& pr, const Swarm& sw, int A, const EvalRe
                          const int32_t* inv, int t, int do_update, cudaStream_t st) {
   if (A <= 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)A, (unsigned)((pr.P + 7) / 8), 1);
+  cfg.gridDim = dim3((unsigned)A, (unsigned)((pr.P + 7) / 8 + (do_update ? 1 : 0)), 1);
   cfg.blockDim = dim3(256, 1, 1);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
