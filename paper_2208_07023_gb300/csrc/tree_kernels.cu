@@ -550,19 +550,26 @@ __global__ void __launch_bounds__(256)
   const int64_t r0 = (int64_t)blockIdx.x * R;
   const int nr = (int)min((int64_t)R, n - r0);
   if (staged) {
-    if (VEC) {
-      const int d4 = d >> 2;
-      for (int q = threadIdx.x; q < nr * d4; q += blockDim.x) {
-        const int r = q / d4, c = q - r * d4;
-        *reinterpret_cast<float4*>(rows + r * stride + 4 * c) =
-            __ldg(reinterpret_cast<const float4*>(X + (r0 + r) * d) + c);
-      }
-    } else {
-      for (int q = threadIdx.x; q < nr * d; q += blockDim.x) {
-        const int r = q / d, c = q - r * d;
-        rows[r * stride + c] = __ldg(X + (r0 + r) * d + c);
+    // every word of the tile on its way at once
+    const int w = VEC ? d >> 2 : d, step_r = (int)blockDim.x / w,
+              step_c = (int)blockDim.x - step_r * w;
+    int r = (int)threadIdx.x / w, c = (int)threadIdx.x - r * w;
+    while (r < nr) {
+      const float* src = X + (r0 + r) * d + (VEC ? 4 * c : c);
+      const uint32_t dst =
+          (uint32_t)__cvta_generic_to_shared(rows + r * stride + (VEC ? 4 * c : c));
+      if (VEC)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src));
+      else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src));
+      r += step_r;
+      c += step_c;
+      if (c >= w) {
+        c -= w;
+        ++r;
       }
     }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
   }
   const int rl = rb * 32 + lane;  // this lane's row of the tile
@@ -776,10 +783,13 @@ cudaError_t launch_predict(const float* X, int64_t n, int d, TreeArrays tr, int 
                             (staged ? (size_t)32 * rb * pred_stride(d, vec) : 0));
   };
   while (RB > 1 && smem(RB, true) > 48 * 1024) RB /= 2;
+  // few rows: smaller tiles, on more SMs
+  while (RB > 1 && (n + 32 * RB - 1) / (32 * RB) < 152) RB /= 2;
   const bool staged = smem(RB, true) <= (size_t)kPredSmem;
   const size_t sm = smem(RB, staged);
   const void* f = vec ? (const void*)k_predict<true> : (const void*)k_predict<false>;
-  if (cudaError_t e = allow_smem(f, (int)sm)) return e;
+  if (sm > 48 * 1024)
+    if (cudaError_t e = allow_smem(f, (int)sm)) return e;
   const unsigned grid = (unsigned)((n + 32 * RB - 1) / (32 * RB));
   const int threads = 32 * RB * WT;
   if (vec)
