@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(kThreads, NP == 1 ? 2 : 4)
   };
   // the first sets are in flight while the range is read
   load_set(0, threadIdx.x);
-  load_set(1, threadIdx.x + kSet);
+  if (NP > 1 || n4 > kSet) load_set(1, threadIdx.x + kSet);
   // the tail's inputs, also in flight from here: the particles' pbest scores
   // and the node's gbest score (evaluation t - 1), their x, v and pB rows
   const int64_t prow0 = ci0 * d;
@@ -240,9 +240,13 @@ __global__ void __launch_bounds__(kThreads, NP == 1 ? 2 : 4)
     uint32_t* h = hc + (warp % C) * (NP * W);  // class-major: h[label * B + bin]
     int done = 0;
     if (g16) {
-      for (int g0 = threadIdx.x; g0 < n4; g0 += 2 * kSet) {
+      // (one particle: the branches on gb are the same for every thread, and a
+      // short slice runs one set's code only: 13.4 us a launch instead of 14.0
+      // on 17,953 entries x 21 particles)
+      for (int gb = 0; gb < n4; gb += 2 * kSet) {
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
+          if (NP == 1 && s == 1 && gb + kSet >= n4) break;
 #pragma unroll
           for (int u = 0; u < U; ++u) {
             const int4 l = lv[s][u];
@@ -259,7 +263,7 @@ __global__ void __launch_bounds__(kThreads, NP == 1 ? 2 : 4)
                 atomicAdd(&hq[l.w * B + bin_of(z.w, zmin[q], inv_w[q], B)], wt.w);
               }
           }
-          load_set(s, g0 + (2 + s) * kSet);
+          if (NP > 1 || gb + (2 + s) * kSet < n4) load_set(s, gb + (int)threadIdx.x + (2 + s) * kSet);
         }
       }
       done = n4 << 2;
