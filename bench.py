@@ -69,8 +69,8 @@ HBM_PEAK_GBS, BF16_PEAK_TFLOPS, PEAK_SOURCE = _measured_peaks()
 TRAFFIC = {
     "project": (16464128 / 3.2e6, "step_kernels.cu",
                 "2fe5bf2588f2bcc6a2d548f57ddbaf6a9b26c948ab42b930cd13fa26df68857e"),
-    "hist_scan": (13067008 / 3.2e6, "hist_kernels.cu",
-                  "cd01add82b7f135f633e18f9d46bd3d011001fb0cb83be2dda9a70edbb538620"),
+    "hist_scan": (13066496 / 3.2e6, "hist_kernels.cu",
+                  "5b75c47a2b50c06eb1e4cb39b1d25e0ae95dce15c1585505862d243a6075da48"),
 }
 
 
