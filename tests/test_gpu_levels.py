@@ -44,3 +44,19 @@ def test_tree_matches_oracle(ctx, crit, n, d):
     elif _check_tree_up_to_near_ties(g, r, op, wl.X, None, wl.y) == 0:
         present = r.kind >= 0
         assert np.allclose(g["leaf_value"][present], r.leaf_value[present], rtol=1e-12, atol=1e-12)
+
+
+@pytest.mark.parametrize("d,trees", [(5, 1), (8, 1), (54, 1), (16, 9), (260, 2)])
+def test_prediction_does_not_depend_on_the_tile(ctx, d, trees):
+    """Tiles of 32 to 256 rows (fewer rows a block where there are few),
+    staged by 4- or 16-byte copies: every row's class and leaves."""
+    from paper_2208_07023_gb300 import binding as S
+    wl = W.gmm(40000, d, 4, seed=d)
+    p = gpu_params(S, "gini", 4, 16, 3, 32, min_leaf=5, max_depth=5, seed=6, n_trees=trees,
+                   bootstrap=trees > 1)
+    f = ctx.train_tree(p, wl.X[:3000], labels=wl.labels[:3000])
+    cls, _, leaf = ctx.predict(f, wl.X, want_leaf=True)
+    for n in (1, 31, 33, 4833, 19457, 38913):
+        c, _, lf = ctx.predict(f, wl.X[:n], want_leaf=True)
+        assert np.array_equal(c, cls[:n]) and np.array_equal(lf, leaf[:n]), n
+    f.free()
