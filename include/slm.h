@@ -611,8 +611,9 @@ slm_status slm_set_projection_tma(slm_ctx* ctx, int32_t on);
 /* on = 1 (the default) or 2: FP32 searches of whole batches (no BF16 form, no
  * persistent node search, no projection tiles forced by slm_force_tiles)
  * project from the rows laid out in blocks of 32, feature-major, once per
- * search (a second copy of the batch's rows; searches without room for it
- * use the kernels of on = 0). Plain searches (no adaptive PSO) whose padded
+ * search (a second copy of the batch's rows, kept by the context for its
+ * next searches until another of its buffers needs the room; searches without
+ * room for it use the kernels of on = 0). Plain searches (no adaptive PSO) whose padded
  * swarm is 16, 32, 48 or 64 particles and whose positions fit in 96 KB of
  * shared memory may also fold the swarm move of Eq. pso-1 into this
  * projection: one iteration is the projection (which first takes the gbest

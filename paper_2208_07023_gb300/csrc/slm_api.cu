@@ -217,7 +217,7 @@ slm_status cuda_fail(slm_ctx* c, cudaError_t e, const char* where) {
 // the device were out of memory (0: never).
 std::atomic<int64_t> g_fail_alloc{0};
 
-cudaError_t ensure(DevBuf& b, size_t bytes) {
+cudaError_t grow(DevBuf& b, size_t bytes) {
   if (bytes == 0) bytes = 16;
   if (bytes <= b.cap) return cudaSuccess;
   if (g_fail_alloc.load() > 0 && g_fail_alloc.fetch_sub(1) == 1) return cudaErrorMemoryAllocation;
@@ -243,6 +243,20 @@ void release(DevBuf& b) {
   b.cap = 0;
 }
 
+// Room for `bytes` in a work buffer. Where the device has none left, the
+// context's blocked copy of a search's rows goes back to it first: no search
+// in flight needs it (plan_step takes it after everything else a search
+// grows), and a search without room for it takes other kernels.
+cudaError_t ensure(slm_ctx* c, DevBuf& b, size_t bytes) {
+  const cudaError_t e = grow(b, bytes);
+  if (e != cudaErrorMemoryAllocation) return e;
+  (void)cudaGetLastError();
+  DevBuf& copy = c->ws[S_XT];
+  if (&b == &copy || !copy.p) return e;
+  release(copy);
+  return grow(b, bytes);
+}
+
 bool is_device_ptr(const void* p) {
   if (!p) return false;
   cudaPointerAttributes a;
@@ -265,7 +279,7 @@ slm_status stage_in(slm_ctx* c, const T* src, size_t count, DevBuf& buf,
     *out = src;
     return SLM_OK;
   }
-  CK(ensure(buf, sizeof(T) * count));
+  CK(ensure(c, buf, sizeof(T) * count));
   CK(cudaMemcpyAsync(buf.p, src, sizeof(T) * count, cudaMemcpyHostToDevice,
                      c->stream));
   *out = static_cast<const T*>(buf.p);
@@ -276,7 +290,7 @@ slm_status stage_in(slm_ctx* c, const T* src, size_t count, DevBuf& buf,
 // address allows, else a copy in `buf`.
 slm_status align16(slm_ctx* c, const float** p, size_t count, DevBuf& buf) {
   if ((reinterpret_cast<uintptr_t>(*p) & 15) == 0) return SLM_OK;
-  CK(ensure(buf, sizeof(float) * count));
+  CK(ensure(c, buf, sizeof(float) * count));
   CK(cudaMemcpyAsync(buf.p, *p, sizeof(float) * count, cudaMemcpyDeviceToDevice, c->stream));
   *p = static_cast<const float*>(buf.p);
   return SLM_OK;
@@ -438,25 +452,25 @@ T* ws_ptr(slm_ctx* c, Slot s) {
 slm_status setup_scoring(slm_ctx* c, Problem& pr, int A,
                          const std::vector<NodeDesc>& nodes,
                          const std::vector<WorkTile>& tiles, Swarm* sw) {
-  CK(ensure(c->ws[S_CUR], sizeof(EvalRes) * (size_t)A * pr.Pp));
-  CK(ensure(c->ws[S_ZMM], sizeof(int32_t) * 2 * (size_t)A * pr.Pp));
-  CK(ensure(c->ws[S_Z], sizeof(float) * (size_t)pr.P * (size_t)(pr.Ez > 0 ? pr.Ez : 4)));
-  CK(ensure(c->ws[S_NODES], sizeof(NodeDesc) * nodes.size()));
-  CK(ensure(c->ws[S_TILES], sizeof(WorkTile) * tiles.size()));
+  CK(ensure(c, c->ws[S_CUR], sizeof(EvalRes) * (size_t)A * pr.Pp));
+  CK(ensure(c, c->ws[S_ZMM], sizeof(int32_t) * 2 * (size_t)A * pr.Pp));
+  CK(ensure(c, c->ws[S_Z], sizeof(float) * (size_t)pr.P * (size_t)(pr.Ez > 0 ? pr.Ez : 4)));
+  CK(ensure(c, c->ws[S_NODES], sizeof(NodeDesc) * nodes.size()));
+  CK(ensure(c, c->ws[S_TILES], sizeof(WorkTile) * tiles.size()));
   CK(cudaMemcpyAsync(c->ws[S_NODES].p, nodes.data(), sizeof(NodeDesc) * nodes.size(),
                      cudaMemcpyHostToDevice, c->stream));
   if (!tiles.empty())
     CK(cudaMemcpyAsync(c->ws[S_TILES].p, tiles.data(), sizeof(WorkTile) * tiles.size(),
                        cudaMemcpyHostToDevice, c->stream));
-  CK(ensure(c->ws[S_ERR], sizeof(int32_t)));
+  CK(ensure(c, c->ws[S_ERR], sizeof(int32_t)));
   CK(cudaMemsetAsync(c->ws[S_ERR].p, 0, sizeof(int32_t), c->stream));
   if (pr.crit == SLM_MSE) {
     const size_t ne = (size_t)(pr.Ez > 0 ? pr.Ez : 4) + 16;
-    CK(ensure(c->ws[S_M1], sizeof(long long) * ne));
-    CK(ensure(c->ws[S_M2], sizeof(long long) * ne));
-    CK(ensure(c->ws[S_MACCW], sizeof(unsigned long long) * (size_t)A));
-    CK(ensure(c->ws[S_MACCY], sizeof(int32_t) * 2 * (size_t)A));
-    CK(ensure(c->ws[S_MSCALE], sizeof(double) * 2 * (size_t)A));
+    CK(ensure(c, c->ws[S_M1], sizeof(long long) * ne));
+    CK(ensure(c, c->ws[S_M2], sizeof(long long) * ne));
+    CK(ensure(c, c->ws[S_MACCW], sizeof(unsigned long long) * (size_t)A));
+    CK(ensure(c, c->ws[S_MACCY], sizeof(int32_t) * 2 * (size_t)A));
+    CK(ensure(c, c->ws[S_MSCALE], sizeof(double) * 2 * (size_t)A));
     pr.m1 = ws_ptr<long long>(c, S_M1);
     pr.m2 = ws_ptr<long long>(c, S_M2);
     pr.mscale = ws_ptr<double>(c, S_MSCALE);
@@ -465,8 +479,8 @@ slm_status setup_scoring(slm_ctx* c, Problem& pr, int A,
     uint32_t* mq = nullptr;
     MseNode* mnode = nullptr;
     if (!pr.w && c->class_hist) {  // scored from the rounded targets (mse_kernels.cu)
-      CK(ensure(c->ws[S_MQ], sizeof(uint32_t) * ne));
-      CK(ensure(c->ws[S_MNODE], sizeof(MseNode) * (size_t)A));
+      CK(ensure(c, c->ws[S_MQ], sizeof(uint32_t) * ne));
+      CK(ensure(c, c->ws[S_MNODE], sizeof(MseNode) * (size_t)A));
       pr.mq = mq = ws_ptr<uint32_t>(c, S_MQ);
       pr.mnode = mnode = ws_ptr<MseNode>(c, S_MNODE);
     }
@@ -493,20 +507,20 @@ slm_status setup_swarm(slm_ctx* c, Problem& pr, int A, int T, bool want_trace,
   Swarm s{};
   if (slm_status st = setup_scoring(c, pr, A, nodes, tiles, &s)) return st;
   const size_t apd = (size_t)A * pr.Pp * pr.d;
-  CK(ensure(c->ws[S_POS], sizeof(float) * apd));
-  CK(ensure(c->ws[S_VEL], sizeof(float) * apd));
-  CK(ensure(c->ws[S_PBEST], sizeof(float) * apd));
-  CK(ensure(c->ws[S_GBEST], sizeof(float) * (size_t)A * pr.d));
-  CK(ensure(c->ws[S_PB], sizeof(EvalRes) * (size_t)A * pr.Pp));
-  CK(ensure(c->ws[S_GB], sizeof(EvalRes) * 2 * (size_t)A));
-  CK(ensure(c->ws[S_GPART], sizeof(int32_t) * (size_t)A));
-  CK(ensure(c->ws[S_GITER], sizeof(int32_t) * (size_t)A));
-  CK(ensure(c->ws[S_DONE], sizeof(int32_t) * (size_t)A));
+  CK(ensure(c, c->ws[S_POS], sizeof(float) * apd));
+  CK(ensure(c, c->ws[S_VEL], sizeof(float) * apd));
+  CK(ensure(c, c->ws[S_PBEST], sizeof(float) * apd));
+  CK(ensure(c, c->ws[S_GBEST], sizeof(float) * (size_t)A * pr.d));
+  CK(ensure(c, c->ws[S_PB], sizeof(EvalRes) * (size_t)A * pr.Pp));
+  CK(ensure(c, c->ws[S_GB], sizeof(EvalRes) * 2 * (size_t)A));
+  CK(ensure(c, c->ws[S_GPART], sizeof(int32_t) * (size_t)A));
+  CK(ensure(c, c->ws[S_GITER], sizeof(int32_t) * (size_t)A));
+  CK(ensure(c, c->ws[S_DONE], sizeof(int32_t) * (size_t)A));
   CK(cudaMemsetAsync(c->ws[S_DONE].p, 0, sizeof(int32_t) * (size_t)A, c->stream));
-  if (want_trace) CK(ensure(c->ws[S_TRACE], sizeof(double) * (size_t)A * (T + 1)));
-  CK(ensure(c->ws[S_APSO], sizeof(ApsoState) * (size_t)A));
+  if (want_trace) CK(ensure(c, c->ws[S_TRACE], sizeof(double) * (size_t)A * (T + 1)));
+  CK(ensure(c, c->ws[S_APSO], sizeof(ApsoState) * (size_t)A));
   if (pr.mq) {
-    CK(ensure(c->ws[S_GNEED], sizeof(float) * (size_t)A * pr.Pp));
+    CK(ensure(c, c->ws[S_GNEED], sizeof(float) * (size_t)A * pr.Pp));
     s.gneed = ws_ptr<float>(c, S_GNEED);
   }
   s.pos = ws_ptr<float>(c, S_POS);
@@ -634,7 +648,7 @@ slm_status setup_hist_plan(slm_ctx* c, const Problem& pr, const std::vector<Node
   for (int a = 0; a < (int)nodes.size(); ++a)
     if (member(a)) moved.push_back(a);
   lst.insert(lst.end(), moved.begin(), moved.end());
-  CK(ensure(c->ws[S_HLIST], sizeof(int32_t) * lst.size()));
+  CK(ensure(c, c->ws[S_HLIST], sizeof(int32_t) * lst.size()));
   CK(cudaMemcpyAsync(c->ws[S_HLIST].p, lst.data(), sizeof(int32_t) * lst.size(),
                      cudaMemcpyHostToDevice, c->stream));
   const int32_t* base = static_cast<const int32_t*>(c->ws[S_HLIST].p);
@@ -671,23 +685,23 @@ slm_status setup_bf16(slm_ctx* c, const Problem& pr, const std::vector<NodeDesc>
     b.pairs_k += (double)nodes[a].seg_len * k;
   }
   b.n_mtiles = (int)mt.size();
-  CK(ensure(c->ws[S_MTILES], sizeof(WorkTile) * mt.size()));
+  CK(ensure(c, c->ws[S_MTILES], sizeof(WorkTile) * mt.size()));
   if (!mt.empty())
     CK(cudaMemcpyAsync(c->ws[S_MTILES].p, mt.data(), sizeof(WorkTile) * mt.size(),
                        cudaMemcpyHostToDevice, c->stream));
-  CK(ensure(c->ws[S_POSB], sizeof(uint16_t) * (size_t)A * pr.Pp * pr.dp));
+  CK(ensure(c, c->ws[S_POSB], sizeof(uint16_t) * (size_t)A * pr.Pp * pr.dp));
   b.posb = ws_ptr<uint16_t>(c, S_POSB);
   CK(prepare_mma_kernels(pr));
   const int cap = mma_grid_cap(pr, c->n_sm);
   if (cap < 1) return fail(c, SLM_EUNSUPPORTED, "the tensor-core pass cannot be scheduled");
   b.grid = std::min(cap, std::max(1, b.n_mtiles));
   if (k > 0) {
-    CK(ensure(c->ws[S_SEL], sizeof(int32_t) * (size_t)A * k));
-    CK(ensure(c->ws[S_INV], sizeof(int32_t) * (size_t)A * pr.Pp));
-    CK(ensure(c->ws[S_POSK], sizeof(float) * (size_t)A * b.kp * pr.d));
-    CK(ensure(c->ws[S_Z2], sizeof(float) * (size_t)k * (size_t)(pr.Ez > 0 ? pr.Ez : 4)));
-    CK(ensure(c->ws[S_ZMM2], sizeof(int32_t) * 2 * (size_t)A * b.kp));
-    CK(ensure(c->ws[S_CUR2], sizeof(EvalRes) * (size_t)A * b.kp));
+    CK(ensure(c, c->ws[S_SEL], sizeof(int32_t) * (size_t)A * k));
+    CK(ensure(c, c->ws[S_INV], sizeof(int32_t) * (size_t)A * pr.Pp));
+    CK(ensure(c, c->ws[S_POSK], sizeof(float) * (size_t)A * b.kp * pr.d));
+    CK(ensure(c, c->ws[S_Z2], sizeof(float) * (size_t)k * (size_t)(pr.Ez > 0 ? pr.Ez : 4)));
+    CK(ensure(c, c->ws[S_ZMM2], sizeof(int32_t) * 2 * (size_t)A * b.kp));
+    CK(ensure(c, c->ws[S_CUR2], sizeof(EvalRes) * (size_t)A * b.kp));
     std::vector<int32_t> zinit(2 * (size_t)A * b.kp);
     for (size_t i = 0; i < zinit.size(); i += 2) {
       zinit[i] = INT32_MAX;
@@ -695,7 +709,7 @@ slm_status setup_bf16(slm_ctx* c, const Problem& pr, const std::vector<NodeDesc>
     }
     CK(cudaMemcpyAsync(c->ws[S_ZMM2].p, zinit.data(), sizeof(int32_t) * zinit.size(),
                        cudaMemcpyHostToDevice, c->stream));
-    CK(ensure(c->ws[S_DONE], sizeof(int32_t) * (size_t)A));
+    CK(ensure(c, c->ws[S_DONE], sizeof(int32_t) * (size_t)A));
     CK(cudaMemsetAsync(c->ws[S_DONE].p, 0, sizeof(int32_t) * (size_t)A, c->stream));
     b.sel = ws_ptr<int32_t>(c, S_SEL);
     b.inv = ws_ptr<int32_t>(c, S_INV);
@@ -792,20 +806,28 @@ std::vector<StepRun> plan_runs(const std::vector<NodeDesc>& nodes, int slices, i
   return runs;
 }
 
-// Blocked rows of the batch and the runs of a projection from them
-// (plan->on; off when there is no room for a second copy of the rows).
+// Blocked rows of the batch and the runs of a projection from them, and the
+// buffers of a folded move (plan->on; off when the device has no room for
+// one of these: the search then takes the row-major kernels). Nothing that
+// the search needs grows after this: ensure() may take the rows back.
 slm_status plan_step(slm_ctx* c, Problem& pr, const std::vector<NodeDesc>& nodes,
                      const std::vector<WorkTile>& tiles, const StepConfig& cfg, int grid,
-                     StepPlan* plan) {
-  const cudaError_t e =
-      ensure(c->ws[S_XT], sizeof(float) * (size_t)step_rows_floats(pr, (int)nodes.size()));
-  if (e == cudaErrorMemoryAllocation) {
-    (void)cudaGetLastError();
-    return SLM_OK;
-  }
-  CK(e);
+                     bool fold, StepPlan* plan) {
+  const size_t A = nodes.size(), apd = A * pr.Pp * pr.d;
   const std::vector<StepRun> runs = plan_runs(nodes, cfg.slices, grid);
-  CK(ensure(c->ws[S_RUNS], sizeof(StepRun) * runs.size()));
+  std::vector<std::pair<Slot, size_t>> room{{S_RUNS, sizeof(StepRun) * runs.size()}};
+  if (fold)
+    room.insert(room.end(), {{S_POS2, sizeof(float) * apd},
+                             {S_IC, sizeof(float) * apd},
+                             {S_S2, sizeof(float) * apd},
+                             {S_IMP, sizeof(int32_t) * 2 * A},
+                             {S_KEYS, sizeof(uint64_t) * A * pr.Pp}});
+  room.push_back({S_XT, sizeof(float) * (size_t)step_rows_floats(pr, (int)A)});
+  for (const auto& r : room) {
+    const cudaError_t e = ensure(c, c->ws[r.first], r.second);
+    if (e == cudaErrorMemoryAllocation) return SLM_OK;
+    CK(e);
+  }
   CK(cudaMemcpyAsync(c->ws[S_RUNS].p, runs.data(), sizeof(StepRun) * runs.size(),
                      cudaMemcpyHostToDevice, c->stream));
   pr.Xt = ws_ptr<float>(c, S_XT);
@@ -814,6 +836,7 @@ slm_status plan_step(slm_ctx* c, Problem& pr, const std::vector<NodeDesc>& nodes
                              ws_ptr<float>(c, S_XT), c->stream);
   }));
   plan->on = true;
+  plan->fold = fold;
   plan->runs = ws_ptr<StepRun>(c, S_RUNS);
   plan->n_runs = (int)runs.size();
   plan->cfg = cfg;
@@ -996,7 +1019,7 @@ slm_status score_batch(slm_ctx* c, const Problem& pr, const Swarm& sw_in,
 // Network work space for a batch of N samples.
 slm_status proposal_work(slm_ctx* c, int N, MlpWork* w) {
   const size_t nh = (size_t)N * kPropH, no = (size_t)N * kPropOut;
-  CK(ensure(c->ws[S_PWORK], sizeof(float) * (4 * nh + 2 * no)));
+  CK(ensure(c, c->ws[S_PWORK], sizeof(float) * (4 * nh + 2 * no)));
   float* b = ws_ptr<float>(c, S_PWORK);
   *w = MlpWork{b, b + nh, b + 2 * nh, b + 2 * nh + no, b + 2 * nh + 2 * no,
                b + 3 * nh + 2 * no};
@@ -1010,10 +1033,10 @@ slm_status batch_stats(slm_ctx* c, const Problem& pr, const std::vector<NodeDesc
   const int K = pr.lab ? pr.K : 4;
   int64_t max_len = 0;
   for (const NodeDesc& nd : nodes) max_len = std::max<int64_t>(max_len, nd.seg_len);
-  CK(ensure(c->ws[S_PSTATS], sizeof(float) * (size_t)A * kPropIn));
-  CK(ensure(c->ws[S_PYR], sizeof(int32_t) * 2 * (size_t)A));
-  CK(ensure(c->ws[S_PACC], sizeof(double) * (size_t)A * (K + 2) * pr.d));
-  CK(ensure(c->ws[S_PWK], sizeof(double) * (size_t)A * K));
+  CK(ensure(c, c->ws[S_PSTATS], sizeof(float) * (size_t)A * kPropIn));
+  CK(ensure(c, c->ws[S_PYR], sizeof(int32_t) * 2 * (size_t)A));
+  CK(ensure(c, c->ws[S_PACC], sizeof(double) * (size_t)A * (K + 2) * pr.d));
+  CK(ensure(c, c->ws[S_PWK], sizeof(double) * (size_t)A * K));
   CK(launch(c, SLM_K_PROPOSAL, 0.0, [&] {
     return launch_node_stats(pr, ws_ptr<NodeDesc>(c, S_NODES), A, max_len, K,
                              ws_ptr<int32_t>(c, S_PYR), ws_ptr<double>(c, S_PACC),
@@ -1456,7 +1479,7 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
     std::vector<int32_t> lst;
     for (int a = 0; a < A; ++a)
       if (resident[a]) lst.push_back(a);
-    CK(ensure(c->ws[S_NLIST], sizeof(int32_t) * lst.size()));
+    CK(ensure(c, c->ws[S_NLIST], sizeof(int32_t) * lst.size()));
     CK(cudaMemcpyAsync(c->ws[S_NLIST].p, lst.data(), sizeof(int32_t) * lst.size(),
                        cudaMemcpyHostToDevice, c->stream));
     const int32_t* dl = static_cast<const int32_t*>(c->ws[S_NLIST].p);
@@ -1476,6 +1499,12 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
     if (!joined) CK(cudaEventRecord(c->ev_join, st));
     c->last_node_search = S;
   }
+  // the histogram kernels' lists (the BF16 form has a warp-per-particle kernel
+  // for regression only)
+  HistPlan hp;
+  if (n_res < A && (!bp.on || (bp.fast && mse_lazy_ok(pr))) &&
+      (s = setup_hist_plan(c, pr, nodes, in, &hp)))
+    return s;
   // FP32 searches of whole batches: projected from blocked rows, the move of
   // a plain search folded in where the batch is short
   StepPlan stp;
@@ -1489,7 +1518,7 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
     if (few_config(bp.pr_k, &cfg)) {
       CK(prepare_step(cfg));
       const int grid = step_grid(cfg, c->n_sm);
-      if (grid > 0 && (s = plan_step(c, bp.pr_k, nodes, tiles, cfg, grid, &bp.step_k))) return s;
+      if (grid > 0 && (s = plan_step(c, bp.pr_k, nodes, tiles, cfg, grid, false, &bp.step_k))) return s;
     }
   }
   if (every && !bp.on) {
@@ -1548,14 +1577,8 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
       CK(prepare_step(cfg));
       grid = step_grid(cfg, c->n_sm);
     }
-    if (grid > 0 && (s = plan_step(c, pr, nodes, tiles, cfg, grid, &stp))) return s;
-    stp.fold = stp.on && sh >= 0;
+    if (grid > 0 && (s = plan_step(c, pr, nodes, tiles, cfg, grid, sh >= 0, &stp))) return s;
     if (stp.fold) {
-      const size_t apd = (size_t)A * pr.Pp * pr.d;
-      CK(ensure(c->ws[S_POS2], sizeof(float) * apd));
-      CK(ensure(c->ws[S_IC], sizeof(float) * apd));
-      CK(ensure(c->ws[S_S2], sizeof(float) * apd));
-      CK(ensure(c->ws[S_IMP], sizeof(int32_t) * 2 * (size_t)A));
       CK(cudaMemsetAsync(c->ws[S_IMP].p, 0, sizeof(int32_t) * 2 * (size_t)A, c->stream));
       stp.pos[0] = sw.pos;
       stp.pos[1] = ws_ptr<float>(c, S_POS2);
@@ -1564,7 +1587,6 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
       sw.s2 = ws_ptr<float>(c, S_S2);
       sw.co = co;
       sw.imp = ws_ptr<int32_t>(c, S_IMP);
-      CK(ensure(c->ws[S_KEYS], sizeof(uint64_t) * (size_t)A * pr.Pp));
       sw.keys = ws_ptr<uint64_t>(c, S_KEYS);
       sw.n_nodes = A;
       c->fused_searches += 1;
@@ -1574,10 +1596,6 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
     int S = batch_split(c, pr, nodes);
     slm_ctx::Tiles tl{};
     if (!bp.on && !stp.on && (s = pick_tiles(c, pr, sw, (int)tiles.size(), A, &tl))) return s;
-    HistPlan hp;
-    // (the BF16 form has a warp-per-particle kernel for regression only)
-    if ((!bp.on || (bp.fast && mse_lazy_ok(pr))) && (s = setup_hist_plan(c, pr, nodes, in, &hp)))
-      return s;
     if (bp.fast && hp.on && hp.n_large) {
       bp.S_large = fast_hist_split(pr, hp.n_large, hp.max_large, c->n_sm);
       bp.S_large_k = fast_hist_split(bp.pr_k, hp.n_large, hp.max_large, c->n_sm);
@@ -1674,7 +1692,7 @@ slm_status prescreen_search(slm_ctx* c, const slm_params* p, Problem& pr,
   const std::vector<WorkTile> tiles = plan_tiles(nodes);
   Swarm su{};
   if (slm_status s = setup_scoring(c, pu, A, nodes, tiles, &su)) return s;
-  CK(ensure(c->ws[S_FPOS], sizeof(float) * (size_t)A * pu.Pp * d));
+  CK(ensure(c, c->ws[S_FPOS], sizeof(float) * (size_t)A * pu.Pp * d));
   su.pos = ws_ptr<float>(c, S_FPOS);
   CK(launch(c, SLM_K_OTHER, 0.0,
             [&] { return launch_unit_positions(su.pos, A, pu.Pp, d, c->stream); }));
@@ -1700,11 +1718,11 @@ slm_status prescreen_search(slm_ctx* c, const slm_params* p, Problem& pr,
     std::sort(order.begin(), order.begin() + n);
     std::copy(order.begin(), order.begin() + n, feat.begin() + (size_t)a * n);
   }
-  CK(ensure(c->ws[S_FEAT], sizeof(int32_t) * feat.size()));
+  CK(ensure(c, c->ws[S_FEAT], sizeof(int32_t) * feat.size()));
   CK(cudaMemcpyAsync(c->ws[S_FEAT].p, feat.data(), sizeof(int32_t) * feat.size(),
                      cudaMemcpyHostToDevice, c->stream));
   const int32_t* dfeat = ws_ptr<int32_t>(c, S_FEAT);
-  CK(ensure(c->ws[W_XS], sizeof(float) * (size_t)(pr.E > 0 ? pr.E : 1) * n));
+  CK(ensure(c, c->ws[W_XS], sizeof(float) * (size_t)(pr.E > 0 ? pr.E : 1) * n));
   float* xs = ws_ptr<float>(c, W_XS);
   CK(launch(c, SLM_K_GATHER, 0.0, [&] {
     return launch_gather_cols(pr.X, d, dfeat, n, ws_ptr<WorkTile>(c, S_TILES),
@@ -1721,7 +1739,7 @@ slm_status prescreen_search(slm_ctx* c, const slm_params* p, Problem& pr,
   q.top_n = 0;
   Swarm sw;
   if (slm_status s = run_search(c, &q, ps, nodes, want_trace, &sw)) return s;
-  CK(ensure(c->ws[S_GFULL], sizeof(float) * (size_t)A * d));
+  CK(ensure(c, c->ws[S_GFULL], sizeof(float) * (size_t)A * d));
   float* gfull = ws_ptr<float>(c, S_GFULL);
   CK(launch(c, SLM_K_OTHER, 0.0,
             [&] { return launch_lift(sw.gbest, dfeat, A, n, d, gfull, c->stream); }));
@@ -1749,7 +1767,7 @@ slm_status read_status(slm_ctx* c, int32_t* out) {
 }
 
 slm_status reset_status(slm_ctx* c) {
-  CK(ensure(c->ws[S_STATUS], sizeof(int32_t)));
+  CK(ensure(c, c->ws[S_STATUS], sizeof(int32_t)));
   CK(cudaMemsetAsync(c->ws[S_STATUS].p, 0, sizeof(int32_t), c->stream));
   return SLM_OK;
 }
@@ -1851,7 +1869,7 @@ slm_status slm_swarm_uniforms(slm_ctx* c, uint64_t seed, uint32_t node_uid,
   float* dst = u;
   const bool dev = is_device_ptr(u);
   if (!dev) {
-    CK(ensure(c->ws[S_OUT], sizeof(float) * cnt));
+    CK(ensure(c, c->ws[S_OUT], sizeof(float) * cnt));
     dst = ws_ptr<float>(c, S_OUT);
   }
   CK(launch(c, SLM_K_OTHER, 0.0, [&] {
@@ -1873,7 +1891,7 @@ slm_status slm_bootstrap(slm_ctx* c, uint64_t seed, uint32_t tree_id, int64_t n,
   uint32_t* dst = w;
   const bool dev = is_device_ptr(w);
   if (!dev) {
-    CK(ensure(c->ws[S_OUT], sizeof(uint32_t) * n));
+    CK(ensure(c, c->ws[S_OUT], sizeof(uint32_t) * n));
     dst = ws_ptr<uint32_t>(c, S_OUT);
   }
   CK(launch(c, SLM_K_OTHER, 0.0,
@@ -1905,7 +1923,7 @@ slm_status prepare_node(slm_ctx* c, const slm_params* p, const float* X, int64_t
   // multiplicities are always copied: the kernels read them 16 bytes at a time
   dw = nullptr;
   if (weights && n_idx > 0) {
-    CK(ensure(c->ws[W_W], sizeof(uint32_t) * (size_t)(n_idx + 16)));
+    CK(ensure(c, c->ws[W_W], sizeof(uint32_t) * (size_t)(n_idx + 16)));
     CK(cudaMemcpyAsync(c->ws[W_W].p, weights, sizeof(uint32_t) * (size_t)n_idx,
                        cudaMemcpyDefault, c->stream));
     dw = ws_ptr<uint32_t>(c, W_W);
@@ -1913,16 +1931,16 @@ slm_status prepare_node(slm_ctx* c, const slm_params* p, const float* X, int64_t
   if (sample_idx) {
     if ((s = stage_in(c, sample_idx, (size_t)n_idx, c->ws[W_IDX], &didx))) return s;
   } else {
-    CK(ensure(c->ws[W_IDX], sizeof(int32_t) * n_idx));
+    CK(ensure(c, c->ws[W_IDX], sizeof(int32_t) * n_idx));
     CK(launch(c, SLM_K_OTHER, 0.0,
               [&] { return launch_iota(ws_ptr<int32_t>(c, W_IDX), n_idx, n_idx, 1, c->stream); }));
     didx = ws_ptr<int32_t>(c, W_IDX);
   }
   if ((s = validate_inputs(c, dlab, n, p->n_classes, sample_idx ? didx : nullptr, n_idx)))
     return s;
-  CK(ensure(c->ws[W_XL], sizeof(float) * (size_t)n_idx * d));
-  CK(ensure(c->ws[W_LABL], sizeof(int32_t) * (size_t)(n_idx + 16)));
-  CK(ensure(c->ws[W_YL], sizeof(float) * (size_t)(n_idx + 16)));
+  CK(ensure(c, c->ws[W_XL], sizeof(float) * (size_t)n_idx * d));
+  CK(ensure(c, c->ws[W_LABL], sizeof(int32_t) * (size_t)(n_idx + 16)));
+  CK(ensure(c, c->ws[W_YL], sizeof(float) * (size_t)(n_idx + 16)));
   float* Xl = ws_ptr<float>(c, W_XL);
   int32_t* ll = dlab ? ws_ptr<int32_t>(c, W_LABL) : nullptr;
   float* yl = dy ? ws_ptr<float>(c, W_YL) : nullptr;
@@ -1934,7 +1952,7 @@ slm_status prepare_node(slm_ctx* c, const slm_params* p, const float* X, int64_t
     // the node's rows once more, as bfloat16 tensor-core operands
     const int dp = round16(d);
     const int64_t nb = std::max<int64_t>(1, (n_idx + kMmaRows - 1) / kMmaRows);
-    CK(ensure(c->ws[W_XB], sizeof(uint16_t) * (size_t)nb * kMmaRows * dp));
+    CK(ensure(c, c->ws[W_XB], sizeof(uint16_t) * (size_t)nb * kMmaRows * dp));
     uint16_t* xb = ws_ptr<uint16_t>(c, W_XB);
     CK(launch(c, SLM_K_GATHER, 0.0, [&] {
       return launch_to_mma_layout(Xl, n_idx, d, dp, kMmaRows, nb, xb, c->stream);
@@ -1989,7 +2007,7 @@ slm_status slm_evaluate_swarm(slm_ctx* c, const slm_params* p, const float* X,
   const std::vector<WorkTile> tiles = plan_tiles(nodes);
   Swarm sw{};
   if (slm_status s = setup_scoring(c, pr, 1, nodes, tiles, &sw)) return s;
-  CK(ensure(c->ws[S_POS], sizeof(float) * pr.Pp * d));
+  CK(ensure(c, c->ws[S_POS], sizeof(float) * pr.Pp * d));
   CK(cudaMemsetAsync(c->ws[S_POS].p, 0, sizeof(float) * pr.Pp * d, c->stream));
   CK(cudaMemcpyAsync(c->ws[S_POS].p, positions, sizeof(float) * n_pos * d,
                      cudaMemcpyDefault, c->stream));
@@ -2007,7 +2025,7 @@ slm_status slm_evaluate_swarm(slm_ctx* c, const slm_params* p, const float* X,
   int32_t* dbins = bins_out;
   const bool bins_dev = bins_out && is_device_ptr(bins_out);
   if (bins_out && !bins_dev) {
-    CK(ensure(c->ws[W_BINS], sizeof(int32_t) * (size_t)n_pos * n_idx));
+    CK(ensure(c, c->ws[W_BINS], sizeof(int32_t) * (size_t)n_pos * n_idx));
     dbins = ws_ptr<int32_t>(c, W_BINS);
   }
   if (slm_status s = score_batch(c, pr, sw, nodes, (int)tiles.size(),
@@ -2136,7 +2154,7 @@ slm_status slm_prob_search(slm_ctx* c, const slm_params* p, const slm_prob* pp, 
   const std::vector<WorkTile> tiles = plan_tiles(nodes);
   Swarm su{};
   if (slm_status s = setup_scoring(c, pr, 1, nodes, tiles, &su)) return s;
-  CK(ensure(c->ws[S_FPOS], sizeof(float) * (size_t)pr.Pp * d));
+  CK(ensure(c, c->ws[S_FPOS], sizeof(float) * (size_t)pr.Pp * d));
   su.pos = ws_ptr<float>(c, S_FPOS);
   // scores rows 0 .. P - 1 of su.pos into su.cur
   auto score = [&](int P) -> slm_status {
@@ -2180,21 +2198,21 @@ slm_status slm_prob_search(slm_ctx* c, const slm_params* p, const slm_prob* pp, 
     m[r] = (int32_t)std::floor(pp->alpha0 * std::exp(-pp->alpha * (double)(r + 1)));
     rf[r] = rank_feat[r];
   }
-  CK(ensure(c->ws[S_PRTAB], tab_bytes));
+  CK(ensure(c, c->ws[S_PRTAB], tab_bytes));
   CK(cudaMemcpyAsync(c->ws[S_PRTAB].p, tab.data(), tab_bytes, cudaMemcpyHostToDevice,
                      c->stream));
   const double* dw = ws_ptr<double>(c, S_PRTAB);
   const int32_t* dm = reinterpret_cast<const int32_t*>(dw + d);
   const int32_t* drf = dm + d;
   const int nb = (I + pp->batch - 1) / pp->batch;
-  CK(ensure(c->ws[S_PRALL], sizeof(float) * (size_t)I * d));
-  CK(ensure(c->ws[S_PRSC], sizeof(EvalRes) * (size_t)I));
+  CK(ensure(c, c->ws[S_PRALL], sizeof(float) * (size_t)I * d));
+  CK(ensure(c, c->ws[S_PRSC], sizeof(EvalRes) * (size_t)I));
   // best score, its index, trace[nb], best vector[d], kept[q], n_kept
   const size_t off_idx = 64, off_trace = 128, off_pos = off_trace + round_up(8 * (size_t)nb, 64),
                off_kept = off_pos + round_up(4 * (size_t)d, 64),
                off_nk = off_kept + round_up(4 * (size_t)std::max(pp->q, 1), 64);
-  CK(ensure(c->ws[S_PRBEST], off_nk + 64));
-  CK(ensure(c->ws[S_PRUNE], (size_t)I));
+  CK(ensure(c, c->ws[S_PRBEST], off_nk + 64));
+  CK(ensure(c, c->ws[S_PRUNE], (size_t)I));
   char* bb = static_cast<char*>(c->ws[S_PRBEST].p);
   EvalRes* dbest = reinterpret_cast<EvalRes*>(bb);
   int32_t* dbest_idx = reinterpret_cast<int32_t*>(bb + off_idx);
@@ -2265,7 +2283,7 @@ slm_status slm_prob_search(slm_ctx* c, const slm_params* p, const slm_prob* pp, 
 static slm_status forest_alloc_trees(slm_ctx* c, slm_forest* f) {
   const size_t TH = (size_t)f->n_trees * f->H;
   const size_t bytes = TH * (4 + 4 * (size_t)f->d + 4 + 4 + 4 + 4 + 8 + 8 + 8 + 8 + 8) + 256;
-  CK(ensure(f->tree_mem, bytes));
+  CK(ensure(c, f->tree_mem, bytes));
   unsigned char* p = static_cast<unsigned char*>(f->tree_mem.p);
   auto take = [&](size_t sz) {
     unsigned char* r = p;
@@ -2377,7 +2395,7 @@ slm_status forest_begin_impl(slm_ctx* c, const slm_params* p, const float* X, in
   if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, c->device) != cudaSuccess) l2 = 0;
   const size_t xbytes = sizeof(float) * (size_t)n * d;
   if (!bf16 && p->n_trees > 1 && xbytes <= (size_t)l2 / 4) {
-    cudaError_t ex = ensure(f->own_X, xbytes);
+    cudaError_t ex = ensure(c, f->own_X, xbytes);
     if (!ex) ex = cudaMemcpyAsync(f->own_X.p, dX, xbytes, cudaMemcpyDeviceToDevice, c->stream);
     if (ex) return bail(cuda_fail(c, ex, "base rows"));
     f->X = static_cast<const float*>(f->own_X.p);
@@ -2388,7 +2406,7 @@ slm_status forest_begin_impl(slm_ctx* c, const slm_params* p, const float* X, in
   // root entries of every tree: sample ids (+ multiplicities) in lidx[1] / lw[1]
   int64_t E = 0, ecap = 0;
   const size_t cap = (size_t)n * f->n_trees;
-  if ((e = ensure(f->lidx[1], 4 * cap))) return bail(cuda_fail(c, e, "level buffers"));
+  if ((e = ensure(c, f->lidx[1], 4 * cap))) return bail(cuda_fail(c, e, "level buffers"));
   if (f->weighted) {
     DevBuf wall, offs, cnts;
     auto cleanup = [&]() {
@@ -2396,8 +2414,8 @@ slm_status forest_begin_impl(slm_ctx* c, const slm_params* p, const float* X, in
       release(offs);
       release(cnts);
     };
-    if ((e = ensure(f->lw[1], 4 * cap)) || (e = ensure(wall, 4 * cap)) ||
-        (e = ensure(offs, 8 * (size_t)f->n_trees)) || (e = ensure(cnts, 4 * (size_t)f->n_trees))) {
+    if ((e = ensure(c, f->lw[1], 4 * cap)) || (e = ensure(c, wall, 4 * cap)) ||
+        (e = ensure(c, offs, 8 * (size_t)f->n_trees)) || (e = ensure(c, cnts, 4 * (size_t)f->n_trees))) {
       cleanup();
       return bail(cuda_fail(c, e, "bootstrap buffers"));
     }
@@ -2430,7 +2448,7 @@ slm_status forest_begin_impl(slm_ctx* c, const slm_params* p, const float* X, in
     cleanup();
     for (int t = 0; t < f->n_trees; ++t) E += round_up(cnt[t], f->align);
     ecap = level_capacity(E, f->n_trees, p->max_depth, f->align, p->min_leaf, true);
-    if ((e = ensure(f->lidx[0], 4 * (size_t)ecap)) || (e = ensure(f->lw[0], 4 * (size_t)ecap)) ||
+    if ((e = ensure(c, f->lidx[0], 4 * (size_t)ecap)) || (e = ensure(c, f->lw[0], 4 * (size_t)ecap)) ||
         (e = cudaMemsetAsync(f->lidx[0].p, 0, 4 * (size_t)ecap, c->stream)) ||
         (e = cudaMemsetAsync(f->lw[0].p, 0, 4 * (size_t)ecap, c->stream)))
       return bail(cuda_fail(c, e, "level buffers"));
@@ -2450,7 +2468,7 @@ slm_status forest_begin_impl(slm_ctx* c, const slm_params* p, const float* X, in
     const int64_t n4 = round_up(n, f->align);
     E = n4 * f->n_trees;
     ecap = level_capacity(E, f->n_trees, p->max_depth, f->align, p->min_leaf, false);
-    if ((e = ensure(f->lidx[0], 4 * (size_t)ecap)) ||
+    if ((e = ensure(c, f->lidx[0], 4 * (size_t)ecap)) ||
         (e = cudaMemsetAsync(f->lidx[0].p, 0, 4 * (size_t)ecap, c->stream)))
       return bail(cuda_fail(c, e, "level buffers"));
     c->launches += 1;
@@ -2462,11 +2480,11 @@ slm_status forest_begin_impl(slm_ctx* c, const slm_params* p, const float* X, in
   // level-resident arrays; every node segment starts at a multiple of 4
   // entries (16 bytes), with room for the padding of a full level
   for (int i = 0; i < 2; ++i) {
-    if ((e = ensure(f->lX[i], sizeof(float) * (size_t)ecap * d)) ||
-        (e = ensure(f->lidx[i], sizeof(int32_t) * (size_t)ecap)) ||
-        (dlab && (e = ensure(f->lab[i], sizeof(int32_t) * (size_t)ecap))) ||
-        (dy && (e = ensure(f->ly[i], sizeof(float) * (size_t)ecap))) ||
-        (f->weighted && (e = ensure(f->lw[i], sizeof(uint32_t) * (size_t)ecap))))
+    if ((e = ensure(c, f->lX[i], sizeof(float) * (size_t)ecap * d)) ||
+        (e = ensure(c, f->lidx[i], sizeof(int32_t) * (size_t)ecap)) ||
+        (dlab && (e = ensure(c, f->lab[i], sizeof(int32_t) * (size_t)ecap))) ||
+        (dy && (e = ensure(c, f->ly[i], sizeof(float) * (size_t)ecap))) ||
+        (f->weighted && (e = ensure(c, f->lw[i], sizeof(uint32_t) * (size_t)ecap))))
       return bail(cuda_fail(c, e, "level buffers"));
   }
   for (int i = 0; i < 2; ++i) {  // padding entries hold defined values
@@ -2476,8 +2494,8 @@ slm_status forest_begin_impl(slm_ctx* c, const slm_params* p, const float* X, in
          (e = cudaMemsetAsync(f->lw[i].p, 0, sizeof(uint32_t) * (size_t)ecap, c->stream))))
       return bail(cuda_fail(c, e, "level buffers"));
   }
-  if ((e = ensure(f->side, (size_t)ecap))) return bail(cuda_fail(c, e, "level buffers"));
-  if (bf16 && (e = ensure(f->lXb, sizeof(uint16_t) * (size_t)round_up(ecap, kMmaRows) *
+  if ((e = ensure(c, f->side, (size_t)ecap))) return bail(cuda_fail(c, e, "level buffers"));
+  if (bf16 && (e = ensure(c, f->lXb, sizeof(uint16_t) * (size_t)round_up(ecap, kMmaRows) *
                                       round16(d))))
     return bail(cuda_fail(c, e, "level buffers"));
   c->launches += 1;
@@ -2536,15 +2554,15 @@ slm_status slm_grow_level(slm_ctx* c, slm_forest* f, int32_t* n_split_out) {
   }
   ltile0[L] = (int32_t)ltiles.size();
   const int n_lt = (int)ltiles.size();
-  CK(ensure(c->ws[S_GLVLNODES], sizeof(LevelNode) * L));
-  CK(ensure(c->ws[S_GLVLSPLIT], sizeof(int32_t) * L));
-  CK(ensure(c->ws[S_GLVLCLS], sizeof(unsigned long long) * (size_t)L * K));
-  CK(ensure(c->ws[S_GLVLPAR], sizeof(double) * 2 * (size_t)L));
-  CK(ensure(c->ws[S_GLTILES], sizeof(WorkTile) * n_lt));
-  CK(ensure(c->ws[S_GLTILE0], sizeof(int32_t) * (L + 1)));
-  CK(ensure(c->ws[S_GACCW], sizeof(unsigned long long) * L));
-  CK(ensure(c->ws[S_GACCY], sizeof(int32_t) * 2 * L));
-  CK(ensure(c->ws[S_GTILESUM], sizeof(double) * 2 * (size_t)n_lt));
+  CK(ensure(c, c->ws[S_GLVLNODES], sizeof(LevelNode) * L));
+  CK(ensure(c, c->ws[S_GLVLSPLIT], sizeof(int32_t) * L));
+  CK(ensure(c, c->ws[S_GLVLCLS], sizeof(unsigned long long) * (size_t)L * K));
+  CK(ensure(c, c->ws[S_GLVLPAR], sizeof(double) * 2 * (size_t)L));
+  CK(ensure(c, c->ws[S_GLTILES], sizeof(WorkTile) * n_lt));
+  CK(ensure(c, c->ws[S_GLTILE0], sizeof(int32_t) * (L + 1)));
+  CK(ensure(c, c->ws[S_GACCW], sizeof(unsigned long long) * L));
+  CK(ensure(c, c->ws[S_GACCY], sizeof(int32_t) * 2 * L));
+  CK(ensure(c, c->ws[S_GTILESUM], sizeof(double) * 2 * (size_t)n_lt));
   CK(cudaMemcpyAsync(c->ws[S_GLVLNODES].p, f->level.data(), sizeof(LevelNode) * L,
                      cudaMemcpyHostToDevice, c->stream));
   if (n_lt)
@@ -2622,14 +2640,14 @@ slm_status slm_grow_level(slm_ctx* c, slm_forest* f, int32_t* n_split_out) {
   }
 
   // 3. partition on gB (per tile), zero-gain test and tree fields (per node)
-  CK(ensure(c->ws[S_GSMAP], sizeof(int32_t) * A));
-  CK(ensure(c->ws[S_GOUT3], sizeof(int32_t) * 3 * A));
-  CK(ensure(c->ws[S_GDST], sizeof(int32_t) * 2 * A));
-  CK(ensure(c->ws[S_GSTILE0], sizeof(int32_t) * (A + 1)));
-  CK(ensure(c->ws[S_GTILELEFT], sizeof(int32_t) * (size_t)n_st));
-  CK(ensure(c->ws[S_GTILEBASE], sizeof(int32_t) * (size_t)n_st));
-  CK(ensure(c->ws[S_GPLK], sizeof(unsigned long long) * (size_t)A * K));
-  CK(ensure(c->ws[S_GPWL], sizeof(unsigned long long) * A));
+  CK(ensure(c, c->ws[S_GSMAP], sizeof(int32_t) * A));
+  CK(ensure(c, c->ws[S_GOUT3], sizeof(int32_t) * 3 * A));
+  CK(ensure(c, c->ws[S_GDST], sizeof(int32_t) * 2 * A));
+  CK(ensure(c, c->ws[S_GSTILE0], sizeof(int32_t) * (A + 1)));
+  CK(ensure(c, c->ws[S_GTILELEFT], sizeof(int32_t) * (size_t)n_st));
+  CK(ensure(c, c->ws[S_GTILEBASE], sizeof(int32_t) * (size_t)n_st));
+  CK(ensure(c, c->ws[S_GPLK], sizeof(unsigned long long) * (size_t)A * K));
+  CK(ensure(c, c->ws[S_GPWL], sizeof(unsigned long long) * A));
   CK(cudaMemcpyAsync(c->ws[S_GSMAP].p, smap.data(), sizeof(int32_t) * A, cudaMemcpyHostToDevice,
                      c->stream));
   CK(cudaMemcpyAsync(c->ws[S_GSTILE0].p, stile0.data(), sizeof(int32_t) * (A + 1),
@@ -2641,7 +2659,7 @@ slm_status slm_grow_level(slm_ctx* c, slm_forest* f, int32_t* n_split_out) {
   // every searched node's tiles (the search uploads only the tiles of the
   // nodes its per-iteration kernels project)
   const std::vector<WorkTile> ptiles = plan_tiles(snodes);
-  CK(ensure(c->ws[S_TILES], sizeof(WorkTile) * ptiles.size()));
+  CK(ensure(c, c->ws[S_TILES], sizeof(WorkTile) * ptiles.size()));
   if (!ptiles.empty())
     CK(cudaMemcpyAsync(c->ws[S_TILES].p, ptiles.data(), sizeof(WorkTile) * ptiles.size(),
                        cudaMemcpyHostToDevice, c->stream));
@@ -2784,7 +2802,7 @@ slm_status slm_predict(slm_ctx* c, const slm_forest* f, const float* X, int64_t 
   size_t off_v = ((hc ? 4 * (size_t)n : 0) + 15) & ~size_t(15);
   size_t off_l = (off_v + (hv ? 8 * (size_t)n : 0) + 15) & ~size_t(15);
   size_t total = off_l + (hl ? 4 * (size_t)n * f->n_trees : 0);
-  CK(ensure(c->ws[S_OUT], total));
+  CK(ensure(c, c->ws[S_OUT], total));
   unsigned char* base = static_cast<unsigned char*>(c->ws[S_OUT].p);
   if (hc) dc = reinterpret_cast<int32_t*>(base);
   if (hv) dv = reinterpret_cast<double*>(base + off_v);
@@ -2877,7 +2895,7 @@ slm_status own_copy(slm_ctx* c, const T* src, size_t count, DevBuf& buf, const T
     *out = src;
     return SLM_OK;
   }
-  CK(ensure(buf, sizeof(T) * count));
+  CK(ensure(c, buf, sizeof(T) * count));
   CK(cudaMemcpyAsync(buf.p, src, sizeof(T) * count, cudaMemcpyHostToDevice, c->stream));
   *out = static_cast<const T*>(buf.p);
   return SLM_OK;
@@ -2914,12 +2932,12 @@ slm_status slm_train_boost(slm_ctx* c, const slm_params* p, const float* X, int6
     if (slm_status s = own_copy(c, labels, (size_t)n, w.lab, &dl)) return s;
     if (slm_status s = validate_inputs(c, dl, n, K, nullptr, 0)) return s;
   }
-  CK(ensure(w.F, sizeof(float) * (size_t)n * K));
-  CK(ensure(w.r, sizeof(float) * (size_t)n * K));
-  CK(ensure(w.v, sizeof(double) * (size_t)n));
+  CK(ensure(c, w.F, sizeof(float) * (size_t)n * K));
+  CK(ensure(c, w.r, sizeof(float) * (size_t)n * K));
+  CK(ensure(c, w.v, sizeof(double) * (size_t)n));
   // (32 doubles more: the sums' scratch)
-  CK(ensure(w.loss, sizeof(double) * ((size_t)n_rounds + 32)));
-  CK(ensure(w.base, sizeof(float)));
+  CK(ensure(c, w.loss, sizeof(double) * ((size_t)n_rounds + 32)));
+  CK(ensure(c, w.base, sizeof(float)));
   float* F = static_cast<float*>(w.F.p);
   float* r = static_cast<float*>(w.r.p);
   double* v = static_cast<double*>(w.v.p);
@@ -3015,7 +3033,7 @@ slm_status slm_boost_predict(slm_ctx* c, const slm_boost* b, const float* X, int
   const int K = b->K;
   const size_t off_f = (sizeof(double) * (size_t)n + 15) & ~size_t(15);
   const size_t off_c = (off_f + sizeof(float) * (size_t)n * K + 15) & ~size_t(15);
-  CK(ensure(c->ws[S_OUT], off_c + sizeof(int32_t) * (size_t)n));
+  CK(ensure(c, c->ws[S_OUT], off_c + sizeof(int32_t) * (size_t)n));
   unsigned char* base = static_cast<unsigned char*>(c->ws[S_OUT].p);
   double* v = reinterpret_cast<double*>(base);
   float* F = value_out && is_device_ptr(value_out) ? value_out
@@ -3097,7 +3115,7 @@ slm_status slm_proposal_create(slm_ctx* c, uint64_t seed, slm_proposal** out) {
   pp->device = c->device;
   // params | grads | Adam m | Adam v (FP32), then the bfloat16 weight copies
   const size_t bytes = sizeof(float) * 4 * kNParams + 2 * (kNW1 + kNW2 + kNW3) + 256;
-  cudaError_t e = ensure(pp->mem, bytes);
+  cudaError_t e = ensure(c, pp->mem, bytes);
   if (e) {
     delete pp;
     return cuda_fail(c, e, "proposal memory");
@@ -3208,7 +3226,7 @@ slm_status slm_proposal_loss_grad(slm_ctx* c, const slm_proposal* pp, const floa
     return s;
   MlpWork w;
   if ((s = proposal_work(c, n, &w))) return s;
-  CK(ensure(c->ws[S_PLOSS], 2 * sizeof(double)));
+  CK(ensure(c, c->ws[S_PLOSS], 2 * sizeof(double)));
   double* dl = ws_ptr<double>(c, S_PLOSS);
   CK(launch(c, SLM_K_PROPOSAL, 0.0, [&] {
     return launch_mlp_loss_grad(pp->m, ds, dd, dt, n, w, pp->g, dl, c->stream);
@@ -3243,11 +3261,11 @@ slm_status slm_proposal_train(slm_ctx* c, slm_proposal* pp, const float* stats,
   const int b = std::min(batch, n);
   MlpWork w;
   if ((s = proposal_work(c, b, &w))) return s;
-  CK(ensure(c->ws[W_PIDX], sizeof(int32_t) * (size_t)n));
-  CK(ensure(c->ws[W_PBS], sizeof(float) * (size_t)b * kPropIn));
-  CK(ensure(c->ws[W_PBD], sizeof(int32_t) * (size_t)b));
-  CK(ensure(c->ws[W_PBT], sizeof(float) * (size_t)b * kPropD));
-  CK(ensure(c->ws[S_PLOSS], 2 * sizeof(double)));
+  CK(ensure(c, c->ws[W_PIDX], sizeof(int32_t) * (size_t)n));
+  CK(ensure(c, c->ws[W_PBS], sizeof(float) * (size_t)b * kPropIn));
+  CK(ensure(c, c->ws[W_PBD], sizeof(int32_t) * (size_t)b));
+  CK(ensure(c, c->ws[W_PBT], sizeof(float) * (size_t)b * kPropD));
+  CK(ensure(c, c->ws[S_PLOSS], 2 * sizeof(double)));
   double* dl = ws_ptr<double>(c, S_PLOSS);
   int32_t* didx = ws_ptr<int32_t>(c, W_PIDX);
   float* bs = ws_ptr<float>(c, W_PBS);
@@ -3304,7 +3322,7 @@ slm_status slm_swarm_seed(slm_ctx* c, uint64_t seed, uint32_t node_uid, int32_t 
   float* dp = pos;
   const bool dev = is_device_ptr(pos);
   if (!dev) {
-    CK(ensure(c->ws[W_PPOS], sizeof(float) * (size_t)P * d));
+    CK(ensure(c, c->ws[W_PPOS], sizeof(float) * (size_t)P * d));
     dp = ws_ptr<float>(c, W_PPOS);
   }
   CK(launch(c, SLM_K_PROPOSAL, 0.0, [&] {
@@ -3336,7 +3354,7 @@ slm_status slm_node_stats(slm_ctx* c, const float* X, int64_t n, int32_t d,
   if (slm_status s = prepare_node(c, &p, X, n, d, labels, y, sample_idx, weights, n_idx, 1, &pr))
     return s;
   const std::vector<NodeDesc> nodes{NodeDesc{0, (int32_t)n_idx, 0u, -1}};
-  CK(ensure(c->ws[S_NODES], sizeof(NodeDesc)));
+  CK(ensure(c, c->ws[S_NODES], sizeof(NodeDesc)));
   CK(cudaMemcpyAsync(c->ws[S_NODES].p, nodes.data(), sizeof(NodeDesc), cudaMemcpyHostToDevice,
                      c->stream));
   float* ds = nullptr;

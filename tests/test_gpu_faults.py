@@ -6,6 +6,9 @@
 * an injected allocation failure at several points of a search and of a
   tree: SLM_ENOMEM, the context stays usable, and repeated failures do not
   grow the device memory in use;
+* a search's blocked copy of its rows, and the buffers of a folded move, are
+  optional: without room for one of them the search takes the row-major
+  kernels with the same result, and a later call that needs the room gets it;
 * batched == unbatched: the root level of a bagged forest (every tree's root
   in one launch) gives each root the result of its own node search with the
   same node id, bootstrap multiplicities and samples; so do the two nodes of
@@ -87,6 +90,71 @@ def test_allocation_failure_returns_enomem_and_context_recovers():
             used = _used_bytes()
         else:  # closed contexts give their memory back
             assert _used_bytes() <= used + (64 << 20)
+
+
+def _refused_growths(run, fused, want, most):
+    """How many of the first `most` growths of a fresh context's work buffers
+    end `run` with SLM_ENOMEM when they fail; the others leave its result."""
+    from paper_2208_07023_gb300 import binding as S
+    n = 0
+    for k in range(1, most):
+        c = context()
+        try:
+            c.set_fused_step(fused)
+            c.test_hooks(-1, k)
+            try:
+                got = run(c)
+            except S.SlmError as e:
+                assert e.status == S.SLM_ENOMEM
+                n += 1
+            else:
+                for key in want:
+                    assert np.array_equal(want[key], got[key]), (k, key)
+        finally:
+            c.test_hooks(-1, 0)
+            c.close()
+    return n
+
+
+@pytest.mark.parametrize("crit,form", [("gini", "folded"), ("gini", "wide"), ("mse", "folded"),
+                                       ("mse", "bf16")])
+def test_blocked_rows_are_optional(crit, form):
+    """folded, unfolded (a swarm of 72) and for the BF16 form's re-scores."""
+    from paper_2208_07023_gb300 import binding as S
+    wl = W.gmm(900, 12, 4, seed=4) if crit == "gini" else W.tanh_regression(900, 12, seed=4)
+    p = S.make_params(crit, 4, n_particles=72 if form == "wide" else 32, n_iters=3, n_bins=32,
+                      min_leaf=5, seed=3, topk=4,
+                      proj=S.SLM_PROJ_BF16_TOPK if form == "bf16" else S.SLM_PROJ_FP32)
+
+    def run(c):
+        return c.node_split(p, wl.X, labels=wl.labels, y=wl.y, node_uid=2, want_trace=True)
+
+    c = context()
+    want = run(c)
+    c.close()
+    assert _refused_growths(run, True, want, 48) <= _refused_growths(run, False, want, 48)
+
+
+def test_blocked_rows_give_way_to_other_buffers():
+    from paper_2208_07023_gb300 import binding as S
+    small, large = W.gmm(2000, 8, 4, seed=4), W.gmm(9000, 20, 4, seed=5)
+    p = gpu_params(S, "gini", 4, 32, 3, 64, min_leaf=5, seed=2)
+
+    def split(c, wl):
+        return c.node_split(p, wl.X, labels=wl.labels, node_uid=1, want_trace=True)
+
+    c = context()
+    try:
+        split(c, small)  # leaves its copy with the context
+        c.test_hooks(-1, 1)  # the next growth finds no room at first
+        got = split(c, large)
+        c.test_hooks(-1, 0)
+        want = split(context(), large)
+        for key in want:
+            assert np.array_equal(want[key], got[key]), key
+    finally:
+        c.test_hooks(-1, 0)
+        c.close()
 
 
 def _members(leaf, h):
