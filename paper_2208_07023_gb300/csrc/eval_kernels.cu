@@ -2260,7 +2260,7 @@ __global__ void __launch_bounds__(kTS)
     int eb = 0;
     s_f1 = ldexp(1.0, s);
     s_f2 = ldexp(1.0, 2 * s - t);
-    if (D > 0.0) frexp(D * (1.0 + 0x1p-40) * s_f1, &eb);
+    if (D > 0.0 && isfinite(D)) frexp(D * (1.0 + 0x1p-40) * s_f1, &eb);
     const int qs = eb > 28 ? eb - 28 : 0;
     s_c = c;
     s_qs = qs;
@@ -2306,6 +2306,7 @@ __global__ void __launch_bounds__(kTS)
 // Per node: the constants of the rounded scores (MseNode) from its sums; W
 // its entries.
 __global__ void k_mse_nodes(int A, const unsigned long long* __restrict__ acc_w,
+                            const int32_t* __restrict__ acc_y,
                             const double* __restrict__ mscale, MseNode* mnode) {
   const int a = blockIdx.x * blockDim.x + threadIdx.x;
   if (a >= A) return;
@@ -2314,9 +2315,14 @@ __global__ void k_mse_nodes(int A, const unsigned long long* __restrict__ acc_w,
   const double sf = (double)m.S * f1, unit = m.inv;
   m.base = n > 0.0 ? (double)m.Q * f2 - sf * sf / n : 0.0;
   m.inv = n > 0.0 && unit > 0.0 ? 1.0 / (n * unit * unit) : 0.0;
-  m.flat = m.S == 0 && m.Q == 0;
-  // targets that are not finite, or scales out of range: score every edge
-  m.full = !isfinite(m.base) || !isfinite(m.inv) || !(m.inv > 0.0);
+  // targets that are not finite (an infinity or a not-a-number is the lowest
+  // or the highest of the ordered range; the moments they give are defined
+  // integers that the rounded targets do not bound), or scales out of range:
+  // score every edge
+  const bool finite = n == 0.0 || (isfinite(ord2f(acc_y[2 * a])) &&
+                                   isfinite(ord2f(acc_y[2 * a + 1])));
+  m.full = !finite || !isfinite(m.base) || !isfinite(m.inv) || !(m.inv > 0.0);
+  m.flat = !m.full && m.S == 0 && m.Q == 0;
   mnode[a] = m;
 }
 
@@ -2333,7 +2339,7 @@ cudaError_t launch_mse_moments(const Problem& pr, const WorkTile* tiles, int n_t
   if (n_tiles > 0) {
     k_mse_range<<<n_tiles, kTS, 0, st>>>(pr, tiles, acc_w, acc_y);
     k_mse_moments<<<n_tiles, kTS, 0, st>>>(pr, tiles, acc_w, acc_y, m1, m2, mscale, mq, mnode);
-    if (mnode) k_mse_nodes<<<(A + 255) / 256, 256, 0, st>>>(A, acc_w, mscale, mnode);
+    if (mnode) k_mse_nodes<<<(A + 255) / 256, 256, 0, st>>>(A, acc_w, acc_y, mscale, mnode);
   }
   return cudaGetLastError();
 }

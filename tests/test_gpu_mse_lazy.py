@@ -3,8 +3,8 @@ of the staged-copy kernel, bit for bit: an edge's rounded interval may only
 rule it out, and every edge left is scored exactly. Sizes at the edges of the
 kernels: the largest warp node (2,048 entries) and the smallest cluster node,
 slices around the switch from 8 to 32 copies per bin, the largest slice of a
-single CTA, bins per lane of every width, and targets that leave many edges
-(two values, one value, one far outlier)."""
+single CTA, bins per lane of every width, targets that leave many edges
+(two values, one value, one far outlier), and targets that are not finite."""
 import numpy as np
 import pytest
 
@@ -34,7 +34,20 @@ def _targets(kind, wl):
         y[len(y) // 2] = 3e6
     if kind == "offset":
         y = (y * np.float32(1e-3) + np.float32(500)).astype(np.float32)
+    if kind in ("inf", "-inf", "nan", "infs"):
+        y[len(y) // 3] = {"-inf": -np.inf, "nan": np.nan}.get(kind, np.inf)
+    if kind == "infs":
+        y[:len(y) // 2:3] = -np.inf
     return y
+
+
+def _same_search(a, b, p, X, y):
+    ra = a.node_split(p, X, y=y, node_uid=8, want_trace=True)
+    rb = b.node_split(p, X, y=y, node_uid=8, want_trace=True)
+    assert np.array_equal(ra["trace"], rb["trace"], equal_nan=True)
+    assert np.array_equal(ra["gbest"].view(np.uint32), rb["gbest"].view(np.uint32))
+    for k in ("valid", "bin", "loss", "n_left", "n_right", "particle", "iter_of_best"):
+        assert ra[k] == rb[k] or (k == "loss" and np.isnan(ra[k]) and np.isnan(rb[k])), k
 
 
 @pytest.mark.parametrize("n,B,min_leaf,kind", [
@@ -53,12 +66,21 @@ def test_search_identical_to_the_exact_histogram(ctxs, n, B, min_leaf, kind, war
     wl = W.tanh_regression(n, 6, seed=n % 83)
     y = _targets(kind, wl)
     p = gpu_params(S, "mse", 0, 19, 9, B, min_leaf=min_leaf, seed=3)
-    ra = a.node_split(p, wl.X, y=y, node_uid=8, want_trace=True)
-    rb = b.node_split(p, wl.X, y=y, node_uid=8, want_trace=True)
-    assert np.array_equal(ra["trace"], rb["trace"])
-    assert np.array_equal(ra["gbest"].view(np.uint32), rb["gbest"].view(np.uint32))
-    for k in ("valid", "bin", "loss", "n_left", "n_right", "particle", "iter_of_best"):
-        assert ra[k] == rb[k], k
+    _same_search(a, b, p, wl.X, y)
+
+
+@pytest.mark.parametrize("n,B,kind", [(700, 32, "inf"), (701, 64, "nan"), (1999, 256, "infs"),
+                                      (9000, 128, "-inf"), (9001, 256, "inf"),
+                                      (20000, 200, "infs"), (20000, 200, "nan")])
+@pytest.mark.parametrize("warp", [False, True])
+def test_targets_that_are_not_finite(ctxs, n, B, kind, warp):
+    """No bound follows from them: every edge is scored."""
+    from paper_2208_07023_gb300 import binding as S
+    a, b = ctxs
+    a.set_small_nodes(4096 if warp else 0, 0)
+    wl = W.tanh_regression(n, 6, seed=n % 83)
+    p = gpu_params(S, "mse", 0, 19, 9, B, min_leaf=2, seed=3)
+    _same_search(a, b, p, wl.X, _targets(kind, wl))
 
 
 @pytest.mark.parametrize("proj,apso", [("fp32", False), ("bf16", False), ("fp32", True)])
