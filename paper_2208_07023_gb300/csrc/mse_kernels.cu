@@ -909,6 +909,25 @@ const void* mse_fn(int C) {
 
 // Copies per bin for slices of `slice` entries.
 int mse_copies_for(int64_t slice) { return slice <= kMseSliceFew ? 8 : 32; }
+// Longest slice of a node of max_len entries in S slices (which start on
+// multiples of 4).
+int64_t mse_launch_slice(int64_t max_len, int S) { return (max_len + S - 1) / S + 4; }
+
+// The fewest slices that a node's counters take, and the most CTAs of a
+// cluster (of the larger kernel, C = 32, which is asked for the most).
+int64_t mse_min_split(int64_t max_len) {
+  return std::max<int64_t>(1, (max_len + kMseSlice - 5) / (kMseSlice - 4));
+}
+int mse_max_cluster(const Problem& pr) {
+  const void* f = mse_fn(32);
+  const size_t smem = mse_hist_smem(pr, 32);
+  int n = 0;
+  if (allow_smem(f, (int)smem) || allow_cluster(f) || cluster_size(&n, f, kThreads, smem)) {
+    (void)cudaGetLastError();
+    n = 8;  // the portable size
+  }
+  return std::max(1, std::min(n, kMseMaxCluster));
+}
 
 }  // namespace
 
@@ -918,13 +937,6 @@ bool mse_lazy_ok(const Problem& pr) {
 
 int mse_warp_max() { return kMqEntries; }
 
-bool mse_lazy_fits(int64_t max_len) { return max_len <= (int64_t)kMseMaxCluster * (kMseSlice - 4); }
-
-int mse_lazy_min_split(int64_t max_len) {
-  return (int)std::min<int64_t>(kMseMaxCluster,
-                                std::max<int64_t>(1, (max_len + kMseSlice - 5) / (kMseSlice - 4)));
-}
-
 cudaError_t prepare_mse_lazy(const Problem& pr) {
   for (int C : {8, 32}) {
     if (cudaError_t e = allow_smem(mse_fn(C), (int)mse_hist_smem(pr, C))) return e;
@@ -933,21 +945,37 @@ cudaError_t prepare_mse_lazy(const Problem& pr) {
   return allow_smem((const void*)k_mse_warp, (int)mse_warp_smem(pr));
 }
 
+bool mse_lazy_fits(const Problem& pr, int64_t max_len) {
+  return mse_min_split(max_len) <= mse_max_cluster(pr);
+}
+
 int mse_lazy_split(const Problem& pr, int A, int64_t max_len, int n_sm) {
-  // as many slices as one wave of CTAs (three per SM) takes, of at least 2048
-  // entries
-  const int64_t wave = 3 * (int64_t)n_sm / ((int64_t)A * pr.P);
-  const int64_t S = std::min<int64_t>({wave, max_len / 2048, kMseMaxCluster});
-  return (int)std::max<int64_t>(S, mse_lazy_min_split(max_len));
+  // As many slices as one wave of CTAs takes, of at least 2048 entries. A wave
+  // is what fits on the SMs: three CTAs each by registers, two by shared memory
+  // from about 360 features on, with 256 bins of 32 copies (51 iterations of a
+  // node of 131,000 x 400 rows, P = 64: 9.87 ms with seven slices, a wave and a
+  // half, and 9.55 with four). First with the few copies of short slices, else
+  // with the many of long ones.
+  auto slices = [&](int C) {
+    int per_sm = 1;
+    if (occupancy(&per_sm, mse_fn(C), kThreads, mse_hist_smem(pr, C)) != cudaSuccess) {
+      (void)cudaGetLastError();
+      per_sm = 1;
+    }
+    const int64_t wave = (int64_t)per_sm * n_sm / ((int64_t)A * pr.P);
+    const int64_t S = std::min<int64_t>({wave, max_len / 2048, mse_max_cluster(pr)});
+    return (int)std::max<int64_t>(S, mse_min_split(max_len));
+  };
+  const int S = slices(8);
+  return mse_copies_for(mse_launch_slice(max_len, S)) == 8 ? S : slices(32);
 }
 
 cudaError_t launch_mse_lazy(const Problem& pr, const Swarm& sw, const NodeDesc* nodes, int A,
                             int64_t max_len, int S, int t, int do_update, cudaStream_t st,
                             const int32_t* list) {
   if (A <= 0) return cudaSuccess;
-  if (S < mse_lazy_min_split(max_len) || S > kMseMaxCluster || !mse_lazy_fits(max_len))
-    return cudaErrorInvalidValue;
-  const int C = mse_copies_for((max_len + S - 1) / S + 4);
+  if (S < mse_min_split(max_len) || S > kMseMaxCluster) return cudaErrorInvalidValue;
+  const int C = mse_copies_for(mse_launch_slice(max_len, S));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(A * S), (unsigned)pr.P, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);

@@ -848,7 +848,7 @@ slm_status plan_step(slm_ctx* c, Problem& pr, const std::vector<NodeDesc>& nodes
 // where the search has them (unweighted), else k_hist_cls / k_hist_mse.
 bool fast_hist_ok(const Problem& pr, int64_t max_len) {
   return hist_cls_ok(pr) &&
-         (mse_lazy_ok(pr) && mse_lazy_fits(max_len) ? true : hist_cls_fits(pr, max_len));
+         (mse_lazy_ok(pr) ? mse_lazy_fits(pr, max_len) : hist_cls_fits(pr, max_len));
 }
 
 cudaError_t prepare_fast_hist(const Problem& pr) {

@@ -271,11 +271,10 @@ cudaError_t launch_hist_cls(const Problem& pr, const Swarm& sw, const NodeDesc* 
 // steps and move terms as launch_hist_scan except that a score that cannot
 // improve its particle's best is recorded as invalid (mse_kernels.cu): a
 // (node, particle) per cluster of S CTAs (nodes of at most max_len entries,
-// mse_lazy_fits, S at least mse_lazy_min_split), or per warp (the nodes
+// mse_lazy_fits, S as mse_lazy_split), or per warp (the nodes
 // list[] names, of at most mse_warp_max() entries).
 bool mse_lazy_ok(const Problem& pr);
-bool mse_lazy_fits(int64_t max_len);
-int mse_lazy_min_split(int64_t max_len);
+bool mse_lazy_fits(const Problem& pr, int64_t max_len);
 int mse_lazy_split(const Problem& pr, int A, int64_t max_len, int n_sm);
 int mse_warp_max();
 cudaError_t prepare_mse_lazy(const Problem& pr);
@@ -606,14 +605,14 @@ cudaError_t launch_swarm_seed_init(const Problem& pr, const Swarm& sw, const Nod
 // Searches plan their launches again at every level; the runtime calls that
 // set a kernel's dynamic shared-memory limit or query its occupancy cost
 // microseconds each, so their results are kept: a limit is raised only when
-// a larger one is needed, an occupancy is queried once per (kernel, block,
-// shared memory) that gives a nonzero answer.
+// a larger one is needed, an occupancy and a cluster size are queried once per
+// (kernel, block, shared memory) that gives a nonzero answer.
 
 struct KernelAttrCache {
   std::mutex mu;
   std::map<std::pair<int, const void*>, int> smem;      // largest limit set
   std::map<std::pair<int, const void*>, bool> cluster;  // non-portable sizes allowed
-  std::map<std::tuple<int, const void*, int, size_t>, int> occ;
+  std::map<std::tuple<int, const void*, int, size_t>, int> occ, cluster_size;
 };
 
 inline KernelAttrCache& kernel_attr_cache() {
@@ -676,6 +675,34 @@ inline cudaError_t occupancy(int* per_sm, const void* fn, int threads, size_t sm
   if (e == cudaSuccess && *per_sm > 0) {  // (zero: perhaps a limit not yet raised)
     std::lock_guard<std::mutex> g(c.mu);
     c.occ[key] = *per_sm;
+  }
+  return e;
+}
+
+// CTAs of the largest cluster of a kernel that the device can schedule
+// (cudaOccupancyMaxPotentialClusterSize), remembered per device. Sizes above 8
+// count once allow_cluster has allowed them.
+inline cudaError_t cluster_size(int* ctas, const void* fn, int threads, size_t smem) {
+  int dev = 0;
+  if (cudaError_t e = cudaGetDevice(&dev)) return e;
+  KernelAttrCache& c = kernel_attr_cache();
+  const auto key = std::make_tuple(dev, fn, threads, smem);
+  {
+    std::lock_guard<std::mutex> g(c.mu);
+    const auto it = c.cluster_size.find(key);
+    if (it != c.cluster_size.end()) {
+      *ctas = it->second;
+      return cudaSuccess;
+    }
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(16, 1, 1);
+  cfg.blockDim = dim3((unsigned)threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  const cudaError_t e = cudaOccupancyMaxPotentialClusterSize(ctas, fn, &cfg);
+  if (e == cudaSuccess && *ctas > 0) {
+    std::lock_guard<std::mutex> g(c.mu);
+    c.cluster_size[key] = *ctas;
   }
   return e;
 }

@@ -83,6 +83,23 @@ def test_targets_that_are_not_finite(ctxs, n, B, kind, warp):
     _same_search(a, b, p, wl.X, _targets(kind, wl))
 
 
+@pytest.mark.parametrize("d,P", [(6, 64), (400, 64), (400, 19)])
+def test_slices_are_one_wave(ctxs, d, P):
+    """Rows of 400 features leave room for two CTAs per SM, not three."""
+    import torch
+    from paper_2208_07023_gb300 import binding as S
+    a, b = ctxs
+    a.set_small_nodes()
+    n = 131000
+    g = torch.Generator(device="cuda").manual_seed(d)
+    X = torch.randn(n, d, generator=g, device="cuda")
+    y = torch.tanh(X[:, 0] + X[:, 1]) + 0.1 * torch.randn(n, generator=g, device="cuda")
+    p = gpu_params(S, "mse", 0, P, 2, 256, min_leaf=5, seed=3)
+    _same_search(a, b, p, X, y)
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    assert a.tuning_stats()["last_hist_cluster"] * P <= (2 if d == 400 else 3) * n_sm
+
+
 @pytest.mark.parametrize("proj,apso", [("fp32", False), ("bf16", False), ("fp32", True)])
 def test_tree_identical_to_the_exact_histogram(ctxs, proj, apso):
     """Levels of hundreds of small nodes (a warp each), beside large ones."""
