@@ -22,6 +22,8 @@
 #include <cuda_runtime.h>
 #include <limits.h>
 
+#include <algorithm>
+
 #include "device_util.cuh"
 #include "slm_internal.cuh"
 
@@ -424,20 +426,26 @@ cudaError_t prepare_mma_kernels(const Problem& pr) {
 
 int mma_grid_cap(const Problem& pr, int n_sm) {
   // resident CTAs per SM from the kernel's own limits: shared memory (static,
-  // dynamic and the per-block reservation), tensor memory, 16 blocks
+  // dynamic and the per-block reservation), tensor memory, registers (given to
+  // a warp 256 at a time), threads. A grid above it runs a second wave with
+  // positions staged and ranges published again (100,000 x 48 rows, P = 32, 51
+  // iterations: 2.64 ms at the 8 CTAs per SM that shared and tensor memory
+  // take, 2.46 at the 4 that the registers take)
   cudaFuncAttributes fa;
-  int dev = 0, per_sm_smem = 0, reserved = 0;
+  int dev = 0, smem = 0, reserved = 0, regs = 0, threads = 0;
   if (cudaFuncGetAttributes(&fa, k_project_mma) != cudaSuccess || cudaGetDevice(&dev) ||
-      cudaDeviceGetAttribute(&per_sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) ||
-      cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev)) {
+      cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) ||
+      cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) ||
+      cudaDeviceGetAttribute(&regs, cudaDevAttrMaxRegistersPerMultiprocessor, dev) ||
+      cudaDeviceGetAttribute(&threads, cudaDevAttrMaxThreadsPerMultiProcessor, dev)) {
     cudaGetLastError();
     return 0;
   }
-  const size_t per_cta = mma_smem_bytes(pr) + fa.sharedSizeBytes + (size_t)reserved;
-  int per_sm = (int)((size_t)per_sm_smem / per_cta);
-  per_sm = per_sm < (int)(512u / (2 * mma_tmem_cols(pr.Pp))) ? per_sm
-                                                             : (int)(512u / (2 * mma_tmem_cols(pr.Pp)));
-  per_sm = per_sm < 16 ? per_sm : 16;
+  const int warp_regs = (fa.numRegs * 32 + 255) / 256 * 256;
+  const int per_sm = std::min({(int)((size_t)smem / (mma_smem_bytes(pr) + fa.sharedSizeBytes +
+                                                     (size_t)reserved)),
+                               (int)(512u / (2 * mma_tmem_cols(pr.Pp))),
+                               regs / (warp_regs * (kMmaThreads / 32)), threads / kMmaThreads});
   return per_sm * n_sm;
 }
 

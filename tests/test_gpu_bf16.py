@@ -244,6 +244,7 @@ def test_bf16_rejects_bad_topk_and_sizes(ctx):
     (128, 16, 40),    # three groups, the last partly particles
     (1000, 33, 64),   # a ragged last tile
     (1280, 64, 250),  # the widest accumulator
+    (250000, 8, 16),  # more tiles than resident CTAs, each with several
 ])
 def test_bf16_epilogue_tiles(ctx, n, d, P):
     """Whole and ragged row tiles and column groups of the tensor-core pass."""
