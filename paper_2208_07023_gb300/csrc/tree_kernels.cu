@@ -521,21 +521,31 @@ __global__ void k_validate(const int32_t* labels, int64_t n, int K, const int32_
 }
 
 // Routes rows through every tree (bin rule of scoring). A CTA takes a tile of
-// rows into shared memory; its warps are RB blocks of 32 rows x WT lanes of
-// trees: a lane walks one row down trees w, w + WT, ... of each chunk of
+// rows, mostly into shared memory; its warps are RB blocks of 32 rows x WT lanes
+// of trees: a lane walks one row down trees w, w + WT, ... of each chunk of
 // kPredTrees, its leaf ids meeting in shared memory, from which one thread per
-// row counts the votes (or adds the leaf values in tree order). With one
-// thread per row walking every tree from global memory, 100,000 rows x 32
-// through 64 trees of depth 8 took 2.40 ms, too few warps, each waiting on
-// its own row's loads; now 0.30 ms, bound by the descents' dependent loads. Features are read 16 bytes at a time (VEC) where d
-// and X's address allow.
+// row counts the votes (or adds the leaf values in tree order). Bound by the
+// descents' dependent loads (100,000 rows x 32 through 64 trees of depth 8:
+// 0.30 ms; one thread per row from global memory, with too few warps, 2.40).
+// Features are read 16 bytes at a time (VEC) where d and X's address allow.
+//
+// F words of a row and of a direction are loaded before any is used, since
+// wide rows leave few warps per SM to hide a load behind (ms for 100,000 rows,
+// depth 6, left to the compiler and now: 601 features, 4 trees 2.43 and 1.12;
+// 680, 2 trees 1.32 and 0.68; 161, 64 trees 5.52 and 3.54; only 400 features
+// with 64 trees lost, 5.91 and 6.13). Up to 128 features of 16-byte rows
+// (F = 1) there are warps enough and registers count: the loop is the
+// compiler's, and its rows' addresses are kept generic (64 features, 64 trees:
+// 1.39 ms; 1.44 through shared addresses, 1.53 two words at a time).
+// ROWS: where the rows are read. MINB: CTAs per SM that the registers allow.
+enum PredRows { kShared, kDirect, kGeneric };
 constexpr int kPredTrees = 64;
 constexpr int kPredSmem = 96 * 1024;  // rows kept in shared memory up to this
 
 __host__ __device__ inline int pred_stride(int d, bool vec) { return vec ? d + 4 : d | 1; }
 
-template <bool VEC>
-__global__ void __launch_bounds__(256)
+template <bool VEC, int F, int ROWS, int MINB>
+__global__ void __launch_bounds__(256, MINB)
     k_predict(const float* __restrict__ X, int64_t n, int d, TreeArrays tr, int n_trees, int H,
               int B, int K, int crit, int32_t* class_out, double* value_out, int32_t* leaf_out,
               int RB, int WT, int staged) {
@@ -549,7 +559,7 @@ __global__ void __launch_bounds__(256)
   const int stride = pred_stride(d, VEC);
   const int64_t r0 = (int64_t)blockIdx.x * R;
   const int nr = (int)min((int64_t)R, n - r0);
-  if (staged) {
+  if (ROWS == kShared || (ROWS == kGeneric && staged)) {
     // every word of the tile on its way at once
     const int w = VEC ? d >> 2 : d, step_r = (int)blockDim.x / w,
               step_c = (int)blockDim.x - step_r * w;
@@ -574,8 +584,54 @@ __global__ void __launch_bounds__(256)
   }
   const int rl = rb * 32 + lane;  // this lane's row of the tile
   const bool in = rl < nr;
-  const float* x = staged ? rows + rl * stride : X + (r0 + (in ? rl : 0)) * d;
+  const float* x = ROWS == kShared || (ROWS == kGeneric && staged)
+                       ? rows + rl * stride
+                       : X + (r0 + (in ? rl : 0)) * d;
   const bool tail = (int)threadIdx.x < nr;  // this thread sums up row threadIdx.x
+  // x . g as one fmaf per feature in increasing order from +0
+  auto dot = [&](const float* __restrict__ g) {
+    float acc = 0.0f;
+    if constexpr (F == 1) {
+#pragma unroll 4
+      for (int j = 0; j < d; j += 4) {
+        const float4 a = *reinterpret_cast<const float4*>(x + j);
+        const float4 b = __ldg(reinterpret_cast<const float4*>(g + j));
+        acc = fmaf(a.x, b.x, acc);
+        acc = fmaf(a.y, b.y, acc);
+        acc = fmaf(a.z, b.z, acc);
+        acc = fmaf(a.w, b.w, acc);
+      }
+    } else {
+      using T = std::conditional_t<VEC, float4, float>;
+      const T* xv = reinterpret_cast<const T*>(x);
+      const T* gv = reinterpret_cast<const T*>(g);
+      const int w = VEC ? d >> 2 : d;
+      auto ld = [&](int j) { return ROWS == kDirect ? __ldg(xv + j) : xv[j]; };
+      auto add = [&](const T& a, const T& b) {
+        if constexpr (VEC) {
+          acc = fmaf(a.x, b.x, acc);
+          acc = fmaf(a.y, b.y, acc);
+          acc = fmaf(a.z, b.z, acc);
+          acc = fmaf(a.w, b.w, acc);
+        } else {
+          acc = fmaf(a, b, acc);
+        }
+      };
+      int j = 0;
+      for (; j + F <= w; j += F) {
+        T a[F], b[F];
+#pragma unroll
+        for (int i = 0; i < F; ++i) {
+          a[i] = ld(j + i);
+          b[i] = __ldg(gv + j + i);
+        }
+#pragma unroll
+        for (int i = 0; i < F; ++i) add(a[i], b[i]);
+      }
+      for (; j < w; ++j) add(ld(j), __ldg(gv + j));
+    }
+    return acc;
+  };
   int votes[kMaxClasses];
   for (int k = 0; k < kMaxClasses; ++k) votes[k] = 0;
   double vsum = 0.0;
@@ -590,21 +646,7 @@ __global__ void __launch_bounds__(256)
           const float* g = tr.dir + slot * d;
           const float zmin = __ldg(tr.zmin + slot), inv_w = __ldg(tr.inv_w + slot);
           const int eb = __ldg(tr.bin + slot);
-          float acc = 0.0f;
-          if (VEC) {
-#pragma unroll 4
-            for (int j = 0; j < d; j += 4) {
-              const float4 a = *reinterpret_cast<const float4*>(x + j);
-              const float4 b = __ldg(reinterpret_cast<const float4*>(g + j));
-              acc = fmaf(a.x, b.x, acc);
-              acc = fmaf(a.y, b.y, acc);
-              acc = fmaf(a.z, b.z, acc);
-              acc = fmaf(a.w, b.w, acc);
-            }
-          } else {
-#pragma unroll 4
-            for (int j = 0; j < d; ++j) acc = fmaf(x[j], __ldg(g + j), acc);
-          }
+          const float acc = dot(g);
           h = bin_of(acc, zmin, inv_w, B) >= eb ? 2 * h + 2 : 2 * h + 1;
         }
         leaf[rl * ls + t] = h;
@@ -785,19 +827,23 @@ cudaError_t launch_predict(const float* X, int64_t n, int d, TreeArrays tr, int 
   while (RB > 1 && smem(RB, true) > 48 * 1024) RB /= 2;
   // few rows: smaller tiles, on more SMs
   while (RB > 1 && (n + 32 * RB - 1) / (32 * RB) < 152) RB /= 2;
-  const bool staged = smem(RB, true) <= (size_t)kPredSmem;
+  // Rows are staged while 32 of them fit. A single tree walks a row about
+  // once per level and gains little: in batches of more tiles than the SMs hold
+  // its wide rows are read where they are (100,000 rows, staged and direct: 200
+  // features 0.17 and 0.16 ms, 512 0.45 to 0.76 and 0.45, 601 2.4 and 0.75; but
+  // 128 0.12 and 0.16, 5,000 rows of 601 0.16 and 0.28).
+  const bool few = (n + 31) / 32 <= 152 * (int64_t)(227 * 1024 / smem(1, true));
+  const size_t most = few || n_trees > 1 ? (size_t)kPredSmem : (size_t)(vec ? 24 : 56) * 1024;
+  const bool staged = smem(1, true) <= most;
   const size_t sm = smem(RB, staged);
-  const void* f = vec ? (const void*)k_predict<true> : (const void*)k_predict<false>;
+  auto* f = !vec ? (staged ? k_predict<false, 8, kShared, 8> : k_predict<false, 8, kDirect, 6>)
+            : d <= 128 ? k_predict<true, 1, kGeneric, 0>
+            : staged   ? k_predict<true, 4, kShared, 5>
+                       : k_predict<true, 2, kDirect, 6>;
   if (sm > 48 * 1024)
-    if (cudaError_t e = allow_smem(f, (int)sm)) return e;
-  const unsigned grid = (unsigned)((n + 32 * RB - 1) / (32 * RB));
-  const int threads = 32 * RB * WT;
-  if (vec)
-    k_predict<true><<<grid, threads, sm, st>>>(X, n, d, tr, n_trees, H, B, K, crit, class_out,
-                                               value_out, leaf_out, RB, WT, staged);
-  else
-    k_predict<false><<<grid, threads, sm, st>>>(X, n, d, tr, n_trees, H, B, K, crit, class_out,
-                                                value_out, leaf_out, RB, WT, staged);
+    if (cudaError_t e = allow_smem((const void*)f, (int)sm)) return e;
+  f<<<(unsigned)((n + 32 * RB - 1) / (32 * RB)), 32 * RB * WT, sm, st>>>(
+      X, n, d, tr, n_trees, H, B, K, crit, class_out, value_out, leaf_out, RB, WT, staged);
   return cudaGetLastError();
 }
 

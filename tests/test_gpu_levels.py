@@ -46,10 +46,13 @@ def test_tree_matches_oracle(ctx, crit, n, d):
         assert np.allclose(g["leaf_value"][present], r.leaf_value[present], rtol=1e-12, atol=1e-12)
 
 
-@pytest.mark.parametrize("d,trees", [(5, 1), (8, 1), (54, 1), (16, 9), (260, 2)])
+@pytest.mark.parametrize("d,trees", [(5, 1), (8, 1), (54, 1), (16, 9), (260, 2), (452, 1),
+                                     (452, 3), (601, 1), (900, 1)])
 def test_prediction_does_not_depend_on_the_tile(ctx, d, trees):
     """Tiles of 32 to 256 rows (fewer rows a block where there are few),
-    staged by 4- or 16-byte copies: every row's class and leaves."""
+    staged by 4- or 16-byte copies, or (one tree in long batches from 192
+    features, or 425 whose rows are not whole 16-byte words; 900 features) read
+    where they are: every row's class and leaves."""
     from paper_2208_07023_gb300 import binding as S
     wl = W.gmm(40000, d, 4, seed=d)
     p = gpu_params(S, "gini", 4, 16, 3, 32, min_leaf=5, max_depth=5, seed=6, n_trees=trees,
