@@ -172,7 +172,7 @@ __device__ __forceinline__ float4 ld4(const __nv_bfloat16* p) {
 // output is one FP32 chain over k in increasing order, whatever the tile, so
 // both shapes give the same bits.
 // A batch of 64 has eight 64 x 64 tiles in the first layer (K = 5376), which
-// took 0.7 ms on 8 of 152 SMs; 16 x 16 tiles spread it over 128, where the
+// took 0.7 ms on eight SMs; 16 x 16 tiles spread it over 128, where the
 // chain's own latency (5376 dependent FMAs of 4 clocks: 10 us) is the floor.
 template <bool TA, bool TB, typename BT, int EPI, int T, int R, int KS>
 __global__ void __launch_bounds__((T / R) * (T / R))
@@ -618,14 +618,14 @@ __global__ void k_gather_rows(const T* __restrict__ src, int64_t cols, const int
 
 __global__ void k_acc_double(double* acc, const double* __restrict__ v) { *acc += *v; }
 
-// 64 x 64 tiles from one CTA per SM of a 152-SM GPU on, 16 x 16 below.
+// 64 x 64 tiles from one CTA per SM on, 16 x 16 below.
 template <bool TA, bool TB, typename BT, int EPI>
 cudaError_t gemm(int M, int N, int K, const float* A, int lda, const BT* B, int ldb,
                  const float* aux, float* C, int ldc, cudaStream_t st) {
   if (M <= 0 || N <= 0) return cudaSuccess;
   auto tiles = [&](int t) { return dim3((unsigned)((N + t - 1) / t), (unsigned)((M + t - 1) / t)); };
   const dim3 g = tiles(64), s = tiles(16);
-  if ((int64_t)g.x * g.y >= 152 || s.y > 65535)
+  if ((int64_t)g.x * g.y >= sm_count() || s.y > 65535)
     k_gemm<TA, TB, BT, EPI, 64, 4, 16><<<g, 256, 0, st>>>(M, N, K, A, lda, B, ldb, aux, C, ldc);
   else
     k_gemm<TA, TB, BT, EPI, 16, 1, 64><<<s, 256, 0, st>>>(M, N, K, A, lda, B, ldb, aux, C, ldc);
@@ -662,13 +662,13 @@ cudaError_t launch_node_stats(const Problem& pr, const NodeDesc* nodes, int A,
 }
 
 // A layer's forward product: few rows by k_gemm_fwd (below one 64 x 64 tile
-// per SM of a 152-SM GPU), else k_gemm.
+// per SM), else k_gemm.
 template <int EPI>
 cudaError_t gemm_fwd(int M, int N, int K, const float* A, const __nv_bfloat16* B,
                      const float* bias, float* C, cudaStream_t st) {
   const int64_t tiles = (int64_t)((N + 63) / 64) * ((M + 63) / 64);
   if (M <= 0) return cudaSuccess;
-  if (tiles >= 152) return gemm<false, false, __nv_bfloat16, EPI>(M, N, K, A, K, B, N, bias, C, N, st);
+  if (tiles >= sm_count()) return gemm<false, false, __nv_bfloat16, EPI>(M, N, K, A, K, B, N, bias, C, N, st);
   k_gemm_fwd<EPI><<<dim3((unsigned)(N / 16), (unsigned)((M + 15) / 16)), 128, 0, st>>>(
       M, N, K, A, B, bias, C);
   return cudaGetLastError();

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -618,6 +619,23 @@ struct KernelAttrCache {
 inline KernelAttrCache& kernel_attr_cache() {
   static KernelAttrCache c;
   return c;
+}
+
+// SMs of the current device (152 on a GB300), remembered per device.
+inline int sm_count() {
+  static std::atomic<int> known[64];
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return 152;
+  }
+  if (dev < 64 && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) {
+    (void)cudaGetLastError();
+    return 152;
+  }
+  if (dev < 64) known[dev].store(n, std::memory_order_relaxed);
+  return n;
 }
 
 // cudaFuncSetAttribute(fn, MaxDynamicSharedMemorySize, bytes) unless this

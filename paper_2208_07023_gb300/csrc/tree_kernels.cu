@@ -826,13 +826,14 @@ cudaError_t launch_predict(const float* X, int64_t n, int d, TreeArrays tr, int 
   };
   while (RB > 1 && smem(RB, true) > 48 * 1024) RB /= 2;
   // few rows: smaller tiles, on more SMs
-  while (RB > 1 && (n + 32 * RB - 1) / (32 * RB) < 152) RB /= 2;
+  const int n_sm = sm_count();
+  while (RB > 1 && (n + 32 * RB - 1) / (32 * RB) < n_sm) RB /= 2;
   // Rows are staged while 32 of them fit. A single tree walks a row about
   // once per level and gains little: in batches of more tiles than the SMs hold
   // its wide rows are read where they are (100,000 rows, staged and direct: 200
   // features 0.17 and 0.16 ms, 512 0.45 to 0.76 and 0.45, 601 2.4 and 0.75; but
   // 128 0.12 and 0.16, 5,000 rows of 601 0.16 and 0.28).
-  const bool few = (n + 31) / 32 <= 152 * (int64_t)(227 * 1024 / smem(1, true));
+  const bool few = (n + 31) / 32 <= n_sm * (int64_t)(227 * 1024 / smem(1, true));
   const size_t most = few || n_trees > 1 ? (size_t)kPredSmem : (size_t)(vec ? 24 : 56) * 1024;
   const bool staged = smem(1, true) <= most;
   const size_t sm = smem(RB, staged);
