@@ -63,3 +63,22 @@ def test_prediction_does_not_depend_on_the_tile(ctx, d, trees):
         c, _, lf = ctx.predict(f, wl.X[:n], want_leaf=True)
         assert np.array_equal(c, cls[:n]) and np.array_equal(lf, leaf[:n]), n
     f.free()
+
+
+@pytest.mark.parametrize("n,d", [(1, 1024), (3, 8), (5, 130), (9, 1001), (17, 1000), (63, 36),
+                                 (255, 1024), (257, 33), (1300, 60), (77903, 3)])
+def test_gather_of_few_and_many_rows(ctx, n, d):
+    """4 to 256 entries a block: a subset's scores are the oracle's."""
+    from paper_2208_07023_gb300 import binding as S
+    wl = W.gmm(max(2 * n, 64), d, 4, seed=d)
+    rng = np.random.default_rng(n)
+    idx = rng.choice(len(wl.X), n, replace=False).astype(np.int32)
+    pos = rng.uniform(-1, 1, (3, d)).astype(np.float32)
+    res, _ = ctx.evaluate_swarm(gpu_params(S, "gini", 4, 3, 0, 16), wl.X, pos, labels=wl.labels,
+                                sample_idx=idx, want_bins=True)
+    ref, _, _ = O.eval_swarm(oracle_params(O, "gini", 4, 3, 0, 16), wl.X, wl.labels, None,
+                             pos.astype(np.float64), idx=idx)
+    for g, r in zip(res, ref):
+        assert g["valid"] == r["valid"]
+        for k in ("bin", "n_left", "n_right", "q_num", "q_den") if r["valid"] else ():
+            assert g[k] == r[k], k
