@@ -448,10 +448,11 @@ T* ws_ptr(slm_ctx* c, Slot s) {
 }
 
 // Scoring buffers of A nodes (one batch): z, ranges, node and tile lists;
-// for MSE also the entries' fixed-point moments (pr.m1, pr.m2, pr.mscale).
+// for MSE also the entries' fixed-point moments (pr.m1, pr.m2, pr.mscale), and
+// in a search their rounded targets (pr.mq, pr.mnode).
 slm_status setup_scoring(slm_ctx* c, Problem& pr, int A,
                          const std::vector<NodeDesc>& nodes,
-                         const std::vector<WorkTile>& tiles, Swarm* sw) {
+                         const std::vector<WorkTile>& tiles, Swarm* sw, bool search = false) {
   CK(ensure(c, c->ws[S_CUR], sizeof(EvalRes) * (size_t)A * pr.Pp));
   CK(ensure(c, c->ws[S_ZMM], sizeof(int32_t) * 2 * (size_t)A * pr.Pp));
   CK(ensure(c, c->ws[S_Z], sizeof(float) * (size_t)pr.P * (size_t)(pr.Ez > 0 ? pr.Ez : 4)));
@@ -478,7 +479,7 @@ slm_status setup_scoring(slm_ctx* c, Problem& pr, int A,
     pr.mnode = nullptr;
     uint32_t* mq = nullptr;
     MseNode* mnode = nullptr;
-    if (!pr.w && c->class_hist) {  // scored from the rounded targets (mse_kernels.cu)
+    if (search && !pr.w && c->class_hist) {  // scored from them (mse_kernels.cu)
       CK(ensure(c, c->ws[S_MQ], sizeof(uint32_t) * ne));
       CK(ensure(c, c->ws[S_MNODE], sizeof(MseNode) * (size_t)A));
       pr.mq = mq = ws_ptr<uint32_t>(c, S_MQ);
@@ -505,7 +506,7 @@ slm_status setup_swarm(slm_ctx* c, Problem& pr, int A, int T, bool want_trace,
                        const std::vector<NodeDesc>& nodes,
                        const std::vector<WorkTile>& tiles, Swarm* sw) {
   Swarm s{};
-  if (slm_status st = setup_scoring(c, pr, A, nodes, tiles, &s)) return st;
+  if (slm_status st = setup_scoring(c, pr, A, nodes, tiles, &s, true)) return st;
   const size_t apd = (size_t)A * pr.Pp * pr.d;
   CK(ensure(c, c->ws[S_POS], sizeof(float) * apd));
   CK(ensure(c, c->ws[S_VEL], sizeof(float) * apd));
