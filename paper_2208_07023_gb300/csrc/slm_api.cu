@@ -1574,7 +1574,7 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
         }
       }
     }
-    if (grid == 0 && step_config(pr, -1, &cfg, blocks / A)) {
+    if (grid == 0 && proj_config(pr, A, blocks, c->n_sm, &cfg)) {
       CK(prepare_step(cfg));
       grid = step_grid(cfg, c->n_sm);
     }

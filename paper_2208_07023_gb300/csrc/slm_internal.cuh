@@ -321,7 +321,7 @@ cudaError_t launch_apso(const Problem& pr, const Swarm& sw, const NodeDesc* node
 // writes x_t to sw.pos, v_t to sw.vel and (slice 0) the gbest records. With
 // sw.node_step the histogram kernel has moved the swarm already: the positions
 // of t come from pos_prev. The gbest step of the last evaluation is left to
-// launch_move(t = T). Not folded (sh = -1): the positions are sw.pos. Then z
+// launch_move(t = T). Not folded (proj_config): the positions are sw.pos. Then z
 // and the ranges of every (block, slice), as k_project (the same fused
 // multiply-adds). runs[n_runs]: each CTA's blocks, a contiguous run in (node,
 // slice, block) order starting at block blk of (node, slice), count >= 1
@@ -339,9 +339,10 @@ struct StepConfig {
   size_t smem = 0;
 };
 bool step_ok(const Problem& pr);
-// Shape sh (0 .. 5) of the folded projection, or (sh = -1) the unfolded one
-// for nodes of about `blocks` blocks of 32 rows.
-bool step_config(const Problem& pr, int sh, StepConfig* c, int64_t blocks = 1 << 20);
+// Shape sh (0 .. 5) of the folded projection.
+bool step_config(const Problem& pr, int sh, StepConfig* c);
+// The unfolded one for A nodes of `blocks` blocks of 32 rows together.
+bool proj_config(const Problem& pr, int A, int64_t blocks, int n_sm, StepConfig* c);
 // Few particles (unfolded, slices of 8): k_project_few.
 bool few_config(const Problem& pr, StepConfig* c);
 cudaError_t launch_project_few(const StepConfig& c, const Problem& pr, const Swarm& sw,

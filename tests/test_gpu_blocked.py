@@ -1,10 +1,10 @@
 """The projection from blocked rows, not folded (the default where a batch is
 long, has more nodes than CTAs, runs adaptive PSO or a swarm that does not
 fold): the results of the row-major projection bit for bit. Swarm widths of
-every particles-per-thread variant, several slices, slices cut down because
-their positions would not fit, feature counts around the 16-feature chunks
-and odd ones, nodes smaller than a block, and levels of many small nodes
-(several warps sharing a block)."""
+every particles-per-thread variant in long batches, short ones (narrow slices), slices cut
+down because their positions would not fit, feature counts around the
+16-feature chunks and odd ones, nodes smaller than a block, and levels of many
+small nodes (several warps sharing a block)."""
 import numpy as np
 import pytest
 
@@ -30,6 +30,11 @@ def ctxs():
     (900, 1024, 70, False),   # slices cut to the positions' room
     (333, 300, 128, False),
     (31, 5, 80, False),       # less than one block
+    (3000, 130, 250, False), (9000, 12, 100, False), (20011, 40, 250, False),
+    # long: the fewest slices, of 5 to 8 particles a thread
+    (90001, 3, 65, False), (90001, 4, 90, False), (90003, 17, 100, False), (90000, 5, 128, False),
+    (90001, 3, 7, True), (90001, 5, 15, True), (70001, 3, 23, True), (70001, 3, 31, True),
+    (70001, 3, 39, True), (70003, 3, 47, True), (70001, 6, 55, True), (70001, 3, 63, True),
     (5000, 23, 7, True), (4097, 33, 15, True), (2500, 50, 23, True), (2500, 48, 31, True),
     (1200, 15, 39, True), (1200, 31, 47, True), (800, 64, 55, True), (4100, 12, 63, True),
 ])
@@ -60,6 +65,24 @@ def test_many_small_nodes_identical(ctxs, P, d):
     for k in ga:
         assert np.array_equal(ga[k], gb[k]), k
     assert (ga["kind"] == 1).sum() > 500
+
+
+@pytest.mark.parametrize("trees,n,P,d", [(2, 900, 72, 33), (5, 61, 100, 20), (17, 700, 250, 9),
+                                         (40, 2000, 96, 130), (300, 200, 100, 7)])
+def test_batches_of_short_nodes_identical(ctxs, trees, n, P, d):
+    """Up to a few blocks a warp: narrow slices of several nodes."""
+    from paper_2208_07023_gb300 import binding as S
+    a, b = ctxs
+    wl = W.gmm(n, d, 3, seed=P)
+    p = gpu_params(S, "gini", 3, P, 3, 64, min_leaf=2, max_depth=2, seed=2, n_trees=trees,
+                   bootstrap=True)
+    fa, fb = (c.train_tree(p, wl.X, labels=wl.labels) for c in (a, b))
+    for t in range(trees):
+        ga, gb = fa.export(t), fb.export(t)
+        for k in ga:
+            assert np.array_equal(ga[k], gb[k]), (t, k)
+    fa.free()
+    fb.free()
 
 
 @pytest.mark.parametrize("n,d,P,k", [
