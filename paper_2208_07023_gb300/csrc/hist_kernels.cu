@@ -1069,13 +1069,12 @@ size_t hist_cls_smem(const Problem& pr, int np) {
   return words * 4 + np * sizeof(float) * 5 * (size_t)hc_dvec(pr.d);
 }
 
-// Particles per CTA.
-int hist_np(const Problem& pr, int A) {
+}  // namespace
+
+int hist_cls_particles(const Problem& pr, int A) {
   if (pr.crit == SLM_MSE) return mse_np(pr, A);
   return (int64_t)A * pr.P >= kHcPairFrom && hist_cls_smem(pr, kHcMaxNP) <= kHcPairSmem ? kHcMaxNP : 1;
 }
-
-}  // namespace
 
 bool hist_cls_ok(const Problem& pr) {
   if (pr.B < 2 || pr.B > kThreads || hist_cls_smem(pr, 1) > 200 * 1024) return false;
@@ -1101,7 +1100,7 @@ cudaError_t prepare_hist_cls(const Problem& pr) {
 }
 
 int hist_cls_split(const Problem& pr, int A, int64_t max_len, int n_sm) {
-  const int np = hist_np(pr, A);
+  const int np = hist_cls_particles(pr, A);
   int per_sm = 1;
   if (occupancy(&per_sm, hist_cls_fn(pr, np), kThreads, hist_cls_smem(pr, np)) != cudaSuccess) {
     cudaGetLastError();
@@ -1120,7 +1119,7 @@ cudaError_t launch_hist_cls(const Problem& pr, const Swarm& sw, const NodeDesc* 
                             int S, int t, int do_update, const double* xtab, cudaStream_t st,
                             const int32_t* list) {
   if (A <= 0) return cudaSuccess;
-  const int np = hist_np(pr, A);  // particles per CTA
+  const int np = hist_cls_particles(pr, A);  // particles per CTA
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(A * S), (unsigned)((pr.P + np - 1) / np), 1);
   cfg.blockDim = dim3(kThreads, 1, 1);

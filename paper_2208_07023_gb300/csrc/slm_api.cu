@@ -1180,7 +1180,8 @@ cudaError_t graph_signature(cudaGraph_t g, std::vector<uint64_t>* sig) {
 // CTAs per (node, particle) of the cluster histogram kernel for a search's
 // FP32 pass: the one-wave rule of hist_split (tuning off), cached for the
 // shape (criterion, bins, classes, particles, multiplicities, log2 of the
-// largest node and of the node count), or tuned now: for every cluster size
+// largest node and of the node count, the kernel and its particles per CTA), or
+// tuned now: for every cluster size
 // the device can schedule (1..16, slices of at least 256 entries) the
 // batch is projected once with the search's tiles and histogrammed once
 // between events; the fastest is kept. The histogram pass only reads the
@@ -1203,7 +1204,8 @@ slm_status pick_split(slm_ctx* c, const Problem& pr, const Swarm& sw,
     return (int64_t)l;
   };
   const std::vector<int64_t> key{pr.crit, pr.B, pr.K, pr.P, pr.w != nullptr, lg(max_len),
-                                 lg((int64_t)nodes.size()), cls ? 1 : 0};
+                                 lg((int64_t)nodes.size()),
+                                 cls ? hist_cls_particles(pr, (int)nodes.size()) : 0};
   auto it = c->tuned_split.find(key);
   if (it != c->tuned_split.end()) {
     *S_out = it->second.S;

@@ -263,6 +263,8 @@ cudaError_t launch_hist_scan(const Problem& pr, const Swarm& sw,
 // 32-bit counters.
 bool hist_cls_ok(const Problem& pr);
 bool hist_cls_fits(const Problem& pr, int64_t max_len);
+// Particles that a CTA scores in a batch of A nodes.
+int hist_cls_particles(const Problem& pr, int A);
 cudaError_t prepare_hist_cls(const Problem& pr);
 int hist_cls_split(const Problem& pr, int A, int64_t max_len, int n_sm);
 cudaError_t launch_hist_cls(const Problem& pr, const Swarm& sw, const NodeDesc* nodes, int A,

@@ -251,3 +251,24 @@ def test_persistent_node_search_gives_the_same_trajectory(ctx, P, n, d):
         assert np.array_equal(a["gbest"].view(np.uint32), b["gbest"].view(np.uint32))
         assert (a["bin"], a["n_left"], a["iter_of_best"], a["particle"]) == \
             (b["bin"], b["n_left"], b["iter_of_best"], b["particle"])
+
+
+def test_histogram_clusters_tuned_apart_for_two_particles_per_block():
+    """9 and 14 nodes share a power of two; from 512 (node, particle) pairs on
+    a block scores two particles, so 432 and 672 pairs are tuned apart."""
+    from paper_2208_07023_gb300 import binding as S
+    wl = W.gmm(9001, 6, 3, seed=5)
+    c = context()
+    try:
+        c.set_small_nodes(0, 0)
+        launches = []
+        for trees in (9, 14, 14, 9, 9):
+            p = gpu_params(S, "gini", 3, 48, 2, 32, min_leaf=5, seed=3, max_depth=1,
+                           n_trees=trees, bootstrap=True)
+            n0 = c.launch_count()
+            c.train_tree(p, wl.X, labels=wl.labels).free()
+            launches.append(c.launch_count() - n0)
+        # (tuning launches the projection and the histogram of every candidate)
+        assert launches[1] > launches[2] and launches[0] > launches[3] == launches[4]
+    finally:
+        c.close()
