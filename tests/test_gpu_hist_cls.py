@@ -1,5 +1,6 @@
 """The latency-oriented histogram kernels (k_hist_cls for classification,
-k_hist_mse for regression; the defaults of FP32 searches) score exactly like
+k_hist_mse for weighted regression, k_mse_hist for unweighted; the defaults of
+FP32 searches) score exactly like
 the staged-copy kernel they replace there: identical traces, gbest, splits,
 trees and bagged forests for Gini, entropy and the squared error, class
 counts spanning every register-array width (2 .. 32), bin counts that are
@@ -108,11 +109,13 @@ def test_unfused_search_identical_with_both_histogram_kernels(ctxs):
     (5003, 16, 48, 256, False),   # the most bins, ragged slices
     (20000, 12, 64, 128, False),  # a cluster of slices per particle
     (37, 4, 16, 16, False),       # a node smaller than one 16-byte group per thread
-    (9000, 20, 40, 100, True),    # multiplicities (bagging)
+    (9000, 20, 40, 100, True),    # multiplicities (bagging: k_hist_mse)
+    (6000, 24, 32, 64, True), (5003, 16, 48, 256, True), (40000, 12, 64, 128, True),
+    (37, 4, 16, 16, True),
 ])
 def test_regression_identical_with_both_histogram_kernels(ctxs, n, d, P, B, weighted):
-    """The squared-error kernel (lane-private copies of the fixed-point bin
-    moments) scores exactly like the staged-copy counting-sort kernel."""
+    """The squared-error kernels (weighted: lane-private copies of the fixed-point
+    bin moments) score exactly like the staged-copy counting-sort kernel."""
     from paper_2208_07023_gb300 import binding as S
     a, b = ctxs
     wl = W.tanh_regression(n, d, seed=n % 89)
@@ -144,39 +147,45 @@ def test_regression_trees_identical_with_both_histogram_kernels(ctxs, bootstrap)
     fb.free()
 
 
-def test_bf16_regression_identical_with_both_histogram_kernels(ctxs):
+@pytest.mark.parametrize("weighted", [False, True])
+def test_bf16_regression_identical_with_both_histogram_kernels(ctxs, weighted):
     """The BF16 form's reduced pass (its last CTA per node selecting the top
-    k) and FP32 re-scoring pass on the squared-error kernel: the same search
+    k) and FP32 re-scoring pass on the squared-error kernels: the same search
     and tree as with the staged-copy kernel."""
     from paper_2208_07023_gb300 import binding as S
     a, b = ctxs
     wl = W.tanh_regression(20000, 32, seed=6)
     p = S.make_params("mse", 0, n_particles=64, n_iters=6, n_bins=128, min_leaf=5, seed=3,
-                      max_depth=6, proj=S.SLM_PROJ_BF16_TOPK, topk=8)
-    ra = a.node_split(p, wl.X, y=wl.y, node_uid=2, want_trace=True)
-    rb = b.node_split(p, wl.X, y=wl.y, node_uid=2, want_trace=True)
+                      max_depth=6, proj=S.SLM_PROJ_BF16_TOPK, topk=8, n_trees=2 if weighted else 1,
+                      bootstrap=weighted)
+    kw = dict(weights=np.arange(20000, dtype=np.uint32) % 3 + 1) if weighted else {}
+    ra = a.node_split(p, wl.X, y=wl.y, node_uid=2, want_trace=True, **kw)
+    rb = b.node_split(p, wl.X, y=wl.y, node_uid=2, want_trace=True, **kw)
     assert np.array_equal(ra["trace"], rb["trace"])
     assert np.array_equal(ra["gbest"], rb["gbest"])
     for k in ("bin", "loss", "n_left", "n_right", "particle", "iter_of_best"):
         assert ra[k] == rb[k], k
     fa = a.train_tree(p, wl.X, y=wl.y)
     fb = b.train_tree(p, wl.X, y=wl.y)
-    same_tree(fa, fb)
+    same_tree(fa, fb, p.n_trees)
     fa.free()
     fb.free()
 
 
-def test_regression_pairs_of_particles_per_block(ctxs):
-    """Wide regression levels (at least 4,096 node-particle pairs) score two
-    particles per block, here with an odd swarm (the last block one
-    particle): the same trees as the staged-copy kernel."""
+@pytest.mark.parametrize("weighted", [False, True])
+def test_regression_pairs_of_particles_per_block(ctxs, weighted):
+    """Wide levels of weighted regression (at least 4,096 node-particle pairs)
+    score two particles per block, here with an odd swarm (the last block one
+    particle): the same trees as the staged-copy kernel. (Unweighted levels
+    have a warp per particle.)"""
     from paper_2208_07023_gb300 import binding as S
     a, b = ctxs
     wl = W.tanh_regression(40000, 12, seed=9)
-    p = gpu_params(S, "mse", 0, 127, 3, 64, min_leaf=8, max_depth=8, seed=5)
+    p = gpu_params(S, "mse", 0, 127, 3, 64, min_leaf=8, max_depth=8, seed=5,
+                   n_trees=2 if weighted else 1, bootstrap=weighted)
     fa = a.train_tree(p, wl.X, y=wl.y)
     fb = b.train_tree(p, wl.X, y=wl.y)
-    same_tree(fa, fb)
+    same_tree(fa, fb, p.n_trees)
     g = fa.export(0)
     assert (g["kind"] == 1).sum() >= 64  # levels of 32+ nodes x 127 particles were scored
     fa.free()

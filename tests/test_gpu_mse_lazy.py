@@ -34,6 +34,9 @@ def _targets(kind, wl):
         y[len(y) // 2] = 3e6
     if kind == "offset":
         y = (y * np.float32(1e-3) + np.float32(500)).astype(np.float32)
+    if kind == "crowd":  # nearly all at the largest rounded target, 2^28 - 1
+        y = np.full_like(y, 0.4999999)
+        y[::1000] = -0.4999999
     if kind in ("inf", "-inf", "nan", "infs"):
         y[len(y) // 3] = {"-inf": -np.inf, "nan": np.nan}.get(kind, np.inf)
     if kind == "infs":
@@ -81,6 +84,32 @@ def test_targets_that_are_not_finite(ctxs, n, B, kind, warp):
     wl = W.tanh_regression(n, 6, seed=n % 83)
     p = gpu_params(S, "mse", 0, 19, 9, B, min_leaf=2, seed=3)
     _same_search(a, b, p, wl.X, _targets(kind, wl))
+
+
+# 250 particles: a CTA per particle as long as the node fits its counters
+@pytest.mark.parametrize("n,B,kind,S_want", [
+    (8188, 256, "plain", 1),   # the longest slice of 8 copies
+    (8189, 256, "plain", 1),   # 32 copies from here on
+    (20001, 200, "two", 1),
+    (30011, 100, "offset", 1),
+    (64996, 256, "plain", 1),  # the largest slice: 2,032 of 2,048 entries a copy
+    (64995, 32, "crowd", 1),   # and sums of the high words near 2^32 in one bin
+    (64996, 2, "crowd", 1),
+    (64997, 64, "outlier", 2),
+])
+def test_long_slices_identical_to_the_exact_histogram(ctxs, n, B, kind, S_want):
+    from paper_2208_07023_gb300 import binding as S
+    a, b = ctxs
+    a.set_small_nodes(0, 0)
+    wl = W.tanh_regression(n, 6, seed=n % 83)
+    X = wl.X
+    if kind == "crowd":  # one far row: the others share a bin
+        X = X.copy()
+        X[0] *= 1e4
+    p = gpu_params(S, "mse", 0, 250, 4, B, min_leaf=1, seed=3)
+    _same_search(a, b, p, X, _targets(kind, wl))
+    a.node_split(p, X, y=_targets(kind, wl), node_uid=8)
+    assert a.tuning_stats()["last_hist_cluster"] == S_want
 
 
 @pytest.mark.parametrize("d,P", [(6, 64), (400, 64), (400, 19)])
