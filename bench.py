@@ -114,8 +114,15 @@ def config_dict(name, cfg, wl, proj, topk, extra=None, args_launch=None):
     if args_launch is not None:
         d["search_loop_graphs"] = args_launch.graphs
         d["projection_tile_mode"] = args_launch.tiles
-        d["projection_staging"] = ("tensor-map tile copies (cp.async.bulk.tensor)"
-                                   if args_launch.tma == "on" else "per-thread cp.async")
+        if proj != "bf16" and args_launch.fused != "off" and ":" not in args_launch.tiles:
+            staging = "blocks of 32 rows, a ring of cp.async chunks per warp"
+        elif proj == "bf16":
+            staging = "bulk copies of tensor-core operands (cp.async.bulk)"
+        elif args_launch.tma == "on":
+            staging = "tensor-map tile copies (cp.async.bulk.tensor)"
+        else:
+            staging = "per-thread cp.async"
+        d["projection_staging"] = staging
     if extra:
         d.update(extra)
     return d
@@ -1090,12 +1097,12 @@ def main():
     ap.add_argument("--topk", type=int, default=8)
     ap.add_argument("--compare-fp32", action="store_true")
     ap.add_argument("--tma", choices=["on", "off"], default="on",
-                    help="FP32 projection staging: tensor-map tile copies (on) or "
-                         "per-thread asynchronous copies (off)")
+                    help="row-major FP32 projection (--fused off or forced tiles): rows by "
+                         "tensor-map tile copies (on) or per-thread asynchronous copies (off)")
     ap.add_argument("--fused", choices=["on", "always", "off"], default="on",
-                    help="plain FP32 searches: swarm move folded into the projection "
-                         "(two launches per iteration) where a level's projection is a "
-                         "few waves (on), wherever possible (always), or never (off)")
+                    help="FP32 searches: projected from blocked rows, a plain swarm's move "
+                         "folded in (two launches per iteration) in short batches (on) or "
+                         "wherever possible (always); or row-major, never folded (off)")
     ap.add_argument("--class-hist", choices=["on", "off"], default="on",
                     help="classification histograms: latency-oriented kernel (on) or the "
                          "staged-copy kernel (off)")
@@ -1121,8 +1128,8 @@ def main():
                     help="run each search's iteration loop as one CUDA graph launch "
                          "(default: the workload's setting, else off)")
     ap.add_argument("--tiles", default="auto",
-                    help="projection tiles: auto (tuned), fixed (16 particles, 2 CTAs/SM) "
-                         "or PG:CPS[:GATHER]")
+                    help="row-major projection tiles: auto (tuned), fixed (16 particles, 2 "
+                         "CTAs/SM) or PG:CPS[:GATHER] (which makes the projection row-major)")
     ap.add_argument("--ncu-case", action="store_true",
                     help="one root-node search with 3 iterations (small case for ncu)")
     args = ap.parse_args()

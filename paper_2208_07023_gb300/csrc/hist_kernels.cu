@@ -80,18 +80,11 @@ struct HcScratch {
 __host__ __device__ inline int hc_dvec(int d) { return (d + 3) & ~3; }
 
 // Words of the histogram region: the copies, or (reused by the BF16 form's
-// top-k selection) P scores and 2 P indices when those need more; a
-// multiple of 4.
+// top-k selection) P scores and P keys when those need more; a multiple of 4.
 __host__ __device__ inline int hc_words(int B, int K, int P) {
   const int copies = 4 * B * K;  // hc_copies(NP) of each of NP particles
   const int topk = (int)((sizeof(EvalRes) + 8) * P / 4);
   return ((copies > topk ? copies : topk) + 3) & ~3;
-}
-
-// A double's total order as an unsigned key (negative values below 0).
-__device__ __forceinline__ uint64_t hc_key(double x) {
-  const uint64_t u = (uint64_t)__double_as_longlong(x);
-  return (u >> 63) ? ~u : u | 0x8000000000000000ull;
 }
 
 __device__ __forceinline__ double xlogx_tab(const double* tab, uint32_t c) {
@@ -447,7 +440,7 @@ __global__ void __launch_bounds__(kThreads, NP == 1 ? 2 : 4)
           const uint64_t nden = (uint64_t)ntot * d_;
           return __float_as_uint(__fdiv_rn((float)(nden - n_), (float)nden));  // >= 0
         }
-        return hc_key(l_);
+        return loss_key(l_);
       };
       uint64_t key = edge_key(bn, bd, bl, bb);
       // the exact winner among this warp's lanes in `cand` (lane order =
@@ -754,7 +747,7 @@ __host__ __device__ inline int mse_particle_words(int B, int NP) {
   return kMseWords * mse_copies(NP) * (B + 1);
 }
 // 32-bit words of the CTA's counters, also the top-k selection's scratch
-// (P scores and 2 P ints), a multiple of 4.
+// (P scores and P keys), a multiple of 4.
 __host__ __device__ inline int mse_count_words(int B, int P, int NP) {
   const int cells = NP * mse_particle_words(B, NP);
   const int topk = (int)((sizeof(EvalRes) + 8) * P / 4);

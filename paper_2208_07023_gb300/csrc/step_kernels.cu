@@ -660,8 +660,9 @@ __global__ void __launch_bounds__(32 * (FOLD ? kFoldWarps : kProjWarps))
 // lane, eight features on their way while eight are multiplied), and a slice's
 // positions at one feature are two broadcast words. A warp takes two blocks
 // at a time. Bound by waiting for the rows: the FP32 re-scores of the BF16
-// form, 200,000 x 128 rows and 8 particles, take 33 us (102 MB; four blocks a
-// warp 36), by the row-major kernel (row tiles through shared memory) 39.
+// form, 200,000 x 128 rows and 8 particles (102 MB), take 33 us of an iteration
+// (24.8 captured by themselves; four blocks a warp 36), by the row-major kernel
+// (row tiles through shared memory) 39.
 constexpr int kFewWarps = 8, kFewP = 8, kFewF = 8;
 constexpr int kFewBlocks = 2;  // blocks of a warp
 
