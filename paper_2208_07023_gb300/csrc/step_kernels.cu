@@ -935,7 +935,11 @@ bool proj_config(const Problem& pr, int A, int64_t blocks, int n_sm, StepConfig*
   };
   fill_config(pr, proj_fn(QP, PB), QP, PB, kProjWarps, c);
   double best = 0.95 * estimate(*c);  // (a narrower slice has to be clearly faster)
-  for (int q = 1; q <= 8; ++q) {
+  // (with more pairs the blocks of one pair follow those of another, and the
+  // nodes of a tree's level differ in size: a 30,011 x 50 regression tree's
+  // level of some 250 nodes lost 5 us of 16 an iteration)
+  const bool few = 4 * (int64_t)A * c->slices <= step_grid(*c, n_sm);
+  for (int q = 1; few && q <= 8; ++q) {
     StepConfig n;
     if ((size_t)8 * q * pr.d * sizeof(float) > (size_t)kStepMaxPosBytes) break;
     fill_config(pr, proj_fn(q, 1), q, 1, kProjWarps, &n);
