@@ -913,20 +913,21 @@ int mse_copies_for(int64_t slice) { return slice <= kMseSliceFew ? 8 : 32; }
 // multiples of 4).
 int64_t mse_launch_slice(int64_t max_len, int S) { return (max_len + S - 1) / S + 4; }
 
-// The fewest slices that a node's counters take, and the most CTAs of a
-// cluster (of the larger kernel, C = 32, which is asked for the most).
+// The fewest slices that a node's counters take.
 int64_t mse_min_split(int64_t max_len) {
   return std::max<int64_t>(1, (max_len + kMseSlice - 5) / (kMseSlice - 4));
 }
-int mse_max_cluster(const Problem& pr) {
-  const void* f = mse_fn(32);
-  const size_t smem = mse_hist_smem(pr, 32);
+// Clusters of S CTAs of the kernel with C copies that run at once.
+int mse_clusters(const Problem& pr, int C, int S) {
+  const void* f = mse_fn(C);
+  const size_t smem = mse_hist_smem(pr, C);
   int n = 0;
-  if (allow_smem(f, (int)smem) || allow_cluster(f) || cluster_size(&n, f, kThreads, smem)) {
+  if (allow_smem(f, (int)smem) || allow_cluster(f) ||
+      active_clusters(&n, f, kThreads, smem, S)) {
     (void)cudaGetLastError();
-    n = 8;  // the portable size
+    return S <= 8 ? 1 : 0;  // (8: the portable size)
   }
-  return std::max(1, std::min(n, kMseMaxCluster));
+  return n;
 }
 
 }  // namespace
@@ -946,28 +947,28 @@ cudaError_t prepare_mse_lazy(const Problem& pr) {
 }
 
 bool mse_lazy_fits(const Problem& pr, int64_t max_len) {
-  return mse_min_split(max_len) <= mse_max_cluster(pr);
+  const int64_t S = mse_min_split(max_len);
+  return S <= kMseMaxCluster && mse_clusters(pr, 32, (int)S) > 0;
 }
 
-int mse_lazy_split(const Problem& pr, int A, int64_t max_len, int n_sm) {
-  // As many slices as one wave of CTAs takes, of at least 2048 entries. A wave
-  // is what fits on the SMs: three CTAs each by registers, two by shared memory
-  // from about 360 features on, with 256 bins of 32 copies (51 iterations of a
-  // node of 131,000 x 400 rows, P = 64: 9.87 ms with seven slices, a wave and a
-  // half, and 9.55 with four). First with the few copies of short slices, else
-  // with the many of long ones.
-  auto slices = [&](int C) {
-    int per_sm = 1;
-    if (occupancy(&per_sm, mse_fn(C), kThreads, mse_hist_smem(pr, C)) != cudaSuccess) {
-      (void)cudaGetLastError();
-      per_sm = 1;
-    }
-    const int64_t wave = (int64_t)per_sm * n_sm / ((int64_t)A * pr.P);
-    const int64_t S = std::min<int64_t>({wave, max_len / 2048, mse_max_cluster(pr)});
-    return (int)std::max<int64_t>(S, mse_min_split(max_len));
-  };
-  const int S = slices(8);
-  return mse_copies_for(mse_launch_slice(max_len, S)) == 8 ? S : slices(32);
+int mse_lazy_split(const Problem& pr, int A, int64_t max_len) {
+  // As many slices as one wave of clusters takes, since the last CTA's exact
+  // pass ends the launch: as many clusters as the device holds at once (of 7
+  // CTAs 59, of 6 74: 64 particles on 80,000 entries, 51 iterations, 2.08 ms
+  // with 7 slices and 1.78 with 6). Above 8 CTAs a cluster needs a quarter of
+  // them to spare (32 particles on 20,000 entries: 1.14 ms with 12 slices, of
+  // which 36 fit, and 0.96 with 9). Slices of at least 1,400 entries, above 8
+  // of 2,048 (4,597 entries, 16 particles: 0.83 ms with 3, 0.88 with 2; 2,500:
+  // 0.75 with one, 0.79 with 2).
+  const int64_t pairs = (int64_t)A * pr.P;
+  const int least = (int)mse_min_split(max_len);
+  int S = (int)std::min<int64_t>(8, max_len / 1400);
+  S = (int)std::max<int64_t>({least, S, std::min<int64_t>(kMseMaxCluster, max_len / 2048)});
+  for (; S > least; --S) {
+    const int64_t n = mse_clusters(pr, mse_copies_for(mse_launch_slice(max_len, S)), S);
+    if (S > 8 ? 3 * n >= 4 * pairs : n >= pairs) break;
+  }
+  return S;
 }
 
 cudaError_t launch_mse_lazy(const Problem& pr, const Swarm& sw, const NodeDesc* nodes, int A,

@@ -859,7 +859,7 @@ cudaError_t prepare_fast_hist(const Problem& pr) {
 }
 
 int fast_hist_split(const Problem& pr, int A, int64_t max_len, int n_sm) {
-  return mse_lazy_ok(pr) ? mse_lazy_split(pr, A, max_len, n_sm)
+  return mse_lazy_ok(pr) ? mse_lazy_split(pr, A, max_len)
                          : hist_cls_split(pr, A, max_len, n_sm);
 }
 
@@ -1615,7 +1615,7 @@ slm_status run_search(slm_ctx* c, const slm_params* p, Problem& pr_in,
         cp.S_large = fast_hist_split(pr, hp.n_large, hp.max_large, c->n_sm);
     }
     if (cp.on && mse_lazy_ok(pr))
-      S = mse_lazy_split(pr, A, max_len, c->n_sm);
+      S = mse_lazy_split(pr, A, max_len);
     else if (!bp.on && !hp.on &&
              (s = pick_split(c, pr, sw, nodes, (int)tiles.size(), tl, &S, cp.on ? &cp : nullptr)))
       return s;

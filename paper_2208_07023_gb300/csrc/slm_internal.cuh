@@ -278,7 +278,7 @@ cudaError_t launch_hist_cls(const Problem& pr, const Swarm& sw, const NodeDesc* 
 // list[] names, of at most mse_warp_max() entries).
 bool mse_lazy_ok(const Problem& pr);
 bool mse_lazy_fits(const Problem& pr, int64_t max_len);
-int mse_lazy_split(const Problem& pr, int A, int64_t max_len, int n_sm);
+int mse_lazy_split(const Problem& pr, int A, int64_t max_len);
 int mse_warp_max();
 cudaError_t prepare_mse_lazy(const Problem& pr);
 cudaError_t launch_mse_lazy(const Problem& pr, const Swarm& sw, const NodeDesc* nodes, int A,
@@ -609,14 +609,15 @@ cudaError_t launch_swarm_seed_init(const Problem& pr, const Swarm& sw, const Nod
 // Searches plan their launches again at every level; the runtime calls that
 // set a kernel's dynamic shared-memory limit or query its occupancy cost
 // microseconds each, so their results are kept: a limit is raised only when
-// a larger one is needed, an occupancy and a cluster size are queried once per
-// (kernel, block, shared memory) that gives a nonzero answer.
+// a larger one is needed, an occupancy is queried once per (kernel, block,
+// shared memory) that gives a nonzero answer, a number of clusters once.
 
 struct KernelAttrCache {
   std::mutex mu;
   std::map<std::pair<int, const void*>, int> smem;      // largest limit set
   std::map<std::pair<int, const void*>, bool> cluster;  // non-portable sizes allowed
-  std::map<std::tuple<int, const void*, int, size_t>, int> occ, cluster_size;
+  std::map<std::tuple<int, const void*, int, size_t>, int> occ;
+  std::map<std::tuple<int, const void*, int, size_t, int>, int> clusters;
 };
 
 inline KernelAttrCache& kernel_attr_cache() {
@@ -700,30 +701,39 @@ inline cudaError_t occupancy(int* per_sm, const void* fn, int threads, size_t sm
   return e;
 }
 
-// CTAs of the largest cluster of a kernel that the device can schedule
-// (cudaOccupancyMaxPotentialClusterSize), remembered per device. Sizes above 8
-// count once allow_cluster has allowed them.
-inline cudaError_t cluster_size(int* ctas, const void* fn, int threads, size_t smem) {
+// Clusters of `ctas` CTAs of a kernel that are resident at once on the device
+// (cudaOccupancyMaxActiveClusters: a cluster stays within a GPC, so this is
+// often less than the SMs' CTAs divided by the cluster's), remembered per
+// device; 0 where it cannot be scheduled. Sizes above 8 count once
+// allow_cluster has allowed them.
+inline cudaError_t active_clusters(int* n, const void* fn, int threads, size_t smem, int ctas) {
   int dev = 0;
   if (cudaError_t e = cudaGetDevice(&dev)) return e;
   KernelAttrCache& c = kernel_attr_cache();
-  const auto key = std::make_tuple(dev, fn, threads, smem);
+  const auto key = std::make_tuple(dev, fn, threads, smem, ctas);
   {
     std::lock_guard<std::mutex> g(c.mu);
-    const auto it = c.cluster_size.find(key);
-    if (it != c.cluster_size.end()) {
-      *ctas = it->second;
+    const auto it = c.clusters.find(key);
+    if (it != c.clusters.end()) {
+      *n = it->second;
       return cudaSuccess;
     }
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(16, 1, 1);
+  cfg.gridDim = dim3((unsigned)ctas, 1, 1);
   cfg.blockDim = dim3((unsigned)threads, 1, 1);
   cfg.dynamicSmemBytes = smem;
-  const cudaError_t e = cudaOccupancyMaxPotentialClusterSize(ctas, fn, &cfg);
-  if (e == cudaSuccess && *ctas > 0) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)ctas;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaOccupancyMaxActiveClusters(n, fn, &cfg);
+  if (e == cudaSuccess) {
     std::lock_guard<std::mutex> g(c.mu);
-    c.cluster_size[key] = *ctas;
+    c.clusters[key] = *n;
   }
   return e;
 }
