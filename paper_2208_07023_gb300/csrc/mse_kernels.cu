@@ -958,11 +958,11 @@ int mse_lazy_split(const Problem& pr, int A, int64_t max_len) {
   // with 7 slices and 1.78 with 6). Above 8 CTAs a cluster needs a quarter of
   // them to spare (32 particles on 20,000 entries: 1.14 ms with 12 slices, of
   // which 36 fit, and 0.96 with 9). Slices of at least 1,400 entries, above 8
-  // of 2,048 (4,597 entries, 16 particles: 0.83 ms with 3, 0.88 with 2; 2,500:
-  // 0.75 with one, 0.79 with 2).
+  // of 2,048; two short ones never pay (4,597 entries, 16 particles: 0.83 ms
+  // with 3, 0.88 with 2; 3,732: 0.79 with one, 0.82 with 2).
   const int64_t pairs = (int64_t)A * pr.P;
   const int least = (int)mse_min_split(max_len);
-  int S = (int)std::min<int64_t>(8, max_len / 1400);
+  int S = max_len < 3 * 1400 ? 1 : (int)std::min<int64_t>(8, max_len / 1400);
   S = (int)std::max<int64_t>({least, S, std::min<int64_t>(kMseMaxCluster, max_len / 2048)});
   for (; S > least; --S) {
     const int64_t n = mse_clusters(pr, mse_copies_for(mse_launch_slice(max_len, S)), S);
