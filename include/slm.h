@@ -542,8 +542,9 @@ slm_status slm_set_tuning(slm_ctx* ctx, int32_t on);
  * bound; 0 makes every wait give up at once: the kernel drains the copies in
  * flight, sets the error word and ends, and the call returns SLM_ETIMEOUT).
  * fail_alloc_after: the fail_alloc_after-th later growth of a library work
- * buffer fails as if the device were out of memory (SLM_ENOMEM; 0: never);
- * process-wide. Synchronises ctx's stream. SLM_EINVAL if
+ * buffer fails as if the device were out of memory (0: never; SLM_ENOMEM, or
+ * the fallback where the search can do without that buffer or the context can
+ * give back its blocked rows, see slm_set_fused_step); process-wide. Synchronises ctx's stream. SLM_EINVAL if
  * fail_alloc_after < 0. */
 slm_status slm_test_hooks(slm_ctx* ctx, int32_t first_wait_polls, int64_t fail_alloc_after);
 
